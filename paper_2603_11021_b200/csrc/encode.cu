@@ -18,19 +18,34 @@ namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr int kEncWarps = 8;               // vectors in flight per CTA, one warp each
+constexpr int kEncCtas = 3;                // CTAs per SM (24 warps)
 constexpr uint32_t kFlagSearchGaveUp = 4u; // LLVQ_FLAG_SEARCH_GAVE_UP
 
 constexpr int kMaxCand = 64;               // cosets re-scored in binary64 per search; more (massive ties) means all 8192 are
 
+// Units of the first stage of the search: costs and moves are whole numbers of 1 / kCostScale.  The largest rounding error
+// of a coordinate costs 1/4, i.e. 2046: the costs of four coordinates stay below 2^13.
+constexpr float kCostScale = 8184.f;
+// Two cosets whose first-stage costs differ by more than this are in the same order in exact arithmetic: a cost carries at
+// most 25 roundings of half a unit (24 coordinates and one move) and 0.1 from the binary32 errors, twice 12.6 is 25.2.
+constexpr uint32_t kCostMargin = 26u;
+constexpr uint32_t kParityCode = 0x7676u;  // a byte-permute selector XOR this trades places with the one of the other parity
+constexpr uint32_t kSelEven = 0x3244u;     // {high half of the first operand} stays high, low half zero; ^ kParityCode: moved low
+
 // Per-warp scratch of the lattice search.
 struct WarpTables {
-    float2 grp[2][4][64];   // [parity][group of 6 coordinates][bit pattern]: {sum of squared errors, smallest cost of
-                            //  moving one coordinate to its other neighbour; its sign bit = parity of the sum of z}
-    float e[24][4];         // squared rounding error of coordinate i for offset b = parity + 2 * codeword bit
-    float d[24][4];         // cost of moving it to the other neighbour: 1 - 2 |error|
-    uint8_t zp[24][4];      // z & 1
+    uint4 pk[24];           // [coordinate, octad by octad] offset b = 0, 2, 1, 3: cost | parity of z << 13 | cost of the other neighbour << 16
+    uint2 nib[2][6][16];    // [parity][4 coordinates][bit pattern n]: {cost | move << 16, parity code | move of pattern ~n << 16}
+    uint4 ent[16][7];       // [parity * 8 + x]: best costs {even sum of z | odd << 16} of octad patterns, 8 per octad (24 words of 28)
     uint32_t cand[kMaxCand];
     uint32_t ncand;
+    uint32_t pad[3];
+};
+
+// What the search needs of the Golay code, in shared memory.
+struct SearchTables {
+    GolayTrio trio;
+    uint2 adr[12][32];      // [j][lane] byte offsets into nib of the low and high nibble of octad pattern j of the 12 a lane scores
 };
 
 // sum of the values of lanes 0..23, added in lane order, one binary64 rounding per addition (every lane gets the sum)
@@ -42,14 +57,55 @@ __device__ __forceinline__ double seq_sum24(double v)
     return acc;
 }
 
-// Cost of coset (pi, codeword j) from the group tables, in units of 16 (binary32).
-__device__ __forceinline__ float coset_cost(const WarpTables& W, uint32_t c, uint32_t pi)
+// The j-th of the 12 octad patterns lane scores: the 24 patterns of (parity, x) are octad 0 a = 0..7, octad 1 b = 0..7,
+// octad 2 c = 0..7; lane < 16 takes the first 12 and lane + 16 the rest.
+__device__ __forceinline__ void lane_pattern(int j, int lane, int& octad, int& which)
 {
-    const float2 a0 = W.grp[pi][0][c & 63u], a1 = W.grp[pi][1][(c >> 6) & 63u], a2 = W.grp[pi][2][(c >> 12) & 63u], a3 = W.grp[pi][3][c >> 18];
-    float cost = (a0.x + a1.x) + (a2.x + a3.x);
-    const uint32_t par = (__float_as_uint(a0.y) ^ __float_as_uint(a1.y) ^ __float_as_uint(a2.y) ^ __float_as_uint(a3.y)) >> 31;
-    if (par != pi) cost += fminf(fminf(fabsf(a0.y), fabsf(a1.y)), fminf(fabsf(a2.y), fabsf(a3.y)));
-    return cost;
+    const int t = 12 * (lane >> 4) + j;
+    octad = t >> 3;
+    which = t & 7;
+}
+
+__device__ __forceinline__ uint32_t lds32(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+
+__device__ __forceinline__ uint2 lds64(uint32_t a)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+
+// The point of coset (pi, codeword c) nearest to u (one coordinate per lane) in binary64, one rounding per operation: the
+// rounded z, with the first coordinate of largest error moved to its other neighbour if the sum rule fails.  alone = no
+// other point of the coset comes within 2e-6 of its rounding errors.
+__device__ __forceinline__ int coset_point(double u, uint32_t c, int pi, int lane, bool& alone)
+{
+    const bool mine = lane < 24;
+    const int b = pi + 2 * (int)((c >> lane) & 1u);
+    const double tt = __dmul_rn(__dsub_rn(u, (double)b), 0.25);
+    const double z = rint(tt);
+    const double err = __dsub_rn(tt, z), mag = fabs(err);
+    int x = mine ? b + 4 * (int)z : 0;
+    const int sum = __reduce_add_sync(kFull, x);
+    if ((sum & 7) != (pi ? 4 : 0)) {
+        // the first coordinate with the largest |error| moves by 4 (binary64 magnitudes compare like their bit patterns)
+        const unsigned long long key = mine ? (unsigned long long)__double_as_longlong(mag) : 0ull;
+        const uint32_t top = __reduce_max_sync(kFull, (uint32_t)(key >> 32));
+        const bool in_top = mine && (uint32_t)(key >> 32) == top;
+        const uint32_t low = __reduce_max_sync(kFull, in_top ? (uint32_t)key : 0u);
+        const int who = __ffs(__ballot_sync(kFull, in_top && (uint32_t)key == low)) - 1;
+        const double largest = __longlong_as_double((long long)((unsigned long long)top << 32 | low));
+        alone = __popc(__ballot_sync(kFull, mine && mag > largest - 1.0e-6)) == 1;
+        if (lane == who) x += err > 0.0 ? 4 : (err < 0.0 ? -4 : 4);
+    } else {
+        alone = __all_sync(kFull, !mine || mag < 0.5 - 1.0e-6);
+    }
+    return x;
 }
 
 // Nearest point of the unbounded lattice to u (one coordinate per lane, lanes 0..23; all in units of the integer
@@ -57,100 +113,161 @@ __device__ __forceinline__ float coset_cost(const WarpTables& W, uint32_t c, uin
 // (mod 2) (the sum rules of Sec. 2.4: all Golay weights are multiples of 4).  For each of the 2 x 4096 cosets the
 // best z is the rounded one, with the coordinate of largest rounding error moved to its other neighbour when the
 // sum rule fails.
-// Two stages.  A binary32 scan of all cosets through tables per group of 6 coordinates (4 reads and about 20
-// instructions per coset) finds the smallest cost; every coset whose binary32 cost is within 2^-12 (+ 2^-13 of the
-// cost) of it -- far more than the binary32 scan can err, costs are at most 1 -- is then evaluated again in binary64,
-// coordinate by coordinate in lane order, one rounding per operation: its point, and the squared distance as the sum
-// over the coordinates in order.  The smallest distance wins, the lowest (parity, codeword position) among equal ones;
+// Two stages.  The first finds the smallest cost over all cosets in whole numbers, along a trio of octads (GolayTrio): per
+// parity and octad pattern {w, ~w} the best cost for an even and for an odd sum of z (a move included where the rounded z has
+// the other parity), packed as two 16-bit halves; over the 512 triples those add up, the even and odd sums of three octads
+// combining to the parity the coset needs.  A minimum over the parities of the three octads never moves more than one
+// coordinate where one move is the better choice, so this is the minimum over the 8192 cosets.  A lane holds (parity, x,
+// half of the a): 32 pairs (a, b), three instructions each with the packed add-and-minimum of this architecture.
+// Every coset within kCostMargin of the smallest cost is then listed (usually one) and evaluated in binary64, coordinate by
+// coordinate in lane order, one rounding per operation: its point, and, if there are several, the squared distance as the
+// sum over the coordinates in order.  The smallest distance wins, the lowest (parity, codeword position) among equal ones;
 // inside a coset the first coordinate with the largest error moves.  The result does not depend on the first stage's
-// rounding.  Returns the coordinate of this lane (0 for lanes >= 24) and the squared norm of the point.
-__device__ int lattice_nearest(WarpTables& W, const uint32_t* __restrict__ golay_s, double u, int lane, int& norm2)
+// rounding.  Returns the coordinate of this lane (0 for lanes >= 24) and the squared norm of the point; unique = every other
+// lattice point is farther from u by a margin far above any binary64 rounding.
+// Bound: instruction issue (about 700 per search; scoring the 8192 cosets one by one took about 6000 and four times the
+// shared-memory traffic: encoding the 699 050 vectors of a 4096 x 4096 matrix took 38.9 ms instead of 2.1, indexing included).
+__device__ __forceinline__ int lattice_nearest(WarpTables& W, const SearchTables& S, const uint32_t* __restrict__ golay,
+                                               const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
 {
-    const float uf = (float)u;
+    const float uq = __shfl_sync(kFull, (float)u, lane < 24 ? S.trio.coord[lane] : lane);   // octad order
     if (lane < 24) {
+        uint32_t w[4];
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const float t = (uf - (float)b) * 0.25f;
+            const float t = (uq - (float)b) * 0.25f;
             const float z = rintf(t);
-            const float err = t - z;
-            W.e[lane][b] = err * err;
-            W.d[lane][b] = 1.f - 2.f * fabsf(err);
-            W.zp[lane][b] = (uint8_t)((int)z & 1);
+            const float err = fabsf(t - z);
+            w[b] = (uint32_t)__float2int_rn(err * err * kCostScale) | (uint32_t)__float2int_rn((1.f - 2.f * err) * kCostScale) << 16 |
+                   (uint32_t)((int)z & 1) << 13;
         }
+        W.pk[lane] = make_uint4(w[0], w[2], w[1], w[3]);
     }
     if (lane == 0) W.ncand = 0u;
     __syncwarp();
-    for (int q = 0; q < 16; ++q) {
-        const int id = q * 32 + lane, pi = id >> 8, g = (id >> 6) & 3, pat = id & 63;
-        float cost = 0.f, delta = 2.f;
-        uint32_t par = 0;
+    // tables per nibble of an octad: lane = (parity, bit pattern), one group of 4 coordinates after the other
+    {
+        const int pi = lane >> 4, n = lane & 15;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(&W.pk[0]) + 8u * (uint32_t)pi;
+        uint32_t a[4];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const int b = pi + 2 * ((pat >> k) & 1), i = 6 * g + k;
-            cost += W.e[i][b];
-            delta = fminf(delta, W.d[i][b]);
-            par ^= W.zp[i][b];
+        for (int k = 0; k < 4; ++k) a[k] = base + 16u * (uint32_t)k + 4u * (uint32_t)((n >> k) & 1);
+#pragma unroll
+        for (int g = 0; g < 6; ++g) {
+            uint32_t v[4], o[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { v[k] = lds32(a[k] + 64u * g); o[k] = lds32((a[k] ^ 4u) + 64u * g); }
+            const uint32_t sum = (v[0] + v[1]) + (v[2] + v[3]);
+            const uint32_t move = __vminu2(__vminu2(v[0], v[1]), __vminu2(v[2], v[3]));
+            const uint32_t move_c = __vminu2(__vminu2(o[0], o[1]), __vminu2(o[2], o[3]));
+            const uint32_t code = ((sum >> 13) & 1u) * kParityCode;
+            W.nib[pi][g][n] = make_uint2((sum & 0x1fffu) | (move & 0xffff0000u), code | (move_c & 0xffff0000u));
         }
-        W.grp[pi][g][pat] = make_float2(cost, __uint_as_float(__float_as_uint(delta) | par << 31));
     }
     __syncwarp();
-    float best = 3.0e38f;
-    for (int s = 0; s < 128; ++s) {
-        const uint32_t c = golay_s[s * 32 + lane];
-        best = fminf(best, fminf(coset_cost(W, c, 0u), coset_cost(W, c, 1u)));
+    // best costs of 12 octad patterns per lane
+    {
+        const uint32_t nib = (uint32_t)__cvta_generic_to_shared(&W.nib[0][0][0]);
+        const int pi = (lane >> 3) & 1;
+        uint32_t e[12], kd = 0u, qc = 0u;
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+            if (j == 0 || j == 4 || j == 8) {                  // the octad may change here: cost of a pattern + that of its complement, and parity between them
+                int octad, which;
+                lane_pattern(j, lane, octad, which);
+                const uint32_t t = nib + (uint32_t)((pi * 6 + 2 * octad) * 16) * 8u;
+                const uint2 l0 = lds64(t), l1 = lds64(t + 120u), h0 = lds64(t + 128u), h1 = lds64(t + 248u);
+                kd = ((l0.x + l1.x + h0.x + h1.x) & 0xffffu) * 0x10001u;
+                qc = l0.y ^ l1.y ^ h0.y ^ h1.y ^ (octad == 2 && pi ? kSelEven ^ kParityCode : kSelEven);
+            }
+            const uint2 at = S.adr[j][lane];
+            const uint2 lo = lds64(nib + at.x), hi = lds64(nib + at.y);
+            const uint32_t sel = lo.y ^ hi.y ^ (lane >= 16 && j >= 4 && pi ? kSelEven ^ kParityCode : kSelEven);   // (octad 2 of parity 1 is stored odd first)
+            const uint32_t cost = __byte_perm(lo.x + hi.x, 0u, 0x1010);
+            const uint32_t w = cost + __byte_perm(__vminu2(lo.x, hi.x), 0u, sel);
+            const uint32_t wc = kd - cost + __byte_perm(__vminu2(lo.y, hi.y), 0u, lo.y ^ hi.y ^ qc);
+            e[j] = __vminu2(w, wc);
+        }
+        uint4* out = &W.ent[lane & 15][3 * (lane >> 4)];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) out[j] = make_uint4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
     }
-    const float mine_best = best;                       // over this lane's 256 codewords
+    __syncwarp();
+    uint32_t best_a[4];
+    {
+        const uint4* in = W.ent[lane & 15];
+        const int h = lane >> 4;                                // this lane's half of the a
+        const uint4 va = in[h], vb0 = in[2], vb1 = in[3], vc0 = in[4 + h], vc1 = in[5 - h];
+        const uint32_t a[4] = {va.x, va.y, va.z, va.w};
+        const uint32_t b[8] = {vb0.x, vb0.y, vb0.z, vb0.w, vb1.x, vb1.y, vb1.z, vb1.w};
+        const uint32_t c[8] = {vc0.x, vc0.y, vc0.z, vc0.w, vc1.x, vc1.y, vc1.z, vc1.w};     // index ^ 4 h
 #pragma unroll
-    for (int o = 16; o; o >>= 1) best = fminf(best, __shfl_xor_sync(kFull, best, o));
-    const float thr = best + (1.f / 4096.f + best * (1.f / 8192.f));
-    // only the lanes whose own minimum is within the margin can hold candidates (usually one lane): the warp goes through
-    // the 256 codewords of each such lane together, 8 per lane
-    for (uint32_t holders = __ballot_sync(kFull, mine_best <= thr); holders; holders &= holders - 1u) {
-        const uint32_t owner = (uint32_t)__ffs(holders) - 1u;
+        for (int i = 0; i < 4; ++i) {
+            best_a[i] = 0xffffffffu;
+            const uint32_t ev = __byte_perm(a[i], 0u, 0x1010), od = __byte_perm(a[i], 0u, 0x3232);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t j = (uint32_t)((q * 32 + lane) * 32) + owner, c = golay_s[j];
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t two = __viaddmin_u16x2(od, __byte_perm(b[j], 0u, 0x1032), ev + b[j]);   // {even, odd} sum of two octads
+                best_a[i] = __viaddmin_u16x2(two, c[i ^ j], best_a[i]);
+            }
+            best_a[i] = min(best_a[i] & 0xffffu, best_a[i] >> 16);
+        }
+    }
+    const uint32_t best = __reduce_min_sync(kFull, min(min(best_a[0], best_a[1]), min(best_a[2], best_a[3])));
+    const uint32_t thr = best + kCostMargin;
+    // list the cosets within the margin: for every (parity, x, a) that holds one, the 64 codewords behind it, two per lane
+    for (int i = 0; i < 4; ++i) {
+        for (uint32_t holders = __ballot_sync(kFull, best_a[i] <= thr); holders; holders &= holders - 1u) {
+            const int owner = __ffs(holders) - 1;
+            const int pi = (owner >> 3) & 1, x = owner & 7, a = 4 * (owner >> 4) + i, b = lane & 7;
+            const uint32_t nib = (uint32_t)__cvta_generic_to_shared(&W.nib[pi][0][0]);
+            const uint32_t p0 = S.trio.pat[0][x * 8 + a] ^ (lane & 8 ? 255u : 0u), p1 = S.trio.pat[1][x * 8 + b] ^ (lane & 16 ? 255u : 0u);
+            uint32_t cost = 0, code = 0, move = 0xffffffffu;
 #pragma unroll
-            for (uint32_t pi = 0; pi < 2; ++pi) {
-                if (coset_cost(W, c, pi) <= thr) {
+            for (int g = 0; g < 4; ++g) {
+                const uint32_t p = g < 2 ? p0 : p1;
+                const uint2 v = lds64(nib + 128u * g + 8u * ((p >> (4 * (g & 1))) & 15u));
+                cost += v.x; code ^= v.y; move = __vminu2(move, v.x);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t p2 = S.trio.pat[2][x * 8 + (a ^ b)] ^ (e ? 255u : 0u);
+                const uint2 v4 = lds64(nib + 512u + 8u * (p2 & 15u)), v5 = lds64(nib + 640u + 8u * (p2 >> 4));
+                const uint32_t mv = __vminu2(move, __vminu2(v4.x, v5.x)) >> 16;
+                const bool odd = ((code ^ v4.y ^ v5.y) & 0xffffu) != 0u;
+                const uint32_t total = ((cost + v4.x + v5.x) & 0xffffu) + (odd != (pi != 0) ? mv : 0u);
+                if (total <= thr) {
                     const uint32_t slot = atomicAdd(&W.ncand, 1u);
-                    if (slot < (uint32_t)kMaxCand) W.cand[slot] = pi << 12 | j;
+                    const uint32_t c = (S.trio.word[0][x * 8 + a] ^ (lane & 8 ? S.trio.ones[0] : 0u)) |
+                                       (S.trio.word[1][x * 8 + b] ^ (lane & 16 ? S.trio.ones[1] : 0u)) |
+                                       (S.trio.word[2][x * 8 + (a ^ b)] ^ (e ? S.trio.ones[2] : 0u));
+                    if (slot < (uint32_t)kMaxCand) W.cand[slot] = (uint32_t)pi << 24 | c;
                 }
             }
         }
     }
     __syncwarp();
     const uint32_t listed = W.ncand;
-    const uint32_t n = listed > (uint32_t)kMaxCand ? 8192u : listed;          // too many near-ties to list: every coset
-    const bool mine = lane < 24;
-    double best_d2 = 1.0e300;
-    uint32_t best_id = 0xffffffffu;
-    int best_x = 0;
-    for (uint32_t t = 0; t < n; ++t) {
-        const uint32_t id = listed > (uint32_t)kMaxCand ? t : W.cand[t];
-        const int pi = (int)(id >> 12);
-        const uint32_t c = golay_s[id & 4095u];
-        const int b = pi + 2 * (int)((c >> (lane & 31)) & 1u);
-        const double tt = __dmul_rn(__dsub_rn(u, (double)b), 0.25);
-        const double z = rint(tt);
-        const double err = __dsub_rn(tt, z);
-        int x = mine ? b + 4 * (int)z : 0;
-        const int sum = __reduce_add_sync(kFull, x);
-        if ((((sum % 8) + 8) % 8) != (pi ? 4 : 0)) {
-            // the first coordinate with the largest |error| moves by 4 (binary64 magnitudes compare like their bit patterns)
-            unsigned long long key = mine ? (unsigned long long)__double_as_longlong(fabs(err)) : 0ull;
-            int who = lane;
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                const unsigned long long ok = __shfl_xor_sync(kFull, key, o);
-                const int ow = __shfl_xor_sync(kFull, who, o);
-                if (ok > key || (ok == key && ow < who)) { key = ok; who = ow; }
-            }
-            if (lane == who) x += err > 0.0 ? 4 : (err < 0.0 ? -4 : 4);
+    int best_x;
+    if (listed == 1u) {
+        const uint32_t k = W.cand[0];
+        best_x = coset_point(u, k & 0xffffffu, (int)(k >> 24), lane, unique);
+    } else {
+        unique = false;
+        const uint32_t n = listed > (uint32_t)kMaxCand ? 8192u : listed;      // too many near-ties to list: every coset
+        double best_d2 = 1.0e300;
+        uint32_t best_id = 0xffffffffu;
+        best_x = 0;
+        for (uint32_t t = 0; t < n; ++t) {
+            uint32_t id = t, c;
+            if (listed > (uint32_t)kMaxCand) c = __ldg(golay + (t & 4095u));
+            else { c = W.cand[t] & 0xffffffu; id = W.cand[t] >> 24 << 12 | __ldg(pos_by_low12 + (c & 0xfffu)); }
+            bool alone;
+            const int x = coset_point(u, c, (int)(id >> 12), lane, alone);
+            const double dd = __dsub_rn(u, (double)x);
+            const double d2 = seq_sum24(lane < 24 ? __dmul_rn(dd, dd) : 0.0);
+            if (d2 < best_d2 || (d2 == best_d2 && id < best_id)) { best_d2 = d2; best_id = id; best_x = x; }
         }
-        const double dd = __dsub_rn(u, (double)x);
-        const double d2 = seq_sum24(mine ? __dmul_rn(dd, dd) : 0.0);
-        if (d2 < best_d2 || (d2 == best_d2 && id < best_id)) { best_d2 = d2; best_id = id; best_x = x; }
     }
     norm2 = __reduce_add_sync(kFull, best_x * best_x);
     __syncwarp();
@@ -164,55 +281,98 @@ __device__ int lattice_nearest(WarpTables& W, const uint32_t* __restrict__ golay
 // the input (EUCLIDEAN) or with the largest cosine (ANGULAR) wins, the first radius on ties.  A zero input gives the
 // point of index 0, (4, 4, 0^22), the first point of the first class of Shell(2) (Sec. 2.3).  Needs m_lo == 2 and
 // m_hi >= 3 (checked on the host).
-__global__ void __launch_bounds__(kEncWarps * 32)
-encode_search_kernel(const uint32_t* __restrict__ golay, const float* __restrict__ v, uint64_t n, int metric, int m_lo, int m_hi,
+// EUCLIDEAN does not need all the radii.  At distance r along the direction d of the input (length R) the nearest point x
+// minimises |x|^2 - 2 r <x, d>; two minimisers at radii r < r' therefore satisfy <x, d> <= <x', d>, and
+// |x'|^2 - 2 R <x', d> <= |x|^2 - 2 R <x, d> for r < r' <= R (symmetrically for R <= r' < r): the radius next to R that yields a
+// point of the code beats all radii beyond it, by the margin that lattice_nearest reports as `unique`.  So the radii are tried
+// outwards from R, on each side until such a point is found (inputs so long that a squared distance no longer resolves the
+// margin try them all).  ANGULAR needs every radius; the exact score is formed only where a binary32 one comes near the best.
+__global__ void __launch_bounds__(kEncWarps * 32, kEncCtas)
+encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const float* __restrict__ v, uint64_t n, int metric, int m_lo, int m_hi,
                      int8_t* __restrict__ points, uint32_t* __restrict__ flags)
 {
     extern __shared__ __align__(16) uint8_t enc_smem[];
-    uint32_t* golay_s = reinterpret_cast<uint32_t*>(enc_smem);
-    WarpTables* tabs = reinterpret_cast<WarpTables*>(enc_smem + 4096 * 4);
-    for (int i = threadIdx.x; i < 4096; i += blockDim.x) golay_s[i] = __ldg(golay + i);
-    __syncthreads();
+    SearchTables& S = *reinterpret_cast<SearchTables*>(enc_smem);
+    WarpTables* tabs = reinterpret_cast<WarpTables*>(enc_smem + (sizeof(SearchTables) + 15) / 16 * 16);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < (int)sizeof(GolayTrio) / 4; i += blockDim.x)
+        reinterpret_cast<uint32_t*>(&S.trio)[i] = __ldg(reinterpret_cast<const uint32_t*>(et.trio) + i);
+    __syncthreads();
+    for (int j = warp; j < 12; j += kEncWarps) {
+        int octad, which;
+        lane_pattern(j, lane, octad, which);
+        const uint32_t p = S.trio.pat[octad][(lane & 7) * 8 + which], t = (uint32_t)((((lane >> 3) & 1) * 6 + 2 * octad) * 128);
+        S.adr[j][lane] = make_uint2(t + (p & 15u) * 8u, t + 128u + (p >> 4) * 8u);
+    }
+    __syncthreads();
     WarpTables& W = tabs[warp];
+    const double reach = sqrt(16.0 * (double)m_hi) + 4.01;
     for (uint64_t vec = (uint64_t)blockIdx.x * kEncWarps + warp; vec < n; vec += (uint64_t)gridDim.x * kEncWarps) {
-        const double vi = lane < 24 ? (double)__ldg(v + vec * 24 + lane) : 0.0;
-        const double n2 = seq_sum24(__dmul_rn(vi, vi));
+        const float vf = lane < 24 ? __ldg(v + vec * 24 + lane) : 0.f;
+        const double vi = (double)vf;
         int bestx = lane == 0 || lane == 1 ? 4 : 0;              // the point of index 0
         bool ok = false, direct = false;
-        const bool finite = n2 < 1.0e300;                        // false for NaN too
-        if (n2 == 0.0) {
+        const bool finite = __all_sync(kFull, isfinite(vf));
+        if (__all_sync(kFull, vf == 0.f)) {
             ok = direct = true;
         } else if (finite && metric == LLVQ_EUCLIDEAN) {
             // no lattice point is farther than 4 from any input (covering radius): beyond radius sqrt(16 m_hi) + 4 the nearest
             // point is certainly outside the code and the decode can be skipped
-            const double reach = sqrt(16.0 * (double)m_hi) + 4.01;
-            if (n2 <= reach * reach) {
+            float n2f = vf * vf;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) n2f += __shfl_xor_sync(kFull, n2f, o);
+            if (n2f <= (float)(reach * reach) + 0.01f) {
                 int norm2;
-                const int x = lattice_nearest(W, golay_s, vi, lane, norm2);
+                bool unique;
+                const int x = lattice_nearest(W, S, golay, et.pos_by_low12, vi, lane, norm2, unique);
                 const int m = norm2 / 16;
                 if (m >= m_lo && m <= m_hi) { ok = direct = true; bestx = x; }
             }
         }
         if (finite && !direct) {
+            const double n2 = seq_sum24(__dmul_rn(vi, vi));
             const double rn = __ddiv_rn(1.0, __dsqrt_rn(n2));
             double best = -1.0e300;
-            bool first = true;
-            for (int m = m_lo; m <= m_hi; ++m) {
+            float best_f = -2.f;
+            int best_m = 0;
+            const bool outwards = metric == LLVQ_EUCLIDEAN && n2 < 1.0e9;
+            // tried outwards: first down from the largest radius not above R, then up from the next one
+            const int m_start = outwards ? max(m_lo - 1, (int)fmin(n2 * 0.0625, (double)m_hi)) : m_hi;
+            int m = m_start, step = -1;
+            if (m < m_lo) { m = m_start + 1; step = 1; }
+            while (true) {
+                if (m < m_lo || m > m_hi) {
+                    if (step > 0 || m_start >= m_hi) break;
+                    m = m_start + 1; step = 1;
+                    continue;
+                }
                 const double rad = __dsqrt_rn(__dmul_rn(16.0, (double)m));
                 int norm2;
-                const int x = lattice_nearest(W, golay_s, __dmul_rn(__dmul_rn(vi, rn), rad), lane, norm2);
+                bool unique;
+                const int x = lattice_nearest(W, S, golay, et.pos_by_low12, __dmul_rn(__dmul_rn(vi, rn), rad), lane, norm2, unique);
                 const int mx = norm2 / 16;
+                const int m_now = m;
+                m += step;
                 if (mx < m_lo || mx > m_hi) continue;
                 double score;
                 if (metric == LLVQ_EUCLIDEAN) {
                     const double dd = __dsub_rn(vi, (double)x);
                     score = -seq_sum24(lane < 24 ? __dmul_rn(dd, dd) : 0.0);
                 } else {
+                    float s = (float)__dmul_rn(vi, rn) * (float)x;
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+                    s *= rsqrtf((float)norm2);
+                    if (s < best_f - 1.0e-5f) continue;          // binary32 errors stay below 3e-6
+                    best_f = fmaxf(best_f, s);
                     const double dot = seq_sum24(lane < 24 ? __dmul_rn(__dmul_rn(vi, rn), (double)x) : 0.0);
                     score = __ddiv_rn(dot, __dsqrt_rn((double)norm2));
                 }
-                if (first || score > best) { best = score; bestx = x; ok = true; first = false; }
+                if (!ok || score > best || (score == best && m_now < best_m)) { best = score; bestx = x; best_m = m_now; ok = true; }
+                if (outwards && unique) {
+                    if (step > 0 || m_start >= m_hi) break;
+                    m = m_start + 1; step = 1;
+                }
             }
         }
         if (!ok) {
@@ -376,11 +536,11 @@ int llvq_encode_blocks(const llvq_ctx* ctx, const float* d_v_f32, uint64_t nbloc
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t smem = 4096 * 4 + kEncWarps * sizeof(WarpTables);
+    const size_t smem = (sizeof(SearchTables) + 15) / 16 * 16 + kEncWarps * sizeof(WarpTables);
     if (cudaFuncSetAttribute(encode_search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return LLVQ_ECUDA;
     const uint64_t ctas = (nblocks + kEncWarps - 1) / kEncWarps;
-    const unsigned grid = (unsigned)std::min<uint64_t>(ctas, (uint64_t)ctx->sm_count * 4);
-    encode_search_kernel<<<grid, kEncWarps * 32, smem, st>>>(ctx->d_golay, d_v_f32, nblocks, metric, ctx->host.m_lo, ctx->host.m_hi,
+    const unsigned grid = (unsigned)std::min<uint64_t>(ctas, (uint64_t)ctx->sm_count * kEncCtas);
+    encode_search_kernel<<<grid, kEncWarps * 32, smem, st>>>(ctx->d_golay, ctx->enc, d_v_f32, nblocks, metric, ctx->host.m_lo, ctx->host.m_hi,
                                                             d_points, ctx->dev.flags);
     if (int e = status_of_launch()) return e;
     return launch_rank(ctx, d_points, nblocks, d_index, st);

@@ -108,6 +108,8 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
             slot = (uint16_t)j;
         }
     }
+    GolayTrio trio{};
+    if (ctx->can_encode) ctx->can_encode = build_golay_trio(h, trio);
     if (!ctx->can_encode) { hkeys.clear(); hcls.clear(); }
     uint64_t sigs[64];
     for (int a = 0; a < 64; ++a) sigs[a] = sig_of_value(a);
@@ -140,7 +142,8 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
         sort_rank.resize(ncls);
         for (uint32_t r = 0; r < ncls; ++r) sort_rank[order[r]] = (uint16_t)r;
     }
-    size_t o_cnt = up(o_srk + sort_rank.size() * 2);
+    size_t o_trio = up(o_srk + sort_rank.size() * 2);
+    size_t o_cnt = up(o_trio + sizeof trio);
     size_t o_scr = up(o_cnt + (size_t)(kCounterWords + 16) * 4 + 256);   // ... and the peers' description of a row-sharded GEMM   // one counter per group of 8 rows (GEMV) / per 128-row tile (GEMM), then the grid arrival counter
     static_assert(kPairSlotOffset == 64ll * kMaxScratchRows, "the pair slots start where the scratch rows end");
     size_t total = o_scr + (size_t)64 * kMaxScratchRows * (4 + 8);       // binary32 scratch rows, then one 64-bit pair slot per GEMV row
@@ -159,6 +162,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
         std::memcpy(blob.data() + o_hc, hcls.data(), hcls.size() * 4);
     }
     if (!sort_rank.empty()) std::memcpy(blob.data() + o_srk, sort_rank.data(), sort_rank.size() * 2);
+    std::memcpy(blob.data() + o_trio, &trio, sizeof trio);
     if (cudaMalloc(&ctx->d_blob, total) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
     if (cudaMemcpy(ctx->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(static_cast<uint8_t*>(ctx->d_blob) + o_cnt, 0, total - o_cnt) != cudaSuccess) {
@@ -181,6 +185,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     ctx->d_sort_rank = sort_rank.empty() ? nullptr : reinterpret_cast<const uint16_t*>(d + o_srk);
     ctx->enc.pos_by_low12 = reinterpret_cast<const uint16_t*>(d + o_p12);
     ctx->enc.sig_of_value = reinterpret_cast<const uint64_t*>(d + o_sig);
+    ctx->enc.trio = reinterpret_cast<const GolayTrio*>(d + o_trio);
     ctx->enc.hash_key = reinterpret_cast<const uint64_t*>(d + o_hk);
     ctx->enc.hash_cls = reinterpret_cast<const uint32_t*>(d + o_hc);
     ctx->enc.hash_mask = hkeys.empty() ? 0u : (uint32_t)(hkeys.size() - 1);

@@ -156,4 +156,16 @@ void build_bucket_table(const HostTables& t, std::vector<uint32_t>& lut);   // u
 uint64_t sig_of_value(int a);
 bool build_class_hash(const HostTables& t, std::vector<uint64_t>& keys, std::vector<uint32_t>& cls);
 
+// The Golay code cut along a trio of octads (three disjoint codewords of weight 8).  Restricted to one octad the codewords
+// are the 128 words of even weight, complementing a codeword on one octad gives another codeword, and up to complements
+// the code is { (s1[x, a], s2[x, b], s3[x, a ^ b]) : x, a, b = 0..7 }: 512 triples, each standing for 8 codewords
+// (Conway & Sloane, "Sphere Packings, Lattices and Groups", ch. 11: the Turyn construction).
+struct GolayTrio {
+    uint32_t word[3][64];   // [octad][x * 8 + a] the codeword's bits on the octad, as bits of the 24 coordinates
+    uint32_t ones[3];       // the octads
+    uint8_t pat[3][64];     // the same bits packed: bit p = coordinate coord[8 * octad + p]
+    uint8_t coord[24];      // coordinates octad by octad, ascending inside an octad
+};
+bool build_golay_trio(const HostTables& t, GolayTrio& out);
+
 }  // namespace llvq
