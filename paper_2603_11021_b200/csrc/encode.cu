@@ -17,35 +17,35 @@ using namespace llvq;
 namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
-constexpr int kEncWarps = 8;               // vectors in flight per CTA, one warp each
-constexpr int kEncCtas = 3;                // CTAs per SM (24 warps)
+constexpr int kEncWarps = 24;              // vectors in flight per CTA (one CTA per SM), one warp each
 constexpr uint32_t kFlagSearchGaveUp = 4u; // LLVQ_FLAG_SEARCH_GAVE_UP
 
+constexpr int kMaxShell = 53;              // llvq_create's limit
 constexpr int kMaxCand = 64;               // cosets re-scored in binary64 per search; more (massive ties) means all 8192 are
 
 // Units of the first stage of the search: costs and moves are whole numbers of 1 / kCostScale.  The largest rounding error
-// of a coordinate costs 1/4, i.e. 2046: the costs of four coordinates stay below 2^13.
+// of a coordinate costs 1/4, i.e. 2046: sixteen of them stay below 2^15.
 constexpr float kCostScale = 8184.f;
 // Two cosets whose first-stage costs differ by more than this are in the same order in exact arithmetic: a cost carries at
 // most 25 roundings of half a unit (24 coordinates and one move) and 0.1 from the binary32 errors, twice 12.6 is 25.2.
 constexpr uint32_t kCostMargin = 26u;
+constexpr uint32_t kParityBit = 0x8000u;   // where a cost carries the parity of its sum of z (adding costs adds the parities mod 2)
 constexpr uint32_t kParityCode = 0x7676u;  // a byte-permute selector XOR this trades places with the one of the other parity
 constexpr uint32_t kSelEven = 0x3244u;     // {high half of the first operand} stays high, low half zero; ^ kParityCode: moved low
 
 // Per-warp scratch of the lattice search.
-struct WarpTables {
-    uint4 pk[24];           // [coordinate, octad by octad] offset b = 0, 2, 1, 3: cost | parity of z << 13 | cost of the other neighbour << 16
-    uint2 nib[2][6][16];    // [parity][4 coordinates][bit pattern n]: {cost | move << 16, parity code | move of pattern ~n << 16}
-    uint4 ent[16][7];       // [parity * 8 + x]: best costs {even sum of z | odd << 16} of octad patterns, 8 per octad (24 words of 28)
-    uint32_t cand[kMaxCand];
+struct __align__(128) WarpTables {
+    uint2 nib[2][6][16];    // [parity][4 coordinates][bit pattern n]: {cost | move << 16, parity code | move of pattern ~n << 16}; rows of 128 bytes
+    uint4 pk[24][2];        // [coordinate, octad by octad][parity] w(b), w(b + 2), w(b + 2), w(b) for offset b = parity:
+                            //  w = cost | parity of z << 15 | cost of the other neighbour << 16
+    uint32_t cand[kMaxCand - 1];
     uint32_t ncand;
-    uint32_t pad[3];
 };
 
-// What the search needs of the Golay code, in shared memory.
-struct SearchTables {
-    GolayTrio trio;
-    uint2 adr[12][32];      // [j][lane] byte offsets into nib of the low and high nibble of octad pattern j of the 12 a lane scores
+// Nibbles of the octad patterns [octad][a = 1..3] (x = 0), times 8 (the row bytes of WarpTables::nib they select): patterns are
+// linear in (x, a), so the address of a pattern is that of (x, a & 4) XOR one of these.
+struct PatternSteps {
+    uint32_t lo[3][4], hi[3][4];
 };
 
 // sum of the values of lanes 0..23, added in lane order, one binary64 rounding per addition (every lane gets the sum)
@@ -57,28 +57,15 @@ __device__ __forceinline__ double seq_sum24(double v)
     return acc;
 }
 
-// The j-th of the 12 octad patterns lane scores: the 24 patterns of (parity, x) are octad 0 a = 0..7, octad 1 b = 0..7,
-// octad 2 c = 0..7; lane < 16 takes the first 12 and lane + 16 the rest.
-__device__ __forceinline__ void lane_pattern(int j, int lane, int& octad, int& which)
-{
-    const int t = 12 * (lane >> 4) + j;
-    octad = t >> 3;
-    which = t & 7;
-}
-
-__device__ __forceinline__ uint32_t lds32(uint32_t a)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
-
 __device__ __forceinline__ uint2 lds64(uint32_t a)
 {
     uint2 v;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
+
+// kParityCode where the parity carried by a cost is odd, else 0 (one multiply-high beside the mask)
+__device__ __forceinline__ uint32_t parity_code(uint32_t cost) { return __umulhi(cost & kParityBit, kParityCode << 17); }
 
 // The point of coset (pi, codeword c) nearest to u (one coordinate per lane) in binary64, one rounding per operation: the
 // rounded z, with the first coordinate of largest error moved to its other neighbour if the sum rule fails.  alone = no
@@ -125,89 +112,91 @@ __device__ __forceinline__ int coset_point(double u, uint32_t c, int pi, int lan
 // inside a coset the first coordinate with the largest error moves.  The result does not depend on the first stage's
 // rounding.  Returns the coordinate of this lane (0 for lanes >= 24) and the squared norm of the point; unique = every other
 // lattice point is farther from u by a margin far above any binary64 rounding.
-// Bound: instruction issue (about 700 per search; scoring the 8192 cosets one by one took about 6000 and four times the
-// shared-memory traffic: encoding the 699 050 vectors of a 4096 x 4096 matrix took 38.9 ms instead of 2.1, indexing included).
-__device__ __forceinline__ int lattice_nearest(WarpTables& W, const SearchTables& S, const uint32_t* __restrict__ golay,
-                                               const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
+// Bound: the integer / logic pipe (78 % busy, 818 instructions per decode; the shared-memory pipe is at 54 %).  Scoring the 8192
+// cosets one by one took about 6000 instructions and was bound by bank conflicts: 38.9 -> 1.13 ms for the 699 050 vectors of a
+// 4096 x 4096 matrix (EUCLIDEAN, indexing included), 32.0 -> 2.06 ms for the 174 763 of 1024 x 4096 (ANGULAR, 12 decodes each).
+// Steps on the way: rows of 128 bytes per (parity, nibble) read by the 16 lanes of one parity instead of rows shared by both
+// parities (1.38 -> 1.31 ms), roundings by additions instead of conversions and 24 warps drawing their vectors from a shared
+// counter instead of fixed strides (-> 1.13 ms).
+__device__ __forceinline__ int lattice_nearest(WarpTables& W, const GolayTrio& S, const PatternSteps& steps,
+                                               const uint32_t (&row)[6], const uint32_t* __restrict__ golay, const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
 {
-    const float uq = __shfl_sync(kFull, (float)u, lane < 24 ? S.trio.coord[lane] : lane);   // octad order
+    const float uq = __shfl_sync(kFull, (float)u, lane < 24 ? S.coord[lane] : lane);   // octad order
     if (lane < 24) {
         uint32_t w[4];
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const float t = (uq - (float)b) * 0.25f;
-            const float z = rintf(t);
-            const float err = fabsf(t - z);
-            w[b] = (uint32_t)__float2int_rn(err * err * kCostScale) | (uint32_t)__float2int_rn((1.f - 2.f * err) * kCostScale) << 16 |
-                   (uint32_t)((int)z & 1) << 13;
+            // rounding by adding 1.5 * 2^23 (the parity of z is then the last bit), whole numbers from adding 2^23: no conversions
+            const float t = (uq - (float)b) * 0.25f, tr = t + 12582912.f;
+            const float err = t - (tr - 12582912.f);
+            const float cost = fmaf(err * err, kCostScale, 8388608.f), move = fmaf(fabsf(err), -2.f * kCostScale, 8388608.f + kCostScale);
+            w[b] = __byte_perm(__float_as_uint(cost), __float_as_uint(move), 0x5410) | (__float_as_uint(tr) << 15 & kParityBit);
         }
-        W.pk[lane] = make_uint4(w[0], w[2], w[1], w[3]);
+        W.pk[lane][0] = make_uint4(w[0], w[2], w[2], w[0]);
+        W.pk[lane][1] = make_uint4(w[1], w[3], w[3], w[1]);
     }
     if (lane == 0) W.ncand = 0u;
     __syncwarp();
+    const int pi = lane >> 4;
+    uint32_t octad_sum[3];                                      // low half: cost of a pattern + that of its complement | parity between them << 15
     // tables per nibble of an octad: lane = (parity, bit pattern), one group of 4 coordinates after the other
     {
-        const int pi = lane >> 4, n = lane & 15;
-        const uint32_t base = (uint32_t)__cvta_generic_to_shared(&W.pk[0]) + 8u * (uint32_t)pi;
-        uint32_t a[4];
+        const int n = lane & 15;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(&W.pk[0][pi]);
+        uint32_t at[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) a[k] = base + 16u * (uint32_t)k + 4u * (uint32_t)((n >> k) & 1);
+        for (int k = 0; k < 4; ++k) at[k] = base + 32u * (uint32_t)k + 8u * (uint32_t)((n >> k) & 1);
 #pragma unroll
         for (int g = 0; g < 6; ++g) {
-            uint32_t v[4], o[4];
+            uint2 v[4];                                         // this pattern's and the complement's choice at each coordinate
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { v[k] = lds32(a[k] + 64u * g); o[k] = lds32((a[k] ^ 4u) + 64u * g); }
-            const uint32_t sum = (v[0] + v[1]) + (v[2] + v[3]);
-            const uint32_t move = __vminu2(__vminu2(v[0], v[1]), __vminu2(v[2], v[3]));
-            const uint32_t move_c = __vminu2(__vminu2(o[0], o[1]), __vminu2(o[2], o[3]));
-            const uint32_t code = ((sum >> 13) & 1u) * kParityCode;
-            W.nib[pi][g][n] = make_uint2((sum & 0x1fffu) | (move & 0xffff0000u), code | (move_c & 0xffff0000u));
+            for (int k = 0; k < 4; ++k) v[k] = lds64(at[k] + 128u * g);
+            const uint32_t sum = (v[0].x + v[1].x) + (v[2].x + v[3].x), sum_c = (v[0].y + v[1].y) + (v[2].y + v[3].y);
+            const uint32_t move = __vminu2(__vimin3_u16x2(v[0].x, v[1].x, v[2].x), v[3].x);
+            const uint32_t move_c = __vminu2(__vimin3_u16x2(v[0].y, v[1].y, v[2].y), v[3].y);
+            W.nib[pi][g][n] = make_uint2((sum & 0x7fffu) | (move & 0xffff0000u), parity_code(sum) | (move_c & 0xffff0000u));
+            octad_sum[g >> 1] = (g & 1 ? octad_sum[g >> 1] : 0u) + sum + sum_c;
         }
     }
     __syncwarp();
-    // best costs of 12 octad patterns per lane
-    {
-        const uint32_t nib = (uint32_t)__cvta_generic_to_shared(&W.nib[0][0][0]);
-        const int pi = (lane >> 3) & 1;
-        uint32_t e[12], kd = 0u, qc = 0u;
+    // best costs of octad patterns: lane = (parity, h, x) scores those with a, b, c = 4 h .. 4 h + 3.  The 16 lanes of a parity
+    // read one row of 128 bytes at a time: no bank conflicts
+    uint32_t e[3][4];
 #pragma unroll
-        for (int j = 0; j < 12; ++j) {
-            if (j == 0 || j == 4 || j == 8) {                  // the octad may change here: cost of a pattern + that of its complement, and parity between them
-                int octad, which;
-                lane_pattern(j, lane, octad, which);
-                const uint32_t t = nib + (uint32_t)((pi * 6 + 2 * octad) * 16) * 8u;
-                const uint2 l0 = lds64(t), l1 = lds64(t + 120u), h0 = lds64(t + 128u), h1 = lds64(t + 248u);
-                kd = ((l0.x + l1.x + h0.x + h1.x) & 0xffffu) * 0x10001u;
-                qc = l0.y ^ l1.y ^ h0.y ^ h1.y ^ (octad == 2 && pi ? kSelEven ^ kParityCode : kSelEven);
-            }
-            const uint2 at = S.adr[j][lane];
-            const uint2 lo = lds64(nib + at.x), hi = lds64(nib + at.y);
-            const uint32_t sel = lo.y ^ hi.y ^ (lane >= 16 && j >= 4 && pi ? kSelEven ^ kParityCode : kSelEven);   // (octad 2 of parity 1 is stored odd first)
+    for (int o = 0; o < 3; ++o) {
+        const uint32_t kd = __byte_perm(octad_sum[o] & 0x7fffu, 0u, 0x1010);
+        const uint32_t sel0 = o == 2 && pi ? kSelEven ^ kParityCode : kSelEven;      // octad 2 of parity 1 is kept odd half first
+        const uint32_t selc = parity_code(octad_sum[o]) ^ sel0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint2 lo = lds64(row[2 * o] ^ steps.lo[o][j]), hi = lds64(row[2 * o + 1] ^ steps.hi[o][j]);
             const uint32_t cost = __byte_perm(lo.x + hi.x, 0u, 0x1010);
-            const uint32_t w = cost + __byte_perm(__vminu2(lo.x, hi.x), 0u, sel);
-            const uint32_t wc = kd - cost + __byte_perm(__vminu2(lo.y, hi.y), 0u, lo.y ^ hi.y ^ qc);
-            e[j] = __vminu2(w, wc);
+            const uint32_t w = cost + __byte_perm(__vminu2(lo.x, hi.x), 0u, lo.y ^ hi.y ^ sel0);
+            const uint32_t wc = kd - cost + __byte_perm(__vminu2(lo.y, hi.y), 0u, lo.y ^ hi.y ^ selc);
+            e[o][j] = __vminu2(w, wc);
         }
-        uint4* out = &W.ent[lane & 15][3 * (lane >> 4)];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) out[j] = make_uint4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
     }
-    __syncwarp();
     uint32_t best_a[4];
     {
-        const uint4* in = W.ent[lane & 15];
-        const int h = lane >> 4;                                // this lane's half of the a
-        const uint4 va = in[h], vb0 = in[2], vb1 = in[3], vc0 = in[4 + h], vc1 = in[5 - h];
-        const uint32_t a[4] = {va.x, va.y, va.z, va.w};
-        const uint32_t b[8] = {vb0.x, vb0.y, vb0.z, vb0.w, vb1.x, vb1.y, vb1.z, vb1.w};
-        const uint32_t c[8] = {vc0.x, vc0.y, vc0.z, vc0.w, vc1.x, vc1.y, vc1.z, vc1.w};     // index ^ 4 h
+        // pairs (a, b) = (4 h + i, (4 h) ^ j): c = i ^ j.  The other half's b and c come from the lane that holds them
+        uint32_t b[8], c[8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            b[j] = e[1][j];
+            b[4 + j] = __shfl_xor_sync(kFull, e[1][j], 8);
+            c[j] = __shfl_sync(kFull, e[2][j], lane & ~8);
+            c[4 + j] = __shfl_sync(kFull, e[2][j], lane | 8);
+        }
+        uint32_t bs[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) bs[j] = __byte_perm(b[j], 0u, 0x1032);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             best_a[i] = 0xffffffffu;
-            const uint32_t ev = __byte_perm(a[i], 0u, 0x1010), od = __byte_perm(a[i], 0u, 0x3232);
+            const uint32_t ev = __byte_perm(e[0][i], 0u, 0x1010), od = __byte_perm(e[0][i], 0u, 0x3232);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint32_t two = __viaddmin_u16x2(od, __byte_perm(b[j], 0u, 0x1032), ev + b[j]);   // {even, odd} sum of two octads
+                const uint32_t two = __viaddmin_u16x2(od, bs[j], ev + b[j]);         // {even, odd} sum of two octads
                 best_a[i] = __viaddmin_u16x2(two, c[i ^ j], best_a[i]);
             }
             best_a[i] = min(best_a[i] & 0xffffu, best_a[i] >> 16);
@@ -219,9 +208,9 @@ __device__ __forceinline__ int lattice_nearest(WarpTables& W, const SearchTables
     for (int i = 0; i < 4; ++i) {
         for (uint32_t holders = __ballot_sync(kFull, best_a[i] <= thr); holders; holders &= holders - 1u) {
             const int owner = __ffs(holders) - 1;
-            const int pi = (owner >> 3) & 1, x = owner & 7, a = 4 * (owner >> 4) + i, b = lane & 7;
-            const uint32_t nib = (uint32_t)__cvta_generic_to_shared(&W.nib[pi][0][0]);
-            const uint32_t p0 = S.trio.pat[0][x * 8 + a] ^ (lane & 8 ? 255u : 0u), p1 = S.trio.pat[1][x * 8 + b] ^ (lane & 16 ? 255u : 0u);
+            const int po = owner >> 4, x = owner & 7, a = 4 * ((owner >> 3) & 1) + i, b = lane & 7;
+            const uint32_t nib = (uint32_t)__cvta_generic_to_shared(&W.nib[po][0][0]);
+            const uint32_t p0 = S.pat[0][x * 8 + a] ^ (lane & 8 ? 255u : 0u), p1 = S.pat[1][x * 8 + b] ^ (lane & 16 ? 255u : 0u);
             uint32_t cost = 0, code = 0, move = 0xffffffffu;
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
@@ -231,17 +220,17 @@ __device__ __forceinline__ int lattice_nearest(WarpTables& W, const SearchTables
             }
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const uint32_t p2 = S.trio.pat[2][x * 8 + (a ^ b)] ^ (e ? 255u : 0u);
+                const uint32_t p2 = S.pat[2][x * 8 + (a ^ b)] ^ (e ? 255u : 0u);
                 const uint2 v4 = lds64(nib + 512u + 8u * (p2 & 15u)), v5 = lds64(nib + 640u + 8u * (p2 >> 4));
                 const uint32_t mv = __vminu2(move, __vminu2(v4.x, v5.x)) >> 16;
                 const bool odd = ((code ^ v4.y ^ v5.y) & 0xffffu) != 0u;
-                const uint32_t total = ((cost + v4.x + v5.x) & 0xffffu) + (odd != (pi != 0) ? mv : 0u);
+                const uint32_t total = ((cost + v4.x + v5.x) & 0xffffu) + (odd != (po != 0) ? mv : 0u);
                 if (total <= thr) {
                     const uint32_t slot = atomicAdd(&W.ncand, 1u);
-                    const uint32_t c = (S.trio.word[0][x * 8 + a] ^ (lane & 8 ? S.trio.ones[0] : 0u)) |
-                                       (S.trio.word[1][x * 8 + b] ^ (lane & 16 ? S.trio.ones[1] : 0u)) |
-                                       (S.trio.word[2][x * 8 + (a ^ b)] ^ (e ? S.trio.ones[2] : 0u));
-                    if (slot < (uint32_t)kMaxCand) W.cand[slot] = (uint32_t)pi << 24 | c;
+                    const uint32_t c = (S.word[0][x * 8 + a] ^ (lane & 8 ? S.ones[0] : 0u)) |
+                                       (S.word[1][x * 8 + b] ^ (lane & 16 ? S.ones[1] : 0u)) |
+                                       (S.word[2][x * 8 + (a ^ b)] ^ (e ? S.ones[2] : 0u));
+                    if (slot < (uint32_t)(kMaxCand - 1)) W.cand[slot] = (uint32_t)po << 24 | c;
                 }
             }
         }
@@ -254,13 +243,13 @@ __device__ __forceinline__ int lattice_nearest(WarpTables& W, const SearchTables
         best_x = coset_point(u, k & 0xffffffu, (int)(k >> 24), lane, unique);
     } else {
         unique = false;
-        const uint32_t n = listed > (uint32_t)kMaxCand ? 8192u : listed;      // too many near-ties to list: every coset
+        const uint32_t n = listed > (uint32_t)(kMaxCand - 1) ? 8192u : listed;      // too many near-ties to list: every coset
         double best_d2 = 1.0e300;
         uint32_t best_id = 0xffffffffu;
         best_x = 0;
         for (uint32_t t = 0; t < n; ++t) {
             uint32_t id = t, c;
-            if (listed > (uint32_t)kMaxCand) c = __ldg(golay + (t & 4095u));
+            if (listed > (uint32_t)(kMaxCand - 1)) c = __ldg(golay + (t & 4095u));
             else { c = W.cand[t] & 0xffffffu; id = W.cand[t] >> 24 << 12 | __ldg(pos_by_low12 + (c & 0xfffu)); }
             bool alone;
             const int x = coset_point(u, c, (int)(id >> 12), lane, alone);
@@ -287,73 +276,84 @@ __device__ __forceinline__ int lattice_nearest(WarpTables& W, const SearchTables
 // point of the code beats all radii beyond it, by the margin that lattice_nearest reports as `unique`.  So the radii are tried
 // outwards from R, on each side until such a point is found (inputs so long that a squared distance no longer resolves the
 // margin try them all).  ANGULAR needs every radius; the exact score is formed only where a binary32 one comes near the best.
-__global__ void __launch_bounds__(kEncWarps * 32, kEncCtas)
-encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const float* __restrict__ v, uint64_t n, int metric, int m_lo, int m_hi,
+__global__ void __launch_bounds__(kEncWarps * 32, 1)
+encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __grid_constant__ PatternSteps steps, const float* __restrict__ v, uint64_t n, int metric, int m_lo, int m_hi,
                      int8_t* __restrict__ points, uint32_t* __restrict__ flags)
 {
-    extern __shared__ __align__(16) uint8_t enc_smem[];
-    SearchTables& S = *reinterpret_cast<SearchTables*>(enc_smem);
-    WarpTables* tabs = reinterpret_cast<WarpTables*>(enc_smem + (sizeof(SearchTables) + 15) / 16 * 16);
+    extern __shared__ __align__(128) uint8_t enc_smem[];
+    WarpTables* tabs = reinterpret_cast<WarpTables*>(enc_smem);
+    GolayTrio& S = *reinterpret_cast<GolayTrio*>(enc_smem + kEncWarps * sizeof(WarpTables));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double radius[kMaxShell + 1];                     // sqrt(16 m)
+    __shared__ uint32_t next_vec;
+    if (threadIdx.x == 0) next_vec = 0u;
+    for (int i = threadIdx.x; i <= m_hi; i += blockDim.x) radius[i] = __dsqrt_rn(__dmul_rn(16.0, (double)i));
     for (int i = threadIdx.x; i < (int)sizeof(GolayTrio) / 4; i += blockDim.x)
-        reinterpret_cast<uint32_t*>(&S.trio)[i] = __ldg(reinterpret_cast<const uint32_t*>(et.trio) + i);
-    __syncthreads();
-    for (int j = warp; j < 12; j += kEncWarps) {
-        int octad, which;
-        lane_pattern(j, lane, octad, which);
-        const uint32_t p = S.trio.pat[octad][(lane & 7) * 8 + which], t = (uint32_t)((((lane >> 3) & 1) * 6 + 2 * octad) * 128);
-        S.adr[j][lane] = make_uint2(t + (p & 15u) * 8u, t + 128u + (p >> 4) * 8u);
-    }
+        reinterpret_cast<uint32_t*>(&S)[i] = __ldg(reinterpret_cast<const uint32_t*>(et.trio) + i);
     __syncthreads();
     WarpTables& W = tabs[warp];
-    const double reach = sqrt(16.0 * (double)m_hi) + 4.01;
-    for (uint64_t vec = (uint64_t)blockIdx.x * kEncWarps + warp; vec < n; vec += (uint64_t)gridDim.x * kEncWarps) {
+    uint32_t row[6];                                             // where the nibbles of pattern (x, 4 h) of every octad are
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+        const uint32_t p = S.pat[o][(lane & 7) * 8 + ((lane >> 1) & 4)], t = (uint32_t)__cvta_generic_to_shared(&W.nib[lane >> 4][2 * o][0]);
+        row[2 * o] = t ^ (p & 15u) * 8u;
+        row[2 * o + 1] = (t + 128u) ^ (p >> 4) * 8u;
+    }
+    const float reach = sqrtf(16.f * (float)m_hi) + 4.01f, reach2 = reach * reach;
+    // a CTA's share is contiguous; its warps draw the vectors one by one (some take several decodes, and the schedulers favour some warps)
+    const uint64_t first = n / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, n % gridDim.x);
+    const uint32_t count = (uint32_t)(n / gridDim.x + (blockIdx.x < n % gridDim.x));
+    while (true) {
+        uint32_t t = 0;
+        if (lane == 0) t = atomicAdd(&next_vec, 1u);
+        t = __shfl_sync(kFull, t, 0);
+        if (t >= count) break;
+        const uint64_t vec = first + t;
         const float vf = lane < 24 ? __ldg(v + vec * 24 + lane) : 0.f;
         const double vi = (double)vf;
         int bestx = lane == 0 || lane == 1 ? 4 : 0;              // the point of index 0
-        bool ok = false, direct = false;
-        const bool finite = __all_sync(kFull, isfinite(vf));
-        if (__all_sync(kFull, vf == 0.f)) {
-            ok = direct = true;
-        } else if (finite && metric == LLVQ_EUCLIDEAN) {
-            // no lattice point is farther than 4 from any input (covering radius): beyond radius sqrt(16 m_hi) + 4 the nearest
-            // point is certainly outside the code and the decode can be skipped
-            float n2f = vf * vf;
+        const bool zero = __all_sync(kFull, vf == 0.f), finite = __all_sync(kFull, isfinite(vf));
+        bool ok = zero;
+        if (!zero && finite) {
+            bool direct = false;                                 // the input itself is decoded (else: its direction at shell radius m)
+            if (metric == LLVQ_EUCLIDEAN) {
+                // no lattice point is farther than 4 from any input (covering radius): beyond radius sqrt(16 m_hi) + 4 the nearest
+                // point is certainly outside the code and the decode can be skipped
+                float n2f = vf * vf;
 #pragma unroll
-            for (int o = 16; o; o >>= 1) n2f += __shfl_xor_sync(kFull, n2f, o);
-            if (n2f <= (float)(reach * reach) + 0.01f) {
+                for (int o = 16; o; o >>= 1) n2f += __shfl_xor_sync(kFull, n2f, o);
+                direct = n2f <= reach2;
+            }
+            double rn = 0.0, best = -1.0e300;
+            float best_f = -2.f;
+            int best_m = 0, m = 0, m_start = 0, step = 0;        // step 0: the radii have not been started
+            bool outwards = false;
+            while (true) {                                       // (one copy of the search in the code: two would not fit the instruction cache)
+                if (!direct) {
+                    if (step == 0) {
+                        const double n2 = seq_sum24(__dmul_rn(vi, vi));
+                        rn = __ddiv_rn(1.0, __dsqrt_rn(n2));
+                        outwards = metric == LLVQ_EUCLIDEAN && n2 < 1.0e9;
+                        // tried outwards: first down from the largest radius not above R, then up from the next one
+                        m = m_start = outwards ? max(m_lo - 1, (int)fmin(n2 * 0.0625, (double)m_hi)) : m_hi;
+                        step = -1;
+                    }
+                    if (step < 0 && m < m_lo) { m = m_start + 1; step = 1; }
+                    if (m > m_hi) break;
+                }
+                const double u = direct ? vi : __dmul_rn(__dmul_rn(vi, rn), radius[m]);
                 int norm2;
                 bool unique;
-                const int x = lattice_nearest(W, S, golay, et.pos_by_low12, vi, lane, norm2, unique);
-                const int m = norm2 / 16;
-                if (m >= m_lo && m <= m_hi) { ok = direct = true; bestx = x; }
-            }
-        }
-        if (finite && !direct) {
-            const double n2 = seq_sum24(__dmul_rn(vi, vi));
-            const double rn = __ddiv_rn(1.0, __dsqrt_rn(n2));
-            double best = -1.0e300;
-            float best_f = -2.f;
-            int best_m = 0;
-            const bool outwards = metric == LLVQ_EUCLIDEAN && n2 < 1.0e9;
-            // tried outwards: first down from the largest radius not above R, then up from the next one
-            const int m_start = outwards ? max(m_lo - 1, (int)fmin(n2 * 0.0625, (double)m_hi)) : m_hi;
-            int m = m_start, step = -1;
-            if (m < m_lo) { m = m_start + 1; step = 1; }
-            while (true) {
-                if (m < m_lo || m > m_hi) {
-                    if (step > 0 || m_start >= m_hi) break;
-                    m = m_start + 1; step = 1;
+                const int x = lattice_nearest(W, S, steps, row, golay, et.pos_by_low12, u, lane, norm2, unique);
+                const bool in_code = norm2 >= 16 * m_lo && norm2 < 16 * m_hi + 16;
+                if (direct) {
+                    if (in_code) { ok = true; bestx = x; break; }
+                    direct = false;
                     continue;
                 }
-                const double rad = __dsqrt_rn(__dmul_rn(16.0, (double)m));
-                int norm2;
-                bool unique;
-                const int x = lattice_nearest(W, S, golay, et.pos_by_low12, __dmul_rn(__dmul_rn(vi, rn), rad), lane, norm2, unique);
-                const int mx = norm2 / 16;
                 const int m_now = m;
                 m += step;
-                if (mx < m_lo || mx > m_hi) continue;
+                if (!in_code) continue;
                 double score;
                 if (metric == LLVQ_EUCLIDEAN) {
                     const double dd = __dsub_rn(vi, (double)x);
@@ -369,9 +369,9 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const flo
                     score = __ddiv_rn(dot, __dsqrt_rn((double)norm2));
                 }
                 if (!ok || score > best || (score == best && m_now < best_m)) { best = score; bestx = x; best_m = m_now; ok = true; }
-                if (outwards && unique) {
-                    if (step > 0 || m_start >= m_hi) break;
-                    m = m_start + 1; step = 1;
+                if (outwards && unique) {                        // this side is done
+                    if (step > 0) break;
+                    m = m_lo - 1;
                 }
             }
         }
@@ -536,11 +536,13 @@ int llvq_encode_blocks(const llvq_ctx* ctx, const float* d_v_f32, uint64_t nbloc
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t smem = (sizeof(SearchTables) + 15) / 16 * 16 + kEncWarps * sizeof(WarpTables);
+    const size_t smem = kEncWarps * sizeof(WarpTables) + sizeof(GolayTrio);
     if (cudaFuncSetAttribute(encode_search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return LLVQ_ECUDA;
-    const uint64_t ctas = (nblocks + kEncWarps - 1) / kEncWarps;
-    const unsigned grid = (unsigned)std::min<uint64_t>(ctas, (uint64_t)ctx->sm_count * kEncCtas);
-    encode_search_kernel<<<grid, kEncWarps * 32, smem, st>>>(ctx->d_golay, ctx->enc, d_v_f32, nblocks, metric, ctx->host.m_lo, ctx->host.m_hi,
+    PatternSteps steps;
+    for (int o = 0; o < 3; ++o)
+        for (int j = 0; j < 4; ++j) { steps.lo[o][j] = (ctx->trio.pat[o][j] & 15u) * 8u; steps.hi[o][j] = (uint32_t)(ctx->trio.pat[o][j] >> 4) * 8u; }
+    const unsigned grid = (unsigned)std::min<uint64_t>(nblocks, (uint64_t)ctx->sm_count);
+    encode_search_kernel<<<grid, kEncWarps * 32, smem, st>>>(ctx->d_golay, ctx->enc, steps, d_v_f32, nblocks, metric, ctx->host.m_lo, ctx->host.m_hi,
                                                             d_points, ctx->dev.flags);
     if (int e = status_of_launch()) return e;
     return launch_rank(ctx, d_points, nblocks, d_index, st);

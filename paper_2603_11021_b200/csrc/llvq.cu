@@ -108,7 +108,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
             slot = (uint16_t)j;
         }
     }
-    GolayTrio trio{};
+    GolayTrio& trio = ctx->trio;
     if (ctx->can_encode) ctx->can_encode = build_golay_trio(h, trio);
     if (!ctx->can_encode) { hkeys.clear(); hcls.clear(); }
     uint64_t sigs[64];

@@ -135,6 +135,40 @@ def test_encode_angular(lib, ctxs, codes, oracle_mod):
     assert lib.llvq_last_error(ctx) == (0, 0)
 
 
+def _edge_inputs(o, kind, n):
+    rng = np.random.default_rng(17)
+    pts = o.unrank([o.N // n * j + 11 * j for j in range(n)]).astype(np.float64)
+    if kind == "midpoints":                               # halfway between two points of the lattice: exact ties between cosets
+        return (pts + np.roll(pts, 1, axis=0)) / 2
+    if kind == "deep_holes":                              # (4, 0^23) is at distance 4 from 48 points: more ties than the list of candidates holds
+        pts[:, 3] += 4.0
+        return pts
+    if kind == "half_integers":                           # rounding ties inside a coset
+        return np.round(rng.standard_normal((n, 24)) * 5.0) / 2
+    if kind == "near_the_sphere":                         # lengths around every shell radius and across the edge of the ball
+        v = rng.standard_normal((n, 24))
+        r = np.sqrt(16.0 * 13) * (0.9 + 0.25 * np.arange(n) / n)
+        return v / np.linalg.norm(v, axis=1, keepdims=True) * r[:, None]
+    if kind == "lattice_directions":                      # scaled lattice points: the direction passes through points at several radii
+        return pts * (1.0 + 2.0 * np.arange(n) / n)[:, None]
+    # from far inside the smallest shell to lengths whose squares swamp the point.  The oracle decodes every input itself first and
+    # rounds its coordinates / 4 to 32-bit integers: |coordinate| < 2^33, i.e. below 1.4e9 for the 6 sigma a draw can reach
+    return rng.standard_normal((n, 24)) * np.logspace(-6, 9, n)[:, None]
+
+
+@pytest.mark.parametrize("metric", ["EUCLIDEAN", "ANGULAR"])
+@pytest.mark.parametrize("kind", ["midpoints", "deep_holes", "half_integers", "near_the_sphere", "lattice_directions", "all_lengths"])
+def test_encode_ties_and_edges_of_the_ball(lib, ctxs, codes, oracle_mod, kind, metric):
+    # where the search could differ from scoring all 8192 cosets at all radii: whole-number costs against ties, radii left out
+    o, ctx = codes[(2, 13)], ctxs[(2, 13)]
+    v = _edge_inputs(o, kind, 157).astype(np.float32)     # one more than the thread blocks of the grid can share evenly
+    pts_ref, idx_ref = o.encode(v.astype(np.float64), getattr(oracle_mod, metric), threads=4)
+    d_pts, d_idx = lib.llvq_encode_blocks(ctx, torch.from_numpy(v).cuda(), getattr(lib, "LLVQ_" + metric))
+    assert np.array_equal(d_pts.cpu().numpy(), pts_ref)
+    assert np.array_equal(_idx_np(d_idx), np.array(idx_ref, dtype=np.uint64))
+    lib.llvq_last_error(ctx)                              # inputs none of whose candidates lie in the code raise the gave-up flag on both sides
+
+
 def test_encode_non_finite_input_is_flagged(lib, ctxs):
     ctx = ctxs[(2, 13)]
     v = torch.zeros((3, 24), dtype=torch.float32, device="cuda")
