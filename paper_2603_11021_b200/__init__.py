@@ -2,17 +2,21 @@
 
 Argument marshalling only: every step of the dequantization path runs in the
 CUDA kernels of ``libllvq.so``.  PyTorch is used for device memory and streams.
+The calls that launch a product, a dequantization or an encoding go through the
+native module ``_native`` (``csrc/binding.cpp``), which checks the tensors and makes
+the output; load-time and multi-GPU calls go through ctypes.
 There is no CPU fallback: if the library is missing or the device is not a CUDA
 device, calls raise.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 
 import torch
 
-from .build import LIB
+from .build import LIB, NATIVE
 
 __all__ = [
     "Context", "llvq_decode_blocks", "llvq_dequant_matrix", "llvq_gemv", "llvq_gemm_small_batch", "llvq_gemm_small_batch_noalloc",
@@ -60,6 +64,7 @@ class LlvqError(RuntimeError):
 
 
 _lib = None
+_native = None      # set when the first context is made
 
 
 class GemvDesc(ctypes.Structure):
@@ -75,6 +80,8 @@ def load_library() -> ctypes.CDLL:
         return _lib
     if not os.path.exists(LIB):
         raise ImportError(f"{LIB} not found: run `python -m paper_2603_11021_b200.build` (needs nvcc); there is no fallback path")
+    if not os.path.exists(NATIVE):
+        raise ImportError(f"{NATIVE} not found: run `python -m paper_2603_11021_b200.build`; there is no fallback path")
     lib = ctypes.CDLL(LIB)
     vp, i64, u64 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_uint64
     lib.llvq_create.argtypes = [ctypes.POINTER(vp), ctypes.c_int, ctypes.c_int, ctypes.c_int]
@@ -145,6 +152,18 @@ def _stream_ptr(stream) -> int:
     return int(stream.cuda_stream)
 
 
+def _stream_arg(stream):
+    """What the native module takes: the stream's address, or None for PyTorch's current stream."""
+    return None if stream is None else int(stream.cuda_stream)
+
+
+def _out(call: str, r):
+    """The native module's answer: an output, or a status to raise."""
+    if type(r) is int:
+        raise LlvqError(call, r)
+    return r
+
+
 def _dev(t: torch.Tensor, name: str) -> int:
     if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous()):
         raise TypeError(f"{name} must be a contiguous CUDA tensor")
@@ -155,10 +174,15 @@ class Context:
     """Tables of the code  union of Shell(m), m_lo <= m <= m_hi,  on one CUDA device."""
 
     def __init__(self, m_lo: int, m_hi: int, device: int = 0):
+        global _native
         self._lib = load_library()
+        if _native is None:
+            _native = importlib.import_module(__name__ + "._native")
+        self._ptr = 0               # address of the llvq_ctx, for the native module
         h = ctypes.c_void_p()
         _check("llvq_create", self._lib.llvq_create(ctypes.byref(h), m_lo, m_hi, device))
         self._h = h
+        self._ptr = h.value
         self.device = device
         self.m_lo, self.m_hi = m_lo, m_hi
         self.index_bits = int(self._lib.llvq_index_bits(h))
@@ -196,6 +220,7 @@ class Context:
         if getattr(self, "_h", None):
             self._lib.llvq_destroy(self._h)
             self._h = None
+            self._ptr = 0
 
     def __del__(self):
         try:
@@ -206,49 +231,19 @@ class Context:
 
 def llvq_decode_blocks(ctx: Context, d_idx: torch.Tensor, nblocks: int, d_points: torch.Tensor | None = None, stream=None):
     """int8 [nblocks, 24] lattice points of the fields of the index stream ``d_idx`` (uint8, CUDA)."""
-    if d_points is None:
-        d_points = torch.empty((nblocks, 24), dtype=torch.int8, device=d_idx.device)
-    assert d_points.dtype == torch.int8 and d_points.numel() >= nblocks * 24
-    assert d_idx.numel() * d_idx.element_size() >= ctx.index_bytes(nblocks)
-    _check("llvq_decode_blocks", ctx._lib.llvq_decode_blocks(ctx._h, _dev(d_idx, "d_idx"), nblocks, _dev(d_points, "d_points"), _stream_ptr(stream)))
-    return d_points
+    return _out("llvq_decode_blocks", _native.decode(ctx._ptr, d_idx, nblocks, d_points, _stream_arg(stream)))
 
 
 def llvq_dequant_matrix(ctx: Context, d_idx: torch.Tensor, d_gain: torch.Tensor, rows: int, cols: int, layout: int,
                         d_w: torch.Tensor | None = None, ld: int | None = None, stream=None):
     """bf16 [rows, cols] dequantized weights; ``d_gain`` is float16 [nblocks]."""
-    ld = cols if ld is None else ld
-    if d_w is None:
-        d_w = torch.empty((rows, ld), dtype=torch.bfloat16, device=d_idx.device)
-    assert d_w.dtype == torch.bfloat16 and d_gain.dtype == torch.float16
-    nblocks = (rows * cols + 23) // 24 if layout == LLVQ_LAYOUT_FLAT else rows * ((cols + 23) // 24)
-    assert d_gain.numel() >= nblocks and d_idx.numel() * d_idx.element_size() >= ctx.index_bytes(nblocks)
-    assert d_w.numel() >= (rows - 1) * ld + cols if rows else True
-    _check("llvq_dequant_matrix", ctx._lib.llvq_dequant_matrix(
-        ctx._h, _dev(d_idx, "d_idx"), _dev(d_gain, "d_gain"), rows, cols, layout, _dev(d_w, "d_w"), ld, _stream_ptr(stream)))
-    return d_w
+    return _out("llvq_dequant_matrix", _native.dequant(ctx._ptr, d_idx, d_gain, rows, cols, layout, d_w, cols if ld is None else ld, _stream_arg(stream)))
 
 
 def llvq_gemv(ctx: Context, d_idx: torch.Tensor, d_gain: torch.Tensor, n_out: int, k_in: int, d_x: torch.Tensor,
               d_y: torch.Tensor | None = None, y_dtype: torch.dtype = torch.float32, stream=None):
     """y = W x with W given by (index stream, gains), ROWWISE blocks; x bf16 [k_in]; y float32 or bf16 [n_out]."""
-    if d_y is None:
-        d_y = torch.empty(n_out, dtype=y_dtype, device=d_idx.device)
-    assert d_x.dtype == torch.bfloat16 and d_x.numel() >= k_in and d_gain.dtype == torch.float16
-    assert d_y.dtype in (torch.float32, torch.bfloat16) and d_y.numel() >= n_out
-    nblocks = n_out * ((k_in + 23) // 24)
-    assert d_gain.numel() >= nblocks and d_idx.numel() * d_idx.element_size() >= ctx.index_bytes(nblocks)
-    code = LLVQ_F32 if d_y.dtype == torch.float32 else LLVQ_BF16
-    _check("llvq_gemv", ctx._lib.llvq_gemv(ctx._h, _dev(d_idx, "d_idx"), _dev(d_gain, "d_gain"), n_out, k_in,
-                                           _dev(d_x, "d_x"), _dev(d_y, "d_y"), code, _stream_ptr(stream)))
-    return d_y
-
-
-def _sg_args(ctx: Context, d_fields, gain_bits: int, d_codebook, d_row_scale, rows: int, nblocks: int):
-    assert d_codebook.dtype == torch.float32 and d_codebook.numel() >= (1 << gain_bits)
-    assert d_row_scale is None or (d_row_scale.dtype == torch.float32 and d_row_scale.numel() >= rows)
-    assert d_fields.numel() * d_fields.element_size() >= int(ctx._lib.llvq_field_bytes(ctx._h, nblocks, gain_bits))
-    return _dev(d_codebook, "d_codebook"), (None if d_row_scale is None else _dev(d_row_scale, "d_row_scale"))
+    return _out("llvq_gemv", _native.gemv(ctx._ptr, d_idx, d_gain, n_out, k_in, d_x, d_y, y_dtype, _stream_arg(stream), False))
 
 
 def llvq_dequant_matrix_sg(ctx: Context, d_fields: torch.Tensor, gain_bits: int, d_codebook: torch.Tensor,
@@ -256,60 +251,30 @@ def llvq_dequant_matrix_sg(ctx: Context, d_fields: torch.Tensor, gain_bits: int,
                            d_w: torch.Tensor | None = None, ld: int | None = None, stream=None):
     """bf16 [rows, cols] weights of the shape-gain form: (row_scale * codebook[k]) * x / |x|, ROWWISE fields
     (shape index | gain index << index_bits); ``d_row_scale`` may be None."""
-    ld = cols if ld is None else ld
-    if d_w is None:
-        d_w = torch.empty((rows, ld), dtype=torch.bfloat16, device=d_fields.device)
-    assert d_w.dtype == torch.bfloat16
-    assert d_w.numel() >= (rows - 1) * ld + cols if rows else True
-    cb, rs = _sg_args(ctx, d_fields, gain_bits, d_codebook, d_row_scale, rows, rows * ((cols + 23) // 24))
-    _check("llvq_dequant_matrix_sg", ctx._lib.llvq_dequant_matrix_sg(
-        ctx._h, _dev(d_fields, "d_fields"), gain_bits, cb, rs, rows, cols, _dev(d_w, "d_w"), ld, _stream_ptr(stream)))
-    return d_w
+    return _out("llvq_dequant_matrix_sg", _native.dequant_sg(ctx._ptr, d_fields, gain_bits, d_codebook, d_row_scale, rows, cols, d_w,
+                                                             cols if ld is None else ld, _stream_arg(stream)))
 
 
 def llvq_gemv_sg(ctx: Context, d_fields: torch.Tensor, gain_bits: int, d_codebook: torch.Tensor,
                  d_row_scale: torch.Tensor | None, n_out: int, k_in: int, d_x: torch.Tensor,
                  d_y: torch.Tensor | None = None, y_dtype: torch.dtype = torch.float32, stream=None):
     """y = W x with W in the shape-gain form of ``llvq_dequant_matrix_sg``."""
-    if d_y is None:
-        d_y = torch.empty(n_out, dtype=y_dtype, device=d_fields.device)
-    assert d_x.dtype == torch.bfloat16 and d_x.numel() >= k_in
-    assert d_y.dtype in (torch.float32, torch.bfloat16) and d_y.numel() >= n_out
-    cb, rs = _sg_args(ctx, d_fields, gain_bits, d_codebook, d_row_scale, n_out, n_out * ((k_in + 23) // 24))
-    code = LLVQ_F32 if d_y.dtype == torch.float32 else LLVQ_BF16
-    _check("llvq_gemv_sg", ctx._lib.llvq_gemv_sg(ctx._h, _dev(d_fields, "d_fields"), gain_bits, cb, rs, n_out, k_in,
-                                                 _dev(d_x, "d_x"), _dev(d_y, "d_y"), code, _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemv_sg", _native.gemv_sg(ctx._ptr, d_fields, gain_bits, d_codebook, d_row_scale, n_out, k_in, d_x, d_y, y_dtype,
+                                                _stream_arg(stream), False))
 
 
 def llvq_gemm_small_batch_sg(ctx: Context, d_fields: torch.Tensor, gain_bits: int, d_codebook: torch.Tensor,
                              d_row_scale: torch.Tensor | None, n_out: int, k_in: int, d_x: torch.Tensor,
                              d_y: torch.Tensor | None = None, stream=None):
     """Y[b, i] = sum_k X[b, k] W[i, k] with W in the shape-gain form of ``llvq_dequant_matrix_sg``; batch <= 64."""
-    assert d_x.dtype == torch.bfloat16 and d_x.dim() == 2 and d_x.shape[1] == k_in
-    batch = d_x.shape[0]
-    if d_y is None:
-        d_y = torch.empty((batch, n_out), dtype=torch.bfloat16, device=d_fields.device)
-    assert d_y.dtype == torch.bfloat16 and d_y.numel() >= batch * n_out
-    cb, rs = _sg_args(ctx, d_fields, gain_bits, d_codebook, d_row_scale, n_out, n_out * ((k_in + 23) // 24))
-    _check("llvq_gemm_small_batch_sg", ctx._lib.llvq_gemm_small_batch_sg(
-        ctx._h, _dev(d_fields, "d_fields"), gain_bits, cb, rs, n_out, k_in, _dev(d_x, "d_x"), batch, _dev(d_y, "d_y"), _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemm_small_batch_sg", _native.gemm_sg(ctx._ptr, d_fields, gain_bits, d_codebook, d_row_scale, n_out, k_in, d_x, d_y,
+                                                            _stream_arg(stream), False))
 
 
 def llvq_gemm_small_batch(ctx: Context, d_idx: torch.Tensor, d_gain: torch.Tensor, n_out: int, k_in: int,
                           d_x: torch.Tensor, d_y: torch.Tensor | None = None, stream=None):
     """Y[b, i] = sum_k X[b, k] W[i, k]; X bf16 [batch, k_in], Y bf16 [batch, n_out], batch <= 64."""
-    assert d_x.dtype == torch.bfloat16 and d_x.dim() == 2 and d_x.shape[1] == k_in and d_gain.dtype == torch.float16
-    batch = d_x.shape[0]
-    if d_y is None:
-        d_y = torch.empty((batch, n_out), dtype=torch.bfloat16, device=d_idx.device)
-    assert d_y.dtype == torch.bfloat16 and d_y.numel() >= batch * n_out
-    nblocks = n_out * ((k_in + 23) // 24)
-    assert d_gain.numel() >= nblocks and d_idx.numel() * d_idx.element_size() >= ctx.index_bytes(nblocks)
-    _check("llvq_gemm_small_batch", ctx._lib.llvq_gemm_small_batch(
-        ctx._h, _dev(d_idx, "d_idx"), _dev(d_gain, "d_gain"), n_out, k_in, _dev(d_x, "d_x"), batch, _dev(d_y, "d_y"), _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemm_small_batch", _native.gemm(ctx._ptr, d_idx, d_gain, n_out, k_in, d_x, d_y, _stream_arg(stream), 0))
 
 
 def llvq_gemm_small_batch_noalloc(ctx: Context, d_idx: torch.Tensor, d_gain: torch.Tensor, n_out: int, k_in: int,
@@ -318,12 +283,7 @@ def llvq_gemm_small_batch_noalloc(ctx: Context, d_idx: torch.Tensor, d_gain: tor
     library uses a fixed built-in scratch array instead of allocated memory, and this wrapper does not allocate
     either, so the output tensor ``d_y`` (bf16 [batch, n_out]) has to be passed in.  Sizes beyond the built-in
     array (see ``include/llvq.h``) raise ``LlvqError`` with LLVQ_EUNSUPPORTED.  Calls must not overlap on the GPU."""
-    assert d_x.dtype == torch.bfloat16 and d_x.dim() == 2 and d_x.shape[1] == k_in and d_gain.dtype == torch.float16
-    batch = d_x.shape[0]
-    assert d_y.dtype == torch.bfloat16 and d_y.numel() >= batch * n_out
-    _check("llvq_gemm_small_batch_noalloc", ctx._lib.llvq_gemm_small_batch_noalloc(
-        ctx._h, _dev(d_idx, "d_idx"), _dev(d_gain, "d_gain"), n_out, k_in, _dev(d_x, "d_x"), batch, _dev(d_y, "d_y"), _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemm_small_batch_noalloc", _native.gemm(ctx._ptr, d_idx, d_gain, n_out, k_in, d_x, d_y, _stream_arg(stream), 2))
 
 
 def llvq_sort_blocks(ctx: Context, d_idx: torch.Tensor, n_out: int, k_in: int, d_sorted: torch.Tensor | None = None, stream=None):
@@ -342,37 +302,18 @@ def llvq_sort_blocks(ctx: Context, d_idx: torch.Tensor, n_out: int, k_in: int, d
 def llvq_gemv_sorted(ctx: Context, d_sorted: torch.Tensor, d_gain: torch.Tensor, n_out: int, k_in: int, d_x: torch.Tensor,
                      d_y: torch.Tensor | None = None, y_dtype: torch.dtype = torch.float32, stream=None):
     """y = W x from the sorted stream of ``llvq_sort_blocks`` and the ROWWISE gains; same result as ``llvq_gemv``."""
-    if d_y is None:
-        d_y = torch.empty(n_out, dtype=y_dtype, device=d_sorted.device)
-    assert d_x.dtype == torch.bfloat16 and d_x.numel() >= k_in and d_gain.dtype == torch.float16
-    assert d_y.dtype in (torch.float32, torch.bfloat16) and d_y.numel() >= n_out
-    assert d_gain.numel() >= n_out * ((k_in + 23) // 24)
-    assert d_sorted.numel() * d_sorted.element_size() >= int(ctx._lib.llvq_sorted_bytes(ctx._h, n_out, k_in))
-    code = LLVQ_F32 if d_y.dtype == torch.float32 else LLVQ_BF16
-    _check("llvq_gemv_sorted", ctx._lib.llvq_gemv_sorted(ctx._h, _dev(d_sorted, "d_sorted"), _dev(d_gain, "d_gain"), n_out, k_in,
-                                                         _dev(d_x, "d_x"), _dev(d_y, "d_y"), code, _stream_ptr(stream)))
-    return d_y
-
-
-def _gemv_multi(call: str, ctx: Context, mats, y_dtype, stream):
-    descs = (GemvDesc * len(mats))()
-    for d, (d_w, d_gain, n_out, k_in, d_x, d_y) in zip(descs, mats):
-        assert d_x.dtype == torch.bfloat16 and d_x.numel() >= k_in and d_gain.dtype == torch.float16
-        assert d_y.dtype == y_dtype and d_y.numel() >= n_out and d_gain.numel() >= n_out * ((k_in + 23) // 24)
-        d.d_weights, d.d_gain_f16, d.n_out, d.k_in = _dev(d_w, "d_weights"), _dev(d_gain, "d_gain"), n_out, k_in
-        d.d_x_bf16, d.d_y = _dev(d_x, "d_x"), _dev(d_y, "d_y")
-    _check(call, getattr(ctx._lib, call)(ctx._h, descs, len(mats), LLVQ_F32 if y_dtype == torch.float32 else LLVQ_BF16, _stream_ptr(stream)))
+    return _out("llvq_gemv_sorted", _native.gemv(ctx._ptr, d_sorted, d_gain, n_out, k_in, d_x, d_y, y_dtype, _stream_arg(stream), True))
 
 
 def llvq_gemv_multi(ctx: Context, mats, y_dtype: torch.dtype = torch.float32, stream=None) -> None:
     """Up to 8 independent products in one launch.  mats: (d_idx, d_gain, n_out, k_in, d_x, d_y) per matrix, all device tensors
     owned by the caller (outputs included); no d_y may be a d_x of the same call."""
-    _gemv_multi("llvq_gemv_multi", ctx, mats, y_dtype, stream)
+    _check("llvq_gemv_multi", _native.gemv_multi(ctx._ptr, mats, y_dtype, _stream_arg(stream), False))
 
 
 def llvq_gemv_sorted_multi(ctx: Context, mats, y_dtype: torch.dtype = torch.float32, stream=None) -> None:
     """The same on streams made by ``llvq_sort_blocks``: (d_sorted, d_gain, n_out, k_in, d_x, d_y) per matrix."""
-    _gemv_multi("llvq_gemv_sorted_multi", ctx, mats, y_dtype, stream)
+    _check("llvq_gemv_sorted_multi", _native.gemv_multi(ctx._ptr, mats, y_dtype, _stream_arg(stream), True))
 
 
 def llvq_sort_blocks_sg(ctx: Context, d_fields: torch.Tensor, gain_bits: int, n_out: int, k_in: int,
@@ -394,18 +335,8 @@ def llvq_gemv_sorted_sg(ctx: Context, d_sorted: torch.Tensor, gain_bits: int, d_
                         d_row_scale: torch.Tensor | None, n_out: int, k_in: int, d_x: torch.Tensor,
                         d_y: torch.Tensor | None = None, y_dtype: torch.dtype = torch.float32, stream=None):
     """y = W x with W in the shape-gain form, from the sorted stream of ``llvq_sort_blocks_sg``; same result as ``llvq_gemv_sg``."""
-    if d_y is None:
-        d_y = torch.empty(n_out, dtype=y_dtype, device=d_sorted.device)
-    assert d_x.dtype == torch.bfloat16 and d_x.numel() >= k_in
-    assert d_y.dtype in (torch.float32, torch.bfloat16) and d_y.numel() >= n_out
-    assert d_codebook.dtype == torch.float32 and d_codebook.numel() >= (1 << gain_bits)
-    assert d_row_scale is None or (d_row_scale.dtype == torch.float32 and d_row_scale.numel() >= n_out)
-    assert d_sorted.numel() * d_sorted.element_size() >= int(ctx._lib.llvq_sorted_bytes(ctx._h, n_out, k_in))
-    code = LLVQ_F32 if d_y.dtype == torch.float32 else LLVQ_BF16
-    _check("llvq_gemv_sorted_sg", ctx._lib.llvq_gemv_sorted_sg(
-        ctx._h, _dev(d_sorted, "d_sorted"), gain_bits, _dev(d_codebook, "d_codebook"),
-        None if d_row_scale is None else _dev(d_row_scale, "d_row_scale"), n_out, k_in, _dev(d_x, "d_x"), _dev(d_y, "d_y"), code, _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemv_sorted_sg", _native.gemv_sg(ctx._ptr, d_sorted, gain_bits, d_codebook, d_row_scale, n_out, k_in, d_x, d_y, y_dtype,
+                                                       _stream_arg(stream), True))
 
 
 def llvq_sort_blocks_gemm(ctx: Context, d_idx: torch.Tensor, n_out: int, k_in: int, d_sorted: torch.Tensor | None = None, stream=None):
@@ -425,16 +356,7 @@ def llvq_sort_blocks_gemm(ctx: Context, d_idx: torch.Tensor, n_out: int, k_in: i
 def llvq_gemm_small_batch_sorted(ctx: Context, d_sorted: torch.Tensor, d_gain: torch.Tensor, n_out: int, k_in: int,
                                  d_x: torch.Tensor, d_y: torch.Tensor | None = None, stream=None):
     """Y[b, i] = sum_k X[b, k] W[i, k] from the sorted stream of ``llvq_sort_blocks_gemm``; same result as ``llvq_gemm_small_batch``."""
-    assert d_x.dtype == torch.bfloat16 and d_x.dim() == 2 and d_x.shape[1] == k_in and d_gain.dtype == torch.float16
-    batch = d_x.shape[0]
-    if d_y is None:
-        d_y = torch.empty((batch, n_out), dtype=torch.bfloat16, device=d_sorted.device)
-    assert d_y.dtype == torch.bfloat16 and d_y.numel() >= batch * n_out
-    assert d_gain.numel() >= n_out * ((k_in + 23) // 24)
-    assert d_sorted.numel() * d_sorted.element_size() >= int(ctx._lib.llvq_sorted_gemm_bytes(ctx._h, n_out, k_in))
-    _check("llvq_gemm_small_batch_sorted", ctx._lib.llvq_gemm_small_batch_sorted(
-        ctx._h, _dev(d_sorted, "d_sorted"), _dev(d_gain, "d_gain"), n_out, k_in, _dev(d_x, "d_x"), batch, _dev(d_y, "d_y"), _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemm_small_batch_sorted", _native.gemm(ctx._ptr, d_sorted, d_gain, n_out, k_in, d_x, d_y, _stream_arg(stream), 1))
 
 
 def llvq_sort_blocks_gemm_sg(ctx: Context, d_fields: torch.Tensor, gain_bits: int, n_out: int, k_in: int,
@@ -455,62 +377,26 @@ def llvq_gemm_small_batch_sorted_sg(ctx: Context, d_sorted: torch.Tensor, gain_b
                                     d_row_scale: torch.Tensor | None, n_out: int, k_in: int, d_x: torch.Tensor,
                                     d_y: torch.Tensor | None = None, stream=None):
     """``llvq_gemm_small_batch_sg`` from the sorted stream of ``llvq_sort_blocks_gemm_sg``."""
-    assert d_x.dtype == torch.bfloat16 and d_x.dim() == 2 and d_x.shape[1] == k_in
-    batch = d_x.shape[0]
-    if d_y is None:
-        d_y = torch.empty((batch, n_out), dtype=torch.bfloat16, device=d_sorted.device)
-    assert d_y.dtype == torch.bfloat16 and d_y.numel() >= batch * n_out
-    assert d_sorted.numel() * d_sorted.element_size() >= int(ctx._lib.llvq_sorted_gemm_bytes(ctx._h, n_out, k_in))
-    assert d_codebook.dtype == torch.float32 and d_codebook.numel() >= (1 << gain_bits)
-    assert d_row_scale is None or (d_row_scale.dtype == torch.float32 and d_row_scale.numel() >= n_out)
-    _check("llvq_gemm_small_batch_sorted_sg", ctx._lib.llvq_gemm_small_batch_sorted_sg(
-        ctx._h, _dev(d_sorted, "d_sorted"), gain_bits, _dev(d_codebook, "d_codebook"),
-        None if d_row_scale is None else _dev(d_row_scale, "d_row_scale"), n_out, k_in, _dev(d_x, "d_x"), batch, _dev(d_y, "d_y"),
-        _stream_ptr(stream)))
-    return d_y
+    return _out("llvq_gemm_small_batch_sorted_sg", _native.gemm_sg(ctx._ptr, d_sorted, gain_bits, d_codebook, d_row_scale, n_out, k_in, d_x, d_y,
+                                                                   _stream_arg(stream), True))
 
 
 def llvq_encode_blocks(ctx: Context, d_v: torch.Tensor, metric: int, d_points: torch.Tensor | None = None,
                        d_index: torch.Tensor | None = None, stream=None):
     """(points int8 [n, 24], indices int64 [n]) of the code points nearest to the rows of ``d_v`` (float32 [n, 24],
     integer-coordinate units) under LLVQ_EUCLIDEAN or LLVQ_ANGULAR scoring."""
-    assert d_v.dtype == torch.float32 and d_v.dim() == 2 and d_v.shape[1] == 24
-    n = d_v.shape[0]
-    if d_points is None:
-        d_points = torch.empty((n, 24), dtype=torch.int8, device=d_v.device)
-    if d_index is None:
-        d_index = torch.empty(n, dtype=torch.int64, device=d_v.device)
-    assert d_points.dtype == torch.int8 and d_points.numel() >= n * 24 and d_index.dtype == torch.int64 and d_index.numel() >= n
-    _check("llvq_encode_blocks", ctx._lib.llvq_encode_blocks(ctx._h, _dev(d_v, "d_v"), n, metric, _dev(d_points, "d_points"),
-                                                             _dev(d_index, "d_index"), _stream_ptr(stream)))
-    return d_points, d_index
+    return _out("llvq_encode_blocks", _native.encode(ctx._ptr, d_v, metric, d_points, d_index, _stream_arg(stream)))
 
 
 def llvq_rank_blocks(ctx: Context, d_points: torch.Tensor, d_index: torch.Tensor | None = None, stream=None):
     """Indices (int64 [n]) of the lattice points ``d_points`` (int8 [n, 24]); the inverse of ``llvq_decode_blocks``."""
-    assert d_points.dtype == torch.int8 and d_points.dim() == 2 and d_points.shape[1] == 24
-    n = d_points.shape[0]
-    if d_index is None:
-        d_index = torch.empty(n, dtype=torch.int64, device=d_points.device)
-    assert d_index.dtype == torch.int64 and d_index.numel() >= n
-    _check("llvq_rank_blocks", ctx._lib.llvq_rank_blocks(ctx._h, _dev(d_points, "d_points"), n, _dev(d_index, "d_index"), _stream_ptr(stream)))
-    return d_index
+    return _out("llvq_rank_blocks", _native.rank(ctx._ptr, d_points, d_index, _stream_arg(stream)))
 
 
 def llvq_pack_fields(ctx: Context, d_index: torch.Tensor, d_gain_index: torch.Tensor | None = None, gain_bits: int = 0,
                      d_fields: torch.Tensor | None = None, stream=None):
     """The stored stream (uint8) of the fields index | gain index << index_bits."""
-    assert d_index.dtype == torch.int64
-    n = d_index.numel()
-    nbytes = int(ctx._lib.llvq_field_bytes(ctx._h, n, gain_bits))
-    if d_fields is None:
-        d_fields = torch.empty(nbytes, dtype=torch.uint8, device=d_index.device)
-    assert d_fields.numel() * d_fields.element_size() >= nbytes
-    assert gain_bits == 0 or (d_gain_index is not None and d_gain_index.dtype == torch.uint8 and d_gain_index.numel() >= n)
-    _check("llvq_pack_fields", ctx._lib.llvq_pack_fields(
-        ctx._h, _dev(d_index, "d_index"), None if d_gain_index is None or gain_bits == 0 else _dev(d_gain_index, "d_gain_index"),
-        gain_bits, n, _dev(d_fields, "d_fields"), _stream_ptr(stream)))
-    return d_fields
+    return _out("llvq_pack_fields", _native.pack(ctx._ptr, d_index, d_gain_index, gain_bits, d_fields, _stream_arg(stream)))
 
 
 def _ptr(p, name: str) -> int:

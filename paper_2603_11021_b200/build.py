@@ -8,6 +8,8 @@ import subprocess
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "libllvq.so")
+NATIVE = os.path.join(PKG, "_native.so")            # the Python module that calls it on PyTorch tensors (csrc/binding.cpp)
+BINDING = os.path.join(PKG, "csrc", "binding.cpp")
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17",
@@ -20,12 +22,15 @@ OBJ_DIR = os.path.join(PKG, "build")
 
 def sources() -> list[str]:
     src = sorted(glob.glob(os.path.join(PKG, "csrc", "*.cu")) + glob.glob(os.path.join(PKG, "csrc", "*.cpp")))
-    return src
+    return [f for f in src if f != BINDING]
+
+
+def _headers() -> list[str]:
+    return glob.glob(os.path.join(ROOT, "include", "*.h"))
 
 
 def _inputs() -> list[str]:
-    return sources() + glob.glob(os.path.join(PKG, "csrc", "*.h")) + glob.glob(os.path.join(PKG, "csrc", "*.cuh")) + \
-        glob.glob(os.path.join(ROOT, "include", "*.h"))
+    return sources() + _headers() + glob.glob(os.path.join(PKG, "csrc", "*.h")) + glob.glob(os.path.join(PKG, "csrc", "*.cuh"))
 
 
 def is_stale() -> bool:
@@ -36,9 +41,30 @@ def is_stale() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Build libllvq.so next to this file; returns its path."""
-    if not force and not is_stale():
-        return LIB
+    """Build libllvq.so and _native.so next to this file; returns the library's path."""
+    if force or is_stale():
+        _build_library(verbose)
+    if force or not os.path.exists(NATIVE) or any(os.path.getmtime(NATIVE) < os.path.getmtime(f) for f in [BINDING] + _headers()):
+        _build_native()
+    return LIB
+
+
+def _build_native() -> None:
+    """The Python module: plain C++ against PyTorch's headers, linked to libllvq.so beside it."""
+    import sysconfig
+    import torch
+    root = os.path.join(os.path.dirname(torch.__file__))
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = NATIVE + f".{os.getpid()}.tmp"
+    subprocess.check_call([
+        os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+        "-I", os.path.join(ROOT, "include"), "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+        "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], BINDING, "-o", tmp, "-L", PKG, "-lllvq",
+        "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, NATIVE)
+
+
+def _build_library(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "nvcc")
     os.makedirs(OBJ_DIR, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose else []
@@ -57,7 +83,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.replace(tmp, LIB)
     for o in objs:
         os.remove(o)
-    return LIB
 
 
 if __name__ == "__main__":

@@ -54,11 +54,11 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
 #define LLVQ_LAUNCH_DOMAINS(BIG, SG, SH)                                                                                      \
     do {                                                                                                                     \
         if (pipe) {                                                                                                          \
-            if (!set_smem(gemm_pipe_kernel<BIG, SG, SH>, smem)) return LLVQ_ECUDA;                                            \
+            if (!set_smem<gemm_pipe_kernel<BIG, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                            \
             if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx, !ctx->fast), \
                            static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, b_double) != cudaSuccess) return LLVQ_ECUDA; \
         } else {                                                                                                             \
-            if (!set_smem(gemm_sorted_kernel<BIG, SG, SH>, smem)) return LLVQ_ECUDA;                                          \
+            if (!set_smem<gemm_sorted_kernel<BIG, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                          \
             if (launch_pdl(gemm_sorted_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx, !ctx->fast), \
                            static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, dpi) != cudaSuccess) return LLVQ_ECUDA; \
         }                                                                                                                    \
@@ -139,7 +139,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_BINNED(SG, SH, RD)                                                                                          \
     do {                                                                                                                        \
-        if (!set_smem(gemm_sorted_kernel<false, SG, SH, true, RD>, smem_bin)) return LLVQ_ECUDA;                                 \
+        if (!set_smem<gemm_sorted_kernel<false, SG, SH, true, RD>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                 \
         if (launch_pdl(gemm_sorted_kernel<false, SG, SH, true, RD>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, false), words, \
                        d_gain_f16, sga, gb, dpi) != cudaSuccess) return LLVQ_ECUDA;                                             \
     } while (0)
@@ -173,11 +173,11 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const unsigned grid_bin = (unsigned)std::min<int64_t>(row_tiles * gb.nstages, ctx->sm_count);
             const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
             if (yo) {
-                if (!set_smem(gemm_sorted_kernel<true, false, true, true, true>, smem_bin)) return LLVQ_ECUDA;
+                if (!set_smem<gemm_sorted_kernel<true, false, true, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
                 if (launch_pdl(gemm_sorted_kernel<true, false, true, true, true>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, true), words,
                                d_gain_f16, SgArgs{}, gb, dpi) != cudaSuccess) return LLVQ_ECUDA;
             } else {
-                if (!set_smem(gemm_sorted_kernel<true, false, false, true, true>, smem_bin)) return LLVQ_ECUDA;
+                if (!set_smem<gemm_sorted_kernel<true, false, false, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
                 if (launch_pdl(gemm_sorted_kernel<true, false, false, true, true>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, true), words,
                                d_gain_f16, SgArgs{}, gb, dpi) != cudaSuccess) return LLVQ_ECUDA;
             }
@@ -199,7 +199,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_PIPE_STORED(BIG, SG, SH)                                                                                    \
     do {                                                                                                                        \
-        if (!set_smem(gemm_pipe_kernel<BIG, SG, SH, true>, smem_pipe)) return LLVQ_ECUDA;                                        \
+        if (!set_smem<gemm_pipe_kernel<BIG, SG, SH, true>>(ctx->device, smem_pipe)) return LLVQ_ECUDA;                                        \
         if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH, true>, grid_pipe, (unsigned)kGemmThreads, smem_pipe, st, fast_args(ctx, !ctx->fast), words, \
                        d_gain_f16, sga, gp, b_double) != cudaSuccess) return LLVQ_ECUDA;                                        \
     } while (0)
@@ -213,20 +213,20 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     }
     if (yo) {
         if (ctx->fast) {
-            if (!set_smem(gemm_kernel<false, false, true>, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemm_kernel<false, false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemm_kernel<false, false, true>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
         } else {
-            if (!set_smem(gemm_kernel<true, false, true>, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemm_kernel<true, false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemm_kernel<true, false, true>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
         }
     } else if (sg) {
-        if (!set_smem(gemm_kernel<false, true>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<gemm_kernel<false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(gemm_kernel<false, true>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, *sg, ga) != cudaSuccess) return LLVQ_ECUDA;
     } else if (ctx->fast) {
-        if (!set_smem(gemm_kernel<false, false>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<gemm_kernel<false, false>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(gemm_kernel<false, false>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
     } else {
-        if (!set_smem(gemm_kernel<true, false>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<gemm_kernel<true, false>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(gemm_kernel<true, false>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
     }
     return launch_status();
@@ -267,7 +267,7 @@ static int sort_blocks_gemm_common(const llvq_ctx* ctx, const void* d_idx, int g
         return launch_status();
     }
     const size_t smem = ctx->fl.total + 16;
-    if (!set_smem(sort_blocks_gemm_kernel, smem)) return LLVQ_ECUDA;
+    if (!set_smem<sort_blocks_gemm_kernel>(ctx->device, smem)) return LLVQ_ECUDA;
     sort_blocks_gemm_kernel<<<g, kDomEntries, smem, (cudaStream_t)stream>>>(fast_args(ctx, !ctx->fast), static_cast<const uint32_t*>(d_idx), ctx->d_sort_rank,
                                                                            gain_bits, n_out, bpr, ndomains, static_cast<unsigned long long*>(d_sorted));
     return launch_status();

@@ -86,7 +86,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
         const FastArgs fa = fast_args(ctx, ext_bin);
 #define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
     do {                                                                                                                   \
-        if (!set_smem(gemv_bin_kernel<BF16, SG, SH>, smem_bin)) return LLVQ_ECUDA;                                          \
+        if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                          \
         if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, n_out, k_in, \
                        bpr, magic, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
@@ -99,7 +99,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const FastArgs fa = fast_args(ctx, ext_direct);
 #define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH)                                                                        \
     do {                                                                                                           \
-        if (!set_smem(gemv_fast_kernel<BIG, BF16, SG, SH>, smem)) return LLVQ_ECUDA;                               \
+        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                               \
         if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, n_out, k_in, bpr, d_x_bf16, yo, \
                        ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;                         \
     } while (0)
@@ -166,7 +166,7 @@ static int sort_blocks_common(const llvq_ctx* ctx, const void* d_fields, int gai
     const int64_t units = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
     const unsigned g = (unsigned)std::min<int64_t>(units, ctx->sm_count);
     const size_t smem = ctx->fl.total + 16;
-    if (!set_smem(sort_blocks_kernel, smem)) return LLVQ_ECUDA;
+    if (!set_smem<sort_blocks_kernel>(ctx->device, smem)) return LLVQ_ECUDA;
     sort_blocks_kernel<<<g, kSortThreads, smem, (cudaStream_t)stream>>>(fast_args(ctx), static_cast<const uint32_t*>(d_fields), ctx->d_sort_rank, gain_bits,
                                                                        n_out, bpr, static_cast<unsigned long long*>(d_sorted));
     return launch_status();
@@ -205,7 +205,7 @@ static int gemv_sorted_common(const llvq_ctx* ctx, const void* d_sorted, const u
     const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_SORTED(BF16, SG, SH)                                                                                \
     do {                                                                                                                \
-        if (!set_smem(gemv_sorted_kernel<BF16, SG, SH>, smem)) return LLVQ_ECUDA;                                        \
+        if (!set_smem<gemv_sorted_kernel<BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                        \
         if (launch_pdl(gemv_sorted_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem, st, fa, sp, d_gain_f16, sga, n_out, k_in, bpr, \
                        magic, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;          \
     } while (0)
@@ -314,10 +314,10 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         const size_t smem_ov = fa.image_bytes + 16 + (size_t)kOverlapSets * ((size_t)xs_words + (size_t)kSortAccCopies * acc_rows) * 4 + kOverlapSets * sizeof(OverlapSet);
         if (one_pass && max_groups <= kGemvGroupsPerPass && smem_ov <= kSmemLimit) {
             if (y_dtype == LLVQ_BF16) {
-                if (!set_smem(gemv_sorted_overlap_kernel<true>, smem_ov)) return LLVQ_ECUDA;
+                if (!set_smem<gemv_sorted_overlap_kernel<true>>(ctx->device, smem_ov)) return LLVQ_ECUDA;
                 if (launch_pdl(gemv_sorted_overlap_kernel<true>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
             } else {
-                if (!set_smem(gemv_sorted_overlap_kernel<false>, smem_ov)) return LLVQ_ECUDA;
+                if (!set_smem<gemv_sorted_overlap_kernel<false>>(ctx->device, smem_ov)) return LLVQ_ECUDA;
                 if (launch_pdl(gemv_sorted_overlap_kernel<false>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
             }
             return launch_status();
@@ -325,18 +325,18 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     }
     if (sorted) {
         if (y_dtype == LLVQ_BF16) {
-            if (!set_smem(gemv_sorted_multi_kernel<true>, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemv_sorted_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemv_sorted_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         } else {
-            if (!set_smem(gemv_sorted_multi_kernel<false>, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemv_sorted_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemv_sorted_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         }
     } else {
         if (y_dtype == LLVQ_BF16) {
-            if (!set_smem(gemv_bin_multi_kernel<true>, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemv_bin_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemv_bin_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, ctx->d_sort_rank, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         } else {
-            if (!set_smem(gemv_bin_multi_kernel<false>, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemv_bin_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemv_bin_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, ctx->d_sort_rank, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         }
     }

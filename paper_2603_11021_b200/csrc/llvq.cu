@@ -265,11 +265,11 @@ int llvq_decode_blocks(const llvq_ctx* ctx, const void* d_idx, uint64_t nblocks,
     const unsigned g = (unsigned)std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count);
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (ctx->fast) {
-        if (!set_smem(decode_blocks_fast_kernel<false>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<decode_blocks_fast_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(decode_blocks_fast_kernel<false>, g, (unsigned)kFastThreads, smem, (cudaStream_t)stream, fast_args(ctx, false), idx, nblocks,
                        reinterpret_cast<uint2*>(d_points)) != cudaSuccess) return LLVQ_ECUDA;
     } else {
-        if (!set_smem(decode_blocks_fast_kernel<true>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<decode_blocks_fast_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(decode_blocks_fast_kernel<true>, g, (unsigned)kFastThreads, smem, (cudaStream_t)stream, fast_args(ctx, false), idx, nblocks,
                        reinterpret_cast<uint2*>(d_points)) != cudaSuccess) return LLVQ_ECUDA;
     }
@@ -299,11 +299,11 @@ int llvq_dequant_matrix(const llvq_ctx* ctx, const void* d_idx, const uint16_t* 
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(d_w_bf16);
     if (ctx->fast) {
-        if (!set_smem(dequant_fast_kernel<false>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<dequant_fast_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(dequant_fast_kernel<false, false>, g, (unsigned)kFastThreads, smem, st, fast_args(ctx, false), idx, d_gain_f16, SgArgs{}, (uint64_t)nblocks,
                        rows, cols, bpr, w, ld) != cudaSuccess) return LLVQ_ECUDA;
     } else {
-        if (!set_smem(dequant_fast_kernel<true>, smem)) return LLVQ_ECUDA;
+        if (!set_smem<dequant_fast_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(dequant_fast_kernel<true, false>, g, (unsigned)kFastThreads, smem, st, fast_args(ctx, false), idx, d_gain_f16, SgArgs{}, (uint64_t)nblocks,
                        rows, cols, bpr, w, ld) != cudaSuccess) return LLVQ_ECUDA;
     }
@@ -333,7 +333,7 @@ int llvq_dequant_matrix_sg(const llvq_ctx* ctx, const void* d_fields, int gain_b
     const size_t smem = ctx->fl.total + 16;
     const uint64_t tiles = (nblocks + kFastThreads - 1) / kFastThreads;
     const unsigned g = (unsigned)std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count);
-    if (!set_smem(dequant_fast_kernel<false, true>, smem)) return LLVQ_ECUDA;
+    if (!set_smem<dequant_fast_kernel<false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
     dequant_fast_kernel<false, true><<<g, kFastThreads, smem, (cudaStream_t)stream>>>(
         fast_args(ctx, false), static_cast<const uint32_t*>(d_fields), nullptr, SgArgs{d_codebook_f32, d_row_scale_f32, gain_bits},
         nblocks, rows, cols, bpr, reinterpret_cast<__nv_bfloat16*>(d_w_bf16), ld);
