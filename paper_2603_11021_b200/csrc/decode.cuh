@@ -84,6 +84,51 @@ __device__ __forceinline__ uint64_t field_of_words(ulonglong2 w, int W)
     return W < 64 ? v & ((1ull << W) - 1) : v;
 }
 
+// The 32-bit words that hold a field, as they are in the stream: requested with the loads of one block while another is being
+// unranked, put together when the block's turn comes.  kBig: indices above 64 bits (four words), else at most 64 bits (three).
+template <bool kBig>
+struct RawField {
+    uint32_t w0, w1, w2, w3, shift;
+};
+
+template <bool kBig>
+__device__ __forceinline__ RawField<kBig> request_field(const uint32_t* __restrict__ stream, uint64_t b, int W, bool in)
+{
+    RawField<kBig> f;
+    const uint64_t bp = b * (uint64_t)W;
+    const uint32_t* p = stream + (bp >> 5);
+    f.shift = (uint32_t)bp & 31u;
+    const uint32_t last = in ? f.shift + (uint32_t)W : 0u;       // bits counted from the first word (0: nothing is read)
+    f.w0 = f.w1 = f.w2 = f.w3 = 0u;
+    if (last > 0u) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(f.w0) : "l"(p));
+    if (last > 32u) asm volatile("ld.global.nc.u32 %0, [%1+4];" : "=r"(f.w1) : "l"(p));
+    if (last > 64u) asm volatile("ld.global.nc.u32 %0, [%1+8];" : "=r"(f.w2) : "l"(p));
+    if (kBig && last > 96u) asm volatile("ld.global.nc.u32 %0, [%1+12];" : "=r"(f.w3) : "l"(p));
+    return f;
+}
+
+// Keeps whatever is formed from the words behind this point.
+template <bool kBig>
+__device__ __forceinline__ void use_field_from_here(RawField<kBig>& f)
+{
+    asm volatile("" : "+r"(f.w0), "+r"(f.w1), "+r"(f.w2), "+r"(f.w3));
+}
+
+template <bool kBig>
+__device__ __forceinline__ void field_value(const RawField<kBig>& f, int W, uint64_t& lo, uint64_t& hi)
+{
+    const uint32_t v0 = __funnelshift_r(f.w0, f.w1, f.shift), v1 = __funnelshift_r(f.w1, f.w2, f.shift);
+    lo = (uint64_t)v1 << 32 | v0;
+    hi = 0u;
+    if (kBig) {
+        const uint32_t v2 = __funnelshift_r(f.w2, f.w3, f.shift);
+        if (W > 64) hi = v2 & ((1u << (W - 64)) - 1u);           // W <= 72
+        else if (W < 64) lo &= (1ull << W) - 1ull;
+    } else if (W < 64) {
+        lo &= (1ull << W) - 1ull;
+    }
+}
+
 // q = p / d, r = p % d with magic = floor((2^64 - 1) / d): the estimate is at most one too small.
 __device__ __forceinline__ void divmod_magic(uint64_t p, uint32_t d, uint64_t magic, uint64_t& q, uint32_t& r)
 {
@@ -136,6 +181,7 @@ __device__ __forceinline__ uint16_t ldg_u16_here(const uint16_t* p)
 
 __device__ __forceinline__ float gain_to_float(uint16_t bits)
 {
+    asm volatile("" : "+h"(bits));          // the conversion stays behind the volatile statements before it (the load may still be in flight there)
     return __half2float(__ushort_as_half(bits));
 }
 

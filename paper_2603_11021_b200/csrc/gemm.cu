@@ -41,8 +41,9 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
     int dpi = ga.npad <= 32 ? 2 : 1;                                         // gemm_sorted_kernel: domains unranked per iteration (shared memory decides)
     const int64_t row_tiles = (n_out + kGemmRows - 1) / kGemmRows;
     ga.scratch_ld = row_tiles * kGemmRows;
-    ga.split = 1;                                                             // unused: the kernel balances domains over the CTAs itself
+    ga.split = 1;
     const unsigned grid = (unsigned)std::min<int64_t>(row_tiles * ga.nstages, ctx->sm_count);
+    ga.sp = make_split(row_tiles * ga.nstages, ga.nstages, grid);
     // gemm_pipe_kernel: two A buffer sets and two X buffer sets, or one X set when two do not fit; else the kernel with the block barrier
     const size_t head = (gemm_image_bytes(ctx) + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
                  x_set = (size_t)kDomStages * ga.npad * kStageK * 2;
@@ -135,6 +136,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
         const size_t smem_bin = head + (size_t)dpi * (a_set + x_set) + (size_t)gb.bin_round * bins;
         if (smem_bin <= 227 * 1024) {
             const unsigned grid_bin = (unsigned)std::min<int64_t>(row_tiles * gb.nstages, ctx->sm_count);
+            gb.sp = make_split(row_tiles * gb.nstages, gb.nstages, grid_bin);
             const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
             const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_BINNED(SG, SH, RD)                                                                                          \
@@ -171,6 +173,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
         const size_t smem_bin = head + (size_t)dpi * (a_set + x_set) + (size_t)gb.bin_round * bins;
         if (smem_bin <= 227 * 1024) {
             const unsigned grid_bin = (unsigned)std::min<int64_t>(row_tiles * gb.nstages, ctx->sm_count);
+            gb.sp = make_split(row_tiles * gb.nstages, gb.nstages, grid_bin);
             const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
             if (yo) {
                 if (!set_smem<gemm_sorted_kernel<true, false, true, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
@@ -195,6 +198,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             gp.nstages = (int)((ga.bpr + kDomBlocks - 1) / kDomBlocks);        // domains per row tile
             gp.split = 1;
             const unsigned grid_pipe = (unsigned)std::min<int64_t>(row_tiles * gp.nstages, ctx->sm_count);
+            gp.sp = make_split(row_tiles * gp.nstages, gp.nstages, grid_pipe);
             const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
             const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_PIPE_STORED(BIG, SG, SH)                                                                                    \

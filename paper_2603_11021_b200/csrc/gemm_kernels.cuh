@@ -1,7 +1,7 @@
 // The fused dequant + small-batch GEMM kernels (tcgen05, accumulator in tensor memory): the kernel with two thread
 // groups on alternating stages, the sorted layouts (sort kernels and the consumer with a block barrier), and the
 // kernel without a block barrier that both entry points run for the 48-bit codes.  Included by gemm.cu inside its
-// unnamed namespace, after kernels_common.cuh and gemv_kernels.cuh (unit_owner, shard_arrive).
+// unnamed namespace, after kernels_common.cuh and gemv_kernels.cuh (shard_arrive).
 #pragma once
 
 // ===========================================================================
@@ -23,7 +23,8 @@ constexpr uint32_t kTmemCols = 128;
 struct GemmArgs {
     int64_t n_out, k_in, bpr;
     int batch, npad;
-    int nstages, split;
+    int nstages, split;        // gemm_kernel: 96-column stages and pieces of K
+    Split sp;                  // the kernels on domains: which CTA works on which
     const uint16_t* x;
     uint16_t* y;               // Y [batch][y_ld] bf16, at the first row of this launch's rows
     int64_t y_ld;
@@ -112,15 +113,16 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
         const int64_t rt = item / ga.split;
         const int f = (int)(item % ga.split);
         const int s_begin = (int)((int64_t)f * ga.nstages / ga.split), s_end = (int)((int64_t)(f + 1) * ga.nstages / ga.split);
-        const int64_t row = rt * kGemmRows + gwarp * 8 + (lane & 7);
+        const int64_t row = (int64_t)rt * kGemmRows + gwarp * 8 + (lane & 7);
         for (int s = s_begin + group; s < s_end; s += 2, ++uses) {
             // ---- A: dequantize one block of 24 weights
             const int64_t cb = (int64_t)s * kStageBlocks + (lane >> 3);
             const bool in = row < ga.n_out && cb < ga.bpr;
             const uint64_t b = in ? (uint64_t)(row * ga.bpr + cb) : 0ull;
             uint32_t w[12];
-            if (kSg) block_pairs_sg(fa, T, stream, sg, b, row, in, w);
-            else block_pairs<kBig>(fa, T, stream, gain, b, in, w);
+            const RawBlock<kBig> raw = request_block<kBig>(stream, kSg ? nullptr : gain, fa.dc.W + (kSg ? sg.bits : 0), b, in);
+            if constexpr (kSg) block_pairs_sg(fa, T, raw.field, sg, row, in, w);
+            else block_pairs<kBig>(fa, T, raw, in, w);
             // the MMAs of this group's previous stage read its buffers: wait for them only now, with the block already unranked
             if (uses > 0 && !mbar_wait(&bar_free[group], (uses - 1u) & 1u)) timeout = true;
             uint8_t* a_dst = a_mine + gwarp * 128 + (lane & 7) * 16;
@@ -154,7 +156,7 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
             if (has0 && !mbar_wait(&bar_done[0], done[0] & 1u)) timeout = true;
             if (has1 && !mbar_wait(&bar_done[1], done[1] & 1u)) timeout = true;
             tc_fence_after();
-            const int64_t orow = rt * kGemmRows + warp * 32 + lane;
+            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
             for (int c0 = 0; c0 < ga.npad && has0; c0 += 16) {
                 float v[16], v1[16];
                 tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
@@ -186,7 +188,7 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
                 __threadfence();
                 for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
                     const int n = i / kGemmRows;
-                    const int64_t orow = rt * kGemmRows + (i % kGemmRows);
+                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
                     if (orow < ga.n_out) {
                         float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
                         gemm_store<kShard>(ga, n, orow, __ldcg(sp));
@@ -233,7 +235,7 @@ sort_blocks_gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const 
         __syncthreads();
         const int64_t rt = dom / nd, d = dom - rt * nd;
         const int i = threadIdx.x;
-        const int64_t row = rt * kGemmRows + (i >> 3), cb = d * kDomBlocks + (i & 7);
+        const int64_t row = (int64_t)rt * kGemmRows + (i >> 3), cb = d * kDomBlocks + (i & 7);
         unsigned long long field = kSortIndexMask;
         uint32_t key = 1023u;
         if (row < n_out && cb < bpr) {
@@ -301,7 +303,7 @@ sort_blocks_gemm_big_kernel(FastArgs fa, const uint32_t* __restrict__ stream, in
     const int i = threadIdx.x;
     for (int64_t dom = blockIdx.x; dom < ndomains; dom += gridDim.x) {
         const int64_t rt = dom / nd, d = dom - rt * nd;
-        const int64_t row = rt * kGemmRows + (i >> 3), cb = d * kDomBlocks + (i & 7);
+        const int64_t row = (int64_t)rt * kGemmRows + (i >> 3), cb = d * kDomBlocks + (i & 7);
         unsigned long long x = kBigNoBlock, y = (unsigned long long)i << kBigClassBits;   // words 0-1 and word 2 of an entry
         uint32_t key = 0x7ffffc00u | (uint32_t)i;                   // no block: after everything else
         if (row < n_out && cb < bpr) {
@@ -396,17 +398,19 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const uint32_t idesc = instr_desc_bf16_m128((uint32_t)ga.npad);
-    const int64_t row_tiles = (ga.n_out + kGemmRows - 1) / kGemmRows;
-    const int64_t nd = ga.nstages;                                         // domains per row tile
+    const uint32_t nd = ga.sp.per_row;                                     // domains per row tile
     // every CTA takes an equal contiguous range of the row_tiles * nd domains (row tile major); the parts of a row
     // tile that end up in different CTAs are summed through the scratch, as in the GEMV
-    const int64_t D = row_tiles * nd, G = gridDim.x;
-    const int64_t dom_begin = blockIdx.x * D / G, dom_end = (blockIdx.x + 1) * D / G;
+    const uint32_t dom_begin = split_begin(ga.sp, blockIdx.x), dom_end = split_begin(ga.sp, blockIdx.x + 1u);
     uint32_t uses = 0, done = 0;
     bool timeout = false;
-    for (int64_t rt = dom_begin / nd; rt * nd < dom_end; ++rt) {
-        const int d_begin = (int)(max(dom_begin, rt * nd) - rt * nd), d_end = (int)(min(dom_end, (rt + 1) * nd) - rt * nd);
-        const uint32_t parts = (uint32_t)(unit_owner((rt + 1) * nd - 1, D, G) - unit_owner(rt * nd, D, G) + 1);   // CTAs that share this row tile
+    // where this thread's 16-byte chunks of an X slice lie: chunk i is (kc, n) = (i / npad, i % npad), i in steps of the block
+    const int bx_kc = (int)threadIdx.x / ga.npad, bx_n = (int)threadIdx.x % ga.npad, bx_step_kc = kGemmThreads / ga.npad, bx_step_n = kGemmThreads % ga.npad;
+    for (uint32_t rt = split_row(ga.sp, dom_begin); rt * nd < dom_end; ++rt) {
+        const uint32_t tile0 = rt * nd, tile1 = tile0 + nd;
+        const int d_begin = (int)(max(dom_begin, tile0) - tile0), d_end = (int)(min(dom_end, tile1) - tile0);
+        // CTAs that share this row tile
+        const uint32_t parts = dom_begin <= tile0 && tile1 <= dom_end ? 1u : split_owner(ga.sp, tile1 - 1u) - split_owner(ga.sp, tile0) + 1u;
         // the entries of an iteration are requested one iteration ahead (they come from DRAM)
         const ulonglong2 no_entry = make_ulonglong2(kSortIndexMask, kBigNoBlock);
         auto entry_at = [&](int d, int q) {
@@ -414,7 +418,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
             if (kBin) {       // a round is one iteration (no room for more): the stream words that hold the field of this thread's block
                               // (position = thread) are requested an iteration ahead into registers; y bit 63 = no block
                 if (kRound) return no_entry;             // longer rounds ask for them in L2 instead, see below
-                const int64_t row = rt * kGemmRows + (threadIdx.x >> 3), cb = (int64_t)(d + q) * kDomBlocks + (threadIdx.x & 7u);
+                const int64_t row = (int64_t)rt * kGemmRows + (threadIdx.x >> 3), cb = (int64_t)(d + q) * kDomBlocks + (threadIdx.x & 7u);
                 if (row < ga.n_out && cb < ga.bpr)
                     return load_field_words(reinterpret_cast<const uint32_t*>(sorted), (uint64_t)(row * ga.bpr + cb), (int)fa.L.W + (kSg ? sg.bits : 0));
                 return no_entry;
@@ -422,7 +426,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
             // warp 0 also issues the MMAs of every iteration: it takes the cheapest chunk of each domain (the last), the other
             // warps pair chunk w - 1 of the first domain with chunk 31 - w of the second
             const int chunk = warp == 0 ? 31 : (q == 0 ? warp - 1 : 31 - warp);
-            const int64_t at = (rt * nd + d + q) * kDomEntries + chunk * 32 + lane;
+            const int64_t at = ((int64_t)rt * nd + d + q) * kDomEntries + chunk * 32 + lane;
             if (kBig) return load_big_entry(sorted, at);
             return make_ulonglong2(__ldg(sorted + at), 0ull);
         };
@@ -440,7 +444,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
                     const int wbits = (int)fa.L.W + (kSg ? sg.bits : 0);
                     const int nr = min(nround, d_end - d0);                  // domains in this round
                     const uint32_t* words = reinterpret_cast<const uint32_t*>(sorted);
-                    const int64_t row = rt * kGemmRows + (threadIdx.x >> 3);
+                    const int64_t row = (int64_t)rt * kGemmRows + (threadIdx.x >> 3);
                     unsigned long long f[kMaxRound];
                     uint32_t f2[kMaxRound];                                  // kBig: class | position << 17
                     uint32_t key[kMaxRound], rank[kMaxRound], cnt[kMaxRound], incl[kMaxRound];
@@ -540,7 +544,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
                 const uint32_t pos = kBig ? (uint32_t)(e.y >> 32) & 1023u : (uint32_t)(e.x >> 48);
                 const bool valid = kBig ? !(e.y >> 63) : (field != kSortIndexMask && I < fa.n_points);
                 const uint32_t r = pos >> 3, c = pos & 7u;
-                const int64_t row = rt * kGemmRows + r, cb = (int64_t)(d0 + q) * kDomBlocks + c;
+                const int64_t row = (int64_t)rt * kGemmRows + r, cb = (int64_t)(d0 + q) * kDomBlocks + c;
                 uint16_t gbits = 0;
                 if (!kSg && valid) gbits = ldg_u16_here(gain + row * ga.bpr + cb);
                 float gn = 0.f;                                               // the gain is converted once the block is unranked
@@ -572,12 +576,12 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
             }
             // ---- B: the slice of X of these stages, 16-byte chunks (8 values along K)
             const int kchunks = nd_now * kDomStages * (kStageK / 8);
-            for (int i = threadIdx.x; i < ga.npad * kchunks; i += kGemmThreads) {
-                const int kc = i / ga.npad, n = i % ga.npad;
-                const int64_t k = (int64_t)d0 * kDomBlocks * 24 + (int64_t)kc * 8;
+            for (int i = threadIdx.x, kc = bx_kc, n = bx_n; i < ga.npad * kchunks; i += kGemmThreads, kc += bx_step_kc, n += bx_step_n) {
+                if (n >= ga.npad) { n -= ga.npad; ++kc; }
+                const int k = d0 * kDomBlocks * 24 + kc * 8;
                 uint4 v = make_uint4(0, 0, 0, 0);
                 if (n < ga.batch && k < ga.k_in) v = __ldg(reinterpret_cast<const uint4*>(ga.x + (int64_t)n * ga.k_in + k));
-                *reinterpret_cast<uint4*>(b_buf + (uint32_t)(kc / (kStageK / 8)) * b_stage + (uint32_t)(kc % (kStageK / 8)) * ga.npad * 16 + n * 16) = v;
+                *reinterpret_cast<uint4*>(b_buf + (uint32_t)i * 16u) = v;              // [kc][n], stage after stage
             }
             fence_async_smem();
             __syncthreads();
@@ -599,7 +603,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
         if (warp < 4 && has) {
             if (!mbar_wait(bar_done, done & 1u)) timeout = true;
             tc_fence_after();
-            const int64_t orow = rt * kGemmRows + warp * 32 + lane;
+            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
             for (int c0 = 0; c0 < ga.npad; c0 += 16) {
                 float v[16];
                 tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
@@ -626,7 +630,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
                 __threadfence();
                 for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
                     const int n = i / kGemmRows;
-                    const int64_t orow = rt * kGemmRows + (i % kGemmRows);
+                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
                     if (orow < ga.n_out) {
                         float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
                         gemm_store<kShard>(ga, n, orow, __ldcg(sp));
@@ -698,10 +702,8 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const uint32_t idesc = instr_desc_bf16_m128((uint32_t)ga.npad);
-    const int64_t row_tiles = (ga.n_out + kGemmRows - 1) / kGemmRows;
-    const int64_t nd = ga.nstages;                                         // domains per row tile
-    const int64_t D = row_tiles * nd, G = gridDim.x;
-    const int64_t dom_begin = blockIdx.x * D / G, dom_end = (blockIdx.x + 1) * D / G;
+    const uint32_t nd = ga.sp.per_row;                                     // domains per row tile
+    const uint32_t dom_begin = split_begin(ga.sp, blockIdx.x), dom_end = split_begin(ga.sp, blockIdx.x + 1u);
     uint32_t g_base = 0, done = 0;                                         // domains this CTA has finished (domain g uses buffer g & 1 for the (g >> 1)-th time)
     bool timeout = false;
     const ulonglong2 no_entry = make_ulonglong2(kSortIndexMask, kBigNoBlock);
@@ -711,9 +713,11 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar_full + b)) : "memory");
     };
 
-    for (int64_t rt = dom_begin / nd; rt * nd < dom_end; ++rt) {
-        const int d_begin = (int)(max(dom_begin, rt * nd) - rt * nd), d_end = (int)(min(dom_end, (rt + 1) * nd) - rt * nd);
-        const uint32_t parts = (uint32_t)(unit_owner((rt + 1) * nd - 1, D, G) - unit_owner(rt * nd, D, G) + 1);   // CTAs that share this row tile
+    for (uint32_t rt = split_row(ga.sp, dom_begin); rt * nd < dom_end; ++rt) {
+        const uint32_t tile0 = rt * nd, tile1 = tile0 + nd;
+        const int d_begin = (int)(max(dom_begin, tile0) - tile0), d_end = (int)(min(dom_end, tile1) - tile0);
+        // CTAs that share this row tile
+        const uint32_t parts = dom_begin <= tile0 && tile1 <= dom_end ? 1u : split_owner(ga.sp, tile1 - 1u) - split_owner(ga.sp, tile0) + 1u;
         const uint32_t n_dom = (uint32_t)(d_end - d_begin), n_tickets = n_dom * 32u;
         if (threadIdx.x == 0) *ticket = kWorkers;                          // the first tickets are the workers' own numbers
         __syncthreads();
@@ -725,15 +729,28 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 const uint32_t gd = g_base + j, b = gd & 1u, bx = b_double ? b : 0u;
                 if (b_double) { if (gd >= 2u && !mbar_wait(bar_free + b, ((gd >> 1) - 1u) & 1u)) timeout = true; }
                 else if (gd >= 1u && !mbar_wait(bar_free + ((gd - 1u) & 1u), ((gd - 1u) >> 1) & 1u)) timeout = true;
-                const int64_t k0 = (int64_t)(d_begin + (int)j) * kDomBlocks * 24;
-                for (int n = lane; n < ga.npad; n += 32) {
-                    const uint16_t* xr = ga.x + (int64_t)n * ga.k_in + k0;
-                    uint8_t* dst = b_buf + bx * kDomStages * b_stage + n * 16;
-#pragma unroll 4
-                    for (int kc = 0; kc < kDomStages * (kStageK / 8); ++kc) {        // 24 asynchronous 16-byte copies per row, zero-filled outside X
-                        const bool in = n < ga.batch && k0 + kc * 8 < ga.k_in;
-                        const uint32_t to = smem_u32(dst + (uint32_t)(kc / (kStageK / 8)) * b_stage + (uint32_t)(kc % (kStageK / 8)) * ga.npad * 16);
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(in ? xr + kc * 8 : ga.x), "r"(in ? 16u : 0u) : "memory");
+                // [kc][n] 16-byte chunks, kc = 0..23.  The loop competes for issue slots with the unranking warps, and with one X
+                // buffer it stands between two domains (28672 x 8192, batch 64: 393 -> 329 us): per chunk one copy and one address step, the size (0 = zero fill)
+                // settled per row except in the last domain of a row of X
+                const uint32_t k0 = (uint32_t)(d_begin + (int)j) * kDomBlocks * 24;
+                const uint32_t have = min((uint32_t)ga.k_in - k0, (uint32_t)(kDomStages * kStageK)) / 8u;          // chunks inside X
+                const int per = ga.npad < 32 ? 2 : 1;                                                           // 16 rows: two lanes per row
+                const int kc0 = per == 2 ? lane >> 4 : 0;
+                for (int n = per == 2 ? lane & 15 : lane; n < ga.npad; n += 32) {
+                    const bool row_in = n < ga.batch;
+                    const uint16_t* src = ga.x + (row_in ? (int64_t)n * ga.k_in : 0) + k0 + 8 * kc0;
+                    uint32_t to = smem_u32(b_buf) + bx * kDomStages * b_stage + (uint32_t)(kc0 * ga.npad + n) * 16u;
+                    const uint32_t step = (uint32_t)(per * ga.npad) * 16u;
+                    if (have == kDomStages * (kStageK / 8) && per == 1) {
+                        const uint32_t size = row_in ? 16u : 0u;
+#pragma unroll
+                        for (int kc = 0; kc < kDomStages * (kStageK / 8); ++kc, to += step)
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(src + 8 * kc), "r"(size) : "memory");
+                    } else {
+                        for (int kc = kc0; kc < kDomStages * (kStageK / 8); kc += per, src += 8 * per, to += step) {
+                            const bool in = row_in && (uint32_t)kc < have;
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(in ? src : ga.x), "r"(in ? 16u : 0u) : "memory");
+                        }
                     }
                 }
                 asm volatile("cp.async.wait_all;" ::: "memory");
@@ -761,29 +778,26 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
             }
         } else {
             // ---- A: unrank chunks until the tile's tickets are gone
+            const int64_t entry0 = (int64_t)(tile0 + d_begin) * kDomEntries + lane;
+            const uint32_t bpr = (uint32_t)ga.bpr;
+            const uint16_t* gain_tile = gain + (int64_t)rt * kGemmRows * ga.bpr;
             auto entry_of = [&](uint32_t t) {
                 if (t >= n_tickets) return no_entry;
-                if (kStored && kBig) {                                       // the index itself, in the form of the sorted layout's entries
-                    const uint32_t pos = (t & 31u) * 32u + lane;
-                    const int64_t row = rt * kGemmRows + (pos >> 3), cb = (int64_t)(d_begin + (int)(t >> 5)) * kDomBlocks + (pos & 7u);
-                    uint64_t lo = 0, hi = kBigNoBlock;
-                    if (row < ga.n_out && cb < ga.bpr) load_index(reinterpret_cast<const uint32_t*>(sorted), (uint64_t)(row * ga.bpr + cb), fa.dc.W, lo, hi);
-                    return make_ulonglong2(lo, hi | (unsigned long long)pos << 32);
-                }
-                if (kStored) {                                               // the field itself, its position in the high 16 bits
-                    const uint32_t pos = (t & 31u) * 32u + lane;
-                    const int64_t row = rt * kGemmRows + (pos >> 3), cb = (int64_t)(d_begin + (int)(t >> 5)) * kDomBlocks + (pos & 7u);
-                    unsigned long long f = kSortIndexMask;
-                    if (row < ga.n_out && cb < ga.bpr)
-                        f = load_field(reinterpret_cast<const uint32_t*>(sorted), (uint64_t)(row * ga.bpr + cb), (int)fa.L.W + (kSg ? sg.bits : 0));
-                    return make_ulonglong2(f | (unsigned long long)pos << 48, 0ull);
-                }
-                const int64_t at = (rt * nd + d_begin + (int)(t >> 5)) * kDomEntries + (t & 31u) * 32u + lane;
-                if (kBig) return load_big_entry(sorted, at);
-                return make_ulonglong2(__ldg(sorted + at), 0ull);
+                if (kBig) return load_big_entry(sorted, entry0 + t * 32u);     // chunk t % 32 of domain t / 32
+                return make_ulonglong2(__ldg(sorted + entry0 + t * 32u), 0ull);
+            };
+            // stored stream: the words of this lane's block of chunk t (position t % 32 * 32 + lane of domain t / 32)
+            const int wbits = fa.dc.W + (kSg ? sg.bits : 0);
+            auto stored_of = [&](uint32_t t, bool& in) {
+                const uint32_t pos = (t & 31u) * 32u + lane, c0 = ((uint32_t)d_begin + (t >> 5)) * kDomBlocks + (pos & 7u), r0 = pos >> 3;
+                in = t < n_tickets && (int64_t)rt * kGemmRows + r0 < ga.n_out && c0 < bpr;
+                return request_field<kBig>(reinterpret_cast<const uint32_t*>(sorted), (uint64_t)rt * kGemmRows * ga.bpr + (r0 * bpr + c0), wbits, in);
             };
             uint32_t tk = (uint32_t)warp - 1u;
-            ulonglong2 e = entry_of(tk);
+            ulonglong2 e = no_entry;
+            RawField<kBig> raw{};
+            bool in = false;
+            if (kStored) raw = stored_of(tk, in); else e = entry_of(tk);
             // sorted 96-bit entries name their class: its record is requested while the previous chunk is still being expanded
             uint4 rec0 = make_uint4(0u, 0u, 0u, 0u), rec1 = rec0;
             if (kBig && !kStored) big_load_record(fa.dc, (int)((uint32_t)(e.y >> 8) & 0xffffffu), !(e.y >> 63), rec0, rec1);
@@ -791,7 +805,17 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 uint32_t tk_next = 0;
                 if (lane == 0) tk_next = atomicAdd(ticket, 1u);
                 tk_next = __shfl_sync(kFullMask, tk_next, 0);
-                const ulonglong2 e_next = entry_of(tk_next);                // requested a chunk ahead (it comes from DRAM)
+                ulonglong2 e_next = no_entry;                               // requested a chunk ahead (it comes from DRAM)
+                RawField<kBig> raw_next{};
+                bool in_next = false;
+                if (kStored) raw_next = stored_of(tk_next, in_next); else e_next = entry_of(tk_next);
+                if (kStored) {                                              // this chunk's blocks in the form of the sorted layout's entries
+                    uint64_t lo, hi;
+                    field_value(raw, wbits, lo, hi);
+                    const unsigned long long pos = (tk & 31u) * 32u + lane;
+                    e = kBig ? make_ulonglong2(lo, (in ? hi : kBigNoBlock) | pos << 32)
+                             : make_ulonglong2((in ? lo : kSortIndexMask) | pos << 48, 0ull);
+                }
                 const uint32_t j = tk >> 5, gd = g_base + j, b = gd & 1u;
                 const int d = d_begin + (int)j;
                 const uint64_t field = e.x & kSortIndexMask;
@@ -804,9 +828,8 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                     if (!valid) atomicAdd(fa.bad_index, 1ull);
                 }
                 const uint32_t r = pos >> 3, c = pos & 7u;
-                const int64_t row = rt * kGemmRows + r, cb = (int64_t)d * kDomBlocks + c;
                 uint16_t gbits = 0;
-                if (!kSg && valid) gbits = ldg_u16_here(gain + row * ga.bpr + cb);
+                if (!kSg && valid) gbits = ldg_u16_here(gain_tile + (r * bpr + (uint32_t)d * kDomBlocks + c));
                 float gn = 0.f;                                               // the gain is converted once the block is unranked
                 uint32_t w[12];
                 if (kBig) {
@@ -838,7 +861,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                     }
                     if (!kSg) gn = gain_to_float(gbits);
                     if (kSg && valid) {
-                        const float scale = sg.row_scale ? __ldg(sg.row_scale + row) : 1.f;
+                        const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rt * kGemmRows + r) : 1.f;
                         gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + (uint32_t)(field >> fa.L.W))),
                                        __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
                     }
@@ -851,7 +874,13 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 for (int jj = 0; jj < 3; ++jj)
                     *reinterpret_cast<uint4*>(a_dst + jj * 2048) = make_uint4(w[4 * jj], w[4 * jj + 1], w[4 * jj + 2], w[4 * jj + 3]);
                 arrive_full(b);
-                tk = tk_next; e = e_next;
+                tk = tk_next;
+                if (kStored) { raw = raw_next; in = in_next; use_field_from_here(raw); }
+                else {
+                    e = e_next;
+                    use_from_here(e.x);
+                    if (kBig) use_from_here(e.y);
+                }
             }
         }
         g_base += n_dom;
@@ -860,7 +889,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
         if (warp < 4 && has) {
             if (!mbar_wait(bar_done, done & 1u)) timeout = true;
             tc_fence_after();
-            const int64_t orow = rt * kGemmRows + warp * 32 + lane;
+            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
             for (int c0 = 0; c0 < ga.npad; c0 += 16) {
                 float v[16];
                 tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
@@ -887,7 +916,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 __threadfence();
                 for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
                     const int n = i / kGemmRows;
-                    const int64_t orow = rt * kGemmRows + (i % kGemmRows);
+                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
                     if (orow < ga.n_out) {
                         float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
                         gemm_store<kShard>(ga, n, orow, __ldcg(sp));

@@ -63,6 +63,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     if (smem > kSmemMax || n_out > 64ll * kMaxScratchRows) return LLVQ_EUNSUPPORTED;
     const int64_t units = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
     const unsigned g = (unsigned)std::min<int64_t>(units, ctx->sm_count);
+    const Split sp = make_split(units, nq, g);
     // warps per CTA: the count in [28, 32] that wastes the fewest warp slots on the units of one CTA
     const int64_t upc = (units + g - 1) / g;
     int warps = 32; double best_eff = 0.0;
@@ -82,13 +83,12 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     bin_smem(ctx, nq, seg_units, smem_bin, ext_bin);
     // (smaller segments sort too few blocks to pay for the sort: the direct kernel takes over when 8192 do not fit)
     if (bin_kernel_serves(ctx, nq, sg)) {
-        const uint32_t magic = nq == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)nq);
         const FastArgs fa = fast_args(ctx, ext_bin);
 #define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
     do {                                                                                                                   \
         if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                          \
-        if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, n_out, k_in, \
-                       bpr, magic, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
+        if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
+                       bpr, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
         if (shard)   { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, true); else LLVQ_LAUNCH_BIN(false, false, true); }
         else if (sg) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, true, false); else LLVQ_LAUNCH_BIN(false, true, false); }
@@ -100,7 +100,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
 #define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH)                                                                        \
     do {                                                                                                           \
         if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                               \
-        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, n_out, k_in, bpr, d_x_bf16, yo, \
+        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, sp, n_out, k_in, bpr, d_x_bf16, yo, \
                        ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;                         \
     } while (0)
     if (shard && ctx->fast) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(false, true, false, true); else LLVQ_LAUNCH_GEMV(false, false, false, true); }
@@ -168,7 +168,7 @@ static int sort_blocks_common(const llvq_ctx* ctx, const void* d_fields, int gai
     const size_t smem = ctx->fl.total + 16;
     if (!set_smem<sort_blocks_kernel>(ctx->device, smem)) return LLVQ_ECUDA;
     sort_blocks_kernel<<<g, kSortThreads, smem, (cudaStream_t)stream>>>(fast_args(ctx), static_cast<const uint32_t*>(d_fields), ctx->d_sort_rank, gain_bits,
-                                                                       n_out, bpr, static_cast<unsigned long long*>(d_sorted));
+                                                                       make_split(units, nq, g), n_out, bpr, static_cast<unsigned long long*>(d_sorted));
     return launch_status();
 }
 
@@ -200,14 +200,14 @@ static int gemv_sorted_common(const llvq_ctx* ctx, const void* d_sorted, const u
     size_t smem; bool ext;
     sorted_smem(ctx, nq, smem, ext);
     const FastArgs fa = fast_args(ctx, ext);
-    const uint32_t magic = nq == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)nq);
+    const Split split = make_split(units, nq, g);
     const unsigned long long* sp = static_cast<const unsigned long long*>(d_sorted);
     const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_SORTED(BF16, SG, SH)                                                                                \
     do {                                                                                                                \
         if (!set_smem<gemv_sorted_kernel<BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                        \
-        if (launch_pdl(gemv_sorted_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem, st, fa, sp, d_gain_f16, sga, n_out, k_in, bpr, \
-                       magic, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;          \
+        if (launch_pdl(gemv_sorted_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem, st, fa, sp, d_gain_f16, sga, split, n_out, k_in, bpr, \
+                       d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;          \
     } while (0)
     const bool shard = yo.n_peer > 0 || yo.n_flag > 0;                  // row-sharded launch: stored-gain form only
     if (shard && sg) return LLVQ_EUNSUPPORTED;
@@ -275,7 +275,7 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         GemvMat& m = mm.m[i];
         m.weights = d.d_weights; m.gain = d.d_gain_f16; m.x = d.d_x_bf16; m.y = d.d_y;
         m.n_out = d.n_out; m.k_in = d.k_in; m.slot0 = slot;
-        m.nq_magic = nq == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)nq);
+        m.sp = make_split(units, nq, (unsigned)ctx->sm_count); m.bpr = (int32_t)bpr;
         m.seg_units = kBinSegUnits;
         slot += (d.n_out + kGemvGroupRows - 1) / kGemvGroupRows * kGemvGroupRows;
     }
@@ -300,15 +300,13 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         // one pass and three sets of (x, row sums) fit beside the tables
         int64_t max_groups = 0, max_nq = 0;
         bool one_pass = true;
-        for (int i = 0; i < n_mats && one_pass; ++i) {
-            const int64_t nq = ((descs[i].k_in + 23) / 24 + 3) / 4;
-            const int64_t U = ((descs[i].n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
+        for (int i = 0; i < n_mats; ++i) {
+            // a CTA's share is at most ceil(U / g) units, hence at most that many + nq - 2 units' worth of row groups, cut at both ends
+            const Split& sp = mm.m[i].sp;
+            const int64_t most = sp.each + (sp.rest ? 1 : 0), nq = sp.per_row;
             max_nq = std::max(max_nq, nq);
-            for (int64_t c = 0; c < g; ++c) {
-                const int64_t ub = c * U / g, ue = (c + 1) * U / g;
-                if (ue - ub > kSortSegUnits) { one_pass = false; break; }
-                max_groups = std::max(max_groups, (ue - 1) / nq - ub / nq + 1);
-            }
+            one_pass = one_pass && most <= kSortSegUnits;
+            max_groups = std::max(max_groups, (most + nq - 2) / nq + 1);
         }
         const int xs_words = (int)(max_nq * 48), acc_rows = (int)(max_groups * kGemvGroupRows);
         const size_t smem_ov = fa.image_bytes + 16 + (size_t)kOverlapSets * ((size_t)xs_words + (size_t)kSortAccCopies * acc_rows) * 4 + kOverlapSets * sizeof(OverlapSet);

@@ -16,9 +16,6 @@ __device__ __forceinline__ void mma_bf16_16816(float c[4], uint32_t a0, uint32_t
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// CTA that owns unit u when G CTAs split U units into ranges [c*U/G, (c+1)*U/G).
-__device__ __forceinline__ int64_t unit_owner(int64_t u, int64_t U, int64_t G) { return ((u + 1) * G - 1) / U; }
-
 template <bool kOutBf16, bool kShard>
 __device__ __forceinline__ void store_y(const YOut& yo, int64_t row, float v)
 {
@@ -42,18 +39,18 @@ __device__ __forceinline__ void store_y(const YOut& yo, int64_t row, float v)
 
 // Stages x for a GEMV CTA: xs[cb * 12 + j] = the bf16 pair (x[24 cb + 2j], x[24 cb + 2j + 1]), zero beyond k_in; `words`
 // = 12 x the number of column blocks staged.  16-byte loads where x allows them.
-__device__ __forceinline__ void stage_x(uint32_t* xs, const uint16_t* __restrict__ x, int64_t k_in, int64_t words)
+__device__ __forceinline__ void stage_x(uint32_t* xs, const uint16_t* __restrict__ x, int64_t k_in, uint32_t words, uint32_t tid, uint32_t nthreads)
 {
     if ((reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-        const int64_t full = k_in / 8;                                       // whole groups of 8 elements
-        for (int64_t v = threadIdx.x; v < words / 4; v += blockDim.x) {
+        const uint32_t full = (uint32_t)(k_in / 8);                          // whole groups of 8 elements
+        for (uint32_t v = tid; v < words / 4; v += nthreads) {
             uint4 q = make_uint4(0u, 0u, 0u, 0u);
             if (v < full) q = __ldg(reinterpret_cast<const uint4*>(x) + v);
             else {
                 uint32_t t[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int64_t e = 8 * v + 2 * j;
+                    const uint32_t e = 8 * v + 2 * j;
                     const uint32_t lo = e < k_in ? __ldg(x + e) : 0u, hi = e + 1 < k_in ? __ldg(x + e + 1) : 0u;
                     t[j] = lo | hi << 16;
                 }
@@ -63,15 +60,15 @@ __device__ __forceinline__ void stage_x(uint32_t* xs, const uint16_t* __restrict
         }
         return;
     }
-    for (int64_t i = threadIdx.x; i < words; i += blockDim.x) {
-        const int64_t e = 2 * i;
+    for (uint32_t i = tid; i < words; i += nthreads) {
+        const uint32_t e = 2 * i;
         const uint32_t lo = e < k_in ? __ldg(x + e) : 0u, hi = e + 1 < k_in ? __ldg(x + e + 1) : 0u;
         xs[i] = lo | hi << 16;
     }
 }
 
-// End of a pass of a GEMV CTA over row groups rg0..rg1 (8 rows each; the CTA owns units [u_begin, u_end) of U, nq
-// units per row group, G CTAs): row_sum(i) is the CTA's sum for row i of the pass.  One warp per row group, lanes
+// End of a pass of a GEMV CTA over row groups rg0..rg1 (8 rows each; the CTA owns units [u_begin, u_end) of sp):
+// row_sum(i) is the CTA's sum for row i of the pass.  One warp per row group, lanes
 // 0..7 its rows, no CTA-wide barrier inside.  A group the CTA covers completely is final.  A group it shares with
 // neighbouring CTAs goes through the scratch row in global memory: add, make the add visible, count the arrival;
 // whoever arrives last reads the total, writes y and leaves scratch and counter zero for the next launch (groups shared
@@ -79,16 +76,17 @@ __device__ __forceinline__ void stage_x(uint32_t* xs, const uint16_t* __restrict
 // The caller puts a __syncthreads() before (sums complete) and after (sums may be cleared) the call.
 // slot0 (a multiple of 8) = first scratch row / pair slot of this matrix when one launch works on several matrices.
 template <bool kOutBf16, bool kShard, typename RowSum>
-__device__ __forceinline__ void finish_pass(const YOut& yo, int64_t rg0, int64_t rg1, int64_t nq, int64_t u_begin, int64_t u_end,
-                                            int64_t U, int64_t G, int64_t n_out, float* __restrict__ scratch,
-                                            uint32_t* __restrict__ counters, RowSum row_sum, int64_t slot0 = 0, int warp_of = -1, int nwarps_of = 0)
+__device__ __forceinline__ void finish_pass(const YOut& yo, const Split& sp, uint32_t rg0, uint32_t rg1, uint32_t u_begin, uint32_t u_end,
+                                            int64_t n_out, float* __restrict__ scratch, uint32_t* __restrict__ counters, RowSum row_sum,
+                                            int64_t slot0 = 0, int warp_of = -1, int nwarps_of = 0)
 {
     // by default the warps of the CTA share the row groups; warp_of / nwarps_of let a subset of the warps (one warp) do it
-    const int warp = warp_of >= 0 ? warp_of : (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const int nwarps = warp_of >= 0 ? nwarps_of : (int)(blockDim.x >> 5);
-    for (int64_t rg = rg0 + warp; rg <= rg1; rg += nwarps) {
-        const bool whole = u_begin <= rg * nq && (rg + 1) * nq <= u_end;
-        const int64_t row = rg * kGemvGroupRows + lane;
+    const uint32_t warp = warp_of >= 0 ? (uint32_t)warp_of : threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t nwarps = warp_of >= 0 ? (uint32_t)nwarps_of : blockDim.x >> 5;
+    for (uint32_t rg = rg0 + warp; rg <= rg1; rg += nwarps) {
+        const uint32_t first = rg * sp.per_row, next = first + sp.per_row;
+        const bool whole = u_begin <= first && next <= u_end;
+        const int64_t row = (int64_t)rg * kGemvGroupRows + lane;
         const bool mine = lane < kGemvGroupRows && row < n_out;
         const float part = lane < kGemvGroupRows ? row_sum((rg - rg0) * kGemvGroupRows + lane) : 0.f;
         if (whole) {
@@ -97,7 +95,7 @@ __device__ __forceinline__ void finish_pass(const YOut& yo, int64_t rg0, int64_t
             }
             continue;
         }
-        const uint32_t parts = (uint32_t)(unit_owner((rg + 1) * nq - 1, U, G) - unit_owner(rg * nq, U, G) + 1);
+        const uint32_t parts = split_owner(sp, next - 1u) - split_owner(sp, first) + 1u;
         if (parts == 2u) {
             // two CTAs share the group (the usual case): one compare-and-swap on a 64-bit slot carries both the sum
             // and the arrival.  Whoever finds the slot empty leaves (its sum, 1) there; the other gets that back from
@@ -168,48 +166,59 @@ __device__ __forceinline__ float dot24_bf16(const uint32_t w[12], const uint32_t
 
 template <bool kBig, bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kGemvThreads, 1)
-gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg,
+gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, Split sp,
                  int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
                  float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
-    const int64_t nq = (bpr + 3) / 4;                               // units along K
+    const uint32_t nq = sp.per_row;                                 // units along K
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
     float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kGemvGroupsPerPass][8]
-    stage_x(xs, x, k_in, nq * 48);
+    stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int kWarps = (int)(blockDim.x >> 5);
-    const int64_t groups = (n_out + kGemvGroupRows - 1) / kGemvGroupRows;
-    const int64_t U = groups * nq, G = gridDim.x;
-    const int64_t u_begin = blockIdx.x * U / G, u_end = (blockIdx.x + 1) * U / G;
-    const int64_t rg_first = u_begin / nq, rg_last = u_begin < u_end ? (u_end - 1) / nq : rg_first - 1;   // no units: no pass
-    for (int64_t rg0 = rg_first; rg0 <= rg_last; rg0 += kGemvGroupsPerPass) {
-        const int64_t rg1 = min(rg0 + kGemvGroupsPerPass - 1, rg_last);
+    const uint32_t kWarps = blockDim.x >> 5;
+    const uint32_t u_begin = split_begin(sp, blockIdx.x), u_end = split_begin(sp, blockIdx.x + 1u);      // at least one unit
+    const uint32_t rg_first = split_row(sp, u_begin), rg_last = split_row(sp, u_end - 1u);
+    for (uint32_t rg0 = rg_first; rg0 <= rg_last; rg0 += kGemvGroupsPerPass) {
+        const uint32_t rg1 = min(rg0 + kGemvGroupsPerPass - 1u, rg_last);
         for (int i = threadIdx.x; i < kGemvGroupsPerPass * kGemvGroupRows; i += (int)blockDim.x) acc[i] = 0.f;
         __syncthreads();
-        const int64_t p_begin = max(u_begin, rg0 * nq), p_end = min(u_end, (rg1 + 1) * nq);
-        int64_t rg = (p_begin + warp) / nq, kq = (p_begin + warp) - rg * nq;      // walked along with u: no division per unit
-        for (int64_t u = p_begin + warp; u < p_end; u += kWarps, kq += kWarps) {
+        const uint32_t p_begin = max(u_begin, rg0 * nq), p_end = min(u_end, (rg1 + 1u) * nq);
+        uint32_t kq, rg = split_row(sp, p_begin + (uint32_t)warp, kq);      // walked along with u: no division per unit
+        // a block's words are requested while the one before it is unranked
+        const int wbits = fa.dc.W + (kSg ? sg.bits : 0);
+        int64_t cb = 0, row = 0;
+        bool in = false;
+        auto request = [&](uint32_t u) {
             while (kq >= nq) { kq -= nq; ++rg; }
-            const int64_t cb = kq * 4 + t;
-            const int64_t row = rg * kGemvGroupRows + g;
-            const bool in = row < n_out && cb < bpr;
-            const uint64_t b = (uint64_t)(row * bpr + cb);
+            cb = kq * 4 + t; row = (int64_t)rg * kGemvGroupRows + g;
+            in = u < p_end && row < n_out && cb < bpr;
+            return request_block<kBig>(stream, kSg ? nullptr : gain, wbits, (uint64_t)(row * bpr + cb), in);
+        };
+        uint32_t u = p_begin + (uint32_t)warp;
+        RawBlock<kBig> raw_next = request(u);
+        while (u < p_end) {
+            RawBlock<kBig> raw = raw_next;
+            use_field_from_here(raw.field);
+            const bool in_now = in;
+            const uint32_t cb_now = (uint32_t)cb, rg_now = rg;
+            u += kWarps; kq += kWarps;
+            raw_next = request(u);
             uint32_t w[12];
-            if (kSg) block_pairs_sg(fa, T, stream, sg, b, row, in, w);
-            else block_pairs<kBig>(fa, T, stream, gain, b, in, w);
-            const uint4* xb = reinterpret_cast<const uint4*>(xs + cb * 12);
+            if constexpr (kSg) block_pairs_sg(fa, T, raw.field, sg, (int64_t)rg_now * kGemvGroupRows + g, in_now, w);
+            else block_pairs<kBig>(fa, T, raw, in_now, w);
+            const uint4* xb = reinterpret_cast<const uint4*>(xs + cb_now * 12u);
             const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
             const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
             float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int q = 0; q < 6; ++q)
                 mma_bf16_16816(c, w[2 * q], 0u, w[2 * q + 1], 0u, xv[2 * q], xv[2 * q + 1]);
-            if (t == 0) atomicAdd(&acc[(rg - rg0) * kGemvGroupRows + g], c[0]);
+            if (t == 0) atomicAdd(&acc[(rg_now - rg0) * kGemvGroupRows + g], c[0]);
         }
         __syncthreads();
         // row groups this CTA covers completely are final; the (at most two) split ones go through the scratch
-        finish_pass<kOutBf16, kShard>(yo, rg0, rg1, nq, u_begin, u_end, U, G, n_out, scratch, counters, [&](int64_t r) { return acc[r]; });
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) { return acc[r]; });
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     }
     if (kShard) shard_arrive(yo);
@@ -234,42 +243,40 @@ constexpr int kSortThreads = 1024;
 constexpr int kSortAccCopies = 4;                    // copies of the row sums in shared memory (a power of two)
 constexpr unsigned long long kSortIndexMask = (1ull << 48) - 1ull;
 
-// Calls f(tu0, tu1, rg0, rg1, first, last) for every segment [tu0, tu1) of CTA `cta` (of G) in order; rg0..rg1 = row
+// Calls f(tu0, tu1, rg0, rg1, first, last) for every segment [tu0, tu1) of CTA `cta` in order; rg0..rg1 = row
 // groups of the pass the segment belongs to (a pass covers at most kGemvGroupsPerPass row groups); first / last =
 // the segment opens / closes its pass.
 template <typename F>
-__device__ __forceinline__ void for_each_sorted_segment(int64_t U, int64_t G, int64_t nq, int64_t cta, F f, int seg_units = kSortSegUnits)
+__device__ __forceinline__ void for_each_sorted_segment(const Split& sp, uint32_t cta, F f, uint32_t seg_units = kSortSegUnits)
 {
-    const int64_t u_begin = cta * U / G, u_end = (cta + 1) * U / G;
+    const uint32_t nq = sp.per_row, u_begin = split_begin(sp, cta), u_end = split_begin(sp, cta + 1u);
     if (u_begin >= u_end) return;
-    const int64_t rg_first = u_begin / nq, rg_last = (u_end - 1) / nq;
-    for (int64_t rg0 = rg_first; rg0 <= rg_last; rg0 += kGemvGroupsPerPass) {
-        const int64_t rg1 = min(rg0 + kGemvGroupsPerPass - 1, rg_last);
-        const int64_t p_begin = max(u_begin, rg0 * nq), p_end = min(u_end, (rg1 + 1) * nq);
-        for (int64_t tu0 = p_begin; tu0 < p_end; tu0 += seg_units)
-            f(tu0, min(tu0 + (int64_t)seg_units, p_end), rg0, rg1, tu0 == p_begin, tu0 + seg_units >= p_end);
+    const uint32_t rg_first = split_row(sp, u_begin), rg_last = split_row(sp, u_end - 1u);
+    for (uint32_t rg0 = rg_first; rg0 <= rg_last; rg0 += kGemvGroupsPerPass) {
+        const uint32_t rg1 = min(rg0 + kGemvGroupsPerPass - 1u, rg_last);
+        const uint32_t p_begin = max(u_begin, rg0 * nq), p_end = min(u_end, (rg1 + 1u) * nq);
+        for (uint32_t tu0 = p_begin; tu0 < p_end; tu0 += seg_units)
+            f(tu0, min(tu0 + seg_units, p_end), rg0, rg1, tu0 == p_begin, tu0 + seg_units >= p_end);
     }
 }
 
 __global__ void __launch_bounds__(kSortThreads, 1)
-sort_blocks_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, int gain_bits, int64_t n_out,
+sort_blocks_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, int gain_bits, Split sp, int64_t n_out,
                    int64_t bpr, unsigned long long* __restrict__ out)
 {
     FAST_PROLOGUE();
     __shared__ uint32_t hist[1024], cursor[1024];                  // one bin per class, in sort order; bin 1023 = no block
-    const int64_t nq = (bpr + 3) / 4;
-    const int64_t groups = (n_out + kGemvGroupRows - 1) / kGemvGroupRows;
-    const int64_t U = groups * nq, G = gridDim.x;
-    for_each_sorted_segment(U, G, nq, blockIdx.x, [&](int64_t tu0, int64_t tu1, int64_t, int64_t, bool, bool) {
+    const uint32_t nq = sp.per_row;
+    for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t, uint32_t, bool, bool) {
         const int entries = (int)(tu1 - tu0) * 32;
         hist[threadIdx.x] = 0; cursor[threadIdx.x] = 0;
         __syncthreads();
         // key and field of entry i of the segment; count = the first pass (out-of-range fields are counted once)
         auto entry_of = [&](int i, bool count, unsigned long long& field) {
-            const int64_t u = tu0 + (i >> 5);
             const int lane = i & 31;
-            const int64_t rg = u / nq, kq = u - rg * nq;
-            const int64_t row = rg * kGemvGroupRows + (lane >> 2), cb = kq * 4 + (lane & 3);
+            uint32_t kq;
+            const uint32_t rg = split_row(sp, tu0 + (uint32_t)(i >> 5), kq);
+            const int64_t row = (int64_t)rg * kGemvGroupRows + (lane >> 2), cb = kq * 4 + (lane & 3);
             field = kSortIndexMask;
             if (row >= n_out || cb >= bpr) return 1023u;
             const uint64_t f = load_field(stream, (uint64_t)(row * bpr + cb), (int)fa.L.W + gain_bits);   // shape index | gain index << W
@@ -292,16 +299,16 @@ sort_blocks_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint1
         // the entries are visited column-block major (all row groups of a column unit, then the next unit): the blocks
         // of a bin then come out roughly ordered by column block, and the 32 lanes of a GEMV warp read few different
         // slices of x
-        const int64_t rg_a = tu0 / nq, nrg = (tu1 - 1) / nq - rg_a + 1;
-        for (int64_t e = threadIdx.x; e < nq * nrg * 32; e += kSortThreads) {
-            const int64_t kq = e / (nrg * 32), rem = e - kq * (nrg * 32);
-            const int64_t u = (rg_a + (rem >> 5)) * nq + kq;
+        const uint32_t rg_a = split_row(sp, tu0), nrg = split_row(sp, tu1 - 1u) - rg_a + 1u;
+        for (uint32_t e = threadIdx.x; e < nq * nrg * 32u; e += kSortThreads) {
+            const uint32_t kq = e / (nrg * 32u), rem = e - kq * (nrg * 32u);
+            const uint32_t u = (rg_a + (rem >> 5)) * nq + kq;
             if (u < tu0 || u >= tu1) continue;
             const int i = (int)(u - tu0) * 32 + (int)(rem & 31);
             unsigned long long field;
             const uint32_t key = entry_of(i, false, field);
             const uint32_t slot = hist[key] + atomicAdd(&cursor[key], 1u);
-            out[tu0 * 32 + slot] = field | (unsigned long long)i << 48;
+            out[(uint64_t)tu0 * 32 + slot] = field | (unsigned long long)i << 48;
         }
         __syncthreads();
     });
@@ -346,8 +353,9 @@ struct GemvMat {
     void* y;
     int64_t n_out, k_in;
     int64_t slot0;              // first scratch row / pair slot of this matrix (a multiple of 8)
-    uint32_t nq_magic;          // floor(2^32 / units per row group)
+    Split sp;
     int32_t seg_units;          // stored stream only: units per binned segment
+    int32_t bpr;                // column blocks per row
 };
 struct GemvMulti {
     GemvMat m[kMaxMultiMats];
@@ -355,12 +363,11 @@ struct GemvMulti {
 };
 
 // Ask for the first chunk of every warp of this CTA in L2 (one request per 128-byte line).
-__device__ __forceinline__ void prefetch_first_chunks(const unsigned long long* sorted, int64_t n_out, int64_t bpr)
+__device__ __forceinline__ void prefetch_first_chunks(const unsigned long long* sorted, const Split& sp)
 {
-    const int64_t nq0 = (bpr + 3) / 4, U0 = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq0;
-    const int64_t ub = blockIdx.x * U0 / gridDim.x, ue = (blockIdx.x + 1) * U0 / gridDim.x;
-    if ((threadIdx.x & 15u) == 0u && ub + (int64_t)(threadIdx.x >> 5) < ue)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(sorted + ub * 32 + threadIdx.x));
+    const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);
+    if ((threadIdx.x & 15u) == 0u && ub + (threadIdx.x >> 5) < ue)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(sorted + (uint64_t)ub * 32 + threadIdx.x));
 }
 
 // The sorted-layout GEMV of one matrix by this CTA (all threads call it; shared memory behind `staging` is reused by the
@@ -368,30 +375,28 @@ __device__ __forceinline__ void prefetch_first_chunks(const unsigned long long* 
 template <bool kOutBf16, bool kSg, bool kShard>
 __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastSmem& T, uint8_t* staging,
                                                  const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, const SgArgs& sg,
-                                                 int64_t n_out, int64_t k_in, int64_t bpr, uint32_t nq_magic, const uint16_t* __restrict__ x,
+                                                 const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, const uint16_t* __restrict__ x,
                                                  const YOut& yo, float* __restrict__ scratch, uint32_t* __restrict__ counters, int64_t slot0)
 {
-    const int64_t nq = (bpr + 3) / 4;
+    const uint32_t nq = sp.per_row;
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
     float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccCopies][kGemvGroupsPerPass][8]: warps spread their adds over the copies
     uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows);
     uint32_t* next_chunk = last_flag + 1;
-    stage_x(xs, x, k_in, nq * 48);
+    stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t kWarps = blockDim.x >> 5;
-    const int64_t groups = (n_out + kGemvGroupRows - 1) / kGemvGroupRows;
-    const int64_t U = groups * nq, G = gridDim.x;
-    const uint32_t nq32 = (uint32_t)nq;
 
-    for_each_sorted_segment(U, G, nq, blockIdx.x, [&](int64_t tu0, int64_t tu1, int64_t rg0, int64_t rg1, bool first, bool last) {
+    for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t rg0, uint32_t rg1, bool first, bool last) {
         if (first)
             for (int i = threadIdx.x; i < kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows; i += (int)blockDim.x) acc[i] = 0.f;
         if (threadIdx.x == 0) *next_chunk = kWarps;
         __syncthreads();
-        const int64_t rg_a = tu0 / nq;
-        const uint32_t kq_a = (uint32_t)(tu0 - rg_a * nq), rg_off = (uint32_t)(rg_a - rg0);
-        const uint32_t nchunks = (uint32_t)(tu1 - tu0);
-        const unsigned long long* seg = sorted + tu0 * 32 + lane;
+        uint32_t kq_a;
+        const uint32_t rg_off = split_row(sp, tu0, kq_a) - rg0;
+        const uint32_t nchunks = tu1 - tu0;
+        const unsigned long long* seg = sorted + (uint64_t)tu0 * 32 + lane;
+        const uint16_t* gain_pass = gain + (int64_t)rg0 * kGemvGroupRows * bpr;
         uint32_t ch = (uint32_t)warp;
         unsigned long long e = ch < nchunks ? __ldg(seg + (uint64_t)ch * 32) : 0ull;
         while (ch < nchunks) {
@@ -405,14 +410,13 @@ __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastS
             const uint32_t pos = (uint32_t)(e >> 48);
             const bool valid = field != kSortIndexMask && I < fa.n_points;
             // where the block sits: unit = pos / 32 of the segment, (row, column block) = lane of the unit
-            const uint32_t v = kq_a + (pos >> 5);
-            uint32_t q = __umulhi(v, nq_magic), kq = v - q * nq32;
-            if (kq >= nq32) { kq -= nq32; ++q; }
+            uint32_t kq;
+            const uint32_t q = split_row(sp, kq_a + (pos >> 5), kq);
             const uint32_t rloc = (rg_off + q) * kGemvGroupRows + ((pos >> 2) & 7u);      // row inside the pass
             const uint32_t cb = kq * 4u + (pos & 3u);
             float gn = 0.f;
             uint16_t gbits = 0;
-            if (!kSg && valid) gbits = ldg_u16_here(gain + ((int64_t)rg0 * kGemvGroupRows + rloc) * bpr + cb);
+            if (!kSg && valid) gbits = ldg_u16_here(gain_pass + (rloc * bpr + cb));
             Decoded r;
             const uint32_t cls = decode_sorted_entry(fa, T, I, valid, r);
             if (!kSg) gn = gain_to_float(gbits);
@@ -429,18 +433,19 @@ __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastS
             const float dot = dot24_bf16(w, xv);
             if (valid) atomicAdd(&acc[(warp & (kSortAccCopies - 1)) * (kGemvGroupsPerPass * kGemvGroupRows) + rloc], dot);
             ch = nxt; e = e_next;
+            use_from_here(e);
         }
         __syncthreads();
         if (!last) return;
         // end of the pass: row groups this CTA covers completely are final; the split ones go through the scratch
-        auto row_sum = [&](int64_t r) {
+        auto row_sum = [&](uint32_t r) {
             float v = 0.f;
 #pragma unroll
             for (int c = 0; c < kSortAccCopies; ++c) v += acc[c * (kGemvGroupsPerPass * kGemvGroupRows) + r];
             return v;
         };
-        const int64_t ub = blockIdx.x * U / G, ue = (blockIdx.x + 1) * U / G;     // recomputed here: nothing 64-bit lives across the main loop
-        finish_pass<kOutBf16, kShard>(yo, rg0, rg1, nq, ub, ue, U, G, n_out, scratch, counters, row_sum, slot0);
+        const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sum, slot0);
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     });
 }
@@ -448,12 +453,12 @@ __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastS
 template <bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg,
-                   int64_t n_out, int64_t k_in, int64_t bpr, uint32_t nq_magic, const uint16_t* __restrict__ x, YOut yo,
+                   Split sp, int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
                    float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
-    prefetch_first_chunks(sorted, n_out, bpr);          // while the table image is on its way
+    prefetch_first_chunks(sorted, sp);                  // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
-    gemv_sorted_body<kOutBf16, kSg, kShard>(fa, T, staging, sorted, gain, sg, n_out, k_in, bpr, nq_magic, x, yo, scratch, counters, 0);
+    gemv_sorted_body<kOutBf16, kSg, kShard>(fa, T, staging, sorted, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0);
     if (kShard) shard_arrive(yo);
 }
 
@@ -462,16 +467,16 @@ template <bool kOutBf16>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_sorted_multi_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
-    prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[0].weights), mm.m[0].n_out, (mm.m[0].k_in + 23) / 24);
+    prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[0].weights), mm.m[0].sp);
     FAST_PROLOGUE();
     for (int i = 0; i < mm.n; ++i) {
         const GemvMat& M = mm.m[i];
         if (i + 1 < mm.n)
-            prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[i + 1].weights), mm.m[i + 1].n_out, (mm.m[i + 1].k_in + 23) / 24);
+            prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[i + 1].weights), mm.m[i + 1].sp);
         YOut yo{};
         yo.y = M.y;
-        gemv_sorted_body<kOutBf16, false, false>(fa, T, staging, static_cast<const unsigned long long*>(M.weights), M.gain, SgArgs{}, M.n_out, M.k_in,
-                                                 (M.k_in + 23) / 24, M.nq_magic, M.x, yo, scratch, counters, M.slot0);
+        gemv_sorted_body<kOutBf16, false, false>(fa, T, staging, static_cast<const unsigned long long*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
+                                                 (uint32_t)M.bpr, M.x, yo, scratch, counters, M.slot0);
         __syncthreads();                                   // the next matrix restages x and clears the row sums
     }
 }
@@ -496,7 +501,7 @@ __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, int xs_words, int acc_rows, float* __restrict__ scratch,
                            uint32_t* __restrict__ counters)
 {
-    prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[0].weights), mm.m[0].n_out, (mm.m[0].k_in + 23) / 24);
+    prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[0].weights), mm.m[0].sp);
     FAST_PROLOGUE();
     // [kOverlapSets] x { x as packed pairs [xs_words] | row sums [kSortAccCopies][acc_rows] } | control words
     const int set_words = xs_words + kSortAccCopies * acc_rows;
@@ -504,26 +509,13 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
     volatile OverlapSet* ctl = reinterpret_cast<volatile OverlapSet*>(sets + kOverlapSets * set_words);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t kWarps = blockDim.x >> 5;
-    const int64_t G = gridDim.x;
 
-    // what this CTA owns of matrix i
-    auto share = [&](int i, int64_t& nq, int64_t& U, int64_t& ub, int64_t& ue) {
-        const GemvMat& M = mm.m[i];
-        nq = ((M.k_in + 23) / 24 + 3) / 4;
-        U = ((M.n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
-        ub = blockIdx.x * U / G; ue = (blockIdx.x + 1) * U / G;
-    };
     // prepare set i % kOverlapSets for matrix i with the calling threads (`nthreads` of them, numbered `tid`)
     auto prepare = [&](int i, int tid, int nthreads) {
         const GemvMat& M = mm.m[i];
         uint32_t* xs = sets + (i % kOverlapSets) * set_words;
         float* acc = reinterpret_cast<float*>(xs + xs_words);
-        const int64_t words = (int64_t)(((M.k_in + 23) / 24 + 3) / 4) * 48;
-        for (int64_t w = tid; w < words; w += nthreads) {
-            const int64_t e = 2 * w;
-            const uint32_t lo = e < M.k_in ? __ldg(M.x + e) : 0u, hi = e + 1 < M.k_in ? __ldg(M.x + e + 1) : 0u;
-            xs[w] = lo | hi << 16;
-        }
+        stage_x(xs, M.x, M.k_in, M.sp.per_row * 48u, (uint32_t)tid, (uint32_t)nthreads);
         for (int r = tid; r < kSortAccCopies * acc_rows; r += nthreads) acc[r] = 0.f;
     };
 
@@ -536,10 +528,10 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
     for (int i = 0; i < mm.n; ++i) {
         const GemvMat& M = mm.m[i];
         const int set = i % kOverlapSets;
-        int64_t nq, U, ub, ue;
-        share(i, nq, U, ub, ue);
-        const int64_t bpr = (M.k_in + 23) / 24;
-        const int64_t rg0 = ub / nq, rg1 = ub < ue ? (ue - 1) / nq : rg0 - 1;
+        const Split& sp = M.sp;
+        const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u), bpr = (uint32_t)M.bpr;      // at least one unit
+        uint32_t kq_a;
+        const uint32_t rg0 = split_row(sp, ub, kq_a);
         // the set is prepared for this matrix long before a warp gets here; a bounded wait all the same
         {
             uint32_t spins = 0;
@@ -549,13 +541,12 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
         }
         const uint32_t* xs = sets + set * set_words;
         float* acc = reinterpret_cast<float*>(sets + set * set_words + xs_words);
-        const uint32_t nchunks = (uint32_t)(ue - ub), nq32 = (uint32_t)nq;
-        const uint32_t kq_a = (uint32_t)(ub - rg0 * nq);
-        const unsigned long long* seg = static_cast<const unsigned long long*>(M.weights) + ub * 32 + lane;
+        const uint32_t nchunks = ue - ub;
+        const unsigned long long* seg = static_cast<const unsigned long long*>(M.weights) + (uint64_t)ub * 32 + lane;
+        const uint16_t* gain_pass = M.gain + (int64_t)rg0 * kGemvGroupRows * bpr;
         if (i + 1 < mm.n && warp == 0) {                    // ask for the next matrix's first chunks in L2
-            int64_t nq2, U2, ub2, ue2;
-            share(i + 1, nq2, U2, ub2, ue2);
-            const unsigned long long* nxt = static_cast<const unsigned long long*>(mm.m[i + 1].weights) + ub2 * 32;
+            const uint32_t ub2 = split_begin(mm.m[i + 1].sp, blockIdx.x), ue2 = split_begin(mm.m[i + 1].sp, blockIdx.x + 1u);
+            const unsigned long long* nxt = static_cast<const unsigned long long*>(mm.m[i + 1].weights) + (uint64_t)ub2 * 32;
             for (int c = lane; c < 64 && ub2 + c / 2 < ue2; c += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt + c * 16));
         }
         uint32_t ch = 0;
@@ -570,14 +561,13 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
             const uint64_t I = e & kSortIndexMask;
             const uint32_t pos = (uint32_t)(e >> 48);
             const bool valid = I != kSortIndexMask && I < fa.n_points;
-            const uint32_t v = kq_a + (pos >> 5);
-            uint32_t q = __umulhi(v, M.nq_magic), kq = v - q * nq32;
-            if (kq >= nq32) { kq -= nq32; ++q; }
+            uint32_t kq;
+            const uint32_t q = split_row(sp, kq_a + (pos >> 5), kq);
             const uint32_t rloc = q * kGemvGroupRows + ((pos >> 2) & 7u);                 // row inside the CTA's share
             const uint32_t cb = kq * 4u + (pos & 3u);
             float gn = 0.f;
             uint16_t gbits = 0;
-            if (valid) gbits = ldg_u16_here(M.gain + ((int64_t)rg0 * kGemvGroupRows + rloc) * bpr + cb);
+            if (valid) gbits = ldg_u16_here(gain_pass + (rloc * bpr + cb));
             Decoded r;
             decode_sorted_entry(fa, T, I, valid, r);
             gn = gain_to_float(gbits);
@@ -589,6 +579,7 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
             const float dot = dot24_bf16(w, xv);
             if (valid) atomicAdd(&acc[(warp & (kSortAccCopies - 1)) * acc_rows + rloc], dot);
             ch = nxt; e = e_next;
+            use_from_here(e);
         }
         // out of chunks: count this warp in; the last one ends the pass and hands the set on
         __threadfence_block();
@@ -599,13 +590,13 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
             __threadfence_block();
             YOut yo{};
             yo.y = M.y;
-            auto row_sum = [&](int64_t rr) {
+            auto row_sum = [&](uint32_t rr) {
                 float vv = 0.f;
 #pragma unroll
                 for (int c = 0; c < kSortAccCopies; ++c) vv += acc[c * acc_rows + rr];
                 return vv;
             };
-            if (ub < ue) finish_pass<kOutBf16, false>(yo, rg0, rg1, nq, ub, ue, U, G, M.n_out, scratch, counters, row_sum, M.slot0, 0, 1);
+            finish_pass<kOutBf16, false>(yo, sp, rg0, split_row(sp, ue - 1u), ub, ue, M.n_out, scratch, counters, row_sum, M.slot0, 0, 1);
             __syncwarp();
             if (i + kOverlapSets < mm.n) {
                 if (lane == 0) { ctl[set].next_chunk = 0u; ctl[set].arrived = 0u; }
@@ -632,13 +623,12 @@ constexpr int kBinPerThread = kBinSegUnits * 32 / kSortThreads;   // 8
 // of time; the binning phases then read it from L2.
 template <bool kSg>
 __device__ __forceinline__ void prefetch_bin_span(const FastArgs& fa, const uint32_t* stream, const uint16_t* gain, const SgArgs& sg,
-                                                  int64_t n_out, int64_t bpr)
+                                                  const Split& sp, int64_t n_out, int64_t bpr)
 {
-    const int64_t nq0 = (bpr + 3) / 4, U0 = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq0;
-    const int64_t ub = blockIdx.x * U0 / gridDim.x, ue = (blockIdx.x + 1) * U0 / gridDim.x;
+    const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);
     if (ub < ue) {
-        const uint64_t b_first = (uint64_t)(ub / nq0) * kGemvGroupRows * (uint64_t)bpr;
-        const uint64_t b_last = (uint64_t)min(((ue - 1) / nq0 + 1) * kGemvGroupRows, n_out) * (uint64_t)bpr;
+        const uint64_t b_first = (uint64_t)split_row(sp, ub) * kGemvGroupRows * (uint64_t)bpr;
+        const uint64_t b_last = (uint64_t)min((int64_t)(split_row(sp, ue - 1u) + 1u) * kGemvGroupRows, n_out) * (uint64_t)bpr;
         const uint64_t wf = (uint64_t)fa.L.W + (kSg ? (uint64_t)sg.bits : 0ull);
         prefetch_span_l2(stream, b_first * wf / 8, (b_last * wf + 7) / 8);
         if (!kSg) prefetch_span_l2(gain, b_first * 2, b_last * 2);
@@ -648,11 +638,11 @@ __device__ __forceinline__ void prefetch_bin_span(const FastArgs& fa, const uint
 template <bool kOutBf16, bool kSg, bool kShard>
 __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem& T, uint8_t* staging, const uint32_t* __restrict__ stream,
                                               const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, const SgArgs& sg,
-                                              int64_t n_out, int64_t k_in, int64_t bpr, uint32_t nq_magic, int seg_units,
+                                              const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, int seg_units,
                                               const uint16_t* __restrict__ x, const YOut& yo, float* __restrict__ scratch,
                                               uint32_t* __restrict__ counters, int64_t slot0)
 {
-    const int64_t nq = (bpr + 3) / 4;
+    const uint32_t nq = sp.per_row;
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
     float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccCopies][kGemvGroupsPerPass][8]
     uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows);
@@ -661,20 +651,17 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
     uint32_t* cursor = hist + 1024;                                  // [1024]
     unsigned long long* ent = reinterpret_cast<unsigned long long*>(cursor + 1024);   // [seg_units * 32] class-local index | position << 48
     uint16_t* ent_cls = reinterpret_cast<uint16_t*>(ent + seg_units * 32);            // [seg_units * 32] class (| gain index << 10), 0xffff = no block
-    stage_x(xs, x, k_in, nq * 48);
+    stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t kWarps = blockDim.x >> 5;
-    const int64_t groups = (n_out + kGemvGroupRows - 1) / kGemvGroupRows;
-    const int64_t U = groups * nq, G = gridDim.x;
-    const uint32_t nq32 = (uint32_t)nq;
-    for_each_sorted_segment(U, G, nq, blockIdx.x, [&](int64_t tu0, int64_t tu1, int64_t rg0, int64_t rg1, bool first, bool last) {
+    for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t rg0, uint32_t rg1, bool first, bool last) {
         if (first)
             for (int i = threadIdx.x; i < kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows; i += (int)blockDim.x) acc[i] = 0.f;
         hist[threadIdx.x] = 0; cursor[threadIdx.x] = 0;
         if (threadIdx.x == 0) *next_chunk = kWarps;
         __syncthreads();
-        const int64_t rg_a = tu0 / nq;
-        const uint32_t kq_a = (uint32_t)(tu0 - rg_a * nq), rg_off = (uint32_t)(rg_a - rg0);
+        uint32_t kq_a;
+        const uint32_t rg_a = split_row(sp, tu0, kq_a), rg_off = rg_a - rg0;
         const int entries = (int)(tu1 - tu0) * 32;
         // ---- S1-S2 for the whole segment and the histogram of the sort keys
         unsigned long long mine_ent[kBinPerThread];
@@ -685,10 +672,9 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
             mine_key[q] = 0xffffffffu; mine_ent[q] = 0ull;
             if (i < entries) {
                 const uint32_t pos = (uint32_t)i;
-                const uint32_t v = kq_a + (pos >> 5);
-                uint32_t qd = __umulhi(v, nq_magic), kq = v - qd * nq32;
-                if (kq >= nq32) { kq -= nq32; ++qd; }
-                const int64_t row = (rg_a + qd) * kGemvGroupRows + ((pos >> 2) & 7u), cb = (int64_t)kq * 4 + (pos & 3u);
+                uint32_t kq;
+                const uint32_t qd = split_row(sp, kq_a + (pos >> 5), kq);
+                const int64_t row = (int64_t)(rg_a + qd) * kGemvGroupRows + ((pos >> 2) & 7u), cb = (int64_t)kq * 4 + (pos & 3u);
                 uint32_t key = 1023u, cls = 0xffffu;
                 uint64_t local = 0;
                 if (row < n_out && cb < bpr) {
@@ -732,8 +718,8 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
         }
         __syncthreads();
         // ---- S3-S8 on the ordered entries
-        const uint32_t nchunks = (uint32_t)(tu1 - tu0);
-        const uint16_t* gain_pass = gain + rg0 * kGemvGroupRows * bpr;
+        const uint32_t nchunks = tu1 - tu0;
+        const uint16_t* gain_pass = gain + (int64_t)rg0 * kGemvGroupRows * bpr;
         for (uint32_t ch = (uint32_t)warp; ch < nchunks;) {
             uint32_t nxt = 0;
             if (lane == 0) nxt = atomicAdd(next_chunk, 1u);
@@ -742,9 +728,8 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
             const uint32_t cls16 = ent_cls[ch * 32 + lane];
             const bool valid = cls16 != 0xffffu;
             const uint32_t pos = (uint32_t)(e >> 48);
-            const uint32_t v = kq_a + (pos >> 5);
-            uint32_t q = __umulhi(v, nq_magic), kq = v - q * nq32;
-            if (kq >= nq32) { kq -= nq32; ++q; }
+            uint32_t kq;
+            const uint32_t q = split_row(sp, kq_a + (pos >> 5), kq);
             const uint32_t rloc = (rg_off + q) * kGemvGroupRows + ((pos >> 2) & 7u);
             const uint32_t cb = kq * 4u + (pos & 3u);
             const uint32_t cls = valid ? (kSg ? cls16 & 1023u : cls16) : 0u;
@@ -755,7 +740,7 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
                     const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rg0 * kGemvGroupRows + rloc) : 1.f;
                     gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + (cls16 >> 10))), __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
                 } else {
-                    gbits = ldg_u16_here(gain_pass + (int64_t)rloc * bpr + cb);
+                    gbits = ldg_u16_here(gain_pass + (rloc * bpr + cb));
                 }
             }
             Decoded r;
@@ -772,27 +757,27 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
         }
         __syncthreads();
         if (!last) return;
-        auto row_sum = [&](int64_t r) {
+        auto row_sum = [&](uint32_t r) {
             float v = 0.f;
 #pragma unroll
             for (int c = 0; c < kSortAccCopies; ++c) v += acc[c * (kGemvGroupsPerPass * kGemvGroupRows) + r];
             return v;
         };
-        const int64_t ub = blockIdx.x * U / G, ue = (blockIdx.x + 1) * U / G;     // recomputed here: nothing 64-bit lives across the main loop
-        finish_pass<kOutBf16, kShard>(yo, rg0, rg1, nq, ub, ue, U, G, n_out, scratch, counters, row_sum, slot0);
+        const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sum, slot0);
         __syncthreads();
-    }, seg_units);
+    }, (uint32_t)seg_units);
 }
 
 template <bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_bin_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, SgArgs sg,
-                int64_t n_out, int64_t k_in, int64_t bpr, uint32_t nq_magic, int seg_units, const uint16_t* __restrict__ x, YOut yo,
+                Split sp, int64_t n_out, int64_t k_in, int64_t bpr, int seg_units, const uint16_t* __restrict__ x, YOut yo,
                 float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
-    prefetch_bin_span<kSg>(fa, stream, gain, sg, n_out, bpr);       // while the table image is on its way
+    prefetch_bin_span<kSg>(fa, stream, gain, sg, sp, n_out, bpr);       // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
-    gemv_bin_body<kOutBf16, kSg, kShard>(fa, T, staging, stream, sort_rank, gain, sg, n_out, k_in, bpr, nq_magic, seg_units, x, yo, scratch, counters, 0);
+    gemv_bin_body<kOutBf16, kSg, kShard>(fa, T, staging, stream, sort_rank, gain, sg, sp, n_out, k_in, (uint32_t)bpr, seg_units, x, yo, scratch, counters, 0);
     if (kShard) shard_arrive(yo);
 }
 
@@ -802,17 +787,17 @@ __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const __grid_constant__ GemvMulti mm, float* __restrict__ scratch,
                       uint32_t* __restrict__ counters)
 {
-    prefetch_bin_span<false>(fa, static_cast<const uint32_t*>(mm.m[0].weights), mm.m[0].gain, SgArgs{}, mm.m[0].n_out, (mm.m[0].k_in + 23) / 24);
+    prefetch_bin_span<false>(fa, static_cast<const uint32_t*>(mm.m[0].weights), mm.m[0].gain, SgArgs{}, mm.m[0].sp, mm.m[0].n_out, mm.m[0].bpr);
     FAST_PROLOGUE();
     for (int i = 0; i < mm.n; ++i) {
         const GemvMat& M = mm.m[i];
         if (i + 1 < mm.n)
-            prefetch_bin_span<false>(fa, static_cast<const uint32_t*>(mm.m[i + 1].weights), mm.m[i + 1].gain, SgArgs{}, mm.m[i + 1].n_out,
-                                     (mm.m[i + 1].k_in + 23) / 24);
+            prefetch_bin_span<false>(fa, static_cast<const uint32_t*>(mm.m[i + 1].weights), mm.m[i + 1].gain, SgArgs{}, mm.m[i + 1].sp,
+                                     mm.m[i + 1].n_out, mm.m[i + 1].bpr);
         YOut yo{};
         yo.y = M.y;
-        gemv_bin_body<kOutBf16, false, false>(fa, T, staging, static_cast<const uint32_t*>(M.weights), sort_rank, M.gain, SgArgs{}, M.n_out, M.k_in,
-                                              (M.k_in + 23) / 24, M.nq_magic, M.seg_units, M.x, yo, scratch, counters, M.slot0);
+        gemv_bin_body<kOutBf16, false, false>(fa, T, staging, static_cast<const uint32_t*>(M.weights), sort_rank, M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
+                                              (uint32_t)M.bpr, M.seg_units, M.x, yo, scratch, counters, M.slot0);
         __syncthreads();
     }
 }

@@ -69,15 +69,77 @@ struct FastArgs {
     DevCode dc;                     // class tables in global memory (big codes)
 };
 
+// How the work of a product is shared out: `units` pieces in rows of `per_row` (GEMV: units of 8 rows x 4 column blocks, a row =
+// the units of a row group; GEMM: domains of 128 rows x 8 column blocks, a row = the domains of a row tile), numbered row by row;
+// CTA c of `ctas` takes the units [c * units / ctas, (c + 1) * units / ctas).  The divisions are taken with constants the host
+// prepares: a 64-bit division is a dependent chain of some hundred instructions, and ten of them, by every warp, stood at the
+// start and the end of each pass (gemv_sorted 512 x 1024: 8.8 -> 7.7 us; three layers of a 7B step in one launch: 106.7 -> 95.8 us).
+struct Split {
+    uint32_t units, ctas, each, rest;        // each = units / ctas, rest = units % ctas
+    uint32_t ctas_magic;                     // ceil(2^32 / ctas): exact quotients of numbers below ctas^2 (ctas < 1625)
+    uint32_t per_row, row_magic;             // floor(2^32 / per_row): quotients at most one too small
+    float ctas_per_unit;
+};
+
+Split make_split(int64_t units, int64_t per_row, unsigned ctas)
+{
+    Split s;
+    s.units = (uint32_t)units; s.ctas = ctas; s.each = s.units / ctas; s.rest = s.units % ctas;
+    s.ctas_magic = (uint32_t)(((1ull << 32) + ctas - 1) / ctas);
+    s.per_row = (uint32_t)per_row;
+    s.row_magic = per_row == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)per_row);
+    s.ctas_per_unit = (float)((double)ctas / (double)units);
+    return s;
+}
+
+// First unit of CTA c (c <= ctas).
+__device__ __forceinline__ uint32_t split_begin(const Split& s, uint32_t c) { return c * s.each + __umulhi(c * s.rest, s.ctas_magic); }
+
+// Row of unit u and its place in the row.
+__device__ __forceinline__ uint32_t split_row(const Split& s, uint32_t u, uint32_t& place)
+{
+    uint32_t q = __umulhi(u, s.row_magic);
+    place = u - q * s.per_row;
+    if (place >= s.per_row) { place -= s.per_row; ++q; }
+    return q;
+}
+__device__ __forceinline__ uint32_t split_row(const Split& s, uint32_t u) { uint32_t place; return split_row(s, u, place); }
+
+// CTA that owns unit u: an estimate within one of it, put right by the ranges themselves.
+__device__ __forceinline__ uint32_t split_owner(const Split& s, uint32_t u)
+{
+    uint32_t c = min((uint32_t)((float)u * s.ctas_per_unit), s.ctas - 1u);
+    while (split_begin(s, c) > u) --c;
+    while (split_begin(s, c + 1u) <= u) ++c;
+    return c;
+}
+
 // One block of 24 weights, end to end, in the two forms the consumers use.  kBig selects the decoder for codes
 // whose class tables live in global memory; otherwise everything is served from the shared-memory image.
 // All 32 lanes of a warp call these together; `in` = the block exists.
-// The table-driven decoder of the codes whose class tables stay in global memory, from the stored stream.
-__device__ __forceinline__ void block_planes_big(const FastArgs& fa, const FastSmem& T, const uint32_t* __restrict__ stream,
-                                                 uint64_t b, bool in, DecodedBig& d)
+// A block's stored field (and gain), requested ahead of its turn.
+template <bool kBig>
+struct RawBlock {
+    RawField<kBig> field;
+    uint16_t gain;
+};
+
+// wbits = bits of a stored field; gain == nullptr: none is read.
+template <bool kBig>
+__device__ __forceinline__ RawBlock<kBig> request_block(const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, int wbits, uint64_t b, bool in)
 {
-    uint64_t lo = 0, hi = 0;
-    if (in) load_index(stream, b, fa.dc.W, lo, hi);
+    RawBlock<kBig> r;
+    r.field = request_field<kBig>(stream, b, wbits, in);
+    r.gain = 0;
+    if (gain != nullptr && in) r.gain = ldg_u16_here(gain + b);
+    return r;
+}
+
+// The table-driven decoder of the codes whose class tables stay in global memory, from the stored stream.
+__device__ __forceinline__ void block_planes_big(const FastArgs& fa, const FastSmem& T, const RawField<true>& f, bool in, DecodedBig& d)
+{
+    uint64_t lo, hi;
+    field_value(f, fa.dc.W, lo, hi);
     const bool valid = in && (hi < fa.dc.n_hi || (hi == fa.dc.n_hi && lo < fa.dc.n_lo));
     if (in && !valid) atomicAdd(fa.bad_index, 1ull);
     uint64_t local = 0;
@@ -85,44 +147,45 @@ __device__ __forceinline__ void block_planes_big(const FastArgs& fa, const FastS
     big_decode_planes(T, fa.dc, cls, local, valid, kFullMask, d);
 }
 
-template <bool kBig>
-__device__ __forceinline__ void block_bytes(const FastArgs& fa, const FastSmem& T, const uint32_t* __restrict__ stream,
-                                            uint64_t b, bool in, uint32_t w[6])
+__device__ __forceinline__ void block_planes(const FastArgs& fa, const FastSmem& T, const RawField<false>& f, bool in, Decoded& d)
 {
-    if (kBig) {
+    uint64_t I, none;
+    field_value(f, (int)fa.L.W, I, none);
+    const bool valid = in && I < fa.n_points;
+    if (in && !valid) atomicAdd(fa.bad_index, 1ull);
+    fast_decode(T, I, valid, d);
+}
+
+template <bool kBig>
+__device__ __forceinline__ void block_bytes(const FastArgs& fa, const FastSmem& T, const RawField<kBig>& f, bool in, uint32_t w[6])
+{
+    if constexpr (kBig) {
         DecodedBig d{};
-        block_planes_big(fa, T, stream, b, in, d);
+        block_planes_big(fa, T, f, in, d);
         Decoded three = d.d;
         three.neg &= ~d.p3;                               // those positions are written by the patch (a negated zero filler would carry)
         expand_bytes(three, w);
         patch_id8_bytes(d, w);
     } else {
-        const uint64_t I = in ? load_field(stream, b, (int)fa.L.W) : 0ull;
-        const bool valid = in && I < fa.n_points;
-        if (in && !valid) atomicAdd(fa.bad_index, 1ull);
         Decoded d;
-        fast_decode(T, I, valid, d);
+        block_planes(fa, T, f, in, d);
         expand_bytes(d, w);
     }
 }
 
 template <bool kBig>
-__device__ __forceinline__ void block_pairs(const FastArgs& fa, const FastSmem& T, const uint32_t* __restrict__ stream,
-                                            const uint16_t* __restrict__ gain, uint64_t b, bool in, uint32_t w[12])
+__device__ __forceinline__ void block_pairs(const FastArgs& fa, const FastSmem& T, const RawBlock<kBig>& r, bool in, uint32_t w[12])
 {
-    const float g = in ? gain_to_float(__ldg(gain + b)) : 0.f;
-    if (kBig) {
+    if constexpr (kBig) {
         DecodedBig d{};
-        block_planes_big(fa, T, stream, b, in, d);
+        block_planes_big(fa, T, r.field, in, d);
+        const float g = gain_to_float(r.gain);
         expand_bf16(d.d, g, w);
         patch_id8_bf16(d, g, w);
     } else {
-        const uint64_t I = in ? load_field(stream, b, (int)fa.L.W) : 0ull;
-        const bool valid = in && I < fa.n_points;
-        if (in && !valid) atomicAdd(fa.bad_index, 1ull);
         Decoded d;
-        fast_decode(T, I, valid, d);
-        expand_bf16(d, g, w);
+        block_planes(fa, T, r.field, in, d);
+        expand_bf16(d, gain_to_float(r.gain), w);
     }
 }
 
@@ -135,10 +198,11 @@ struct SgArgs {
     int bits;
 };
 
-__device__ __forceinline__ void block_pairs_sg(const FastArgs& fa, const FastSmem& T, const uint32_t* __restrict__ stream,
-                                               const SgArgs& sg, uint64_t b, int64_t row, bool in, uint32_t w[12])
+__device__ __forceinline__ void block_pairs_sg(const FastArgs& fa, const FastSmem& T, const RawField<false>& raw,
+                                               const SgArgs& sg, int64_t row, bool in, uint32_t w[12])
 {
-    const uint64_t f = in ? load_field(stream, b, (int)fa.L.W + sg.bits) : 0ull;
+    uint64_t f, none;
+    field_value(raw, (int)fa.L.W + sg.bits, f, none);
     const uint64_t I = f & ((1ull << fa.L.W) - 1ull);                 // W < 64 whenever gain bits are present or not: checked on the host
     const uint32_t k = (uint32_t)(f >> fa.L.W);
     const bool valid = in && I < fa.n_points;
@@ -160,6 +224,10 @@ __device__ __forceinline__ void block_pairs_sg(const FastArgs& fa, const FastSme
 // loaded its table image, before it reads anything a predecessor may have written (x, the scratch, the counters).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Keeps what is computed from v (a load in flight) behind this point: the compiler otherwise pulls the first steps of the next
+// round of a loop up to the load and waits for it there.
+__device__ __forceinline__ void use_from_here(unsigned long long& v) { asm volatile("" : "+l"(v)); }
 
 // Ask for the 128-byte lines of [p + first, p + last) in L2; the whole CTA calls this.
 __device__ __forceinline__ void prefetch_span_l2(const void* p, uint64_t first, uint64_t last)

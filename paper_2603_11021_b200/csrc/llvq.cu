@@ -10,40 +10,81 @@ decode_blocks_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, uint
 {
     FAST_PROLOGUE();
     const uint64_t ntiles = (nblocks + kFastThreads - 1) / kFastThreads;
+    uint64_t b = (uint64_t)blockIdx.x * kFastThreads + threadIdx.x;
+    RawField<kBig> raw = request_field<kBig>(stream, b, fa.dc.W, b < nblocks);
     for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint64_t b = tile * kFastThreads + threadIdx.x;
         const bool in = b < nblocks;
+        const uint64_t b_next = b + (uint64_t)gridDim.x * kFastThreads;
+        RawField<kBig> raw_next = request_field<kBig>(stream, b_next, fa.dc.W, b_next < nblocks);
         uint32_t w[6];
-        block_bytes<kBig>(fa, T, stream, b, in, w);
+        block_bytes<kBig>(fa, T, raw, in, w);
         if (in) {
             out[b * 3 + 0] = make_uint2(w[0], w[1]);
             out[b * 3 + 1] = make_uint2(w[2], w[3]);
             out[b * 3 + 2] = make_uint2(w[4], w[5]);
         }
+        b = b_next; raw = raw_next;
+        use_field_from_here(raw);
     }
 }
 
 // FLAT (bpr == 0): block b covers elements 24b.. of the flattened matrix.
-// ROWWISE: block b = r * bpr + cb covers columns 24cb.. of row r.
+// ROWWISE: block b = r * bpr + cb covers columns 24cb.. of row r.  A thread's blocks are gridDim.x * kFastThreads apart: (r, cb)
+// moves by the same (step_r, step_c) every time, so there is one division per thread and none per block.
+struct RowWalk {
+    uint32_t bpr, bpr_magic;      // bpr_magic = floor(2^32 / bpr)
+    uint32_t step_r, step_c;      // gridDim.x * kFastThreads = step_r * bpr + step_c
+};
+
+RowWalk row_walk(int64_t bpr, unsigned grid)
+{
+    RowWalk w{};
+    if (bpr == 0) return w;
+    const uint64_t step = (uint64_t)grid * kFastThreads;
+    w.bpr = (uint32_t)bpr;
+    w.bpr_magic = bpr == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)bpr);
+    w.step_r = (uint32_t)(step / (uint64_t)bpr); w.step_c = (uint32_t)(step % (uint64_t)bpr);
+    return w;
+}
+
 template <bool kBig, bool kSg = false>
 __global__ void __launch_bounds__(kFastThreads, 1)
 dequant_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, uint64_t nblocks,
-                    int64_t rows, int64_t cols, int64_t bpr, __nv_bfloat16* __restrict__ out, int64_t ld)
+                    int64_t rows, int64_t cols, RowWalk walk, __nv_bfloat16* __restrict__ out, int64_t ld)
 {
     FAST_PROLOGUE();
+    uint32_t r = 0, cb = 0;
+    if (walk.bpr) {
+        const uint32_t b0 = blockIdx.x * kFastThreads + threadIdx.x;
+        r = __umulhi(b0, walk.bpr_magic);
+        cb = b0 - r * walk.bpr;
+        if (cb >= walk.bpr) { cb -= walk.bpr; ++r; }
+    }
     const uint64_t ntiles = (nblocks + kFastThreads - 1) / kFastThreads;
     const uint64_t total = (uint64_t)rows * (uint64_t)cols;
+    const int wbits = fa.dc.W + (kSg ? sg.bits : 0);
+    uint64_t b = (uint64_t)blockIdx.x * kFastThreads + threadIdx.x, b_next = b;
+    RawBlock<kBig> raw_next = request_block<kBig>(stream, kSg ? nullptr : gain, wbits, b, b < nblocks);
     for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint64_t b = tile * kFastThreads + threadIdx.x;
+        // a block's words are requested while the one before it is unranked
+        RawBlock<kBig> raw = raw_next;
+        use_field_from_here(raw.field);
+        b = b_next;
         const bool in = b < nblocks;
+        b_next = b + (uint64_t)gridDim.x * kFastThreads;
+        raw_next = request_block<kBig>(stream, kSg ? nullptr : gain, wbits, b_next, b_next < nblocks);
         uint32_t w[12];
-        if (kSg) block_pairs_sg(fa, T, stream, sg, b, in ? (int64_t)(b / (uint64_t)bpr) : 0, in, w);   // ROWWISE only
-        else block_pairs<kBig>(fa, T, stream, gain, b, in, w);        // whole warp: the decoders vote
-        if (!in) continue;
+        if constexpr (kSg) block_pairs_sg(fa, T, raw.field, sg, in ? (int64_t)r : 0, in, w);   // ROWWISE only
+        else block_pairs<kBig>(fa, T, raw, in, w);                    // whole warp: the decoders vote
         __nv_bfloat16* dst;
         int64_t left;
-        if (bpr == 0) { dst = out + b * 24; left = (int64_t)(total - b * 24); }
-        else { const int64_t r = (int64_t)(b / (uint64_t)bpr), cb = (int64_t)(b % (uint64_t)bpr); dst = out + r * ld + cb * 24; left = cols - cb * 24; }
+        if (walk.bpr == 0) { dst = out + b * 24; left = (int64_t)(total - b * 24); }
+        else {
+            dst = out + (int64_t)r * ld + (int64_t)cb * 24; left = cols - (int64_t)cb * 24;
+            cb += walk.step_c; r += walk.step_r;
+            if (cb >= walk.bpr) { cb -= walk.bpr; ++r; }
+        }
+        if (!in) continue;
         if (left >= 24 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
             uint4* d4 = reinterpret_cast<uint4*>(dst);
             d4[0] = make_uint4(w[0], w[1], w[2], w[3]);
@@ -301,11 +342,11 @@ int llvq_dequant_matrix(const llvq_ctx* ctx, const void* d_idx, const uint16_t* 
     if (ctx->fast) {
         if (!set_smem<dequant_fast_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(dequant_fast_kernel<false, false>, g, (unsigned)kFastThreads, smem, st, fast_args(ctx, false), idx, d_gain_f16, SgArgs{}, (uint64_t)nblocks,
-                       rows, cols, bpr, w, ld) != cudaSuccess) return LLVQ_ECUDA;
+                       rows, cols, row_walk(bpr, g), w, ld) != cudaSuccess) return LLVQ_ECUDA;
     } else {
         if (!set_smem<dequant_fast_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
         if (launch_pdl(dequant_fast_kernel<true, false>, g, (unsigned)kFastThreads, smem, st, fast_args(ctx, false), idx, d_gain_f16, SgArgs{}, (uint64_t)nblocks,
-                       rows, cols, bpr, w, ld) != cudaSuccess) return LLVQ_ECUDA;
+                       rows, cols, row_walk(bpr, g), w, ld) != cudaSuccess) return LLVQ_ECUDA;
     }
     return launch_status();
 }
@@ -336,7 +377,7 @@ int llvq_dequant_matrix_sg(const llvq_ctx* ctx, const void* d_fields, int gain_b
     if (!set_smem<dequant_fast_kernel<false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
     dequant_fast_kernel<false, true><<<g, kFastThreads, smem, (cudaStream_t)stream>>>(
         fast_args(ctx, false), static_cast<const uint32_t*>(d_fields), nullptr, SgArgs{d_codebook_f32, d_row_scale_f32, gain_bits},
-        nblocks, rows, cols, bpr, reinterpret_cast<__nv_bfloat16*>(d_w_bf16), ld);
+        nblocks, rows, cols, row_walk(bpr, g), reinterpret_cast<__nv_bfloat16*>(d_w_bf16), ld);
     return launch_status();
 }
 
