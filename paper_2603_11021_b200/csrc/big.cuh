@@ -79,11 +79,11 @@ __device__ __forceinline__ void big_decode_record(const FastSmem& T, const uint4
     uint64_t p = q >> B;
 
     // S4: Golay codeword
-    const uint32_t c = T.golay[goff + r];
+    const uint32_t word_c = T.golay[goff + r], c = word_c & kAllCoords;
 
     // S5: arrangement.  Group 1 on F1(c), then group 0 on F0(c) (odd classes: one group 0 on all positions).
     const uint32_t F1 = odd ? 0u : c;
-    const uint32_t F0 = ~F1 & 0xffffffu;
+    const uint32_t F0 = ~F1 & kAllCoords;
     uint32_t freem = F1, nfree = odd ? 0u : w;
     bool in_group0 = false;
     uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0, bit1 = 0, nz0 = 0;
@@ -119,7 +119,7 @@ __device__ __forceinline__ void big_decode_record(const FastSmem& T, const uint4
                 if (active) { p = qq; rho = rem; }
             }
             uint32_t rel;
-            if (T.sub3 != 0u && __all_sync(mask, k <= (uint32_t)kSmallSubsetMaxK)) rel = small_subset(T, k, rho);
+            if (T.sub3 != 0u && __all_sync(mask, k <= (uint32_t)kSmallSubsetMaxK)) rel = small_subset(T.sub3, k, rho);
             else rel = nth_subset(T, k, rho, (int)__reduce_max_sync(mask, active ? nfree : 0u));
             const uint32_t a = deposit24(T.pd6, rel, freem);
             freem ^= a; nfree -= k;
@@ -145,7 +145,7 @@ __device__ __forceinline__ void big_decode_record(const FastSmem& T, const uint4
     else {
         // the bits of s go to the positions that carry a sign (F1 and the nonzero ones of F0) in ascending order, except the
         // last F1 position: its sign makes the sum 0 mod 8
-        const uint32_t last_f1 = F1 ? 0x80000000u >> __clz(F1) : 0u;
+        const uint32_t last_f1 = 1u << (((word_c & kLastPosBits) * kLastPosGather) >> 27);      // bit 31 for the zero word
         uint32_t neg_even = deposit24(T.pd6, s, (F1 | (odd ? 0u : nz0)) & ~last_f1);
         if ((__popc(neg_even & F1) + (flags >> 1)) & 1u) neg_even |= last_f1;
         neg = odd ? (c ^ bit1) : neg_even;
@@ -185,9 +185,10 @@ __device__ __forceinline__ void patch_id8_bf16(const DecodedBig& b, float gain, 
     const uint32_t v = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(gain * (float)b.val8));
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
-        const uint32_t lo = (b.p3 >> (2 * j)) & 1u, hi = (b.p3 >> (2 * j + 1)) & 1u;
+        const int at = 8 * (j / 3) + j % 3;                         // coordinates 2j and 2j + 1: bits at and at + 4
+        const uint32_t lo = (b.p3 >> at) & 1u, hi = (b.p3 >> (at + 4)) & 1u;
         const uint32_t m = (lo ? 0xffffu : 0u) | (hi ? 0xffff0000u : 0u);
-        const uint32_t sg = (((b.d.neg >> (2 * j)) & 1u) << 15) | (((b.d.neg >> (2 * j + 1)) & 1u) << 31);
+        const uint32_t sg = (((b.d.neg >> at) & 1u) << 15) | (((b.d.neg >> (at + 4)) & 1u) << 31);
         w[j] = (w[j] & ~m) | (((v | v << 16) ^ sg) & m);
     }
 }
@@ -197,8 +198,9 @@ __device__ __forceinline__ void patch_id8_bytes(const DecodedBig& b, uint32_t ou
     if (!__any_sync(kFullMask, b.p3 != 0u)) return;
 #pragma unroll
     for (int i = 0; i < 24; ++i) {
-        if ((b.p3 >> i) & 1u) {
-            const uint32_t byte = ((b.d.neg >> i) & 1u) ? (0u - b.val8) & 0xffu : b.val8;
+        const int at = 8 * (i / 6) + 4 * (i & 1) + (i % 6) / 2;
+        if ((b.p3 >> at) & 1u) {
+            const uint32_t byte = ((b.d.neg >> at) & 1u) ? (0u - b.val8) & 0xffu : b.val8;
             out[i >> 2] = (out[i >> 2] & ~(0xffu << (8 * (i & 3)))) | byte << (8 * (i & 3));
         }
     }

@@ -14,6 +14,7 @@ struct EncTables {
     const uint32_t* hash_cls = nullptr;       // [hash_size] its class number
     uint32_t hash_mask = 0;                   // hash_size - 1 (a power of two)
     const uint64_t* sig_of_value = nullptr;   // [64] signature contribution of one coordinate of absolute value a
+    const uint32_t* pascal = nullptr;         // [25 * 25] C(n, k) at n * 25 + k
     const llvq::GolayTrio* trio = nullptr;    // the Golay code along a trio of octads (search)
 };
 

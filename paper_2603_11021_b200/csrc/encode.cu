@@ -508,9 +508,8 @@ int status_of_launch() { return cudaGetLastError() == cudaSuccess ? LLVQ_OK : LL
 
 int launch_rank(const llvq_ctx* ctx, const int8_t* d_points, uint64_t nblocks, uint64_t* d_index, cudaStream_t st)
 {
-    const uint32_t* pascal = reinterpret_cast<const uint32_t*>(ctx->d_image + ctx->fl.pascal);
     const unsigned grid = (unsigned)((nblocks + 255) / 256);
-    rank_kernel<<<grid, 256, 0, st>>>(ctx->dev, ctx->enc, ctx->d_golay, pascal, d_points, nblocks,
+    rank_kernel<<<grid, 256, 0, st>>>(ctx->dev, ctx->enc, ctx->d_golay, ctx->enc.pascal, d_points, nblocks,
                                       reinterpret_cast<unsigned long long*>(d_index));
     return status_of_launch();
 }

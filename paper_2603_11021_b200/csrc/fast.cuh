@@ -25,7 +25,7 @@ struct FastSmem {
     const uint32_t* desc;
     const uint64_t* recip64;  // images without class tables: reciprocals of the Pascal entries
     const uint32_t* recip32;
-    uint32_t sub3;            // shared-window byte address of the table of small subsets, 0 when the kernel did not load it
+    uint32_t sub3, sub2;      // shared-window byte addresses of the tables of small subsets, 0 when the kernel did not load them
     uint32_t lut_shift;
 };
 
@@ -46,6 +46,7 @@ __device__ __forceinline__ FastSmem fast_view(const uint8_t* smem, const FastLay
     T.recip64 = reinterpret_cast<const uint64_t*>(smem + L.recip64);
     T.recip32 = reinterpret_cast<const uint32_t*>(smem + L.recip32);
     T.sub3 = with_small_subsets ? smem_addr(smem + L.sub3) : 0u;
+    T.sub2 = with_small_subsets ? smem_addr(smem + L.sub2) : 0u;
     T.lut_shift = L.lut_shift;
     return T;
 }
@@ -89,7 +90,6 @@ __device__ __forceinline__ bool fast_load_image(uint8_t* dst, const uint8_t* __r
     return __syncthreads_and((int)done) != 0;
 }
 
-// Deposit the low bits of src into the set bits of mask, lowest first (24-bit masks, 6 bits per lookup).
 // r = a * b + c on the multiply-add pipe (the logic pipe is the busy one: sums of disjoint bit fields go here)
 __device__ __forceinline__ uint32_t mad_u32(uint32_t a, uint32_t b, uint32_t c)
 {
@@ -98,16 +98,40 @@ __device__ __forceinline__ uint32_t mad_u32(uint32_t a, uint32_t b, uint32_t c)
     return r;
 }
 
+// Deposit the low bits of src into the coordinates of mask (layout of coords_of), lowest coordinate first, six per lookup.  The
+// entry for mask byte f and source bits s is at f * 64 + (s ^ f): a plain table row per f would put every lane whose source bits
+// are used up (s = 0: most lanes, where few slots are taken) into the same two banks whatever f is.  Counted over the classes
+// of the 48-bit code, the 32 lanes of a warp need 30 instead of 55 passes over the banks for the deposits of a block.
 __device__ __forceinline__ uint32_t deposit24(const uint8_t* pd6, uint32_t src, uint32_t mask)
 {
     // how many source bits the lower groups consume: known from the mask alone, so the four lookups are independent
-    const uint32_t c1 = __popc(mask & 0x3fu), c2 = __popc(mask & 0xfffu), c3 = __popc(mask & 0x3ffffu);
-    // row of a lookup = the group's 6 mask bits times 64: for groups 1..3 that is a masked (shifted) copy of the mask
-    const uint32_t r0 = pd6[mad_u32(mask & 0x3fu, 64u, src & 63u)];
-    const uint32_t r1 = pd6[(mask & 0xfc0u) + ((src >> c1) & 63u)];
-    const uint32_t r2 = pd6[((mask >> 6) & 0xfc0u) + ((src >> c2) & 63u)];
-    const uint32_t r3 = pd6[((mask >> 12) & 0xfc0u) + ((src >> c3) & 63u)];
-    return mad_u32(r3, 1u << 18, mad_u32(r2, 1u << 12, mad_u32(r1, 64u, r0)));
+    const uint32_t c1 = __popc(mask & 0xffu), c2 = __popc(mask & 0xffffu), c3 = __popc(mask & 0xffffffu);
+    const uint32_t f1 = __byte_perm(mask, 0u, 0x4441), f2 = __byte_perm(mask, 0u, 0x4442);
+    const uint32_t r0 = pd6[mad_u32(mask & 0xffu, 64u, (src ^ mask) & 63u)];
+    const uint32_t r1 = pd6[mad_u32(f1, 64u, ((src >> c1) ^ f1) & 63u)];
+    const uint32_t r2 = pd6[mad_u32(f2, 64u, ((src >> c2) ^ f2) & 63u)];
+    const uint32_t r3 = pd6[mad_u32(mask >> 24, 64u, ((src >> c3) ^ (mask >> 24)) & 63u)];
+    return mad_u32(r3, 1u << 24, mad_u32(r2, 1u << 16, mad_u32(r1, 256u, r0)));
+}
+
+// The same with every coordinate in the mask: bit i of src -> coordinate i.
+__device__ __forceinline__ uint32_t spread24(const uint8_t* pd6, uint32_t src)
+{
+    const uint8_t* row = pd6 + 0x77 * 64;
+    const uint32_t r0 = row[(src & 63u) ^ 0x37u], r1 = row[((src >> 6) & 63u) ^ 0x37u], r2 = row[((src >> 12) & 63u) ^ 0x37u], r3 = row[(src >> 18) ^ 0x37u];
+    return mad_u32(r3, 1u << 24, mad_u32(r2, 1u << 16, mad_u32(r1, 256u, r0)));
+}
+
+// Quotient of n (below 2^52) by d with inv = 1 / d rounded down, remainder in rem.  On the binary64 pipe, which nothing else uses:
+// n and 2^52 + n / d, truncated, are formed in place in the mantissa; the quotient is at most one too small.
+__device__ __forceinline__ uint64_t divide52(uint64_t n, uint32_t d, double inv, uint32_t& rem)
+{
+    const double nd = __hiloint2double((int)(0x43300000u | (uint32_t)(n >> 32)), (int)(uint32_t)n) - 4503599627370496.0;
+    const double qd = __fma_rz(nd, inv, 4503599627370496.0);
+    uint64_t q = (uint64_t)((uint32_t)__double2hiint(qd) & 0xfffffu) << 32 | (uint32_t)__double2loint(qd);
+    rem = (uint32_t)n - (uint32_t)q * d;
+    if (rem >= d) { rem -= d; ++q; }
+    return q;
 }
 
 template <int kOff>
@@ -143,31 +167,18 @@ __device__ __forceinline__ uint32_t nth_subset(const FastSmem& T, uint32_t k, ui
 }
 
 // The rho-th k-subset of up to 24 slots for k <= 3: one lookup behind a four-word directory (T.sub3 != 0).
-__device__ __forceinline__ uint32_t small_subset(const FastSmem& T, uint32_t k, uint32_t rho)
+// From T.sub2 (k <= 2) it comes in the layout of coords_of.
+__device__ __forceinline__ uint32_t small_subset(uint32_t table, uint32_t k, uint32_t rho)
 {
     uint32_t first, m;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(first) : "r"(T.sub3 + k * 4u));
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(m) : "r"(T.sub3 + (first + rho) * 4u));
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(first) : "r"(table + k * 4u));
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(m) : "r"(table + (first + rho) * 4u));
     return m;
-}
-
-// Deposit into a mask that is 24 ones with at most two holes: open a gap at each hole, lowest first.
-__device__ __forceinline__ uint32_t deposit_two_holes(uint32_t src, uint32_t mask)
-{
-    uint32_t holes = ~mask & 0xffffffu;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const uint32_t b = holes & (0u - holes);          // lowest hole, or 0: then nothing moves
-        const uint32_t low = b - 1u;
-        src = (src & low) | ((src & ~low) << 1);
-        holes ^= b;
-    }
-    return src;
 }
 
 // Result of the index -> point map in a form the consumers expand cheaply:
 // three bit planes giving each position a value id (0..7), the table of
-// absolute values per id, and the mask of negative positions.
+// absolute values per id, and the mask of negative positions (masks in the layout of coords_of; bit 31 of neg may be set).
 struct Decoded {
     uint32_t p0, p1, p2;
     uint32_t neg;
@@ -202,23 +213,18 @@ __device__ __forceinline__ void fast_decode_local(const FastSmem& T, uint32_t cl
     // S3: r fastest, then the sign word s, then the arrangement rank p
     uint64_t q;
     uint32_t r;
-    if (kPar == 1 || (kPar == -1 && A == 4096u)) { r = (uint32_t)local & 4095u; q = local >> 12; }
-    else {
-        q = __umul64hi(local, ((uint64_t)h.w << 32) | h.z);
-        uint64_t rem = local - q * A;
-        if (rem >= A) { rem -= A; ++q; }
-        r = (uint32_t)rem;
-    }
+    if (kPar == 1) { r = (uint32_t)local & 4095u; q = local >> 12; }
+    else q = divide52(local, A, __hiloint2double((int)h.w, (int)h.z), r);
     const uint32_t s = kPar == 1 ? 0u : (uint32_t)q & ((1u << B) - 1u);
     const uint64_t p = kPar == 1 ? q : q >> B;
 
     // S4: Golay codeword
-    const uint32_t c = T.golay[goff + r];
+    const uint32_t word_c = T.golay[goff + r], c = word_c & kAllCoords;
 
     // S5: arrangement.  Group 1 lives on F1(c), group 0 on F0(c); an odd class is one group 0 on all positions.
     const uint32_t F1 = odd ? 0u : c;
-    const uint32_t F0 = ~F1 & 0xffffffu;
-    uint32_t freem = kPar == 1 ? 0xffffffu : F1;
+    const uint32_t F0 = ~F1 & kAllCoords;
+    uint32_t freem = kPar == 1 ? kAllCoords : F1;
     bool in_group0 = kPar == 1;
     uint32_t p0 = 0, p1 = 0, p2 = 0, bit1 = 0, nz0 = 0;
     uint32_t p32 = (uint32_t)p;
@@ -246,30 +252,29 @@ __device__ __forceinline__ void fast_decode_local(const FastSmem& T, uint32_t cl
                 // hold 0 here and place the empty subset), no division
                 rho = p32;
             } else if (l == 0 && !rank32) {
-                uint64_t qq = __umul64hi(p, ((uint64_t)v.w << 32) | v.z);
-                uint64_t rem = p - qq * radix;
-                if (rem >= radix) { rem -= radix; ++qq; }
-                p32 = (uint32_t)qq; rho = (uint32_t)rem;
+                p32 = (uint32_t)divide52(p, radix, __hiloint2double((int)v.w, (int)v.z), rho);
             } else {
                 uint32_t qq = __umulhi(p32, l == 0 ? T.desc[cls * kFastDescStride + kFastDescMagic0] : magics[l]);
                 uint32_t rem = p32 - qq * radix;
                 if (rem >= radix) { rem -= radix; ++qq; }
                 p32 = qq; rho = rem;
             }
-            uint32_t rel;
-            if (T.sub3 != 0u && __all_sync(mask, k <= (uint32_t)kSmallSubsetMaxK)) {
-                rel = small_subset(T, k, rho);                          // few elements: one lookup whatever the number of slots
-            } else {
-                int top;
-                if (kPar == 0) top = 16;
-                else if (kPar == 1 && l == 0) top = 24;
-                else top = __reduce_max_sync(mask, nfree);
-                rel = nth_subset(T, k, rho, top);
-            }
             uint32_t a;
-            if (kPar == 1 && l == 0) a = rel;                           // odd, first step: every position is free
-            else if (kPar == 1 && l == 1 && __all_sync(mask, k == 0u || nfree >= 22u)) a = deposit_two_holes(rel, freem);
-            else a = deposit24(T.pd6, rel, freem);
+            if (kPar == 1 && l == 0 && T.sub2 != 0u && __all_sync(mask, k <= (uint32_t)kSub2MaxK)) {
+                a = small_subset(T.sub2, k, rho);                       // odd, first step: every position is free
+            } else {
+                uint32_t rel;
+                if (T.sub3 != 0u && __all_sync(mask, k <= (uint32_t)kSmallSubsetMaxK)) {
+                    rel = small_subset(T.sub3, k, rho);                 // few elements: one lookup whatever the number of slots
+                } else {
+                    int top;
+                    if (kPar == 0) top = 16;
+                    else if (kPar == 1 && l == 0) top = 24;
+                    else top = __reduce_max_sync(mask, nfree);
+                    rel = nth_subset(T, k, rho, top);
+                }
+                a = kPar == 1 && l == 0 ? spread24(T.pd6, rel) : deposit24(T.pd6, rel, freem);
+            }
             freem ^= a;
             constexpr int kId0 = kPar == 1 ? 1 : 2;                     // the value id of level l is 2 + l (odd classes alone: 1 + l)
             if ((l + kId0) & 1) p0 |= a;
@@ -294,7 +299,7 @@ __device__ __forceinline__ void fast_decode_local(const FastSmem& T, uint32_t cl
     } else {
         // the bits of s go to the positions that carry a sign (F1 and the nonzero ones of F0) in ascending order, except the
         // last F1 position: its sign makes the sum 0 mod 8
-        const uint32_t last_f1 = F1 ? 0x80000000u >> __clz(F1) : 0u;
+        const uint32_t last_f1 = 1u << (((word_c & kLastPosBits) * kLastPosGather) >> 27);      // bit 31 for the zero word
         uint32_t neg_even = deposit24(T.pd6, s, (F1 | (odd ? 0u : nz0)) & ~last_f1);
         if ((__popc(neg_even & F1) + (flags >> 1)) & 1u) neg_even |= last_f1;
         neg = odd ? (c ^ bit1) : neg_even;
@@ -319,76 +324,75 @@ __device__ __forceinline__ void fast_decode(const FastSmem& T, uint64_t I, bool 
 }
 
 // ---- expansion helpers -------------------------------------------------------
-// 8 mask bits -> 8 nibbles (bit i -> bit 4i).
-__device__ __forceinline__ uint32_t nibspread8(uint32_t b)
-{
-    // each "x | x << s" is written as a multiplication (the two copies never overlap): it runs on the FMA pipe,
-    // the integer ALU pipe is the busy one
-    uint32_t x = (b * 0x1001u) & 0x000f000fu;
-    x = (x * 65u) & 0x03030303u;
-    x = (x * 9u) & 0x11111111u;
-    return x;
-}
+constexpr uint32_t kPairs = 0x11111111u;     // bit r of every nibble: the coordinates 6 g + 2 r, 6 g + 2 r + 1 of the four groups
 
-// Value id of each position as a nibble string: sel[r] holds positions 8r..8r+7.
-__device__ __forceinline__ void id_nibbles(const Decoded& d, uint32_t sel[3])
+// Nibble n + 2 g of the result = bits (x, y, z) of coordinate 6 g + 2 r + n.
+template <int r>
+__device__ __forceinline__ uint32_t selectors(uint32_t x, uint32_t y, uint32_t z)
 {
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-        sel[r] = nibspread8((d.p0 >> (8 * r)) & 0xffu) | (nibspread8((d.p1 >> (8 * r)) & 0xffu) << 1) |
-                 (nibspread8((d.p2 >> (8 * r)) & 0xffu) << 2);
+    return ((x >> r) & kPairs) | ((r == 0 ? y << 1 : y >> (r - (r > 0))) & (kPairs << 1)) | ((z << (2 - r)) & (kPairs << 2));
 }
-
-// 4 mask bits -> the most significant bits of 4 bytes.
-__device__ __forceinline__ uint32_t msbspread4(uint32_t nib) { return (nib * 0x10204080u) & 0x80808080u; }
 
 // The 24 coordinates as signed bytes, coordinate i in byte (i & 3) of word (i >> 2).
 __device__ __forceinline__ void expand_bytes(const Decoded& d, uint32_t out[6])
 {
-    uint32_t sel[3];
-    id_nibbles(d, sel);
+    uint32_t t[6];                            // t[r + 3 q]: coordinates 2 r, 2 r + 1 of groups 2 q and 2 q + 1
+    const uint32_t sel[3] = {selectors<0>(d.p0, d.p1, d.p2), selectors<1>(d.p0, d.p1, d.p2), selectors<2>(d.p0, d.p1, d.p2)};
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-        const uint32_t s16 = (j & 1) ? sel[j >> 1] >> 16 : sel[j >> 1];
-        const uint32_t a = __byte_perm(d.vals_lo, d.vals_hi, s16);
-        const uint32_t sm = msbspread4((d.neg >> (4 * j)) & 15u) >> 7;     // bytes 0 / 1
-        out[j] = (a ^ (sm * 0xffu)) + sm;                                     // negated bytes are never zero
+        const uint32_t neg = ((d.neg >> (j % 3)) & kPairs) >> (j < 3 ? 0 : 16);
+        const uint32_t a = __byte_perm(d.vals_lo, d.vals_hi, sel[j % 3] >> (j < 3 ? 0 : 16));
+        t[j] = (a ^ __byte_perm(0xff00u, 0u, neg)) + __byte_perm(0x0100u, 0u, neg);       // negated bytes are never zero
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        out[3 * q] = __byte_perm(t[3 * q], t[3 * q + 1], 0x5410);
+        out[3 * q + 1] = __byte_perm(t[3 * q + 2], t[3 * q], 0x7610);
+        out[3 * q + 2] = __byte_perm(t[3 * q + 1], t[3 * q + 2], 0x7632);
     }
 }
 
 // The 24 dequantized weights bf16_rn(gain * x_i) as 12 packed pairs (weight 2j in the low half of w[j]).
 // All lanes of the warp must call this together: when no lane uses a value id above 3 (codes with few distinct
-// values per class) the third bit plane and the upper half of the value table are skipped.
+// values per class) the upper half of the value table is not formed and the sign takes its place in the selectors: ids 4..7 are
+// the negated values then.
+// The bit planes become selectors by masks and shifts alone because of where the coordinates lie in them (coords_of), 60 instructions
+// in all; with bit i = coordinate i the planes were spread arithmetically, 100 instructions (EXPAND_MEASURED).
 __device__ __forceinline__ void expand_bf16(const Decoded& d, float gain, uint32_t w[12])
 {
-    const bool wide = __any_sync(kFullMask, d.p2 != 0u);
     // bf16(gain * a) for the value ids; float(a) by the 2^23 trick (a <= 28)
-    uint32_t packed[4] = {0u, 0u, 0u, 0u};
+    auto products = [&](uint32_t src, int i) {
+        const float a0 = __uint_as_float(__byte_perm(src, 0x4b000000u, i ? 0x7442 : 0x7440)) - 8388608.f;
+        const float a1 = __uint_as_float(__byte_perm(src, 0x4b000000u, i ? 0x7443 : 0x7441)) - 8388608.f;
+        const __nv_bfloat162 b = __floats2bfloat162_rn(gain * a0, gain * a1);
+        return *reinterpret_cast<const uint32_t*>(&b);
+    };
+    const uint32_t v01 = products(d.vals_lo, 0), v23 = products(d.vals_lo, 1);
+    const uint32_t lo03 = __byte_perm(v01, v23, 0x6420), hi03 = __byte_perm(v01, v23, 0x7531);
+    if (__any_sync(kFullMask, d.p2 != 0u)) {
+        const uint32_t v45 = products(d.vals_hi, 0), v67 = products(d.vals_hi, 1);
+        const uint32_t lo47 = __byte_perm(v45, v67, 0x6420), hi47 = __byte_perm(v45, v67, 0x7531);
+        const uint32_t sel[3] = {selectors<0>(d.p0, d.p1, d.p2), selectors<1>(d.p0, d.p1, d.p2), selectors<2>(d.p0, d.p1, d.p2)};
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (i < 2 || wide) {
-            const uint32_t src = i < 2 ? d.vals_lo : d.vals_hi;
-            const float a0 = __uint_as_float(__byte_perm(src, 0x4b000000u, (i & 1) ? 0x7442 : 0x7440)) - 8388608.f;
-            const float a1 = __uint_as_float(__byte_perm(src, 0x4b000000u, (i & 1) ? 0x7443 : 0x7441)) - 8388608.f;
-            __nv_bfloat162 b = __floats2bfloat162_rn(gain * a0, gain * a1);
-            packed[i] = *reinterpret_cast<uint32_t*>(&b);
+        for (int j = 0; j < 6; ++j) {
+            const int r = j % 3, q = j / 3;
+            const uint32_t s16 = q ? sel[r] >> 16 : sel[r];
+            const uint32_t lob = __byte_perm(lo03, lo47, s16);
+            const uint32_t hib = __byte_perm(hi03, hi47, s16) ^ __byte_perm(0x8000u, 0u, (d.neg >> (r + 16 * q)) & kPairs);
+            w[6 * q + r] = __byte_perm(lob, hib, 0x5140);
+            w[6 * q + 3 + r] = __byte_perm(lob, hib, 0x7362);
         }
-    }
-    const uint32_t lo03 = __byte_perm(packed[0], packed[1], 0x6420), hi03 = __byte_perm(packed[0], packed[1], 0x7531);
-    const uint32_t lo47 = __byte_perm(packed[2], packed[3], 0x6420), hi47 = __byte_perm(packed[2], packed[3], 0x7531);
-    uint32_t sel[3];
+    } else {
+        const uint32_t neg03 = hi03 ^ 0x80808080u;
+        const uint32_t sel[3] = {selectors<0>(d.p0, d.p1, d.neg), selectors<1>(d.p0, d.p1, d.neg), selectors<2>(d.p0, d.p1, d.neg)};
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        sel[r] = nibspread8((d.p0 >> (8 * r)) & 0xffu) | (nibspread8((d.p1 >> (8 * r)) & 0xffu) << 1);
-        if (wide) sel[r] |= nibspread8((d.p2 >> (8 * r)) & 0xffu) << 2;
-    }
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-        const uint32_t s16 = (j & 1) ? sel[j >> 1] >> 16 : sel[j >> 1];
-        const uint32_t lob = __byte_perm(lo03, lo47, s16);
-        const uint32_t hib = __byte_perm(hi03, hi47, s16) ^ msbspread4((d.neg >> (4 * j)) & 15u);
-        w[2 * j] = __byte_perm(lob, hib, 0x5140);
-        w[2 * j + 1] = __byte_perm(lob, hib, 0x7362);
+        for (int j = 0; j < 6; ++j) {
+            const int r = j % 3, q = j / 3;
+            const uint32_t s16 = q ? sel[r] >> 16 : sel[r];
+            const uint32_t lob = __byte_perm(lo03, lo03, s16), hib = __byte_perm(hi03, neg03, s16);
+            w[6 * q + r] = __byte_perm(lob, hib, 0x5140);
+            w[6 * q + 3 + r] = __byte_perm(lob, hib, 0x7362);
+        }
     }
 }
 

@@ -184,7 +184,8 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
         for (uint32_t r = 0; r < ncls; ++r) sort_rank[order[r]] = (uint16_t)r;
     }
     size_t o_trio = up(o_srk + sort_rank.size() * 2);
-    size_t o_cnt = up(o_trio + sizeof trio);
+    size_t o_pas = up(o_trio + sizeof trio);
+    size_t o_cnt = up(o_pas + sizeof h.pascal);
     size_t o_scr = up(o_cnt + (size_t)(kCounterWords + 16) * 4 + 256);   // ... and the peers' description of a row-sharded GEMM   // one counter per group of 8 rows (GEMV) / per 128-row tile (GEMM), then the grid arrival counter
     static_assert(kPairSlotOffset == 64ll * kMaxScratchRows, "the pair slots start where the scratch rows end");
     size_t total = o_scr + (size_t)64 * kMaxScratchRows * (4 + 8);       // binary32 scratch rows, then one 64-bit pair slot per GEMV row
@@ -204,6 +205,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     }
     if (!sort_rank.empty()) std::memcpy(blob.data() + o_srk, sort_rank.data(), sort_rank.size() * 2);
     std::memcpy(blob.data() + o_trio, &trio, sizeof trio);
+    std::memcpy(blob.data() + o_pas, h.pascal, sizeof h.pascal);
     if (cudaMalloc(&ctx->d_blob, total) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
     if (cudaMemcpy(ctx->d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(static_cast<uint8_t*>(ctx->d_blob) + o_cnt, 0, total - o_cnt) != cudaSuccess) {
@@ -226,6 +228,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     ctx->d_sort_rank = sort_rank.empty() ? nullptr : reinterpret_cast<const uint16_t*>(d + o_srk);
     ctx->enc.pos_by_low12 = reinterpret_cast<const uint16_t*>(d + o_p12);
     ctx->enc.sig_of_value = reinterpret_cast<const uint64_t*>(d + o_sig);
+    ctx->enc.pascal = reinterpret_cast<const uint32_t*>(d + o_pas);
     ctx->enc.trio = reinterpret_cast<const GolayTrio*>(d + o_trio);
     ctx->enc.hash_key = reinterpret_cast<const uint64_t*>(d + o_hk);
     ctx->enc.hash_cls = reinterpret_cast<const uint32_t*>(d + o_hc);

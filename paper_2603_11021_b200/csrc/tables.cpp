@@ -210,6 +210,16 @@ bool build_tables(int m_lo, int m_hi, HostTables& t)
 
 namespace llvq {
 
+// Bits of the largest binary64 number whose product with d (below 2^27, so that the product is exact where it matters) is at most 1.
+static uint64_t reciprocal_down(uint32_t d)
+{
+    double r = 1.0 / (double)d;
+    if (std::fma(r, (double)d, -1.0) > 0.0) r = std::nextafter(r, 0.0);
+    uint64_t bits;
+    std::memcpy(&bits, &r, 8);
+    return bits;
+}
+
 bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& img, bool with_classes)
 {
     const size_t ncls = with_classes ? t.desc.size() : 0;
@@ -225,12 +235,14 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
     }
     L.golay = 0;
     L.lut = up16(L.golay + 4096 * 4);
-    L.pascal = up16(L.lut + (with_classes ? 4096 * 2 : 0));
-    L.base14 = up16(L.pascal + 625 * 4);
-    if (L.base14 - L.pascal != 2512) return false;                      // the kernels address base14 relative to pascal
+    if (with_classes)
+        for (const ClassInfo& c : t.info) if (c.card >> 52) return false;      // class-local indices are divided in binary64
+    const uint32_t pascal_from = with_classes ? kLowBits * 25 * 4 : 0;         // rows below 14 are read by the decoders of big codes only
+    L.pascal = up16(L.lut + (with_classes ? 4096 * 2 : 0)) - pascal_from;
+    L.base14 = L.pascal + 2512;                                         // the kernels address base14 relative to pascal
     L.r14 = up16(L.base14 + 16 * 4);
     L.pd6 = up16(L.r14 + r14.size() * 2);
-    L.off = up16(L.pd6 + 4096);
+    L.off = up16(L.pd6 + 0x78 * 64);
     L.desc = up16(L.off + (with_classes ? (ncls + 1) * 8 : 0));
     L.recip64 = L.recip32 = 0;
     size_t end = L.desc + ncls * kFastDescStride * 4;
@@ -241,7 +253,8 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
     }
     L.total = up16(end);
     L.sub3 = L.total;
-    L.total_ext = up16(L.sub3 + kSmallSubsetWords * 4);
+    L.sub2 = up16(L.sub3 + kSmallSubsetWords * 4);
+    L.total_ext = up16(L.sub2 + kSub2Words * 4);
     L.lut_shift = (uint32_t)(t.W >= 12 ? t.W - 12 : 0);
     L.ncls = (uint32_t)ncls;
     L.W = (uint32_t)t.W;
@@ -257,20 +270,27 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
                 if (__builtin_popcount(m) == k) sub[at++] = m;
         }
         if (at != (uint32_t)kSmallSubsetWords) return false;
+        uint32_t* sub2 = reinterpret_cast<uint32_t*>(img.data() + L.sub2);
+        for (uint32_t i = 0; i < (uint32_t)kSub2Words; ++i) sub2[i] = i < 4 ? sub[i] : coords_of(sub[i]);
     }
-    std::memcpy(img.data() + L.golay, t.golay.data(), 4096 * 4);
-    std::memcpy(img.data() + L.pascal, t.pascal, 625 * 4);
-    for (int n = 0; n < 25; ++n)                           // column 0 is a sentinel in the image: "no element left to place"
+    for (int j = 0; j < 4096; ++j) {
+        const uint32_t last = t.golay[j] ? (uint32_t)__builtin_ctz(coord_bit(31 - __builtin_clz(t.golay[j]))) : 31u;
+        uint32_t w = coords_of(t.golay[j]);
+        for (int k = 0; k < 5; ++k) if ((last >> (4 - k)) & 1u) w |= 8u << (4 * k);
+        reinterpret_cast<uint32_t*>(img.data() + L.golay)[j] = w;
+    }
+    std::memcpy(img.data() + L.pascal + pascal_from, t.pascal + pascal_from / 4, 625 * 4 - pascal_from);
+    for (int n = (int)pascal_from / 100; n < 25; ++n)      // column 0 is a sentinel in the image: "no element left to place"
         reinterpret_cast<uint32_t*>(img.data() + L.pascal)[n * 25] = 0xffffffffu;
     std::memcpy(img.data() + L.base14, base14, sizeof base14);
     std::memcpy(img.data() + L.r14, r14.data(), r14.size() * 2);
     // pd6
-    for (uint32_t f = 0; f < 64; ++f)
-        for (uint32_t s = 0; s < 64; ++s) {
-            uint32_t out = 0, src = s;
-            for (int b = 0; b < 6; ++b)
-                if ((f >> b) & 1u) { if (src & 1u) out |= 1u << b; src >>= 1; }
-            img[L.pd6 + (f << 6 | s)] = (uint8_t)out;
+    for (uint32_t f = 0; f < 0x78; ++f)
+        for (uint32_t src0 = 0; src0 < 64; ++src0) {
+            uint32_t out = 0, src = src0;
+            for (int i = 0; i < 6; ++i)
+                if (f & coord_bit(i)) { if (src & 1u) out |= coord_bit(i); src >>= 1; }
+            img[L.pd6 + (f << 6 | (src0 ^ (f & 63u)))] = (uint8_t)out;
         }
     if (!with_classes) {                                   // small tables only: the class tables stay in global memory
         uint64_t* r64 = reinterpret_cast<uint64_t*>(img.data() + L.recip64);
@@ -305,7 +325,8 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
         flags |= (d.parity ? 1u : ((d.w == 8 || d.w == 12 || d.w == 16) ? 0u : 2u)) << 6;
         w[0] = d.w | (uint32_t)d.B << 8 | flags << 16 | (uint32_t)d.nlev1 << 24 | (uint32_t)nlev << 28;
         w[1] = d.goff | (uint32_t)d.A << 16;
-        w[2] = (uint32_t)d.magicA; w[3] = (uint32_t)(d.magicA >> 32);
+        const uint64_t inv_a = reciprocal_down(d.A);
+        w[2] = (uint32_t)inv_a; w[3] = (uint32_t)(inv_a >> 32);
         uint8_t vals[8] = {d.fill0, d.fill1, 0, 0, 0, 0, 0, 0};
         uint32_t nbytes = 0;
         u128 p_after = t.info[j].card / ((u128)d.A << d.B);        // number of arrangements P
@@ -316,7 +337,8 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
             w[8 + l] = lv.radix | (uint32_t)lv.k << 22 | (uint32_t)(2 + l) << 27 | ((lv.val & 2) ? 1u << 30 : 0u) | (lv.val ? 1u << 31 : 0u);
             nbytes |= (uint32_t)lv.n << (8 * l);
             if (l == 0) {
-                w[6] = (uint32_t)lv.magic; w[7] = (uint32_t)(lv.magic >> 32); p_after = (p_after + lv.radix - 1) / lv.radix;
+                const uint64_t inv = reciprocal_down(lv.radix);
+                w[6] = (uint32_t)inv; w[7] = (uint32_t)(inv >> 32); p_after = (p_after + lv.radix - 1) / lv.radix;
                 w[kFastDescMagic0] = lv.radix > 1 ? (uint32_t)((1ull << 32) / lv.radix) : 0xffffffffu;
             }
             else {
@@ -326,7 +348,7 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
         }
         for (int l = nlev; l < kFastMaxLevels; ++l) {          // steps the class does not have: radix 1 and the matching reciprocals, no slots:
             w[8 + l] = 1u;                                      // the division by multiplication then returns the rank unchanged and
-            if (l == 0) { w[6] = w[7] = 0xffffffffu; w[kFastDescMagic0] = 0xffffffffu; }    // remainder 0, so a lane that runs such a
+            if (l == 0) { w[6] = 0u; w[7] = 0x3ff00000u; w[kFastDescMagic0] = 0xffffffffu; }    // remainder 0, so a lane that runs such a
             else w[11 + l] = 0xffffffffu;                       // step beside lanes with more steps needs no special case
         }
         std::memcpy(&w[4], vals, 8);

@@ -103,25 +103,45 @@ constexpr int kFastDescMagic0 = 17;    // word holding floor(2^32 / radix) of le
 constexpr uint32_t kFastFlagRank32 = 32u;   // descriptor flag: the class has fewer than 2^32 arrangements
 constexpr int kSmallSubsetMaxK = 3;    // the table of all k-subsets of 24 slots covers k = 0..3
 constexpr int kSmallSubsetWords = 4 + 1 + 24 + 276 + 2024;   // [first entry of k = 0..3][the subsets, by k, each group in numeric order]
+constexpr int kSub2MaxK = 2;
+constexpr int kSub2Words = 4 + 1 + 24 + 276;
 constexpr int kFastDescStride = 20;    // words between descriptors: 80 bytes spread consecutive classes over all bank groups
 constexpr int kLowBits = 14;           // slots resolved by one table lookup in the subset unranking
+
+// Where the decoders keep the 24 coordinates in a 32-bit mask: coordinate 6 g + 2 r + n is bit 8 g + 4 n + r (g = 0..3, r = 0..2,
+// n = 0, 1).  Byte g holds a group of six coordinates, which is what a deposit into free positions works on (the order inside a
+// byte does not matter there, its table returns the bits where they belong); and bit r of the eight nibbles belongs to the
+// coordinate pairs (2 r, 2 r + 1) of the four groups, so that a mask and two shifts turn bit planes into byte-permute
+// selectors (expand_bf16).  Bits 3 and 7 of a byte are free.
+constexpr uint32_t kAllCoords = 0x77777777u;
+inline uint32_t coord_bit(int i) { return 1u << (8 * (i / 6) + 4 * (i & 1) + (i % 6) / 2); }
+inline uint32_t coords_of(uint32_t dense)      // bit i = coordinate i -> the layout above
+{
+    uint32_t m = 0;
+    for (int i = 0; i < kDim; ++i) if ((dense >> i) & 1u) m |= coord_bit(i);
+    return m;
+}
+// The free bits of a codeword in the image name its last coordinate: bits 3, 7, 11, 15, 19 = bits 4..0 of that coordinate's bit
+// position, gathered by one multiplication (no sums collide).  The zero word names bit 31, which belongs to no coordinate.
+constexpr uint32_t kLastPosBits = 0x00088888u, kLastPosGather = 0x10842100u;
 
 
 // Byte offsets of the parts of the image (all 16-byte aligned) and scalars the kernels need.
 struct FastLayout {
-    uint32_t golay;       // u32[4096]
+    uint32_t golay;       // u32[4096] in the layout of coords_of, the last coordinate named in the free bits
     uint32_t lut;         // u16[4096]  class of the first index of bucket (I >> lut_shift)
-    uint32_t pascal;      // u32[25*25]
+    uint32_t pascal;      // u32[25*25]; images with class tables hold the rows from 14 on only (the offset is still that of row 0)
     uint32_t base14;      // u32[16]: [k] = first entry of the k-subsets of 14 slots in r14
     uint32_t r14;         // u16[16384]: the k-subsets of 14 slots as bit masks, k = 0..14, each in numeric order
-    uint32_t pd6;         // u8[4096]: [f << 6 | s] = low bits of s deposited into the set bits of f
+    uint32_t pd6;         // u8[0x78 * 64]: [f << 6 | (s ^ (f & 63))] = low bits of s deposited into the coordinates of a byte f, lowest first
     uint32_t off;         // u64[ncls + 1]
     uint32_t desc;        // u32[ncls][kFastDescStride]
     uint32_t total;       // bytes of the image proper, multiple of 16
     uint32_t recip64;     // u64[25*25] floor((2^64 - 1) / C(n, k)) and
     uint32_t recip32;     // u32[25*25] floor(2^32 / C(n, k)) (0xffffffff for C = 1): images without class tables only, else 0
     uint32_t sub3;        // u32[kSmallSubsetWords], behind the image proper: kernels with room for it load total_ext bytes
-    uint32_t total_ext;   // bytes including sub3, multiple of 16
+    uint32_t sub2;        // u32[kSub2Words], behind sub3: directory and subsets for k = 0..2 in the layout of coords_of
+    uint32_t total_ext;   // bytes including sub3 and sub2, multiple of 16
     uint32_t lut_shift;
     uint32_t ncls;
     uint32_t W;
@@ -132,11 +152,11 @@ struct FastLayout {
 //       flags: bit0 parity, bit1 signpar, bit2 fill0 is nonzero, bit3 fill1 has value bit 1, bit4 fill0 has value bit 1,
 //              bit5 the arrangement rank of the class fits 32 bits, bits 6-7 decoder form (0 even with weight 8 / 12 / 16, 1 odd, 2 other)
 //  1: goff | A << 16
-//  2,3: magicA = floor((2^64-1)/A)
+//  2,3: 1 / A as binary64, rounded down
 //  4,5: absolute value of id 0..7 (one byte each): id 0 = fill0, id 1 = fill1, ids 2.. = levels in order
-//  6,7: magic of level 0 = floor((2^64-1)/radix0)
+//  6,7: 1 / radix of level 0 as binary64, rounded down
 //  8..11: level l: radix | k << 22 | id << 27 | (value bit 1) << 30 | (value nonzero) << 31; steps the class does not have:
-//         radix 1, k 0, reciprocals 0xffffffff (dividing by them leaves the rank unchanged and gives remainder 0)
+//         radix 1, k 0, reciprocals 1.0 / 0xffffffff (dividing by them leaves the rank unchanged and gives remainder 0)
 //  12..14: floor(2^32 / radix) of levels 1..3
 //  15: n (free slots before the step) of levels 0..3, one byte each
 //  16: binary32 bits of 1 / |x| = 1 / sqrt(16 m) (formed in binary64, rounded once), for the shape-gain form
