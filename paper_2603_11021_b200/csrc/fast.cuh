@@ -134,6 +134,14 @@ __device__ __forceinline__ uint64_t divide52(uint64_t n, uint32_t d, double inv,
     return q;
 }
 
+// Byte permute with a selector made at run time (__byte_perm clears bit 3 of every nibble first: here it is zero, or welcome).
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
+{
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+
 template <int kOff>
 __device__ __forceinline__ uint32_t lds_at(uint32_t addr)
 {
@@ -333,6 +341,10 @@ __device__ __forceinline__ uint32_t selectors(uint32_t x, uint32_t y, uint32_t z
     return ((x >> r) & kPairs) | ((r == 0 ? y << 1 : y >> (r - (r > 0))) & (kPairs << 1)) | ((z << (2 - r)) & (kPairs << 2));
 }
 
+// Byte i of the result = 0xff where bit 4 i of x is set, else 0 (i = 0..3).  The other bits of x may be anything: as part of the
+// selector they choose an equal byte or ask for its sign, which is the byte again.
+__device__ __forceinline__ uint32_t ones_where(uint32_t x) { return prmt(0xff00ff00u, 0xff00ff00u, x); }
+
 // The 24 coordinates as signed bytes, coordinate i in byte (i & 3) of word (i >> 2).
 __device__ __forceinline__ void expand_bytes(const Decoded& d, uint32_t out[6])
 {
@@ -340,9 +352,9 @@ __device__ __forceinline__ void expand_bytes(const Decoded& d, uint32_t out[6])
     const uint32_t sel[3] = {selectors<0>(d.p0, d.p1, d.p2), selectors<1>(d.p0, d.p1, d.p2), selectors<2>(d.p0, d.p1, d.p2)};
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
-        const uint32_t neg = ((d.neg >> (j % 3)) & kPairs) >> (j < 3 ? 0 : 16);
-        const uint32_t a = __byte_perm(d.vals_lo, d.vals_hi, sel[j % 3] >> (j < 3 ? 0 : 16));
-        t[j] = (a ^ __byte_perm(0xff00u, 0u, neg)) + __byte_perm(0x0100u, 0u, neg);       // negated bytes are never zero
+        const uint32_t neg = ones_where(d.neg >> (j % 3 + (j < 3 ? 0 : 16)));
+        const uint32_t a = prmt(d.vals_lo, d.vals_hi, sel[j % 3] >> (j < 3 ? 0 : 16));
+        t[j] = (a ^ neg) + (neg & 0x01010101u);                                   // negated bytes are never zero
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -377,8 +389,8 @@ __device__ __forceinline__ void expand_bf16(const Decoded& d, float gain, uint32
         for (int j = 0; j < 6; ++j) {
             const int r = j % 3, q = j / 3;
             const uint32_t s16 = q ? sel[r] >> 16 : sel[r];
-            const uint32_t lob = __byte_perm(lo03, lo47, s16);
-            const uint32_t hib = __byte_perm(hi03, hi47, s16) ^ __byte_perm(0x8000u, 0u, (d.neg >> (r + 16 * q)) & kPairs);
+            const uint32_t lob = prmt(lo03, lo47, s16);
+            const uint32_t hib = prmt(hi03, hi47, s16) ^ (ones_where(d.neg >> (r + 16 * q)) & 0x80808080u);
             w[6 * q + r] = __byte_perm(lob, hib, 0x5140);
             w[6 * q + 3 + r] = __byte_perm(lob, hib, 0x7362);
         }
@@ -389,7 +401,7 @@ __device__ __forceinline__ void expand_bf16(const Decoded& d, float gain, uint32
         for (int j = 0; j < 6; ++j) {
             const int r = j % 3, q = j / 3;
             const uint32_t s16 = q ? sel[r] >> 16 : sel[r];
-            const uint32_t lob = __byte_perm(lo03, lo03, s16), hib = __byte_perm(hi03, neg03, s16);
+            const uint32_t lob = prmt(lo03, lo03, s16), hib = prmt(hi03, neg03, s16);
             w[6 * q + r] = __byte_perm(lob, hib, 0x5140);
             w[6 * q + 3 + r] = __byte_perm(lob, hib, 0x7362);
         }

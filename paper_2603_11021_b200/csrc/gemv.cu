@@ -14,17 +14,20 @@ constexpr size_t kSmemLimit = 227 * 1024;
 // Shared memory of gemv_bin_kernel for `su` units per segment, and whether the table of small subsets still fits.
 void bin_smem(const llvq_ctx* ctx, int64_t nq, int su, size_t& bytes, bool& ext)
 {
-    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows * 4 + 16 + 2 * 1024 * 4 + (size_t)su * 32 * (8 + 2);
+    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + 16 + 2 * 1024 * 4 + (size_t)su * 32 * (8 + 2);
     ext = ctx->fl.total_ext + rest <= kSmemLimit;
     bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest;
 }
 
-// The same for gemv_sorted_kernel.
-void sorted_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext)
+// The same for gemv_sorted_kernel; acc_floats = room for the row sums, cut down to one copy per row where rows are so long that x
+// needs the space.
+void sorted_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext, uint32_t& acc_floats)
 {
-    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows * 4 + 16;
-    ext = ctx->fl.total_ext + rest <= kSmemLimit;
-    bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest;
+    const size_t rest = 16 + (size_t)nq * 48 * 4 + 16;
+    acc_floats = kSortAccFloats;
+    while (acc_floats > kGemvGroupsPerPass * kGemvGroupRows && ctx->fl.total + rest + acc_floats * 4 > kSmemLimit) acc_floats /= 2;
+    ext = ctx->fl.total_ext + rest + acc_floats * 4 <= kSmemLimit;
+    bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest + acc_floats * 4;
 }
 
 bool bin_kernel_serves(const llvq_ctx* ctx, int64_t nq, const SgArgs* sg)
@@ -56,7 +59,10 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const int64_t bpr = (k_in + 23) / 24;
     const int64_t nq = (bpr + 3) / 4;
     const size_t kSmemMax = 227 * 1024;
-    const size_t rest = 16 + (size_t)nq * 48 * 4 + kGemvGroupsPerPass * kGemvGroupRows * 4 + 16;
+    // row groups per pass: the row sums take 32 bytes each beside x, so rows too long for 128 of them get passes of 8
+    const size_t rest_x = 16 + (size_t)nq * 48 * 4 + 16;
+    const uint32_t per_pass = ctx->fl.total + rest_x + kGemvGroupsPerPass * kGemvGroupRows * 4 <= kSmemMax ? kGemvGroupsPerPass : 8;
+    const size_t rest = rest_x + per_pass * kGemvGroupRows * 4;
     // room for the table of small subsets (not for the 72-bit code: its warps hold 32 unrelated classes that almost never take it together)
     const bool ext_direct = ctx->fast && ctx->fl.total_ext + rest <= kSmemMax;
     const size_t smem = (ext_direct ? ctx->fl.total_ext : ctx->fl.total) + rest;
@@ -100,7 +106,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
 #define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH)                                                                        \
     do {                                                                                                           \
         if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                               \
-        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, sp, n_out, k_in, bpr, d_x_bf16, yo, \
+        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, sp, per_pass, n_out, k_in, bpr, d_x_bf16, yo, \
                        ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;                         \
     } while (0)
     if (shard && ctx->fast) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(false, true, false, true); else LLVQ_LAUNCH_GEMV(false, false, false, true); }
@@ -118,8 +124,8 @@ bool sortable(const llvq_ctx* ctx, int64_t k_in)
 {
     if (!ctx->fast || !ctx->d_sort_rank || ctx->host.W > 48 || ctx->host.N >= (u128)kSortIndexMask) return false;
     const int64_t nq = ((k_in + 23) / 24 + 3) / 4;
-    size_t smem; bool ext;
-    sorted_smem(ctx, nq, smem, ext);
+    size_t smem; bool ext; uint32_t acc_floats;
+    sorted_smem(ctx, nq, smem, ext, acc_floats);
     return smem <= kSmemLimit && nq < (1ll << 24);
 }
 
@@ -197,8 +203,8 @@ static int gemv_sorted_common(const llvq_ctx* ctx, const void* d_sorted, const u
     const int64_t bpr = (k_in + 23) / 24, nq = (bpr + 3) / 4;
     const int64_t units = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
     const unsigned g = (unsigned)std::min<int64_t>(units, ctx->sm_count);
-    size_t smem; bool ext;
-    sorted_smem(ctx, nq, smem, ext);
+    size_t smem; bool ext; uint32_t acc_floats;
+    sorted_smem(ctx, nq, smem, ext, acc_floats);
     const FastArgs fa = fast_args(ctx, ext);
     const Split split = make_split(units, nq, g);
     const unsigned long long* sp = static_cast<const unsigned long long*>(d_sorted);
@@ -207,7 +213,7 @@ static int gemv_sorted_common(const llvq_ctx* ctx, const void* d_sorted, const u
     do {                                                                                                                \
         if (!set_smem<gemv_sorted_kernel<BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                        \
         if (launch_pdl(gemv_sorted_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem, st, fa, sp, d_gain_f16, sga, split, n_out, k_in, bpr, \
-                       d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;          \
+                       acc_floats, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;          \
     } while (0)
     const bool shard = yo.n_peer > 0 || yo.n_flag > 0;                  // row-sharded launch: stored-gain form only
     if (shard && sg) return LLVQ_EUNSUPPORTED;
@@ -251,8 +257,8 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     if (n_mats > kMaxMultiMats) return LLVQ_EUNSUPPORTED;
     GemvMulti mm{};
     mm.n = n_mats;
-    size_t smem = 0; bool ext = true;
-    int64_t slot = 0;
+    uint32_t acc_floats = kSortAccFloats;
+    int64_t slot = 0, max_nq = 0;
     for (int i = 0; i < n_mats; ++i) {
         const llvq_gemv_desc& d = descs[i];
         if (int e = check_common(ctx, d.d_weights)) return e;
@@ -262,16 +268,8 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         const int64_t units = ((d.n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
         // every matrix must give every CTA work: the sorted layout was made for that many CTAs
         if (units < ctx->sm_count) return LLVQ_EUNSUPPORTED;
-        size_t bytes; bool e1;
-        if (sorted) {
-            if (!sortable(ctx, d.k_in)) return LLVQ_EUNSUPPORTED;
-            sorted_smem(ctx, nq, bytes, e1);
-        } else {
-            if (!bin_kernel_serves(ctx, nq, nullptr)) return LLVQ_EUNSUPPORTED;
-            bin_smem(ctx, nq, kBinSegUnits, bytes, e1);
-        }
-        ext = ext && e1;
-        smem = std::max(smem, bytes);
+        if (sorted ? !sortable(ctx, d.k_in) : !bin_kernel_serves(ctx, nq, nullptr)) return LLVQ_EUNSUPPORTED;
+        max_nq = std::max(max_nq, nq);
         GemvMat& m = mm.m[i];
         m.weights = d.d_weights; m.gain = d.d_gain_f16; m.x = d.d_x_bf16; m.y = d.d_y;
         m.n_out = d.n_out; m.k_in = d.k_in; m.slot0 = slot;
@@ -280,15 +278,9 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         slot += (d.n_out + kGemvGroupRows - 1) / kGemvGroupRows * kGemvGroupRows;
     }
     if (slot > 64ll * kMaxScratchRows) return LLVQ_EUNSUPPORTED;
-    if (!ext) {                                          // one image size for the whole launch: recompute without the extension
-        smem = 0;
-        for (int i = 0; i < n_mats; ++i) {
-            const int64_t nq = ((descs[i].k_in + 23) / 24 + 3) / 4;
-            const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows * 4 + 16 +
-                                (sorted ? 0 : 2 * 1024 * 4 + (size_t)kBinSegUnits * 32 * (8 + 2));
-            smem = std::max(smem, ctx->fl.total + rest);
-        }
-    }
+    size_t smem; bool ext;                               // the longest rows decide for the whole launch
+    if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);
+    else bin_smem(ctx, max_nq, kBinSegUnits, smem, ext);
     if (smem > kSmemLimit) return LLVQ_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
@@ -298,25 +290,29 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     if (sorted && n_mats >= 2) {
         // the kernel without a barrier between the matrices, when every CTA's share of every matrix is one segment and
         // one pass and three sets of (x, row sums) fit beside the tables
-        int64_t max_groups = 0, max_nq = 0;
+        int64_t max_groups = 0;
         bool one_pass = true;
         for (int i = 0; i < n_mats; ++i) {
             // a CTA's share is at most ceil(U / g) units, hence at most that many + nq - 2 units' worth of row groups, cut at both ends
             const Split& sp = mm.m[i].sp;
             const int64_t most = sp.each + (sp.rest ? 1 : 0), nq = sp.per_row;
-            max_nq = std::max(max_nq, nq);
             one_pass = one_pass && most <= kSortSegUnits;
             max_groups = std::max(max_groups, (most + nq - 2) / nq + 1);
         }
         const int xs_words = (int)(max_nq * 48), acc_rows = (int)(max_groups * kGemvGroupRows);
-        const size_t smem_ov = fa.image_bytes + 16 + (size_t)kOverlapSets * ((size_t)xs_words + (size_t)kSortAccCopies * acc_rows) * 4 + kOverlapSets * sizeof(OverlapSet);
+        uint32_t shift = 4;                              // copies of every row sum: up to sixteen (one warp alone sums them up), at least four
+        auto ov_bytes = [&] {
+            return fa.image_bytes + 16 + (size_t)kOverlapSets * ((size_t)xs_words + ((size_t)acc_rows << shift)) * 4 + kOverlapSets * sizeof(OverlapSet);
+        };
+        while (shift > 2 && ov_bytes() > kSmemLimit) --shift;
+        const size_t smem_ov = ov_bytes();
         if (one_pass && max_groups <= kGemvGroupsPerPass && smem_ov <= kSmemLimit) {
             if (y_dtype == LLVQ_BF16) {
                 if (!set_smem<gemv_sorted_overlap_kernel<true>>(ctx->device, smem_ov)) return LLVQ_ECUDA;
-                if (launch_pdl(gemv_sorted_overlap_kernel<true>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
+                if (launch_pdl(gemv_sorted_overlap_kernel<true>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, shift, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
             } else {
                 if (!set_smem<gemv_sorted_overlap_kernel<false>>(ctx->device, smem_ov)) return LLVQ_ECUDA;
-                if (launch_pdl(gemv_sorted_overlap_kernel<false>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
+                if (launch_pdl(gemv_sorted_overlap_kernel<false>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, shift, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
             }
             return launch_status();
         }
@@ -324,10 +320,10 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     if (sorted) {
         if (y_dtype == LLVQ_BF16) {
             if (!set_smem<gemv_sorted_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_sorted_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
+            if (launch_pdl(gemv_sorted_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         } else {
             if (!set_smem<gemv_sorted_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_sorted_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
+            if (launch_pdl(gemv_sorted_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         }
     } else {
         if (y_dtype == LLVQ_BF16) {

@@ -68,16 +68,16 @@ __device__ __forceinline__ void stage_x(uint32_t* xs, const uint16_t* __restrict
 }
 
 // End of a pass of a GEMV CTA over row groups rg0..rg1 (8 rows each; the CTA owns units [u_begin, u_end) of sp):
-// row_sum(i) is the CTA's sum for row i of the pass.  One warp per row group, lanes
+// row_sums(i), called by a whole warp, gives lanes 0..7 the CTA's sums for rows i..i + 7 of the pass.  One warp per row group, lanes
 // 0..7 its rows, no CTA-wide barrier inside.  A group the CTA covers completely is final.  A group it shares with
 // neighbouring CTAs goes through the scratch row in global memory: add, make the add visible, count the arrival;
 // whoever arrives last reads the total, writes y and leaves scratch and counter zero for the next launch (groups shared
 // by exactly two CTAs take a shorter way, below).
 // The caller puts a __syncthreads() before (sums complete) and after (sums may be cleared) the call.
 // slot0 (a multiple of 8) = first scratch row / pair slot of this matrix when one launch works on several matrices.
-template <bool kOutBf16, bool kShard, typename RowSum>
+template <bool kOutBf16, bool kShard, typename RowSums>
 __device__ __forceinline__ void finish_pass(const YOut& yo, const Split& sp, uint32_t rg0, uint32_t rg1, uint32_t u_begin, uint32_t u_end,
-                                            int64_t n_out, float* __restrict__ scratch, uint32_t* __restrict__ counters, RowSum row_sum,
+                                            int64_t n_out, float* __restrict__ scratch, uint32_t* __restrict__ counters, RowSums row_sums,
                                             int64_t slot0 = 0, int warp_of = -1, int nwarps_of = 0)
 {
     // by default the warps of the CTA share the row groups; warp_of / nwarps_of let a subset of the warps (one warp) do it
@@ -88,7 +88,7 @@ __device__ __forceinline__ void finish_pass(const YOut& yo, const Split& sp, uin
         const bool whole = u_begin <= first && next <= u_end;
         const int64_t row = (int64_t)rg * kGemvGroupRows + lane;
         const bool mine = lane < kGemvGroupRows && row < n_out;
-        const float part = lane < kGemvGroupRows ? row_sum((rg - rg0) * kGemvGroupRows + lane) : 0.f;
+        const float part = row_sums((rg - rg0) * kGemvGroupRows);
         if (whole) {
             if (mine) {
                 store_y<kOutBf16, kShard>(yo, row, part);
@@ -166,22 +166,22 @@ __device__ __forceinline__ float dot24_bf16(const uint32_t w[12], const uint32_t
 
 template <bool kBig, bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kGemvThreads, 1)
-gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, Split sp,
+gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, Split sp, uint32_t groups_per_pass,
                  int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
                  float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
     const uint32_t nq = sp.per_row;                                 // units along K
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
-    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kGemvGroupsPerPass][8]
+    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [groups_per_pass][8]
     stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const uint32_t kWarps = blockDim.x >> 5;
     const uint32_t u_begin = split_begin(sp, blockIdx.x), u_end = split_begin(sp, blockIdx.x + 1u);      // at least one unit
     const uint32_t rg_first = split_row(sp, u_begin), rg_last = split_row(sp, u_end - 1u);
-    for (uint32_t rg0 = rg_first; rg0 <= rg_last; rg0 += kGemvGroupsPerPass) {
-        const uint32_t rg1 = min(rg0 + kGemvGroupsPerPass - 1u, rg_last);
-        for (int i = threadIdx.x; i < kGemvGroupsPerPass * kGemvGroupRows; i += (int)blockDim.x) acc[i] = 0.f;
+    for (uint32_t rg0 = rg_first; rg0 <= rg_last; rg0 += groups_per_pass) {
+        const uint32_t rg1 = min(rg0 + groups_per_pass - 1u, rg_last);
+        for (uint32_t i = threadIdx.x; i < groups_per_pass * kGemvGroupRows; i += blockDim.x) acc[i] = 0.f;
         __syncthreads();
         const uint32_t p_begin = max(u_begin, rg0 * nq), p_end = min(u_end, (rg1 + 1u) * nq);
         uint32_t kq, rg = split_row(sp, p_begin + (uint32_t)warp, kq);      // walked along with u: no division per unit
@@ -218,7 +218,7 @@ gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_
         }
         __syncthreads();
         // row groups this CTA covers completely are final; the (at most two) split ones go through the scratch
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) { return acc[r]; });
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) { return lane < kGemvGroupRows ? acc[r + lane] : 0.f; });
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     }
     if (kShard) shard_arrive(yo);
@@ -240,8 +240,30 @@ constexpr uint32_t kKindEven = 0u, kKindOdd = 1u, kKindOther = 2u, kKindNull = 3
 // ===========================================================================
 constexpr int kSortSegUnits = 2048;                  // 65536 blocks
 constexpr int kSortThreads = 1024;
-constexpr int kSortAccCopies = 4;                    // copies of the row sums in shared memory (a power of two)
+// Row sums of a pass in shared memory: acc[row << shift | lane & mask], as many copies of every row (a power of two, up to one per
+// lane) as kSortAccFloats floats hold.  An addition of floats in shared memory is a compare-and-swap loop that goes round once for
+// every lane of the warp that meets the same address: 32 blocks of a warp fall into some 80 rows, and with one copy per warp
+// parity instead of per lane that took 18 instructions and 15 passes over the banks per addition (ACC_MEASURED).
+constexpr uint32_t kSortAccFloats = 4 * kGemvGroupsPerPass * kGemvGroupRows;
 constexpr unsigned long long kSortIndexMask = (1ull << 48) - 1ull;
+
+__device__ __forceinline__ uint32_t acc_shift(uint32_t rows, uint32_t floats)
+{
+    uint32_t c = 5;
+    while (c > 0 && (rows << c) > floats) --c;
+    return c;
+}
+
+// Sums over the copies of rows first..first + 7, in lanes 0..7; the whole warp calls this.
+__device__ __forceinline__ float acc_row_sums(const float* acc, uint32_t first, uint32_t shift)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    float v = 0.f;
+    for (uint32_t c = lane & 3u; c < (1u << shift); c += 4) v += acc[(first + (lane >> 2)) << shift | c];      // four lanes per row
+    v += __shfl_xor_sync(kFullMask, v, 1);
+    v += __shfl_xor_sync(kFullMask, v, 2);
+    return __shfl_sync(kFullMask, v, (lane & 7u) * 4u);
+}
 
 // Calls f(tu0, tu1, rg0, rg1, first, last) for every segment [tu0, tu1) of CTA `cta` in order; rg0..rg1 = row
 // groups of the pass the segment belongs to (a pass covers at most kGemvGroupsPerPass row groups); first / last =
@@ -296,15 +318,14 @@ sort_blocks_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint1
             for (int k = 0; k < 1024; ++k) { const uint32_t c = hist[k]; hist[k] = run; run += c; }
         }
         __syncthreads();
-        // the entries are visited column-block major (all row groups of a column unit, then the next unit): the blocks
-        // of a bin then come out roughly ordered by column block, and the 32 lanes of a GEMV warp read few different
-        // slices of x
+        // the entries are visited column block by column block (all rows of one, then the next): the blocks of a bin then come out
+        // roughly ordered by column block, and the eight lanes that read x together read few different slices of it
         const uint32_t rg_a = split_row(sp, tu0), nrg = split_row(sp, tu1 - 1u) - rg_a + 1u;
         for (uint32_t e = threadIdx.x; e < nq * nrg * 32u; e += kSortThreads) {
-            const uint32_t kq = e / (nrg * 32u), rem = e - kq * (nrg * 32u);
-            const uint32_t u = (rg_a + (rem >> 5)) * nq + kq;
+            const uint32_t cb = e / (nrg * 8u), row = e - cb * (nrg * 8u);
+            const uint32_t u = (rg_a + (row >> 3)) * nq + (cb >> 2);
             if (u < tu0 || u >= tu1) continue;
-            const int i = (int)(u - tu0) * 32 + (int)(rem & 31);
+            const int i = (int)(u - tu0) * 32 + (int)((row & 7u) * 4u + (cb & 3u));
             unsigned long long field;
             const uint32_t key = entry_of(i, false, field);
             const uint32_t slot = hist[key] + atomicAdd(&cursor[key], 1u);
@@ -376,20 +397,21 @@ template <bool kOutBf16, bool kSg, bool kShard>
 __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastSmem& T, uint8_t* staging,
                                                  const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, const SgArgs& sg,
                                                  const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, const uint16_t* __restrict__ x,
-                                                 const YOut& yo, float* __restrict__ scratch, uint32_t* __restrict__ counters, int64_t slot0)
+                                                 const YOut& yo, float* __restrict__ scratch, uint32_t* __restrict__ counters, int64_t slot0,
+                                                 uint32_t acc_floats)
 {
     const uint32_t nq = sp.per_row;
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
-    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccCopies][kGemvGroupsPerPass][8]: warps spread their adds over the copies
-    uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows);
-    uint32_t* next_chunk = last_flag + 1;
+    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [acc_floats]
+    uint32_t* next_chunk = reinterpret_cast<uint32_t*>(acc + acc_floats);
     stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t kWarps = blockDim.x >> 5;
 
     for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t rg0, uint32_t rg1, bool first, bool last) {
+        const uint32_t shift = acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, acc_floats);
         if (first)
-            for (int i = threadIdx.x; i < kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows; i += (int)blockDim.x) acc[i] = 0.f;
+            for (uint32_t i = threadIdx.x; i < (rg1 - rg0 + 1u) * kGemvGroupRows << shift; i += blockDim.x) acc[i] = 0.f;
         if (threadIdx.x == 0) *next_chunk = kWarps;
         __syncthreads();
         uint32_t kq_a;
@@ -431,21 +453,16 @@ __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastS
             const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
             const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
             const float dot = dot24_bf16(w, xv);
-            if (valid) atomicAdd(&acc[(warp & (kSortAccCopies - 1)) * (kGemvGroupsPerPass * kGemvGroupRows) + rloc], dot);
+            if (valid) atomicAdd(&acc[rloc << shift | ((uint32_t)lane & ((1u << shift) - 1u))], dot);
             ch = nxt; e = e_next;
             use_from_here(e);
         }
         __syncthreads();
         if (!last) return;
         // end of the pass: row groups this CTA covers completely are final; the split ones go through the scratch
-        auto row_sum = [&](uint32_t r) {
-            float v = 0.f;
-#pragma unroll
-            for (int c = 0; c < kSortAccCopies; ++c) v += acc[c * (kGemvGroupsPerPass * kGemvGroupRows) + r];
-            return v;
-        };
+        auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
         const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sum, slot0);
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     });
 }
@@ -453,19 +470,19 @@ __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastS
 template <bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg,
-                   Split sp, int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
+                   Split sp, int64_t n_out, int64_t k_in, int64_t bpr, uint32_t acc_floats, const uint16_t* __restrict__ x, YOut yo,
                    float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
     prefetch_first_chunks(sorted, sp);                  // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
-    gemv_sorted_body<kOutBf16, kSg, kShard>(fa, T, staging, sorted, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0);
+    gemv_sorted_body<kOutBf16, kSg, kShard>(fa, T, staging, sorted, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0, acc_floats);
     if (kShard) shard_arrive(yo);
 }
 
 // Several independent matrices in one launch (no output of one may be an input of another).
 template <bool kOutBf16>
 __global__ void __launch_bounds__(kSortThreads, 1)
-gemv_sorted_multi_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, float* __restrict__ scratch, uint32_t* __restrict__ counters)
+gemv_sorted_multi_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, uint32_t acc_floats, float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
     prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[0].weights), mm.m[0].sp);
     FAST_PROLOGUE();
@@ -476,7 +493,7 @@ gemv_sorted_multi_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, floa
         YOut yo{};
         yo.y = M.y;
         gemv_sorted_body<kOutBf16, false, false>(fa, T, staging, static_cast<const unsigned long long*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
-                                                 (uint32_t)M.bpr, M.x, yo, scratch, counters, M.slot0);
+                                                 (uint32_t)M.bpr, M.x, yo, scratch, counters, M.slot0, acc_floats);
         __syncthreads();                                   // the next matrix restages x and clears the row sums
     }
 }
@@ -498,13 +515,13 @@ struct OverlapSet {
 
 template <bool kOutBf16>
 __global__ void __launch_bounds__(kSortThreads, 1)
-gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, int xs_words, int acc_rows, float* __restrict__ scratch,
+gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, int xs_words, int acc_rows, uint32_t shift, float* __restrict__ scratch,
                            uint32_t* __restrict__ counters)
 {
     prefetch_first_chunks(static_cast<const unsigned long long*>(mm.m[0].weights), mm.m[0].sp);
     FAST_PROLOGUE();
-    // [kOverlapSets] x { x as packed pairs [xs_words] | row sums [kSortAccCopies][acc_rows] } | control words
-    const int set_words = xs_words + kSortAccCopies * acc_rows;
+    // [kOverlapSets] x { x as packed pairs [xs_words] | row sums [acc_rows << shift] } | control words
+    const int set_words = xs_words + (acc_rows << shift);
     uint32_t* sets = reinterpret_cast<uint32_t*>(staging);
     volatile OverlapSet* ctl = reinterpret_cast<volatile OverlapSet*>(sets + kOverlapSets * set_words);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -516,7 +533,7 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
         uint32_t* xs = sets + (i % kOverlapSets) * set_words;
         float* acc = reinterpret_cast<float*>(xs + xs_words);
         stage_x(xs, M.x, M.k_in, M.sp.per_row * 48u, (uint32_t)tid, (uint32_t)nthreads);
-        for (int r = tid; r < kSortAccCopies * acc_rows; r += nthreads) acc[r] = 0.f;
+        for (int r = tid; r < acc_rows << shift >> 2; r += nthreads) reinterpret_cast<float4*>(acc)[r] = make_float4(0.f, 0.f, 0.f, 0.f);
     };
 
     if (threadIdx.x < kOverlapSets) { ctl[threadIdx.x].next_chunk = 0u; ctl[threadIdx.x].arrived = 0u; ctl[threadIdx.x].ready = 0u; }
@@ -577,7 +594,7 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
             const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
             const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
             const float dot = dot24_bf16(w, xv);
-            if (valid) atomicAdd(&acc[(warp & (kSortAccCopies - 1)) * acc_rows + rloc], dot);
+            if (valid) atomicAdd(&acc[rloc << shift | ((uint32_t)lane & ((1u << shift) - 1u))], dot);
             ch = nxt; e = e_next;
             use_from_here(e);
         }
@@ -590,13 +607,8 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
             __threadfence_block();
             YOut yo{};
             yo.y = M.y;
-            auto row_sum = [&](uint32_t rr) {
-                float vv = 0.f;
-#pragma unroll
-                for (int c = 0; c < kSortAccCopies; ++c) vv += acc[c * acc_rows + rr];
-                return vv;
-            };
-            finish_pass<kOutBf16, false>(yo, sp, rg0, split_row(sp, ue - 1u), ub, ue, M.n_out, scratch, counters, row_sum, M.slot0, 0, 1);
+            auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
+            finish_pass<kOutBf16, false>(yo, sp, rg0, split_row(sp, ue - 1u), ub, ue, M.n_out, scratch, counters, row_sums, M.slot0, 0, 1);
             __syncwarp();
             if (i + kOverlapSets < mm.n) {
                 if (lane == 0) { ctl[set].next_chunk = 0u; ctl[set].arrived = 0u; }
@@ -644,8 +656,8 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
 {
     const uint32_t nq = sp.per_row;
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
-    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccCopies][kGemvGroupsPerPass][8]
-    uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows);
+    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccFloats]
+    uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccFloats);
     uint32_t* next_chunk = last_flag + 1;
     uint32_t* hist = last_flag + 4;                                  // [1024] bins in sort order; later their first slots
     uint32_t* cursor = hist + 1024;                                  // [1024]
@@ -655,8 +667,9 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t kWarps = blockDim.x >> 5;
     for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t rg0, uint32_t rg1, bool first, bool last) {
+        const uint32_t shift = acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, kSortAccFloats);
         if (first)
-            for (int i = threadIdx.x; i < kSortAccCopies * kGemvGroupsPerPass * kGemvGroupRows; i += (int)blockDim.x) acc[i] = 0.f;
+            for (uint32_t i = threadIdx.x; i < (rg1 - rg0 + 1u) * kGemvGroupRows << shift; i += blockDim.x) acc[i] = 0.f;
         hist[threadIdx.x] = 0; cursor[threadIdx.x] = 0;
         if (threadIdx.x == 0) *next_chunk = kWarps;
         __syncthreads();
@@ -752,19 +765,14 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
             const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
             const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
             const float dot = dot24_bf16(w, xv);
-            if (valid) atomicAdd(&acc[(warp & (kSortAccCopies - 1)) * (kGemvGroupsPerPass * kGemvGroupRows) + rloc], dot);
+            if (valid) atomicAdd(&acc[rloc << shift | ((uint32_t)lane & ((1u << shift) - 1u))], dot);
             ch = nxt;
         }
         __syncthreads();
         if (!last) return;
-        auto row_sum = [&](uint32_t r) {
-            float v = 0.f;
-#pragma unroll
-            for (int c = 0; c < kSortAccCopies; ++c) v += acc[c * (kGemvGroupsPerPass * kGemvGroupRows) + r];
-            return v;
-        };
+        auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
         const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sum, slot0);
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
         __syncthreads();
     }, (uint32_t)seg_units);
 }
