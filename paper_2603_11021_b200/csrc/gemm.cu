@@ -8,6 +8,25 @@ namespace {
 #include "gemv_kernels.cuh"
 #include "gemm_kernels.cuh"
 
+// The tensor map of X [batch][k_in] bf16 (16-byte aligned, k_in a multiple of 8): boxes of 64 columns x npad rows, 128-byte swizzle.
+bool make_x_map(const uint16_t* d_x, int64_t k_in, int batch, int npad, CUtensorMap* map)
+{
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {                    // the driver's function, without linking against the driver library
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) fn = nullptr;
+        return reinterpret_cast<Encode>(fn);
+    }();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)k_in, (cuuint64_t)batch}, strides[1] = {(cuuint64_t)k_in * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)npad}, steps[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(d_x), dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // The codes whose class tables stay in global memory have room for the table of small subsets beside the GEMM's buffers.
 size_t gemm_image_bytes(const llvq_ctx* ctx) { return ctx->fast ? ctx->fl.total : ctx->fl.total_ext; }
 
@@ -57,14 +76,16 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
         if (pipe) {                                                                                                          \
             if (!set_smem<gemm_pipe_kernel<BIG, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                            \
             if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx, !ctx->fast), \
-                           static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, b_double) != cudaSuccess) return LLVQ_ECUDA; \
+                           static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, b_double, xmap) != cudaSuccess) return LLVQ_ECUDA; \
         } else {                                                                                                             \
             if (!set_smem<gemm_sorted_kernel<BIG, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                          \
             if (launch_pdl(gemm_sorted_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx, !ctx->fast), \
-                           static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, dpi) != cudaSuccess) return LLVQ_ECUDA; \
+                           static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA; \
         }                                                                                                                    \
     } while (0)
     const SgArgs sga = sg ? *sg : SgArgs{};
+    CUtensorMap xmap;
+    if (!make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
     if (yo) {                                            // row-sharded: stored-gain form only
         if (sg) return LLVQ_EUNSUPPORTED;
         if (ctx->fast) LLVQ_LAUNCH_DOMAINS(false, false, true); else LLVQ_LAUNCH_DOMAINS(true, false, true);
@@ -117,6 +138,8 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     if (smem > 227 * 1024) return LLVQ_EUNSUPPORTED;
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (yo && sg) return LLVQ_EUNSUPPORTED;              // row-sharded: stored-gain form only
+    CUtensorMap xmap;
+    if (!make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
     // codes with their class tables in shared memory and many classes (a warp of 32 unrelated blocks is what costs there):
     // the kernel that puts every domain of 1024 blocks into the order of the sorted layout before unranking it, as many
     // domains at a time (up to 4) as shared memory has room for beside the operand buffers
@@ -143,7 +166,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     do {                                                                                                                        \
         if (!set_smem<gemm_sorted_kernel<false, SG, SH, true, RD>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                 \
         if (launch_pdl(gemm_sorted_kernel<false, SG, SH, true, RD>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, false), words, \
-                       d_gain_f16, sga, gb, dpi) != cudaSuccess) return LLVQ_ECUDA;                                             \
+                       d_gain_f16, sga, gb, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA;                                             \
     } while (0)
             if (gb.bin_round > dpi) {                    // rounds of several iterations
                 if (yo) LLVQ_LAUNCH_BINNED(false, true, true);
@@ -178,11 +201,11 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             if (yo) {
                 if (!set_smem<gemm_sorted_kernel<true, false, true, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
                 if (launch_pdl(gemm_sorted_kernel<true, false, true, true, true>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, true), words,
-                               d_gain_f16, SgArgs{}, gb, dpi) != cudaSuccess) return LLVQ_ECUDA;
+                               d_gain_f16, SgArgs{}, gb, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA;
             } else {
                 if (!set_smem<gemm_sorted_kernel<true, false, false, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
                 if (launch_pdl(gemm_sorted_kernel<true, false, false, true, true>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, true), words,
-                               d_gain_f16, SgArgs{}, gb, dpi) != cudaSuccess) return LLVQ_ECUDA;
+                               d_gain_f16, SgArgs{}, gb, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA;
             }
             return launch_status();
         }
@@ -205,7 +228,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     do {                                                                                                                        \
         if (!set_smem<gemm_pipe_kernel<BIG, SG, SH, true>>(ctx->device, smem_pipe)) return LLVQ_ECUDA;                                        \
         if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH, true>, grid_pipe, (unsigned)kGemmThreads, smem_pipe, st, fast_args(ctx, !ctx->fast), words, \
-                       d_gain_f16, sga, gp, b_double) != cudaSuccess) return LLVQ_ECUDA;                                        \
+                       d_gain_f16, sga, gp, b_double, xmap) != cudaSuccess) return LLVQ_ECUDA;                                        \
     } while (0)
             if (!ctx->fast) { if (yo) LLVQ_LAUNCH_PIPE_STORED(true, false, true); else LLVQ_LAUNCH_PIPE_STORED(true, false, false); }
             else if (yo) LLVQ_LAUNCH_PIPE_STORED(false, false, true);

@@ -222,6 +222,27 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
 constexpr int kDomBlocks = 8;                          // column blocks per domain
 constexpr int kDomEntries = kGemmRows * kDomBlocks;    // 1024
 constexpr int kDomStages = 2;                          // 96-column MMA stages per domain
+// The slice of X that goes with a domain, 192 columns x the padded batch: three panels of 64 columns, each one TMA box with the
+// 128-byte swizzle (rows and columns outside X come as zeros).  One thread asks for them; copied by a warp, 16 bytes per lane and
+// row, the slices took 85 of the 212 passes per chunk through the load / store pipe that bounds the kernel at batch 64
+// (28672 x 8192: 308 -> 250 us).
+constexpr int kXPanels = kDomBlocks * 24 / 64;
+
+__device__ __forceinline__ void request_x(uint32_t dst, const CUtensorMap* map, int domain, int npad, uint64_t* bar)
+{
+    mbar_expect(bar, (uint32_t)(kXPanels * npad * 128));
+#pragma unroll
+    for (int i = 0; i < kXPanels; ++i) tma_load_2d(dst + (uint32_t)(i * npad * 128), map, domain * (kDomBlocks * 24) + i * 64, 0, bar);
+}
+
+// The 12 MMAs of a domain: A tile at a_addr (two 96-column stages), X slice at b_addr; fresh = the accumulator starts at zero.
+__device__ __forceinline__ void domain_mmas(uint32_t tmem, uint32_t a_addr, uint32_t b_addr, int npad, uint32_t idesc, bool fresh)
+{
+#pragma unroll
+    for (int t = 0; t < kDomBlocks * 24 / 16; ++t)
+        umma_bf16(tmem, smem_desc(a_addr + (uint32_t)t * 4096u, 2048, 128), smem_desc_sw128(b_addr + (uint32_t)((t >> 2) * npad * 128 + (t & 3) * 32)), idesc,
+                  !fresh || t > 0 ? 1u : 0u);
+}
 
 __global__ void __launch_bounds__(kDomEntries, 1)
 sort_blocks_gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, int gain_bits, int64_t n_out,
@@ -353,14 +374,17 @@ sort_blocks_gemm_big_kernel(FastArgs fa, const uint32_t* __restrict__ stream, in
 // reads from L2) run side by side.
 template <bool kBig, bool kSg = false, bool kShard = false, bool kBin = false, bool kRound = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga, int dpi)
+gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga, int dpi,
+                   const __grid_constant__ CUtensorMap xmap)
 {
     static_assert(!(kBin && kBig && (kSg || !kRound)), "in-kernel ordering for the codes with tables in global memory: stored gains, rounds");
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem_1k[];
+    uint8_t* const smem = smem_1k;
     const uint32_t img_bytes = fa.image_bytes;
     uint64_t* bar_img = reinterpret_cast<uint64_t*>(smem + img_bytes);
     uint64_t* bar_free = bar_img + 1;                                     // the MMAs reading the A / B buffers are done
     uint64_t* bar_done = bar_img + 2;                                     // the accumulator of this item is complete
+    uint64_t* bar_x = bar_img + 3;                                        // the X slices of the iteration are in the buffer
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_img + 5);
     uint32_t* last_flag = tmem_slot + 1;
     const uint32_t a_off = (img_bytes + 64 + 1023) & ~1023u;
@@ -389,7 +413,7 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
     if (kBin)
         for (int i = threadIdx.x; i < nround * ga.nbins; i += kGemmThreads) bin_hist[i] = 0u;
     if (threadIdx.x == 0) {
-        mbar_init(bar_free, 1); mbar_init(bar_done, 1);
+        mbar_init(bar_free, 1); mbar_init(bar_done, 1); mbar_init(bar_x, (uint32_t)dpi);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
@@ -404,8 +428,6 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
     const uint32_t dom_begin = split_begin(ga.sp, blockIdx.x), dom_end = split_begin(ga.sp, blockIdx.x + 1u);
     uint32_t uses = 0, done = 0;
     bool timeout = false;
-    // where this thread's 16-byte chunks of an X slice lie: chunk i is (kc, n) = (i / npad, i % npad), i in steps of the block
-    const int bx_kc = (int)threadIdx.x / ga.npad, bx_n = (int)threadIdx.x % ga.npad, bx_step_kc = kGemmThreads / ga.npad, bx_step_n = kGemmThreads % ga.npad;
     for (uint32_t rt = split_row(ga.sp, dom_begin); rt * nd < dom_end; ++rt) {
         const uint32_t tile0 = rt * nd, tile1 = tile0 + nd;
         const int d_begin = (int)(max(dom_begin, tile0) - tile0), d_end = (int)(min(dom_end, tile1) - tile0);
@@ -568,32 +590,27 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
                     expand_bf16(dec, gn, w);
                 }
                 // the previous MMAs read the buffers: wait for them only now, with the first chunk already unranked
-                if (q == 0 && uses > 0 && !mbar_wait(bar_free, (uses - 1u) & 1u)) timeout = true;
+                if (q == 0) {
+                    if (uses > 0 && !mbar_wait(bar_free, (uses - 1u) & 1u)) timeout = true;
+                    if (threadIdx.x == 0)
+                        for (int st = 0; st < dpi; ++st) {
+                            if (st < nd_now) request_x(smem_u32(b_buf) + (uint32_t)st * kDomStages * b_stage, &xmap, d0 + st, ga.npad, bar_x);
+                            else mbar_expect(bar_x, 0u);
+                        }
+                }
                 uint8_t* a_dst = a_buf + (uint32_t)(q * kDomStages + (c >> 2)) * kAStage + (r >> 3) * 128u + (r & 7u) * 16u + 3u * (c & 3u) * 2048u;
 #pragma unroll
                 for (int j = 0; j < 3; ++j)
                     *reinterpret_cast<uint4*>(a_dst + j * 2048) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
             }
-            // ---- B: the slice of X of these stages, 16-byte chunks (8 values along K)
-            const int kchunks = nd_now * kDomStages * (kStageK / 8);
-            for (int i = threadIdx.x, kc = bx_kc, n = bx_n; i < ga.npad * kchunks; i += kGemmThreads, kc += bx_step_kc, n += bx_step_n) {
-                if (n >= ga.npad) { n -= ga.npad; ++kc; }
-                const int k = d0 * kDomBlocks * 24 + kc * 8;
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (n < ga.batch && k < ga.k_in) v = __ldg(reinterpret_cast<const uint4*>(ga.x + (int64_t)n * ga.k_in + k));
-                *reinterpret_cast<uint4*>(b_buf + (uint32_t)i * 16u) = v;              // [kc][n], stage after stage
-            }
             fence_async_smem();
             __syncthreads();
             if (threadIdx.x == 0) {
+                if (!mbar_wait(bar_x, uses & 1u)) timeout = true;
                 tc_fence_after();
-                const uint32_t a_addr = smem_u32(a_buf), b_addr = smem_u32(b_buf);
-                for (int st = 0; st < nd_now * kDomStages; ++st)
-#pragma unroll
-                    for (int j = 0; j < kStageK / 16; ++j)
-                        umma_bf16(tmem, smem_desc(a_addr + st * kAStage + j * 4096, 2048, 128),
-                                  smem_desc(b_addr + st * b_stage + j * 2 * ga.npad * 16, ga.npad * 16, 128), idesc,
-                                  (d0 > d_begin || st > 0 || j > 0) ? 1u : 0u);
+                for (int st = 0; st < nd_now; ++st)
+                    domain_mmas(tmem, smem_u32(a_buf) + (uint32_t)st * kDomStages * kAStage, smem_u32(b_buf) + (uint32_t)st * kDomStages * b_stage, ga.npad,
+                                idesc, d0 == d_begin && st == 0);
                 umma_commit(bar_free);
                 if (d0 + dpi >= d_end) umma_commit(bar_done);
             }
@@ -656,17 +673,18 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
 // row tile are handed out by a ticket counter (ticket t = chunk t % 32 of the tile's domain t / 32, so from expensive
 // to cheap inside a domain), a warp always holding its next ticket with that chunk's entries already requested.
 // It unranks the chunk, waits (rarely) until the MMAs that read this buffer two domains ago are done, writes its
-// part of A and arrives on the buffer's "full" barrier.  Warp 0 stages the X slice of the next domain, arrives too,
-// and its first thread issues the MMAs of a domain as soon as that barrier completes.
+// part of A and arrives on the buffer's "full" barrier.  The first thread of warp 0 asks for the X slice of the next domain, whose
+// bytes that barrier counts too, and issues the MMAs of a domain as soon as it completes.
 // kStored: the same structure on the stored stream (`sorted` then points at it): a chunk is 32 consecutive blocks of the
 // domain in natural order (4 rows x 8 column blocks), unranked by the any-class decoder.
 template <bool kBig, bool kSg = false, bool kShard = false, bool kStored = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga,
-                 int b_double)
+                 int b_double, const __grid_constant__ CUtensorMap xmap)
 {
     static_assert(!(kStored && kBig && kSg), "no shape-gain form for the codes with tables in global memory");
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem_1k[];
+    uint8_t* const smem = smem_1k;
     const uint32_t img_bytes = fa.image_bytes;
     uint64_t* bar_img = reinterpret_cast<uint64_t*>(smem + img_bytes);
     uint64_t* bar_full = bar_img + 1;                                     // [2] 32 chunks of A and the X slice are in the buffer
@@ -723,59 +741,28 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
         __syncthreads();
         if (warp == 0) {
             // ---- X slices and MMAs
-            // the slice of domain j of this tile, 16-byte chunks (8 values along K).  With two X buffers it may be written once
-            // the MMAs of two domains ago are done; with one (wide batches: no room for two), only after the previous domain's
-            auto stage_b = [&](uint32_t j) {
-                const uint32_t gd = g_base + j, b = gd & 1u, bx = b_double ? b : 0u;
-                if (b_double) { if (gd >= 2u && !mbar_wait(bar_free + b, ((gd >> 1) - 1u) & 1u)) timeout = true; }
-                else if (gd >= 1u && !mbar_wait(bar_free + ((gd - 1u) & 1u), ((gd - 1u) >> 1) & 1u)) timeout = true;
-                // [kc][n] 16-byte chunks, kc = 0..23.  The loop competes for issue slots with the unranking warps, and with one X
-                // buffer it stands between two domains (28672 x 8192, batch 64: 393 -> 329 us): per chunk one copy and one address step, the size (0 = zero fill)
-                // settled per row except in the last domain of a row of X
-                const uint32_t k0 = (uint32_t)(d_begin + (int)j) * kDomBlocks * 24;
-                const uint32_t have = min((uint32_t)ga.k_in - k0, (uint32_t)(kDomStages * kStageK)) / 8u;          // chunks inside X
-                const int per = ga.npad < 32 ? 2 : 1;                                                           // 16 rows: two lanes per row
-                const int kc0 = per == 2 ? lane >> 4 : 0;
-                for (int n = per == 2 ? lane & 15 : lane; n < ga.npad; n += 32) {
-                    const bool row_in = n < ga.batch;
-                    const uint16_t* src = ga.x + (row_in ? (int64_t)n * ga.k_in : 0) + k0 + 8 * kc0;
-                    uint32_t to = smem_u32(b_buf) + bx * kDomStages * b_stage + (uint32_t)(kc0 * ga.npad + n) * 16u;
-                    const uint32_t step = (uint32_t)(per * ga.npad) * 16u;
-                    if (have == kDomStages * (kStageK / 8) && per == 1) {
-                        const uint32_t size = row_in ? 16u : 0u;
-#pragma unroll
-                        for (int kc = 0; kc < kDomStages * (kStageK / 8); ++kc, to += step)
-                            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(src + 8 * kc), "r"(size) : "memory");
-                    } else {
-                        for (int kc = kc0; kc < kDomStages * (kStageK / 8); kc += per, src += 8 * per, to += step) {
-                            const bool in = row_in && (uint32_t)kc < have;
-                            asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(in ? src : ga.x), "r"(in ? 16u : 0u) : "memory");
-                        }
-                    }
-                }
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                arrive_full(b);
-            };
-            if (n_dom > 0) stage_b(0);
-            for (uint32_t j = 0; j < n_dom; ++j) {
-                if (b_double && j + 1 < n_dom) stage_b(j + 1);
-                const uint32_t gd = g_base + j, b = gd & 1u, bx = b_double ? b : 0u;
-                if (lane == 0) {
+            // With two X buffers a domain's slice may be written once the MMAs of two domains ago are done; with one (wide batches: no
+            // room for two), only after the previous domain's
+            if (lane == 0) {
+                auto stage_b = [&](uint32_t j) {
+                    const uint32_t gd = g_base + j, b = gd & 1u, bx = b_double ? b : 0u;
+                    if (b_double) { if (gd >= 2u && !mbar_wait(bar_free + b, ((gd >> 1) - 1u) & 1u)) timeout = true; }
+                    else if (gd >= 1u && !mbar_wait(bar_free + ((gd - 1u) & 1u), ((gd - 1u) >> 1) & 1u)) timeout = true;
+                    request_x(smem_u32(b_buf) + bx * kDomStages * b_stage, &xmap, d_begin + (int)j, ga.npad, bar_full + b);
+                };
+                if (n_dom > 0) stage_b(0);
+                for (uint32_t j = 0; j < n_dom; ++j) {
+                    if (b_double && j + 1 < n_dom) stage_b(j + 1);
+                    const uint32_t gd = g_base + j, b = gd & 1u, bx = b_double ? b : 0u;
                     if (!mbar_wait(bar_full + b, (gd >> 1) & 1u)) timeout = true;
                     tc_fence_after();
-                    const uint32_t a_addr = smem_u32(a_buf) + b * kDomStages * kAStage, b_addr = smem_u32(b_buf) + bx * kDomStages * b_stage;
-                    for (int st = 0; st < kDomStages; ++st)
-#pragma unroll
-                        for (int jj = 0; jj < kStageK / 16; ++jj)
-                            umma_bf16(tmem, smem_desc(a_addr + st * kAStage + jj * 4096, 2048, 128),
-                                      smem_desc(b_addr + st * b_stage + jj * 2 * ga.npad * 16, ga.npad * 16, 128), idesc,
-                                      (j > 0 || st > 0 || jj > 0) ? 1u : 0u);
+                    domain_mmas(tmem, smem_u32(a_buf) + b * kDomStages * kAStage, smem_u32(b_buf) + bx * kDomStages * b_stage, ga.npad, idesc, j == 0);
                     umma_commit(bar_free + b);
                     if (j + 1 == n_dom) umma_commit(bar_done);
+                    if (!b_double && j + 1 < n_dom) stage_b(j + 1);
                 }
-                __syncwarp();
-                if (!b_double && j + 1 < n_dom) stage_b(j + 1);
             }
+            __syncwarp();
         } else {
             // ---- A: unrank chunks until the tile's tickets are gone
             const int64_t entry0 = (int64_t)(tile0 + d_begin) * kDomEntries + lane;

@@ -1,7 +1,9 @@
 // Thin wrappers over the Blackwell tensor-core instructions used by the small-batch GEMM:
-// tcgen05.mma with both operands in shared memory (K-major, no swizzle) and the
-// accumulator in tensor memory, plus the mbarrier / fence / TMEM plumbing.
+// tcgen05.mma with both operands in shared memory (K-major, without swizzle or with the 128-byte swizzle) and the
+// accumulator in tensor memory, plus the mbarrier / fence / TMEM / tiled-TMA plumbing.
 #pragma once
+#include <cuda.h>
+
 #include <cstdint>
 
 namespace llvq {
@@ -52,6 +54,26 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 {
     return (uint64_t)((addr >> 4) & 0x3fffu) | (uint64_t)((lbo >> 4) & 0x3fffu) << 16 | (uint64_t)((sbo >> 4) & 0x3fffu) << 32 |
            1ull << 46;
+}
+
+// Shared-memory operand, K-major, rows of 64 bf16 values (128 bytes) swizzled as TMA leaves them (CU_TENSOR_MAP_SWIZZLE_128B):
+// 8-row groups of 1024 bytes, one after the other; the panel starts on a 1024-byte boundary, addr advances 32 bytes per MMA.
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
+{
+    return (uint64_t)((addr >> 4) & 0x3fffu) | 1ull << 16 | (uint64_t)(1024u >> 4) << 32 | 1ull << 46 | 2ull << 61;
+}
+
+// Tiled TMA load of one box of a 2-d tensor map at (x, y) (x in elements, a multiple of 8) into shared memory, counted on bar.
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar)
+{
+    asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
+}
+
+// Arrive once on bar and add `bytes` to what its phase waits for.
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
 // bf16 x bf16 -> f32, both operands K-major, M = 128, N = n (multiple of 16).
