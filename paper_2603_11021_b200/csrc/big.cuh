@@ -9,6 +9,13 @@
 
 namespace llvq {
 
+// Top 16 bits of a W-bit index (hi:lo): the bucket of the class table.
+__device__ __forceinline__ uint32_t big_bucket(const DevCode& dc, uint64_t lo, uint64_t hi)
+{
+    const int sh = dc.W > 16 ? dc.W - 16 : 0;
+    return (uint32_t)(sh >= 64 ? hi >> (sh - 64) : (sh ? (lo >> sh) | (hi << (64 - sh)) : lo)) & 0xffffu;
+}
+
 // S2: class of index (hi:lo) < N: bucket table on the top 16 bits, then bisection between the classes of this
 // bucket's and the next bucket's first index.
 __device__ __forceinline__ int big_find_class(const DevCode& dc, uint64_t lo, uint64_t hi, uint64_t& local)

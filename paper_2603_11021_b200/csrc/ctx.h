@@ -31,6 +31,7 @@ struct llvq_ctx {
     bool fast = false;               // class tables fit the shared-memory image; otherwise they are read from global memory
     llvq::FastLayout fl{};
     const uint8_t* d_image = nullptr;
+    uint64_t largest_class = 0;      // points of the largest class
     bool can_encode = false;         // m_lo == 2, m_hi >= 6, indices fit 64 bits
     EncTables enc{};
     llvq::GolayTrio trio{};

@@ -91,13 +91,13 @@ struct RawField {
     uint32_t w0, w1, w2, w3, shift;
 };
 
+// The field that starts `bits` bits behind the word p0.
 template <bool kBig>
-__device__ __forceinline__ RawField<kBig> request_field(const uint32_t* __restrict__ stream, uint64_t b, int W, bool in)
+__device__ __forceinline__ RawField<kBig> request_field_at(const uint32_t* __restrict__ p0, uint32_t bits, int W, bool in)
 {
     RawField<kBig> f;
-    const uint64_t bp = b * (uint64_t)W;
-    const uint32_t* p = stream + (bp >> 5);
-    f.shift = (uint32_t)bp & 31u;
+    const uint32_t* p = p0 + (bits >> 5);
+    f.shift = bits & 31u;
     const uint32_t last = in ? f.shift + (uint32_t)W : 0u;       // bits counted from the first word (0: nothing is read)
     f.w0 = f.w1 = f.w2 = f.w3 = 0u;
     if (last > 0u) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(f.w0) : "l"(p));
@@ -105,6 +105,13 @@ __device__ __forceinline__ RawField<kBig> request_field(const uint32_t* __restri
     if (last > 64u) asm volatile("ld.global.nc.u32 %0, [%1+8];" : "=r"(f.w2) : "l"(p));
     if (kBig && last > 96u) asm volatile("ld.global.nc.u32 %0, [%1+12];" : "=r"(f.w3) : "l"(p));
     return f;
+}
+
+template <bool kBig>
+__device__ __forceinline__ RawField<kBig> request_field(const uint32_t* __restrict__ stream, uint64_t b, int W, bool in)
+{
+    const uint64_t bp = b * (uint64_t)W;
+    return request_field_at<kBig>(stream + (bp >> 5), (uint32_t)bp & 31u, W, in);
 }
 
 // Keeps whatever is formed from the words behind this point.

@@ -5,6 +5,7 @@
 
 namespace {
 
+#include "order.cuh"
 #include "gemv_kernels.cuh"
 #include "gemm_kernels.cuh"
 

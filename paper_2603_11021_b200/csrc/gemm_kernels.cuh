@@ -297,13 +297,6 @@ constexpr unsigned long long kBigNoBlock = 1ull << 63;
 constexpr int kBigEntryWords = 3;
 constexpr int kBigClassBits = 17;
 
-// Top 16 bits of a W-bit index (hi:lo): the bucket of the class table.
-__device__ __forceinline__ uint32_t big_bucket(const DevCode& dc, uint64_t lo, uint64_t hi)
-{
-    const int sh = dc.W > 16 ? dc.W - 16 : 0;
-    return (uint32_t)(sh >= 64 ? hi >> (sh - 64) : (sh ? (lo >> sh) | (hi << (64 - sh)) : lo)) & 0xffffu;
-}
-
 // Entry `at` of a sorted stream of 96-bit entries, in the two-word form the kernels use.
 __device__ __forceinline__ ulonglong2 load_big_entry(const void* sorted, int64_t at)
 {

@@ -7,19 +7,23 @@ int llvq_internal_gemv_domains(const llvq_ctx* ctx, const void* d_sorted, const 
 
 namespace {
 
+#include "order.cuh"
 #include "gemv_kernels.cuh"
 
 constexpr size_t kSmemLimit = 227 * 1024;
 
-// Shared memory of gemv_bin_kernel for `su` units per segment, and whether the table of small subsets still fits.
-void bin_smem(const llvq_ctx* ctx, int64_t nq, int su, size_t& bytes, bool& ext)
+// Whether gemv_order_kernel takes a matrix of nq units per row group; its shared memory, and whether the table of small subsets
+// still fits.
+bool order_smem(const llvq_ctx* ctx, int64_t nq, int gain_bits, OrderArgs& oa, size_t& bytes, bool& ext)
 {
-    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + 16 + 2 * 1024 * 4 + (size_t)su * 32 * (8 + 2);
-    ext = ctx->fl.total_ext + rest <= kSmemLimit;
+    if (nq >= (1ll << 24) || !order_args(ctx, gain_bits, &oa)) return false;
+    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + gemv_order_bytes(oa, !ctx->fast);
+    ext = ctx->fast && ctx->fl.total_ext + rest <= kSmemLimit;       // (big codes: their lanes almost never agree on a small subset)
     bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest;
+    return bytes <= kSmemLimit;
 }
 
-// The same for gemv_sorted_kernel; acc_floats = room for the row sums, cut down to one copy per row where rows are so long that x
+// The shared memory of gemv_sorted_kernel; acc_floats = room for the row sums, cut down to one copy per row where rows are so long that x
 // needs the space.
 void sorted_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext, uint32_t& acc_floats)
 {
@@ -28,14 +32,6 @@ void sorted_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext, uint
     while (acc_floats > kGemvGroupsPerPass * kGemvGroupRows && ctx->fl.total + rest + acc_floats * 4 > kSmemLimit) acc_floats /= 2;
     ext = ctx->fl.total_ext + rest + acc_floats * 4 <= kSmemLimit;
     bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest + acc_floats * 4;
-}
-
-bool bin_kernel_serves(const llvq_ctx* ctx, int64_t nq, const SgArgs* sg)
-{
-    size_t bytes; bool ext;
-    bin_smem(ctx, nq, kBinSegUnits, bytes, ext);
-    return (!sg || sg->bits <= 5) && ctx->fast && ctx->d_sort_rank && ctx->host.desc.size() >= 64 && ctx->host.W <= 48 && bytes <= kSmemLimit &&
-           nq < (1ll << 24);
 }
 
 // Shared by llvq_gemv, llvq_gemv_sg and llvq_gemv_rowshard: exactly one of d_gain_f16 / sg is used.
@@ -82,24 +78,25 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const SgArgs sga = sg ? *sg : SgArgs{};
     const bool shard = yo.n_peer > 0 || yo.n_flag > 0;                  // row-sharded launch: stored-gain form only
     if (shard && sg) return LLVQ_EUNSUPPORTED;
-    // fast-path codes with many classes (mixed warps are what costs there): the kernel that bins the blocks of a segment by
-    // class before unranking them; codes with a handful of classes keep the direct kernel
-    int seg_units = kBinSegUnits;
-    size_t smem_bin; bool ext_bin;
-    bin_smem(ctx, nq, seg_units, smem_bin, ext_bin);
-    // (smaller segments sort too few blocks to pay for the sort: the direct kernel takes over when 8192 do not fit)
-    if (bin_kernel_serves(ctx, nq, sg)) {
-        const FastArgs fa = fast_args(ctx, ext_bin);
-#define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
+    // codes with many classes (a warp of unrelated blocks is what costs there): the kernel that orders the blocks before it unranks
+    // them; codes with a handful of classes, and rows too long for its buffers, keep the direct kernel
+    OrderArgs oa;
+    size_t smem_order; bool ext_order;
+    if (order_smem(ctx, nq, sg ? sg->bits : 0, oa, smem_order, ext_order)) {
+        const FastArgs fa = fast_args(ctx, ext_order);
+#define LLVQ_LAUNCH_ORDER(BIG, BF16, SG, SH)                                                                               \
     do {                                                                                                                   \
-        if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                          \
-        if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
-                       bpr, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
+        if (!set_smem<gemv_order_kernel<BIG, BF16, SG, SH>>(ctx->device, smem_order)) return LLVQ_ECUDA;                   \
+        if (launch_pdl(gemv_order_kernel<BIG, BF16, SG, SH>, g, (unsigned)kSortThreads, smem_order, st, fa, idx, oa, d_gain_f16, sga, sp, n_out, k_in, \
+                       bpr, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;              \
     } while (0)
-        if (shard)   { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, true); else LLVQ_LAUNCH_BIN(false, false, true); }
-        else if (sg) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, true, false); else LLVQ_LAUNCH_BIN(false, true, false); }
-        else         { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, false); else LLVQ_LAUNCH_BIN(false, false, false); }
-#undef LLVQ_LAUNCH_BIN
+        const bool bf16 = y_dtype == LLVQ_BF16;
+        if (shard && ctx->fast) { if (bf16) LLVQ_LAUNCH_ORDER(false, true, false, true); else LLVQ_LAUNCH_ORDER(false, false, false, true); }
+        else if (shard)         { if (bf16) LLVQ_LAUNCH_ORDER(true, true, false, true);  else LLVQ_LAUNCH_ORDER(true, false, false, true); }
+        else if (sg)            { if (bf16) LLVQ_LAUNCH_ORDER(false, true, true, false); else LLVQ_LAUNCH_ORDER(false, false, true, false); }
+        else if (ctx->fast)     { if (bf16) LLVQ_LAUNCH_ORDER(false, true, false, false); else LLVQ_LAUNCH_ORDER(false, false, false, false); }
+        else                    { if (bf16) LLVQ_LAUNCH_ORDER(true, true, false, false);  else LLVQ_LAUNCH_ORDER(true, false, false, false); }
+#undef LLVQ_LAUNCH_ORDER
         return launch_status();
     }
     const FastArgs fa = fast_args(ctx, ext_direct);
@@ -268,19 +265,19 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         const int64_t units = ((d.n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
         // every matrix must give every CTA work: the sorted layout was made for that many CTAs
         if (units < ctx->sm_count) return LLVQ_EUNSUPPORTED;
-        if (sorted ? !sortable(ctx, d.k_in) : !bin_kernel_serves(ctx, nq, nullptr)) return LLVQ_EUNSUPPORTED;
+        if (sorted && !sortable(ctx, d.k_in)) return LLVQ_EUNSUPPORTED;
         max_nq = std::max(max_nq, nq);
         GemvMat& m = mm.m[i];
         m.weights = d.d_weights; m.gain = d.d_gain_f16; m.x = d.d_x_bf16; m.y = d.d_y;
         m.n_out = d.n_out; m.k_in = d.k_in; m.slot0 = slot;
         m.sp = make_split(units, nq, (unsigned)ctx->sm_count); m.bpr = (int32_t)bpr;
-        m.seg_units = kBinSegUnits;
         slot += (d.n_out + kGemvGroupRows - 1) / kGemvGroupRows * kGemvGroupRows;
     }
     if (slot > 64ll * kMaxScratchRows) return LLVQ_EUNSUPPORTED;
     size_t smem; bool ext;                               // the longest rows decide for the whole launch
+    OrderArgs oa{};
     if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);
-    else bin_smem(ctx, max_nq, kBinSegUnits, smem, ext);
+    else if (!ctx->fast || !order_smem(ctx, max_nq, 0, oa, smem, ext)) return LLVQ_EUNSUPPORTED;
     if (smem > kSmemLimit) return LLVQ_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
@@ -327,11 +324,11 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         }
     } else {
         if (y_dtype == LLVQ_BF16) {
-            if (!set_smem<gemv_bin_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_bin_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, ctx->d_sort_rank, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
+            if (!set_smem<gemv_order_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
+            if (launch_pdl(gemv_order_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, oa, mm, (uint32_t)max_nq, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         } else {
-            if (!set_smem<gemv_bin_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_bin_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, ctx->d_sort_rank, mm, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
+            if (!set_smem<gemv_order_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
+            if (launch_pdl(gemv_order_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, oa, mm, (uint32_t)max_nq, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         }
     }
     return launch_status();

@@ -229,11 +229,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // round of a loop up to the load and waits for it there.
 __device__ __forceinline__ void use_from_here(unsigned long long& v) { asm volatile("" : "+l"(v)); }
 
-// Ask for the 128-byte lines of [p + first, p + last) in L2; the whole CTA calls this.
-__device__ __forceinline__ void prefetch_span_l2(const void* p, uint64_t first, uint64_t last)
+// Ask for the 128-byte lines of [p + first, p + last) in L2; called by `nthreads` threads numbered `tid`.
+__device__ __forceinline__ void prefetch_span_l2(const void* p, uint64_t first, uint64_t last, uint32_t tid, uint32_t nthreads)
 {
     const uint8_t* base = static_cast<const uint8_t*>(p);
-    for (uint64_t o = (first & ~127ull) + (uint64_t)threadIdx.x * 128; o < last; o += (uint64_t)blockDim.x * 128)
+    for (uint64_t o = (first & ~127ull) + (uint64_t)tid * 128; o < last; o += (uint64_t)nthreads * 128)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(base + o));
 }
 

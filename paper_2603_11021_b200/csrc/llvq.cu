@@ -222,6 +222,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     ctx->dev.flags = reinterpret_cast<uint32_t*>(d + o_err + 8);
     ctx->dev.n_lo = (uint64_t)h.N; ctx->dev.n_hi = (uint64_t)(h.N >> 64);
     ctx->dev.nclasses = (int)ncls;
+    for (const ClassInfo& c : h.info) ctx->largest_class = std::max(ctx->largest_class, (uint64_t)c.card);
     ctx->dev.W = h.W;
     ctx->d_image = d + o_img;
     ctx->d_golay = reinterpret_cast<const uint32_t*>(d + o_gol);
