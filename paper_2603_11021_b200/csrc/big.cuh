@@ -9,20 +9,20 @@
 
 namespace llvq {
 
-// Top 16 bits of a W-bit index (hi:lo): the bucket of the class table.
+// Top bits of a W-bit index (hi:lo): the bucket of the class table.
 __device__ __forceinline__ uint32_t big_bucket(const DevCode& dc, uint64_t lo, uint64_t hi)
 {
-    const int sh = dc.W > 16 ? dc.W - 16 : 0;
-    return (uint32_t)(sh >= 64 ? hi >> (sh - 64) : (sh ? (lo >> sh) | (hi << (64 - sh)) : lo)) & 0xffffu;
+    const int sh = dc.W - kBigBucketBits;                // 1..52
+    if (sh <= 0) return (uint32_t)lo;
+    return (uint32_t)((lo >> sh) | (hi << (64 - sh)));
 }
 
-// S2: class of index (hi:lo) < N: bucket table on the top 16 bits, then bisection between the classes of this
-// bucket's and the next bucket's first index.
+// S2: class of index (hi:lo) < N: bucket table, then bisection between the classes of this bucket's and the next bucket's first
+// index.
 __device__ __forceinline__ int big_find_class(const DevCode& dc, uint64_t lo, uint64_t hi, uint64_t& local)
 {
-    const int sh = dc.W > 16 ? dc.W - 16 : 0;
-    const uint32_t bucket = (uint32_t)(sh >= 64 ? hi >> (sh - 64) : (sh ? (lo >> sh) | (hi << (64 - sh)) : lo)) & 0xffffu;
-    int a = (int)__ldg(dc.lut16 + bucket), b = (int)__ldg(dc.lut16 + bucket + 1);
+    const uint32_t bucket = big_bucket(dc, lo, hi);
+    int a = (int)__ldg(dc.lut + bucket), b = (int)__ldg(dc.lut + bucket + 1);
     while (a < b) {
         const int mid = (a + b + 1) >> 1;
         const uint64_t ol = __ldg(dc.off_lo + mid);
@@ -114,10 +114,10 @@ __device__ __forceinline__ void big_decode_record(const FastSmem& T, const uint4
                 // and places the empty subset), no division
                 rho = (uint32_t)p;
             } else if (__any_sync(mask, (uint32_t)(p >> 32) != 0u)) {
-                const uint64_t qq0 = __umul64hi(p, lds_u64(r64_a + cell * 8u));
-                uint64_t qq = qq0, rem = p - qq * radix;
-                if (rem >= radix) { rem -= radix; ++qq; }
-                if (active) { p = qq; rho = (uint32_t)rem; }
+                // (no class of the largest supported code has more than 2^50.2 arrangements)
+                uint32_t rem;
+                const uint64_t qq = divide52(p, radix, __longlong_as_double((long long)lds_u64(r64_a + cell * 8u)), rem);
+                if (active) { p = qq; rho = rem; }
             } else {
                 const uint32_t p32 = (uint32_t)p;
                 uint32_t qq = __umulhi(p32, lds_u32(r32_a + cell * 4u));

@@ -16,7 +16,7 @@ struct DevCode {
     const BigDesc* big;             // [nclasses] compact records (codes whose class tables stay in global memory)
     const uint64_t* off_lo;         // [nclasses + 1] low 64 bits of the class offsets
     const uint32_t* off_hi;         // [nclasses + 1] bits 64.. of the class offsets
-    const uint32_t* lut16;          // [65537] class of the first index of bucket (I >> (W - 16)), then the last class
+    const uint32_t* lut;            // [2^kBigBucketBits + 1] class of the first index of bucket (I >> (W - kBigBucketBits)), then the last class; codes with class tables in global memory
     unsigned long long* bad_index;  // device counter of fields with I >= N
     uint32_t* flags;                // device error flags
     uint64_t n_lo, n_hi;            // N

@@ -17,8 +17,8 @@ constexpr size_t kSmemLimit = 227 * 1024;
 bool order_smem(const llvq_ctx* ctx, int64_t nq, int gain_bits, OrderArgs& oa, size_t& bytes, bool& ext)
 {
     if (nq >= (1ll << 24) || !order_args(ctx, gain_bits, &oa)) return false;
-    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + gemv_order_bytes(oa, !ctx->fast);
-    ext = ctx->fast && ctx->fl.total_ext + rest <= kSmemLimit;       // (big codes: their lanes almost never agree on a small subset)
+    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + gemv_order_bytes(oa);
+    ext = ctx->fl.total_ext + rest <= kSmemLimit;
     bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest;
     return bytes <= kSmemLimit;
 }
@@ -79,23 +79,21 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const bool shard = yo.n_peer > 0 || yo.n_flag > 0;                  // row-sharded launch: stored-gain form only
     if (shard && sg) return LLVQ_EUNSUPPORTED;
     // codes with many classes (a warp of unrelated blocks is what costs there): the kernel that orders the blocks before it unranks
-    // them; codes with a handful of classes, and rows too long for its buffers, keep the direct kernel
+    // them; the others, and rows too long for its buffers, go to the direct kernel
     OrderArgs oa;
     size_t smem_order; bool ext_order;
     if (order_smem(ctx, nq, sg ? sg->bits : 0, oa, smem_order, ext_order)) {
         const FastArgs fa = fast_args(ctx, ext_order);
-#define LLVQ_LAUNCH_ORDER(BIG, BF16, SG, SH)                                                                               \
+#define LLVQ_LAUNCH_ORDER(BF16, SG, SH)                                                                               \
     do {                                                                                                                   \
-        if (!set_smem<gemv_order_kernel<BIG, BF16, SG, SH>>(ctx->device, smem_order)) return LLVQ_ECUDA;                   \
-        if (launch_pdl(gemv_order_kernel<BIG, BF16, SG, SH>, g, (unsigned)kSortThreads, smem_order, st, fa, idx, oa, d_gain_f16, sga, sp, n_out, k_in, \
+        if (!set_smem<gemv_order_kernel<BF16, SG, SH>>(ctx->device, smem_order)) return LLVQ_ECUDA;                   \
+        if (launch_pdl(gemv_order_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_order, st, fa, idx, oa, d_gain_f16, sga, sp, n_out, k_in, \
                        bpr, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;              \
     } while (0)
         const bool bf16 = y_dtype == LLVQ_BF16;
-        if (shard && ctx->fast) { if (bf16) LLVQ_LAUNCH_ORDER(false, true, false, true); else LLVQ_LAUNCH_ORDER(false, false, false, true); }
-        else if (shard)         { if (bf16) LLVQ_LAUNCH_ORDER(true, true, false, true);  else LLVQ_LAUNCH_ORDER(true, false, false, true); }
-        else if (sg)            { if (bf16) LLVQ_LAUNCH_ORDER(false, true, true, false); else LLVQ_LAUNCH_ORDER(false, false, true, false); }
-        else if (ctx->fast)     { if (bf16) LLVQ_LAUNCH_ORDER(false, true, false, false); else LLVQ_LAUNCH_ORDER(false, false, false, false); }
-        else                    { if (bf16) LLVQ_LAUNCH_ORDER(true, true, false, false);  else LLVQ_LAUNCH_ORDER(true, false, false, false); }
+        if (shard)   { if (bf16) LLVQ_LAUNCH_ORDER(true, false, true); else LLVQ_LAUNCH_ORDER(false, false, true); }
+        else if (sg) { if (bf16) LLVQ_LAUNCH_ORDER(true, true, false); else LLVQ_LAUNCH_ORDER(false, true, false); }
+        else         { if (bf16) LLVQ_LAUNCH_ORDER(true, false, false); else LLVQ_LAUNCH_ORDER(false, false, false); }
 #undef LLVQ_LAUNCH_ORDER
         return launch_status();
     }
@@ -277,7 +275,7 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     size_t smem; bool ext;                               // the longest rows decide for the whole launch
     OrderArgs oa{};
     if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);
-    else if (!ctx->fast || !order_smem(ctx, max_nq, 0, oa, smem, ext)) return LLVQ_EUNSUPPORTED;
+    else if (!order_smem(ctx, max_nq, 0, oa, smem, ext)) return LLVQ_EUNSUPPORTED;
     if (smem > kSmemLimit) return LLVQ_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;

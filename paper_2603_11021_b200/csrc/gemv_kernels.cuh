@@ -630,11 +630,8 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
 constexpr int kOrderTeams = 4;
 constexpr int kTeamThreads = kSortThreads / kOrderTeams;
 
-// Bytes of the teams' areas in shared memory: chunk counters, then per team two histograms, the entries of a piece (and their second words).
-__host__ __device__ inline size_t gemv_order_bytes(const OrderArgs& oa, bool big)
-{
-    return 16 + (size_t)kOrderTeams * (2 * 4 * oa.words + kOrderBlocks * (big ? 12 : 8));
-}
+// Bytes of the teams' areas in shared memory: chunk counters, two histograms per team, the entries of a piece per team.
+__host__ __device__ inline size_t gemv_order_bytes(const OrderArgs& oa) { return 16 + (size_t)kOrderTeams * (2 * 4 * oa.words + kOrderBlocks * 8); }
 
 // The span of the index stream and of the gains that this CTA's row groups cover is contiguous: request it from DRAM ahead
 // of time; the ordering then reads it from L2.
@@ -653,7 +650,7 @@ __device__ __forceinline__ void prefetch_stored_span(const FastArgs& fa, const u
 }
 
 // One matrix; `piece` = pieces this team has been through.
-template <bool kBig, bool kOutBf16, bool kSg, bool kShard>
+template <bool kOutBf16, bool kSg, bool kShard>
 __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSmem& T, const OrderArgs& oa, uint32_t* xs, uint8_t* areas,
                                                 const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, const SgArgs& sg, const Split& sp,
                                                 int64_t n_out, int64_t k_in, uint32_t bpr, const uint16_t* __restrict__ x, const YOut& yo,
@@ -661,12 +658,11 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
 {
     constexpr uint32_t kTeamWarps = kTeamThreads / 32;
     float* acc = reinterpret_cast<float*>(xs + sp.per_row * 48u);   // [kSortAccFloats]
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x & (kTeamThreads - 1);
+    const uint32_t lane = threadIdx.x & 31, tid = threadIdx.x & (kTeamThreads - 1);
     const int team = (int)(threadIdx.x / kTeamThreads);
     uint32_t* next_chunk = reinterpret_cast<uint32_t*>(areas) + team;
     uint32_t* hist = reinterpret_cast<uint32_t*>(areas + 16) + (uint32_t)team * 2u * oa.words;
     unsigned long long* ent = reinterpret_cast<unsigned long long*>(areas + 16 + kOrderTeams * 2 * 4 * oa.words) + team * kOrderBlocks;
-    uint32_t* ent2 = reinterpret_cast<uint32_t*>(areas + 16 + kOrderTeams * (2 * 4 * oa.words + kOrderBlocks * 8)) + team * kOrderBlocks;
     stage_x(xs, x, k_in, sp.per_row * 48u, threadIdx.x, blockDim.x);
     for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t p_begin, uint32_t p_end, uint32_t rg0, uint32_t rg1, bool, bool) {
         const uint32_t shift = acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, kSortAccFloats);
@@ -688,58 +684,38 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
             o.b = (o.row - rg0 * kGemvGroupRows) * bpr + kq * 4u + (c & 3u);
             o.pos = (c >> 2) * 32u + r * 4u + (c & 3u);
             o.there = (c >> 2) < nchunks && kq * 4u + (c & 3u) < bpr;
-            order_piece<kBig, kSg, kTeamThreads>(fa, T, sg, oa, stream, hist + (piece & 1u) * oa.words, hist + ((piece & 1u) ^ 1u) * oa.words, ent, ent2, team, tid,
+            order_piece<kSg, kTeamThreads>(fa, T, sg, oa, stream, hist + (piece & 1u) * oa.words, hist + ((piece & 1u) ^ 1u) * oa.words, ent, team, tid,
                                                  o, (uint32_t)n_out, 2u * bpr, 2u, 8u, [&] { if (tid == 0) *next_chunk = kTeamWarps; });
             uint32_t kq_a;
             const uint32_t rg_off = split_row(sp, u0, kq_a) - rg0;
-            uint32_t ch = tid >> 5, e2 = 0;
-            uint64_t e = 0;
-            uint4 rec0 = make_uint4(0u, 0u, 0u, 0u), rec1 = rec0;
-            auto take = [&](uint32_t at) {
-                e = ent[(at * 32u + lane) & (kOrderBlocks - 1u)];
-                if (kBig) { e2 = at < nchunks ? ent2[at * 32u + lane] : 1u << 31; big_load_record(fa.dc, (int)(e2 & 0x1ffffu), !(e2 >> 31), rec0, rec1); }
-            };
-            take(ch);
+            uint32_t ch = tid >> 5;
             while (ch < nchunks) {
                 uint32_t nxt = 0;
                 if (lane == 0) nxt = atomicAdd(next_chunk, 1u);
                 nxt = __shfl_sync(kFullMask, nxt, 0);
-                OrderedBlock b{};
-                if (!kBig) b = ordered_block<kSg>(fa, sg, oa, e);
-                const bool valid = kBig ? !(e2 >> 31) : b.valid;
-                const uint32_t pos = kBig ? (e2 >> 17) & 1023u : b.pos;
+                const OrderedBlock b = ordered_block<kSg>(fa, sg, oa, ent[ch * 32u + lane]);
                 uint32_t kqb;
-                const uint32_t q = split_row(sp, kq_a + (pos >> 5), kqb);
-                const uint32_t rloc = (rg_off + q) * kGemvGroupRows + ((pos >> 2) & 7u);      // row inside the pass
-                const uint32_t cb = kqb * 4u + (pos & 3u);
+                const uint32_t q = split_row(sp, kq_a + (b.pos >> 5), kqb);
+                const uint32_t rloc = (rg_off + q) * kGemvGroupRows + ((b.pos >> 2) & 7u);    // row inside the pass
+                const uint32_t cb = kqb * 4u + (b.pos & 3u);
                 float gn = 0.f;
                 uint16_t gbits = 0;
-                if (!kSg && valid) gbits = ldg_u16_here(gain_pass + (rloc * bpr + cb));
+                if (!kSg && b.valid) gbits = ldg_u16_here(gain_pass + (rloc * bpr + cb));
                 uint32_t w[12];
-                if constexpr (kBig) {
-                    DecodedBig dec{};
-                    big_decode_record(T, rec0, rec1, valid ? e : 0ull, valid, kFullMask, dec);
-                    take(nxt);                              // the record of the next chunk's class is on its way while this one is multiplied
-                    gn = gain_to_float(gbits);
-                    expand_bf16(dec.d, gn, w);
-                    patch_id8_bf16(dec, gn, w);
-                } else {
-                    if (kSg && valid) {
-                        const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rg0 * kGemvGroupRows + rloc) : 1.f;
-                        gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + b.gain_index)), __uint_as_float(T.desc[b.cls * kFastDescStride + kFastDescRnorm]));
-                    }
-                    Decoded d;
-                    decode_known_class(T, valid ? b.cls : 0u, b.local, valid, d);
-                    if (!kSg) gn = gain_to_float(gbits);
-                    expand_bf16(d, gn, w);
+                if (kSg && b.valid) {
+                    const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rg0 * kGemvGroupRows + rloc) : 1.f;
+                    gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + b.gain_index)), __uint_as_float(T.desc[b.cls * kFastDescStride + kFastDescRnorm]));
                 }
+                Decoded d;
+                decode_known_class(T, b.valid ? b.cls : 0u, b.local, b.valid, d);
+                if (!kSg) gn = gain_to_float(gbits);
+                expand_bf16(d, gn, w);
                 const uint4* xb = reinterpret_cast<const uint4*>(xs + cb * 12u);
                 const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
                 const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
                 const float dot = dot24_bf16(w, xv);
-                if (valid) atomicAdd(&acc[rloc << shift | (lane & ((1u << shift) - 1u))], dot);
+                if (b.valid) atomicAdd(&acc[rloc << shift | (lane & ((1u << shift) - 1u))], dot);
                 ch = nxt;
-                if (!kBig) take(ch);
             }
         }
         __syncthreads();
@@ -756,7 +732,7 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
     for (uint32_t i = threadIdx.x; i < kOrderTeams * 2 * oa.words; i += blockDim.x) reinterpret_cast<uint32_t*>(areas + 16)[i] = 0u; \
     uint32_t piece = 0;
 
-template <bool kBig, bool kOutBf16, bool kSg = false, bool kShard = false>
+template <bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_order_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa, const uint16_t* __restrict__ gain, SgArgs sg,
                   Split sp, int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
@@ -765,7 +741,7 @@ gemv_order_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa
     prefetch_stored_span<kSg>(fa, stream, gain, sg, sp, n_out, bpr);       // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
     ORDER_PROLOGUE(sp.per_row);
-    gemv_order_body<kBig, kOutBf16, kSg, kShard>(fa, T, oa, xs, areas, stream, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0, piece);
+    gemv_order_body<kOutBf16, kSg, kShard>(fa, T, oa, xs, areas, stream, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0, piece);
     if (kShard) shard_arrive(yo);
 }
 
@@ -785,7 +761,7 @@ gemv_order_multi_kernel(FastArgs fa, OrderArgs oa, const __grid_constant__ GemvM
                                         mm.m[i + 1].n_out, mm.m[i + 1].bpr);
         YOut yo{};
         yo.y = M.y;
-        gemv_order_body<false, kOutBf16, false, false>(fa, T, oa, xs, areas, static_cast<const uint32_t*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
+        gemv_order_body<kOutBf16, false, false>(fa, T, oa, xs, areas, static_cast<const uint32_t*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
                                                        (uint32_t)M.bpr, M.x, yo, scratch, counters, M.slot0, piece);
     }
 }

@@ -125,8 +125,8 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     std::vector<uint8_t> image;
     ctx->fast = build_fast_image(h, ctx->fl, image, true);
     if (!ctx->fast && !build_fast_image(h, ctx->fl, image, false)) { delete ctx; return LLVQ_EUNSUPPORTED; }
-    std::vector<uint32_t> lut16;
-    build_bucket_table(h, lut16);
+    std::vector<uint32_t> lut;                           // class lookup of the codes whose class tables stay in global memory
+    if (!ctx->fast) build_bucket_table(h, lut);
     // class records in global memory: the full descriptors where the encoder's indexing kernel reads them (codes with their
     // tables in shared memory), the compact 32-byte records for the codes whose decoders read them from global memory
     std::vector<BigDesc> big;
@@ -161,7 +161,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     size_t o_offlo = up(o_offhi + (ncls + 1) * 4);
     size_t o_cls = up(o_offlo + (ncls + 1) * 8);
     size_t o_lut = up(o_cls + cls_bytes);
-    size_t o_err = up(o_lut + lut16.size() * 4);
+    size_t o_err = up(o_lut + lut.size() * 4);
     size_t o_img = up(o_err + 256);
     size_t o_gol = up(o_img + image.size());
     size_t o_p12 = up(o_gol + 4096 * 4);
@@ -194,7 +194,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     std::memcpy(blob.data() + o_offlo, off_lo.data(), (ncls + 1) * 8);
     if (full_descs) std::memcpy(blob.data() + o_cls, h.desc.data(), ncls * sizeof(ClassDesc));
     if (!big.empty()) std::memcpy(blob.data() + o_cls + big_at, big.data(), big.size() * sizeof(BigDesc));
-    std::memcpy(blob.data() + o_lut, lut16.data(), lut16.size() * 4);
+    if (!lut.empty()) std::memcpy(blob.data() + o_lut, lut.data(), lut.size() * 4);
     std::memcpy(blob.data() + o_img, image.data(), image.size());
     std::memcpy(blob.data() + o_gol, h.golay.data(), 4096 * 4);
     std::memcpy(blob.data() + o_p12, pos12.data(), 4096 * 2);
@@ -216,7 +216,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     ctx->dev.off_lo = reinterpret_cast<const uint64_t*>(d + o_offlo);
     ctx->dev.cls = full_descs ? reinterpret_cast<const ClassDesc*>(d + o_cls) : nullptr;
     ctx->dev.big = big.empty() ? nullptr : reinterpret_cast<const BigDesc*>(d + o_cls + big_at);
-    ctx->dev.lut16 = reinterpret_cast<const uint32_t*>(d + o_lut);
+    ctx->dev.lut = reinterpret_cast<const uint32_t*>(d + o_lut);
     ctx->d_err = reinterpret_cast<unsigned long long*>(d + o_err);
     ctx->dev.bad_index = ctx->d_err;
     ctx->dev.flags = reinterpret_cast<uint32_t*>(d + o_err + 8);

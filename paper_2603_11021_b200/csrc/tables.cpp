@@ -297,7 +297,7 @@ bool build_fast_image(const HostTables& t, FastLayout& L, std::vector<uint8_t>& 
         uint32_t* r32 = reinterpret_cast<uint32_t*>(img.data() + L.recip32);
         for (int i = 0; i < 625; ++i) {
             const uint32_t c = t.pascal[i];
-            r64[i] = c ? ~0ull / c : 0ull;
+            r64[i] = c ? reciprocal_down(c) : 0ull;
             r32[i] = c > 1 ? (uint32_t)((1ull << 32) / c) : 0xffffffffu;
         }
         return true;
@@ -388,15 +388,15 @@ void build_big_descs(const HostTables& t, std::vector<BigDesc>& out)
     }
 }
 
-// Class of the first index of every bucket (I >> (W - 16)), plus a final entry = last class: the class of an
+// Class of the first index of every bucket (I >> (W - kBigBucketBits)), plus a final entry = last class: the class of an
 // index lies between the entries of its bucket and of the next one.
 void build_bucket_table(const HostTables& t, std::vector<uint32_t>& lut)
 {
     const size_t ncls = t.desc.size();
-    const int shift = t.W > 16 ? t.W - 16 : 0;
-    lut.assign(65537, (uint32_t)(ncls - 1));
+    const int shift = std::max(t.W - kBigBucketBits, 0);
+    lut.assign(((size_t)1 << kBigBucketBits) + 1, (uint32_t)(ncls - 1));
     size_t c = 0;
-    for (uint32_t b = 0; b < 65536; ++b) {
+    for (uint32_t b = 0; b < 1u << kBigBucketBits; ++b) {
         u128 first = (u128)b << shift;
         if (first >= t.N) break;
         while (c + 1 < ncls && t.offset[c + 1] <= first) ++c;

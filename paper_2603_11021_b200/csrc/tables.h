@@ -95,6 +95,8 @@ bool build_tables(int m_lo, int m_hi, HostTables& out);
 // ---------------------------------------------------------------------------
 namespace llvq {
 
+constexpr int kBigBucketBits = 20;     // buckets of the class lookup of codes with class tables in global memory (4 MB, in L2): the bisection between a bucket's first
+                                       // and last class takes 1.4 steps per warp of the 72-bit code (2^16 buckets: 4.4); some buckets hold thousands of classes
 constexpr int kFastMaxLevels = 4;      // unranking steps per class on the fast path
 constexpr int kFastDescWords = 20;     // words of a class descriptor that carry data
 constexpr int kFastDescValsOdd = 18;   // words 18, 19: absolute value of id 0..7 in the numbering of the odd-only decoder form
@@ -137,7 +139,7 @@ struct FastLayout {
     uint32_t off;         // u64[ncls + 1]
     uint32_t desc;        // u32[ncls][kFastDescStride]
     uint32_t total;       // bytes of the image proper, multiple of 16
-    uint32_t recip64;     // u64[25*25] floor((2^64 - 1) / C(n, k)) and
+    uint32_t recip64;     // binary64[25*25] 1 / C(n, k) rounded down and
     uint32_t recip32;     // u32[25*25] floor(2^32 / C(n, k)) (0xffffffff for C = 1): images without class tables only, else 0
     uint32_t sub3;        // u32[kSmallSubsetWords], behind the image proper: kernels with room for it load total_ext bytes
     uint32_t sub2;        // u32[kSub2Words], behind sub3: directory and subsets for k = 0..2 in the layout of coords_of
@@ -167,7 +169,7 @@ struct FastLayout {
 // tables do not fit shared memory keep those in global memory.
 bool build_fast_image(const HostTables& t, FastLayout& layout, std::vector<uint8_t>& image, bool with_classes = true);
 void build_big_descs(const HostTables& t, std::vector<BigDesc>& out);
-void build_bucket_table(const HostTables& t, std::vector<uint32_t>& lut);   // u32[65537], see tables.cpp
+void build_bucket_table(const HostTables& t, std::vector<uint32_t>& lut);   // see tables.cpp
 
 // Encoder side (point -> class).  Signature of a class: sum over its 24 absolute values of a fixed pseudo-random
 // 64-bit number per value (the multiset fixes shell and parity).  build_class_hash() fills an open-addressing
