@@ -12,6 +12,26 @@ namespace {
 
 constexpr size_t kSmemLimit = 227 * 1024;
 
+// Shared memory of gemv_bin_kernel for `su` units per segment, and whether the table of small subsets still fits.
+void bin_smem(const llvq_ctx* ctx, int64_t nq, int su, size_t& bytes, bool& ext)
+{
+    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + 16 + 2 * 1024 * 4 + (size_t)su * 32 * (8 + 2);
+    ext = ctx->fl.total_ext + rest <= kSmemLimit;
+    bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest;
+}
+
+bool bin_kernel_serves(const llvq_ctx* ctx, int64_t nq, const SgArgs* sg)
+{
+    size_t bytes; bool ext;
+    bin_smem(ctx, nq, kBinSegUnits, bytes, ext);
+    return (!sg || sg->bits <= 5) && ctx->fast && ctx->d_sort_rank && ctx->host.desc.size() >= 64 && ctx->host.W <= 48 && bytes <= kSmemLimit &&
+           nq < (1ll << 24);
+}
+
+// Stored streams of codes with many classes: gemv_bin_kernel while a CTA's range is one of its segments (it orders the whole range at
+// once, so the warps share classes best), else gemv_order_kernel, whose teams order small pieces and unrank others meanwhile.
+bool one_segment(int64_t units_per_cta) { return units_per_cta <= kBinSegUnits; }
+
 // Whether gemv_order_kernel takes a matrix of nq units per row group; its shared memory, and whether the table of small subsets
 // still fits.
 bool order_smem(const llvq_ctx* ctx, int64_t nq, int gain_bits, OrderArgs& oa, size_t& bytes, bool& ext)
@@ -78,11 +98,29 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const SgArgs sga = sg ? *sg : SgArgs{};
     const bool shard = yo.n_peer > 0 || yo.n_flag > 0;                  // row-sharded launch: stored-gain form only
     if (shard && sg) return LLVQ_EUNSUPPORTED;
-    // codes with many classes (a warp of unrelated blocks is what costs there): the kernel that orders the blocks before it unranks
-    // them; the others, and rows too long for its buffers, go to the direct kernel
+    // codes with many classes (a warp of unrelated blocks is what costs there): the kernels that order the blocks before they unrank
+    // them; the others, and rows too long for their buffers, go to the direct kernel
+    int seg_units = kBinSegUnits;
+    size_t smem_bin; bool ext_bin;
+    bin_smem(ctx, nq, seg_units, smem_bin, ext_bin);
     OrderArgs oa;
     size_t smem_order; bool ext_order;
-    if (order_smem(ctx, nq, sg ? sg->bits : 0, oa, smem_order, ext_order)) {
+    const bool order = order_smem(ctx, nq, sg ? sg->bits : 0, oa, smem_order, ext_order);
+    if (bin_kernel_serves(ctx, nq, sg) && (one_segment(upc) || !order)) {
+        const FastArgs fa = fast_args(ctx, ext_bin);
+#define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
+    do {                                                                                                                   \
+        if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                          \
+        if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
+                       bpr, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
+    } while (0)
+        if (shard)   { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, true); else LLVQ_LAUNCH_BIN(false, false, true); }
+        else if (sg) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, true, false); else LLVQ_LAUNCH_BIN(false, true, false); }
+        else         { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, false); else LLVQ_LAUNCH_BIN(false, false, false); }
+#undef LLVQ_LAUNCH_BIN
+        return launch_status();
+    }
+    if (order) {
         const FastArgs fa = fast_args(ctx, ext_order);
 #define LLVQ_LAUNCH_ORDER(BF16, SG, SH)                                                                               \
     do {                                                                                                                   \
@@ -254,6 +292,7 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     mm.n = n_mats;
     uint32_t acc_floats = kSortAccFloats;
     int64_t slot = 0, max_nq = 0;
+    bool bin = true;                                     // stored streams: which of the two kernels (see one_segment)
     for (int i = 0; i < n_mats; ++i) {
         const llvq_gemv_desc& d = descs[i];
         if (int e = check_common(ctx, d.d_weights)) return e;
@@ -264,6 +303,7 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         // every matrix must give every CTA work: the sorted layout was made for that many CTAs
         if (units < ctx->sm_count) return LLVQ_EUNSUPPORTED;
         if (sorted && !sortable(ctx, d.k_in)) return LLVQ_EUNSUPPORTED;
+        bin = bin && one_segment((units + ctx->sm_count - 1) / ctx->sm_count);
         max_nq = std::max(max_nq, nq);
         GemvMat& m = mm.m[i];
         m.weights = d.d_weights; m.gain = d.d_gain_f16; m.x = d.d_x_bf16; m.y = d.d_y;
@@ -275,7 +315,12 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     size_t smem; bool ext;                               // the longest rows decide for the whole launch
     OrderArgs oa{};
     if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);
-    else if (!order_smem(ctx, max_nq, 0, oa, smem, ext)) return LLVQ_EUNSUPPORTED;
+    else {
+        const bool order = order_smem(ctx, max_nq, 0, oa, smem, ext);
+        bin = bin_kernel_serves(ctx, max_nq, nullptr) && (bin || !order);
+        if (!bin && !order) return LLVQ_EUNSUPPORTED;
+        if (bin) bin_smem(ctx, max_nq, kBinSegUnits, smem, ext);
+    }
     if (smem > kSmemLimit) return LLVQ_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
@@ -321,13 +366,15 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
             if (launch_pdl(gemv_sorted_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         }
     } else {
-        if (y_dtype == LLVQ_BF16) {
-            if (!set_smem<gemv_order_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_order_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, oa, mm, (uint32_t)max_nq, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
-        } else {
-            if (!set_smem<gemv_order_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_order_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, oa, mm, (uint32_t)max_nq, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
-        }
+#define LLVQ_LAUNCH_MULTI(K, ...)                                                                                                  \
+    do {                                                                                                                           \
+        if (!set_smem<K>(ctx->device, smem)) return LLVQ_ECUDA;                                                                     \
+        if (launch_pdl(K, g, (unsigned)kSortThreads, smem, st, fa, __VA_ARGS__, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
+    } while (0)
+        const bool bf16 = y_dtype == LLVQ_BF16;
+        if (bin) { if (bf16) LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<true>, ctx->d_sort_rank, mm); else LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<false>, ctx->d_sort_rank, mm); }
+        else     { if (bf16) LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel<true>, oa, mm, (uint32_t)max_nq); else LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel<false>, oa, mm, (uint32_t)max_nq); }
+#undef LLVQ_LAUNCH_MULTI
     }
     return launch_status();
 }

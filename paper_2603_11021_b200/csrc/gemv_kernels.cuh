@@ -624,8 +624,10 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
 // Fused GEMV on the stored stream with the blocks ordered inside the kernel (order.cuh): the work split of gemv_fast_kernel.  A
 // CTA's range of a pass is cut into an equal contiguous share per team of 8 warps, a share into pieces of 32 units (1024 blocks); a
 // team orders a piece, its warps take 32 consecutive entries at a time, run the one unranker form they need, and each lane
-// forms its own dot product, as in gemv_sorted_kernel.  The first pieces are of 8, 16, 24 and 32 units, so that the teams do
-// not order at the same time.
+// forms its own dot product, as in gemv_sorted_kernel.  A share's pieces are of equal size (the teams drift apart by
+// themselves: first pieces of 8, 16, 24 and 32 units made shares of two pieces slower and long ones no faster).  28672 x 8192:
+// 278 -> 235 us, 8192 x 8192: 82 -> 71 us against gemv_bin_kernel, which orders up to 8192 blocks at a time as a phase of the
+// whole block and is the faster one while that is the CTA's whole range (4096 x 4096: 23.5 against 26 us).
 // ===========================================================================
 constexpr int kOrderTeams = 4;
 constexpr int kTeamThreads = kSortThreads / kOrderTeams;
@@ -671,11 +673,12 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
         const uint32_t units = p_end - p_begin;
         const uint32_t t_begin = p_begin + (uint32_t)team * units / kOrderTeams, t_end = p_begin + ((uint32_t)team + 1u) * units / kOrderTeams;
         const uint16_t* gain_pass = gain + (int64_t)rg0 * kGemvGroupRows * bpr;
-        uint32_t size = 32u * ((uint32_t)team + 1u) / kOrderTeams;
-        for (uint32_t u0 = t_begin; u0 < t_end; u0 += size, size = 32u, ++piece) {
+        const uint32_t npieces = (t_end - t_begin + 31u) / 32u, size = npieces ? (t_end - t_begin + npieces - 1u) / npieces : 1u;
+        for (uint32_t u0 = t_begin; u0 < t_end; u0 += size, ++piece) {
             const uint32_t nchunks = min(size, t_end - u0);
-            // a thread has one column block of the piece (of 128) and every second row of it: a warp reads 32 neighbouring fields
-            const uint32_t c = tid & 127u, r = tid >> 7;
+            // a thread has one column block of the piece (of up to 128, 64 or 32) and every second, fourth or single row of it: a warp
+            // reads 32 neighbouring fields, and a small piece is spread over all threads
+            const uint32_t narrow = nchunks <= 8u ? 2u : nchunks <= 16u ? 1u : 0u, c = tid & (127u >> narrow), r = tid >> (7u - narrow);
             uint32_t kq;
             const uint32_t rg = split_row(sp, u0 + (c >> 2), kq);
             OrderSpot o;
@@ -685,7 +688,7 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
             o.pos = (c >> 2) * 32u + r * 4u + (c & 3u);
             o.there = (c >> 2) < nchunks && kq * 4u + (c & 3u) < bpr;
             order_piece<kSg, kTeamThreads>(fa, T, sg, oa, stream, hist + (piece & 1u) * oa.words, hist + ((piece & 1u) ^ 1u) * oa.words, ent, team, tid,
-                                                 o, (uint32_t)n_out, 2u * bpr, 2u, 8u, [&] { if (tid == 0) *next_chunk = kTeamWarps; });
+                                                 o, min((uint32_t)n_out, (rg + 1u) * kGemvGroupRows), bpr << (1u + narrow), 2u << narrow, 8u << narrow, [&] { if (tid == 0) *next_chunk = kTeamWarps; });
             uint32_t kq_a;
             const uint32_t rg_off = split_row(sp, u0, kq_a) - rg0;
             uint32_t ch = tid >> 5;
@@ -763,5 +766,178 @@ gemv_order_multi_kernel(FastArgs fa, OrderArgs oa, const __grid_constant__ GemvM
         yo.y = M.y;
         gemv_order_body<kOutBf16, false, false>(fa, T, oa, xs, areas, static_cast<const uint32_t*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
                                                        (uint32_t)M.bpr, M.x, yo, scratch, counters, M.slot0, piece);
+    }
+}
+
+// ===========================================================================
+// Fused GEMV on the stored stream with the blocks binned inside the kernel: the work split of gemv_fast_kernel, but a
+// CTA first looks up the class of every block of a segment of up to kBinSegUnits units (S1-S2), orders the
+// (class-local index, class, position) triples by the sorted layout's key with a counting sort in shared memory,
+// and then proceeds like gemv_sorted_kernel on those entries (S3-S8): a warp takes 32 consecutive entries, runs
+// the one unranker form they need and each lane forms its own dot product.
+// ===========================================================================
+constexpr int kBinSegUnits = 256;                    // at most 8192 blocks per segment (halved while shared memory is short)
+constexpr int kBinPerThread = kBinSegUnits * 32 / kSortThreads;   // 8
+
+template <bool kOutBf16, bool kSg, bool kShard>
+__device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem& T, uint8_t* staging, const uint32_t* __restrict__ stream,
+                                              const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, const SgArgs& sg,
+                                              const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, int seg_units,
+                                              const uint16_t* __restrict__ x, const YOut& yo, float* __restrict__ scratch,
+                                              uint32_t* __restrict__ counters, int64_t slot0)
+{
+    const uint32_t nq = sp.per_row;
+    uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
+    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccFloats]
+    uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccFloats);
+    uint32_t* next_chunk = last_flag + 1;
+    uint32_t* hist = last_flag + 4;                                  // [1024] bins in sort order; later their first slots
+    uint32_t* cursor = hist + 1024;                                  // [1024]
+    unsigned long long* ent = reinterpret_cast<unsigned long long*>(cursor + 1024);   // [seg_units * 32] class-local index | position << 48
+    uint16_t* ent_cls = reinterpret_cast<uint16_t*>(ent + seg_units * 32);            // [seg_units * 32] class (| gain index << 10), 0xffff = no block
+    stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t kWarps = blockDim.x >> 5;
+    for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t rg0, uint32_t rg1, bool first, bool last) {
+        const uint32_t shift = acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, kSortAccFloats);
+        if (first)
+            for (uint32_t i = threadIdx.x; i < (rg1 - rg0 + 1u) * kGemvGroupRows << shift; i += blockDim.x) acc[i] = 0.f;
+        hist[threadIdx.x] = 0; cursor[threadIdx.x] = 0;
+        if (threadIdx.x == 0) *next_chunk = kWarps;
+        __syncthreads();
+        uint32_t kq_a;
+        const uint32_t rg_a = split_row(sp, tu0, kq_a), rg_off = rg_a - rg0;
+        const int entries = (int)(tu1 - tu0) * 32;
+        // ---- S1-S2 for the whole segment and the histogram of the sort keys
+        unsigned long long mine_ent[kBinPerThread];
+        uint32_t mine_key[kBinPerThread];
+#pragma unroll
+        for (int q = 0; q < kBinPerThread; ++q) {
+            const int i = (int)threadIdx.x + q * kSortThreads;
+            mine_key[q] = 0xffffffffu; mine_ent[q] = 0ull;
+            if (i < entries) {
+                const uint32_t pos = (uint32_t)i;
+                uint32_t kq;
+                const uint32_t qd = split_row(sp, kq_a + (pos >> 5), kq);
+                const int64_t row = (int64_t)(rg_a + qd) * kGemvGroupRows + ((pos >> 2) & 7u), cb = (int64_t)kq * 4 + (pos & 3u);
+                uint32_t key = 1023u, cls = 0xffffu;
+                uint64_t local = 0;
+                if (row < n_out && cb < bpr) {
+                    const uint64_t f = load_field(stream, (uint64_t)(row * bpr + cb), (int)fa.L.W + (kSg ? sg.bits : 0));
+                    const uint64_t I = kSg ? f & ((1ull << fa.L.W) - 1ull) : f;
+                    if (I < fa.n_points) {
+                        cls = fast_find_class(T, I, local);
+                        key = __ldg(sort_rank + cls);
+                        if (kSg) cls |= (uint32_t)(f >> fa.L.W) << 10;           // the gain index rides with the class
+                    } else atomicAdd(fa.bad_index, 1ull);
+                }
+                mine_key[q] = key | cls << 16;
+                mine_ent[q] = local | (unsigned long long)pos << 48;
+                atomicAdd(&hist[key], 1u);
+            }
+        }
+        __syncthreads();
+        // exclusive prefix sum of the 1024 bins: one bin per thread
+        {
+            const uint32_t c = hist[threadIdx.x];
+            uint32_t incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(kFullMask, incl, o); if (lane >= o) incl += t; }
+            if (lane == 31) cursor[warp] = incl;                       // warp totals, parked in the cursor array for a moment
+            __syncthreads();
+            uint32_t before = 0;
+            for (int w2 = 0; w2 < warp; ++w2) before += cursor[w2];
+            __syncthreads();
+            hist[threadIdx.x] = before + incl - c;
+            cursor[threadIdx.x] = 0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kBinPerThread; ++q) {
+            if (mine_key[q] != 0xffffffffu) {
+                const uint32_t key = mine_key[q] & 0xffffu;
+                const uint32_t slot = hist[key] + atomicAdd(&cursor[key], 1u);
+                ent[slot] = mine_ent[q];
+                ent_cls[slot] = (uint16_t)(mine_key[q] >> 16);
+            }
+        }
+        __syncthreads();
+        // ---- S3-S8 on the ordered entries
+        const uint32_t nchunks = tu1 - tu0;
+        const uint16_t* gain_pass = gain + (int64_t)rg0 * kGemvGroupRows * bpr;
+        for (uint32_t ch = (uint32_t)warp; ch < nchunks;) {
+            uint32_t nxt = 0;
+            if (lane == 0) nxt = atomicAdd(next_chunk, 1u);
+            nxt = __shfl_sync(kFullMask, nxt, 0);
+            const unsigned long long e = ent[ch * 32 + lane];
+            const uint32_t cls16 = ent_cls[ch * 32 + lane];
+            const bool valid = cls16 != 0xffffu;
+            const uint32_t pos = (uint32_t)(e >> 48);
+            uint32_t kq;
+            const uint32_t q = split_row(sp, kq_a + (pos >> 5), kq);
+            const uint32_t rloc = (rg_off + q) * kGemvGroupRows + ((pos >> 2) & 7u);
+            const uint32_t cb = kq * 4u + (pos & 3u);
+            const uint32_t cls = valid ? (kSg ? cls16 & 1023u : cls16) : 0u;
+            float gn = 0.f;
+            uint16_t gbits = 0;
+            if (valid) {
+                if (kSg) {
+                    const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rg0 * kGemvGroupRows + rloc) : 1.f;
+                    gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + (cls16 >> 10))), __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
+                } else {
+                    gbits = ldg_u16_here(gain_pass + (rloc * bpr + cb));
+                }
+            }
+            Decoded r;
+            decode_known_class(T, cls, e & ((1ull << 48) - 1ull), valid, r);
+            if (!kSg) gn = gain_to_float(gbits);
+            uint32_t w[12];
+            expand_bf16(r, gn, w);
+            const uint4* xb = reinterpret_cast<const uint4*>(xs + cb * 12u);
+            const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
+            const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
+            const float dot = dot24_bf16(w, xv);
+            if (valid) atomicAdd(&acc[rloc << shift | ((uint32_t)lane & ((1u << shift) - 1u))], dot);
+            ch = nxt;
+        }
+        __syncthreads();
+        if (!last) return;
+        auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
+        const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
+        __syncthreads();
+    }, (uint32_t)seg_units);
+}
+
+template <bool kOutBf16, bool kSg = false, bool kShard = false>
+__global__ void __launch_bounds__(kSortThreads, 1)
+gemv_bin_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, SgArgs sg,
+                Split sp, int64_t n_out, int64_t k_in, int64_t bpr, int seg_units, const uint16_t* __restrict__ x, YOut yo,
+                float* __restrict__ scratch, uint32_t* __restrict__ counters)
+{
+    prefetch_stored_span<kSg>(fa, stream, gain, sg, sp, n_out, bpr);       // while the table image is on its way
+    FAST_PROLOGUE(if (kShard) shard_arrive(yo));
+    gemv_bin_body<kOutBf16, kSg, kShard>(fa, T, staging, stream, sort_rank, gain, sg, sp, n_out, k_in, (uint32_t)bpr, seg_units, x, yo, scratch, counters, 0);
+    if (kShard) shard_arrive(yo);
+}
+
+// Several independent matrices on their stored streams in one launch.
+template <bool kOutBf16>
+__global__ void __launch_bounds__(kSortThreads, 1)
+gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const __grid_constant__ GemvMulti mm, float* __restrict__ scratch,
+                      uint32_t* __restrict__ counters)
+{
+    prefetch_stored_span<false>(fa, static_cast<const uint32_t*>(mm.m[0].weights), mm.m[0].gain, SgArgs{}, mm.m[0].sp, mm.m[0].n_out, mm.m[0].bpr);
+    FAST_PROLOGUE();
+    for (int i = 0; i < mm.n; ++i) {
+        const GemvMat& M = mm.m[i];
+        if (i + 1 < mm.n)
+            prefetch_stored_span<false>(fa, static_cast<const uint32_t*>(mm.m[i + 1].weights), mm.m[i + 1].gain, SgArgs{}, mm.m[i + 1].sp,
+                                     mm.m[i + 1].n_out, mm.m[i + 1].bpr);
+        YOut yo{};
+        yo.y = M.y;
+        gemv_bin_body<kOutBf16, false, false>(fa, T, staging, static_cast<const uint32_t*>(M.weights), sort_rank, M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
+                                              (uint32_t)M.bpr, kBinSegUnits, M.x, yo, scratch, counters, M.slot0);
+        __syncthreads();
     }
 }
