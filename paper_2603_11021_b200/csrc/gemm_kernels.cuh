@@ -916,3 +916,184 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
+
+// The product on the stored stream of the 48-bit codes: two teams of 16 warps take the domains of a row tile in turn.  A team orders
+// its domain's 1024 blocks (order.cuh; the entries lie in its own A buffer, which its previous MMAs have left by then), every
+// warp takes two chunks of them into registers, unranks them, writes its part of A, and the team's first thread issues the MMAs
+// into the team's own accumulator.  The teams meet only at the end of a row tile: while one orders, which leaves most issue slots
+// empty, the other unranks.  x_double: an X buffer per team, asked for ahead; else one that the teams use in turn (wide batches).
+constexpr int kGemmTeams = 2;
+constexpr int kGemmTeamThreads = kGemmThreads / kGemmTeams;
+
+template <bool kSg = false, bool kShard = false>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga, int x_double,
+                 const __grid_constant__ CUtensorMap xmap)
+{
+    extern __shared__ __align__(1024) uint8_t smem_1k[];
+    uint8_t* const smem = smem_1k;
+    const uint32_t img_bytes = fa.image_bytes;
+    uint64_t* bar_img = reinterpret_cast<uint64_t*>(smem + img_bytes);
+    uint64_t* bar_free = bar_img + 1;                                     // [2] the MMAs of the team's last domain are done (its A buffer and X are free)
+    uint64_t* bar_x = bar_img + 3;                                        // [2] the X slice of the team's domain has arrived
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_img + 5);
+    uint32_t* last_flag = tmem_slot + 1;
+    const uint32_t a_off = (img_bytes + 64 + 1023) & ~1023u;
+    constexpr uint32_t kASet = kDomStages * kGemmRows * kStageK * 2;       // 49152
+    uint8_t* a_buf = smem + a_off;                                        // [2 teams] x 49152
+    const uint32_t x_set = (uint32_t)ga.npad * kDomStages * kStageK * 2;
+    uint8_t* b_buf = a_buf + kGemmTeams * kASet;                          // [2 teams, or 1]
+    uint32_t* hists = reinterpret_cast<uint32_t*>(b_buf + (x_double ? 2u : 1u) * x_set);      // [2 teams][2][words]
+
+    pdl_launch_dependents();
+    const bool image_ok = fast_load_image(smem, fa.image, fa.image_bytes, bar_img, fa.flags);
+    pdl_wait();                                        // also when the image did not arrive: the dependents of this launch rely on it
+    if (!image_ok) {
+        if (kShard) shard_arrive(*ga.shard);           // the peers must not wait for this rank
+        return;
+    }
+    const FastSmem T = fast_view(smem, fa.L);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, team = (int)threadIdx.x / kGemmTeamThreads;
+    const uint32_t tid = threadIdx.x % kGemmTeamThreads, twarp = tid >> 5;
+    for (uint32_t i = threadIdx.x; i < kGemmTeams * 2 * oa.words; i += kGemmThreads) hists[i] = 0u;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) { mbar_init(bar_free + i, 1); mbar_init(bar_x + i, 1); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t idesc = instr_desc_bf16_m128((uint32_t)ga.npad);
+    uint8_t* const a_mine = a_buf + (uint32_t)team * kASet;
+    uint8_t* const x_mine = b_buf + (x_double ? (uint32_t)team * x_set : 0u);
+    unsigned long long* const ent = reinterpret_cast<unsigned long long*>(a_mine);
+    const uint32_t nd = ga.sp.per_row, bpr = (uint32_t)ga.bpr;
+    const uint32_t dom_begin = split_begin(ga.sp, blockIdx.x), dom_end = split_begin(ga.sp, blockIdx.x + 1u);
+    uint32_t mine = 0, base[2] = {0, 0};               // domains this team has done; domains either team had done before this row tile
+    bool timeout = false;
+
+    for (uint32_t rt = split_row(ga.sp, dom_begin); rt * nd < dom_end; ++rt) {
+        const uint32_t tile0 = rt * nd, tile1 = tile0 + nd;
+        const uint32_t d_begin = max(dom_begin, tile0) - tile0, d_end = min(dom_end, tile1) - tile0;
+        // CTAs that share this row tile
+        const uint32_t parts = dom_begin <= tile0 && tile1 <= dom_end ? 1u : split_owner(ga.sp, tile1 - 1u) - split_owner(ga.sp, tile0) + 1u;
+        const uint16_t* gain_tile = gain + (int64_t)rt * kGemmRows * ga.bpr;
+        bool fresh = true;
+        for (uint32_t d = d_begin + (uint32_t)team; d < d_end; d += kGemmTeams, ++mine) {
+            // ---- order
+            OrderSpot o;
+            o.row = rt * kGemmRows + (tid >> 3);
+            o.b0 = (uint64_t)rt * kGemmRows * ga.bpr;
+            o.b = (tid >> 3) * bpr + d * kDomBlocks + (tid & 7u);
+            o.pos = tid;
+            o.there = d * kDomBlocks + (tid & 7u) < bpr;
+            order_piece<kSg, kGemmTeamThreads>(fa, T, sg, oa, stream, hists + ((uint32_t)team * 2u + (mine & 1u)) * oa.words,
+                                               hists + ((uint32_t)team * 2u + ((mine & 1u) ^ 1u)) * oa.words, ent, team, tid, o, (uint32_t)ga.n_out,
+                                               64u * bpr, 64u, (uint32_t)kGemmTeamThreads, [&] {
+                // the entries go over what the previous MMAs read
+                if (mine > 0 && !mbar_wait(bar_free + team, (mine - 1u) & 1u)) timeout = true;
+                if (x_double && tid == 0) request_x(smem_u32(x_mine), &xmap, (int)d, ga.npad, bar_x + team);
+            });
+            // ---- A: two chunks per warp, one from the expensive and one from the cheap end
+            const unsigned long long e[2] = {ent[twarp * 32u + lane], ent[(31u - twarp) * 32u + lane]};
+            team_barrier(team, kGemmTeamThreads);                         // all entries are in registers: A may overwrite them
+#pragma unroll 1
+            for (int q = 0; q < 2; ++q) {
+                const OrderedBlock b = ordered_block<kSg>(fa, sg, oa, q == 0 ? e[0] : e[1]);
+                const uint32_t r = b.pos >> 3, c = b.pos & 7u;
+                uint16_t gbits = 0;
+                if (!kSg && b.valid) gbits = ldg_u16_here(gain_tile + (r * bpr + d * kDomBlocks + c));
+                float gn = 0.f;                                           // the gain is converted once the block is unranked
+                Decoded dec;
+                decode_known_class(T, b.valid ? b.cls : 0u, b.local, b.valid, dec);
+                if (!kSg) gn = gain_to_float(gbits);
+                if (kSg && b.valid) {
+                    const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rt * kGemmRows + r) : 1.f;
+                    gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + b.gain_index)), __uint_as_float(T.desc[b.cls * kFastDescStride + kFastDescRnorm]));
+                }
+                uint32_t w[12];
+                expand_bf16(dec, gn, w);
+                uint8_t* a_dst = a_mine + (c >> 2) * (kASet / 2) + (r >> 3) * 128u + (r & 7u) * 16u + 3u * (c & 3u) * 2048u;
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    *reinterpret_cast<uint4*>(a_dst + j * 2048) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+            }
+            fence_async_smem();
+            team_barrier(team, kGemmTeamThreads);
+            // ---- MMAs
+            if (tid == 0) {
+                if (!x_double) {
+                    // the domain before this one in the tile is the other team's: its MMAs have to be through with X
+                    const uint32_t i = d - d_begin, before = team == 0 ? base[1] + (i >> 1) - 1u : base[0] + (i >> 1);
+                    if (i > 0u && !mbar_wait(bar_free + (team ^ 1), before & 1u)) timeout = true;
+                    request_x(smem_u32(x_mine), &xmap, (int)d, ga.npad, bar_x + team);
+                }
+                if (!mbar_wait(bar_x + team, mine & 1u)) timeout = true;
+                tc_fence_after();
+                domain_mmas(tmem + 64u * (uint32_t)team, smem_u32(a_mine), smem_u32(x_mine), ga.npad, idesc, fresh);
+                umma_commit(bar_free + team);
+            }
+            fresh = false;
+        }
+        const uint32_t n0 = (d_end - d_begin + 1u) / 2u, n1 = (d_end - d_begin) / 2u;
+        // ---- epilogue: accumulators -> scratch (split-K) or Y
+        __syncthreads();                                                  // both teams' MMAs of this tile are issued
+        if (warp < 4 && n0 > 0) {
+            if (!mbar_wait(bar_free, (base[0] + n0 - 1u) & 1u)) timeout = true;
+            if (n1 > 0 && !mbar_wait(bar_free + 1, (base[1] + n1 - 1u) & 1u)) timeout = true;
+            tc_fence_after();
+            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
+            for (int c0 = 0; c0 < ga.npad; c0 += 16) {
+                float v[16];
+                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
+                if (n1 > 0) {
+                    float v1[16];
+                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + 64u + (uint32_t)c0, v1);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] += v1[i];
+                }
+                if (orow < ga.n_out) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const int n = c0 + i;
+                        if (n < ga.batch) {
+                            if (parts == 1u) gemm_store<kShard>(ga, n, orow, v[i]);
+                            else atomicAdd(ga.scratch + (int64_t)n * ga.scratch_ld + orow, v[i]);
+                        }
+                    }
+                }
+            }
+            tc_fence_before();
+        }
+        base[0] += n0; base[1] += n1;
+        if (parts > 1u) {
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) *last_flag = (atomicAdd(ga.counters + rt, 1u) == parts - 1u);
+            __syncthreads();
+            if (*last_flag) {
+                __threadfence();
+                for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
+                    const int n = i / kGemmRows;
+                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
+                    if (orow < ga.n_out) {
+                        float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
+                        gemm_store<kShard>(ga, n, orow, __ldcg(sp));
+                        __stcg(sp, 0.f);
+                    }
+                }
+                if (threadIdx.x == 0) ga.counters[rt] = 0u;
+            }
+        }
+        __syncthreads();
+    }
+    if (timeout) atomicOr(fa.flags, 1u);
+    if (kShard) {
+        __threadfence_system();                           // this thread's stores to the peers' copies, before the CTA counts itself in
+        shard_arrive(*ga.shard);
+    }
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+}
