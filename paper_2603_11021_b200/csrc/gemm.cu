@@ -143,7 +143,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     if (!make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
     OrderArgs oa;
     if (order_args(ctx, sg ? sg->bits : 0, &oa)) {
-        const size_t head = (img + 64 + 1023) & ~size_t(1023), a_sets = (size_t)kGemmTeams * kDomStages * kGemmRows * kStageK * 2,
+        const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_sets = (size_t)kGemmTeams * kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2, hists = (size_t)kGemmTeams * 2 * oa.words * 4;
         const int x_double = head + a_sets + 2 * x_set + hists <= 227 * 1024;
         const size_t smem_team = head + a_sets + (x_double ? 2 : 1) * x_set + hists;
@@ -154,15 +154,16 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const unsigned grid_team = (unsigned)std::min<int64_t>(row_tiles * gt.nstages, ctx->sm_count);
             gt.sp = make_split(row_tiles * gt.nstages, gt.nstages, grid_team);
             const SgArgs sga = sg ? *sg : SgArgs{};
-#define LLVQ_LAUNCH_TEAM(SG, SH)                                                                                              \
+#define LLVQ_LAUNCH_TEAM(BIG, SG, SH)                                                                                              \
     do {                                                                                                                     \
-        if (!set_smem<gemm_team_kernel<SG, SH>>(ctx->device, smem_team)) return LLVQ_ECUDA;                                   \
-        if (launch_pdl(gemm_team_kernel<SG, SH>, grid_team, (unsigned)kGemmThreads, smem_team, st, fast_args(ctx, false), idx, oa, d_gain_f16, sga, gt, \
+        if (!set_smem<gemm_team_kernel<BIG, SG, SH>>(ctx->device, smem_team)) return LLVQ_ECUDA;                                   \
+        if (launch_pdl(gemm_team_kernel<BIG, SG, SH>, grid_team, (unsigned)kGemmThreads, smem_team, st, fast_args(ctx, false), idx, oa, d_gain_f16, sga, gt, \
                        x_double, xmap) != cudaSuccess) return LLVQ_ECUDA;                                                     \
     } while (0)
-            if (yo) LLVQ_LAUNCH_TEAM(false, true);
-            else if (sg) LLVQ_LAUNCH_TEAM(true, false);
-            else LLVQ_LAUNCH_TEAM(false, false);
+            if (yo) { if (ctx->fast) LLVQ_LAUNCH_TEAM(false, false, true); else LLVQ_LAUNCH_TEAM(true, false, true); }
+            else if (sg) LLVQ_LAUNCH_TEAM(false, true, false);
+            else if (ctx->fast) LLVQ_LAUNCH_TEAM(false, false, false);
+            else LLVQ_LAUNCH_TEAM(true, false, false);
 #undef LLVQ_LAUNCH_TEAM
             return launch_status();
         }

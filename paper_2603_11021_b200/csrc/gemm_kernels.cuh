@@ -917,7 +917,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
     if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
-// The product on the stored stream of the 48-bit codes: two teams of 16 warps take the domains of a row tile in turn.  A team orders
+// The product on the stored stream of codes with many classes: two teams of 16 warps take the domains of a row tile in turn.  A team orders
 // its domain's 1024 blocks (order.cuh; the entries lie in its own A buffer, which its previous MMAs have left by then), every
 // warp takes two chunks of them into registers, unranks them, writes its part of A, and the team's first thread issues the MMAs
 // into the team's own accumulator.  The teams meet only at the end of a row tile: while one orders, which leaves most issue slots
@@ -925,7 +925,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
 constexpr int kGemmTeams = 2;
 constexpr int kGemmTeamThreads = kGemmThreads / kGemmTeams;
 
-template <bool kSg = false, bool kShard = false>
+template <bool kBig, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga, int x_double,
                  const __grid_constant__ CUtensorMap xmap)
@@ -969,6 +969,7 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
     uint8_t* const a_mine = a_buf + (uint32_t)team * kASet;
     uint8_t* const x_mine = b_buf + (x_double ? (uint32_t)team * x_set : 0u);
     unsigned long long* const ent = reinterpret_cast<unsigned long long*>(a_mine);
+    uint32_t* const ent2 = reinterpret_cast<uint32_t*>(ent + kOrderBlocks);
     const uint32_t nd = ga.sp.per_row, bpr = (uint32_t)ga.bpr;
     const uint32_t dom_begin = split_begin(ga.sp, blockIdx.x), dom_end = split_begin(ga.sp, blockIdx.x + 1u);
     uint32_t mine = 0, base[2] = {0, 0};               // domains this team has done; domains either team had done before this row tile
@@ -989,8 +990,8 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
             o.b = (tid >> 3) * bpr + d * kDomBlocks + (tid & 7u);
             o.pos = tid;
             o.there = d * kDomBlocks + (tid & 7u) < bpr;
-            order_piece<kSg, kGemmTeamThreads>(fa, T, sg, oa, stream, hists + ((uint32_t)team * 2u + (mine & 1u)) * oa.words,
-                                               hists + ((uint32_t)team * 2u + ((mine & 1u) ^ 1u)) * oa.words, ent, team, tid, o, (uint32_t)ga.n_out,
+            order_piece<kBig, kSg, kGemmTeamThreads>(fa, T, sg, oa, stream, hists + ((uint32_t)team * 2u + (mine & 1u)) * oa.words,
+                                               hists + ((uint32_t)team * 2u + ((mine & 1u) ^ 1u)) * oa.words, ent, ent2, team, tid, o, (uint32_t)ga.n_out,
                                                64u * bpr, 64u, (uint32_t)kGemmTeamThreads, [&] {
                 // the entries go over what the previous MMAs read
                 if (mine > 0 && !mbar_wait(bar_free + team, (mine - 1u) & 1u)) timeout = true;
@@ -998,23 +999,48 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
             });
             // ---- A: two chunks per warp, one from the expensive and one from the cheap end
             const unsigned long long e[2] = {ent[twarp * 32u + lane], ent[(31u - twarp) * 32u + lane]};
+            uint32_t e2[2] = {0u, 0u};
+            uint4 rec0, rec1;
+            if (kBig) {
+                e2[0] = ent2[twarp * 32u + lane]; e2[1] = ent2[(31u - twarp) * 32u + lane];
+                big_load_record(fa.dc, (int)(e2[0] & 0x1ffffu), !(e2[0] >> 31), rec0, rec1);
+            }
             team_barrier(team, kGemmTeamThreads);                         // all entries are in registers: A may overwrite them
+            // one X buffer: it may be asked for once the MMAs of the tile's domain before this one (the other team's) are through with it;
+            // looked at between the two chunks, waited for only when this domain's own MMAs are due
+            const uint32_t i_tile = d - d_begin, before = team == 0 ? base[1] + (i_tile >> 1) - 1u : base[0] + (i_tile >> 1);
+            bool asked = x_double != 0;
 #pragma unroll 1
             for (int q = 0; q < 2; ++q) {
-                const OrderedBlock b = ordered_block<kSg>(fa, sg, oa, q == 0 ? e[0] : e[1]);
+                if (q == 1 && !asked && tid == 0 && (i_tile == 0u || mbar_test(bar_free + (team ^ 1), before & 1u))) {
+                    request_x(smem_u32(x_mine), &xmap, (int)d, ga.npad, bar_x + team);
+                    asked = true;
+                }
+                OrderedBlock b{};
+                if (!kBig) b = ordered_block<kSg>(fa, sg, oa, q == 0 ? e[0] : e[1]);
+                else { const uint32_t y = q == 0 ? e2[0] : e2[1]; b.valid = !(y >> 31); b.pos = (y >> 17) & 1023u; }
                 const uint32_t r = b.pos >> 3, c = b.pos & 7u;
                 uint16_t gbits = 0;
                 if (!kSg && b.valid) gbits = ldg_u16_here(gain_tile + (r * bpr + d * kDomBlocks + c));
                 float gn = 0.f;                                           // the gain is converted once the block is unranked
-                Decoded dec;
-                decode_known_class(T, b.valid ? b.cls : 0u, b.local, b.valid, dec);
-                if (!kSg) gn = gain_to_float(gbits);
-                if (kSg && b.valid) {
-                    const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rt * kGemmRows + r) : 1.f;
-                    gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + b.gain_index)), __uint_as_float(T.desc[b.cls * kFastDescStride + kFastDescRnorm]));
-                }
                 uint32_t w[12];
-                expand_bf16(dec, gn, w);
+                if constexpr (kBig) {
+                    DecodedBig dec{};
+                    big_decode_record(T, rec0, rec1, b.valid ? (q == 0 ? e[0] : e[1]) : 0ull, b.valid, kFullMask, dec);
+                    if (q == 0) big_load_record(fa.dc, (int)(e2[1] & 0x1ffffu), !(e2[1] >> 31), rec0, rec1);
+                    gn = gain_to_float(gbits);
+                    expand_bf16(dec.d, gn, w);
+                    patch_id8_bf16(dec, gn, w);
+                } else {
+                    Decoded dec;
+                    decode_known_class(T, b.valid ? b.cls : 0u, b.local, b.valid, dec);
+                    if (!kSg) gn = gain_to_float(gbits);
+                    if (kSg && b.valid) {
+                        const float scale = sg.row_scale ? __ldg(sg.row_scale + (int64_t)rt * kGemmRows + r) : 1.f;
+                        gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + b.gain_index)), __uint_as_float(T.desc[b.cls * kFastDescStride + kFastDescRnorm]));
+                    }
+                    expand_bf16(dec, gn, w);
+                }
                 uint8_t* a_dst = a_mine + (c >> 2) * (kASet / 2) + (r >> 3) * 128u + (r & 7u) * 16u + 3u * (c & 3u) * 2048u;
 #pragma unroll
                 for (int j = 0; j < 3; ++j)
@@ -1024,10 +1050,8 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
             team_barrier(team, kGemmTeamThreads);
             // ---- MMAs
             if (tid == 0) {
-                if (!x_double) {
-                    // the domain before this one in the tile is the other team's: its MMAs have to be through with X
-                    const uint32_t i = d - d_begin, before = team == 0 ? base[1] + (i >> 1) - 1u : base[0] + (i >> 1);
-                    if (i > 0u && !mbar_wait(bar_free + (team ^ 1), before & 1u)) timeout = true;
+                if (!asked) {
+                    if (i_tile > 0u && !mbar_wait(bar_free + (team ^ 1), before & 1u)) timeout = true;
                     request_x(smem_u32(x_mine), &xmap, (int)d, ga.npad, bar_x + team);
                 }
                 if (!mbar_wait(bar_x + team, mine & 1u)) timeout = true;

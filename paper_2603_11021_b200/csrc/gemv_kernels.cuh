@@ -687,7 +687,7 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
             o.b = (o.row - rg0 * kGemvGroupRows) * bpr + kq * 4u + (c & 3u);
             o.pos = (c >> 2) * 32u + r * 4u + (c & 3u);
             o.there = (c >> 2) < nchunks && kq * 4u + (c & 3u) < bpr;
-            order_piece<kSg, kTeamThreads>(fa, T, sg, oa, stream, hist + (piece & 1u) * oa.words, hist + ((piece & 1u) ^ 1u) * oa.words, ent, team, tid,
+            order_piece<false, kSg, kTeamThreads>(fa, T, sg, oa, stream, hist + (piece & 1u) * oa.words, hist + ((piece & 1u) ^ 1u) * oa.words, ent, nullptr, team, tid,
                                                  o, min((uint32_t)n_out, (rg + 1u) * kGemvGroupRows), bpr << (1u + narrow), 2u << narrow, 8u << narrow, [&] { if (tid == 0) *next_chunk = kTeamWarps; });
             uint32_t kq_a;
             const uint32_t rg_off = split_row(sp, u0, kq_a) - rg0;

@@ -9,10 +9,10 @@
 #pragma once
 
 constexpr int kOrderBlocks = 1024;                          // blocks of a piece
-constexpr uint32_t kOrderPosShift = 22;                     // position in the top 10 bits of an entry's high word
+constexpr uint32_t kOrderPosShift = 22;                     // position in the top 10 bits of an entry's high word (class tables in shared memory)
 
 struct OrderArgs {
-    const uint16_t* sort_rank;      // sort key of every class
+    const uint16_t* sort_rank;      // sort key of every class (class tables in shared memory), else null
     uint32_t words;                 // bins of a histogram (32 times an odd number); the last bin is "no block"
     uint32_t cls_shift, gain_shift; // high word of an entry: class-local index >> 32 | class << cls_shift | gain index << gain_shift | position << 22
 };
@@ -29,11 +29,12 @@ struct OrderSpot {
 __device__ __forceinline__ void team_barrier(int team, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(threads) : "memory"); }
 
 // Orders one piece; the kThreads threads of team `team` call this together, numbered tid.  hist / hist_next: this piece's
-// histogram (zero on entry) and the next one's (zeroed here).  The entries go to ent; on return the piece is complete.
+// histogram (zero on entry) and the next one's (zeroed here).  The entries go to ent (with kBig the class-local index) and, with
+// kBig, ent2 (class | position << 17, bit 31 = no block); on return the piece is complete.
 // before_write(): what has to be awaited before ent may be written.
-template <bool kSg, int kThreads, typename Before>
+template <bool kBig, bool kSg, int kThreads, typename Before>
 __device__ __forceinline__ void order_piece(const FastArgs& fa, const FastSmem& T, const SgArgs& sg, const OrderArgs& oa, const uint32_t* __restrict__ stream,
-                                            uint32_t* hist, uint32_t* hist_next, unsigned long long* ent, int team, uint32_t tid,
+                                            uint32_t* hist, uint32_t* hist_next, unsigned long long* ent, uint32_t* ent2, int team, uint32_t tid,
                                             const OrderSpot& o, uint32_t n_out, uint32_t b_step, uint32_t row_step, uint32_t pos_step, Before before_write)
 {
     constexpr int kEach = kOrderBlocks / kThreads;
@@ -43,7 +44,7 @@ __device__ __forceinline__ void order_piece(const FastArgs& fa, const FastSmem& 
     uint64_t local[kEach];
     uint32_t hi[kEach], key[kEach], rank[kEach];             // hi: what the entry keeps beside the class-local index and the position
     {
-        RawField<false> raw[kEach];
+        RawField<kBig> raw[kEach];
         const uint64_t bits0 = o.b0 * (uint64_t)wbits;
         const uint32_t* base = stream + (bits0 >> 5);
         const uint32_t bits = o.b * (uint32_t)wbits + ((uint32_t)bits0 & 31u), step = b_step * (uint32_t)wbits;
@@ -51,25 +52,77 @@ __device__ __forceinline__ void order_piece(const FastArgs& fa, const FastSmem& 
 #pragma unroll
         for (int q = 0; q < kEach; ++q) {
             const bool there = o.there && o.row + (uint32_t)q * row_step < n_out;
-            raw[q] = request_field_at<false>(base, bits + (uint32_t)q * step, wbits, there);
+            raw[q] = request_field_at<kBig>(base, bits + (uint32_t)q * step, wbits, there);
             in |= (uint32_t)there << q;
         }
+        if constexpr (kBig) {
+            // the searches of the thread's blocks go side by side: each is a chain of reads from L2 (bucket, offsets, offset, record)
+            uint64_t lo[kEach];
+            uint32_t high[kEach], a[kEach], z[kEach], h[kEach], valid = 0;
 #pragma unroll
-        for (int q = 0; q < kEach; ++q) {
-            uint64_t lo, high;
-            field_value(raw[q], wbits, lo, high);
-            const bool there = (in >> q) & 1u;
-            const uint64_t I = kSg ? lo & ((1ull << fa.L.W) - 1ull) : lo;
-            const bool valid = there && I < fa.n_points;
-            if (there && !valid) atomicAdd(fa.bad_index, 1ull);
-            uint32_t cls = fa.L.ncls;                                 // no block
-            key[q] = none; local[q] = 0;
-            if (valid) {
-                cls = fast_find_class(T, I, local[q]);
-                key[q] = __ldg(oa.sort_rank + cls);
+            for (int q = 0; q < kEach; ++q) {
+                uint64_t h64;
+                field_value(raw[q], wbits, lo[q], h64);
+                high[q] = (uint32_t)h64;
+                const bool v = ((in >> q) & 1u) && (h64 < fa.dc.n_hi || (h64 == fa.dc.n_hi && lo[q] < fa.dc.n_lo));
+                if (((in >> q) & 1u) && !v) atomicAdd(fa.bad_index, 1ull);
+                valid |= (uint32_t)v << q;
+                a[q] = z[q] = 0u;
+                if (v) {
+                    const uint32_t bucket = big_bucket(fa.dc, lo[q], h64);
+                    a[q] = __ldg(fa.dc.lut + bucket); z[q] = __ldg(fa.dc.lut + bucket + 1);
+                }
             }
-            hi[q] = cls << oa.cls_shift;
-            if (kSg) hi[q] |= (uint32_t)(lo >> fa.L.W) << oa.gain_shift;
+            while (true) {
+                bool more = false;
+#pragma unroll
+                for (int q = 0; q < kEach; ++q) more = more || a[q] < z[q];
+                if (!more) break;
+                uint64_t ol[kEach];
+                uint32_t oh[kEach];
+#pragma unroll
+                for (int q = 0; q < kEach; ++q) {
+                    const uint32_t mid = (a[q] + z[q] + 1u) >> 1;
+                    ol[q] = 0; oh[q] = 0;
+                    if (a[q] < z[q]) { ol[q] = __ldg(fa.dc.off_lo + mid); oh[q] = __ldg(fa.dc.off_hi + mid); }
+                }
+#pragma unroll
+                for (int q = 0; q < kEach; ++q) {
+                    const uint32_t mid = (a[q] + z[q] + 1u) >> 1;
+                    if (a[q] < z[q]) { if (oh[q] < high[q] || (oh[q] == high[q] && ol[q] <= lo[q])) a[q] = mid; else z[q] = mid - 1u; }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < kEach; ++q) {
+                local[q] = 0; h[q] = 0;
+                if ((valid >> q) & 1u) { local[q] = lo[q] - __ldg(fa.dc.off_lo + a[q]); h[q] = __ldg(reinterpret_cast<const uint32_t*>(fa.dc.big + a[q])); }
+            }
+#pragma unroll
+            for (int q = 0; q < kEach; ++q) {
+                const bool v = (valid >> q) & 1u;
+                const uint32_t nlev = h[q] >> 28, nlev1 = (h[q] >> 24) & 7u, parity = (h[q] >> 16) & 1u;
+                // coarse shape of the unranking; two bins per shape (by lane): the few common shapes would queue at one word each
+                key[q] = v ? ((1u - parity) << 6 | (7u - min(nlev, 7u)) << 3 | nlev1) * 2u + (lane & 1u) : none;
+                hi[q] = v ? a[q] : 1u << 31;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < kEach; ++q) {
+                uint64_t lo, high;
+                field_value(raw[q], wbits, lo, high);
+                const bool there = (in >> q) & 1u;
+                const uint64_t I = kSg ? lo & ((1ull << fa.L.W) - 1ull) : lo;
+                const bool valid = there && I < fa.n_points;
+                if (there && !valid) atomicAdd(fa.bad_index, 1ull);
+                uint32_t cls = fa.L.ncls;                                 // no block
+                key[q] = none; local[q] = 0;
+                if (valid) {
+                    cls = fast_find_class(T, I, local[q]);
+                    key[q] = __ldg(oa.sort_rank + cls);
+                }
+                hi[q] = cls << oa.cls_shift;
+                if (kSg) hi[q] |= (uint32_t)(lo >> fa.L.W) << oa.gain_shift;
+            }
         }
     }
 #pragma unroll
@@ -94,7 +147,12 @@ __device__ __forceinline__ void order_piece(const FastArgs& fa, const FastSmem& 
 #pragma unroll
     for (int q = 0; q < kEach; ++q) {
         const uint32_t pos = o.pos + (uint32_t)q * pos_step, slot = hist[key[q]] + rank[q];
-        ent[slot] = local[q] | (unsigned long long)(hi[q] | pos << kOrderPosShift) << 32;
+        if (kBig) {
+            ent[slot] = local[q];
+            ent2[slot] = hi[q] | pos << 17;
+        } else {
+            ent[slot] = local[q] | (unsigned long long)(hi[q] | pos << kOrderPosShift) << 32;
+        }
     }
     team_barrier(team, kThreads);
 }
@@ -120,13 +178,16 @@ __device__ __forceinline__ OrderedBlock ordered_block(const FastArgs& fa, const 
 }
 
 // How a code's stored stream is ordered (host).  False where it is not: few classes (a warp of unrelated blocks costs little there),
-// class tables in global memory (looking up the classes and ordering by the shape of the unranking took as many instructions
-// as it saved: GEMV 4096 x 4096 of the 72-bit code 49.7 us against 44.2 unordered), or entries that do not fit.
+// or entries that do not fit.
 bool order_args(const llvq_ctx* ctx, int gain_bits, OrderArgs* oa)
 {
     *oa = OrderArgs{};
     const size_t ncls = ctx->host.desc.size();
-    if (!ctx->fast || !ctx->d_sort_rank || ncls < 64 || ncls > 1023 || ctx->host.W + gain_bits > 64) return false;
+    if (!ctx->fast) {
+        oa->words = 288;                                     // 128 shapes x 2 and "no block"
+        return gain_bits == 0 && ctx->host.W > 64 && ctx->host.W <= 72 && ncls <= (1u << 17);
+    }
+    if (!ctx->d_sort_rank || ncls < 64 || ncls > 1023 || ctx->host.W + gain_bits > 64) return false;
     auto bits = [](uint64_t v) { uint32_t b = 0; while (v >> b) ++b; return b; };
     const uint32_t local_high = std::max(bits(ctx->largest_class - 1), 32u) - 32u;
     oa->sort_rank = ctx->d_sort_rank;

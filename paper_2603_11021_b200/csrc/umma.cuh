@@ -29,6 +29,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
     return done != 0;
 }
 
+// Whether the phase has completed, without waiting.
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity)
+{
+    uint32_t done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return done != 0;
+}
+
 // ---- tensor memory ------------------------------------------------------------
 // One full warp allocates `cols` (power of two >= 32) columns; the base address is written to *slot (shared memory).
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t cols)
