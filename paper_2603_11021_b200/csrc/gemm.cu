@@ -28,9 +28,6 @@ bool make_x_map(const uint16_t* d_x, int64_t k_in, int batch, int npad, CUtensor
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The codes whose class tables stay in global memory have room for the table of small subsets beside the GEMM's buffers.
-size_t gemm_image_bytes(const llvq_ctx* ctx) { return ctx->fast ? ctx->fl.total : ctx->fl.total_ext; }
-
 int check_gemm_args(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f16, int64_t n_out, int64_t k_in,
                     const uint16_t* d_x_bf16, int batch, const uint16_t* d_y_bf16)
 {
@@ -49,7 +46,7 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     GemmArgs ga;
-    ga.y = d_y_bf16; ga.y_ld = n_out; ga.shard = nullptr; ga.y_f32 = y_f32; ga.sort_rank = nullptr; ga.nbins = 0; ga.bin_round = 0;
+    ga.y = d_y_bf16; ga.y_ld = n_out; ga.shard = nullptr; ga.y_f32 = y_f32;
     if (yo) {                                             // the description travels ahead of the kernel on the same stream
         ga.y = static_cast<uint16_t*>(yo->y); ga.y_ld = y_ld; ga.shard = static_cast<const YOut*>(ctx->d_shard);
         put_shard_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(*yo, static_cast<YOut*>(ctx->d_shard));   // by value: safe under stream capture
@@ -65,37 +62,32 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
     const unsigned grid = (unsigned)std::min<int64_t>(row_tiles * ga.nstages, ctx->sm_count);
     ga.sp = make_split(row_tiles * ga.nstages, ga.nstages, grid);
     // gemm_pipe_kernel: two A buffer sets and two X buffer sets, or one X set when two do not fit; else the kernel with the block barrier
-    const size_t head = (gemm_image_bytes(ctx) + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
+    const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
                  x_set = (size_t)kDomStages * ga.npad * kStageK * 2;
     int pipe = 0, b_double = 0;
     size_t smem = head + (size_t)dpi * (a_set + x_set);
-    if (head + 2 * a_set + 2 * x_set <= 227 * 1024) { pipe = 1; b_double = 1; smem = head + 2 * a_set + 2 * x_set; }
+    if (head + 2 * a_set + 2 * x_set <= (ctx->fast ? 227u : 200u) * 1024) { pipe = 1; b_double = 1; smem = head + 2 * a_set + 2 * x_set; }
     else if (head + 2 * a_set + x_set <= 227 * 1024) { pipe = 1; smem = head + 2 * a_set + x_set; }
-    if (smem > 227 * 1024) return LLVQ_EUNSUPPORTED;
-#define LLVQ_LAUNCH_DOMAINS(BIG, SG, SH)                                                                                      \
+    if (smem > 227 * 1024 || (!ctx->fast && !pipe)) return LLVQ_EUNSUPPORTED;      // (the pipeline's buffers fit for every code of the second kind)
+#define LLVQ_LAUNCH_DOMAINS(K, LAST)                                                                                          \
     do {                                                                                                                     \
-        if (pipe) {                                                                                                          \
-            if (!set_smem<gemm_pipe_kernel<BIG, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                            \
-            if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx, !ctx->fast), \
-                           static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, b_double, xmap) != cudaSuccess) return LLVQ_ECUDA; \
-        } else {                                                                                                             \
-            if (!set_smem<gemm_sorted_kernel<BIG, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                          \
-            if (launch_pdl(gemm_sorted_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx, !ctx->fast), \
-                           static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA; \
-        }                                                                                                                    \
+        if (!set_smem<K>(ctx->device, smem)) return LLVQ_ECUDA;                                                               \
+        if (launch_pdl(K, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx), static_cast<const unsigned long long*>(p), d_gain_f16, \
+                       sga, ga, LAST, xmap) != cudaSuccess) return LLVQ_ECUDA;                                                \
     } while (0)
     const SgArgs sga = sg ? *sg : SgArgs{};
     CUtensorMap xmap;
     if (!make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
-    if (yo) {                                            // row-sharded: stored-gain form only
-        if (sg) return LLVQ_EUNSUPPORTED;
-        if (ctx->fast) LLVQ_LAUNCH_DOMAINS(false, false, true); else LLVQ_LAUNCH_DOMAINS(true, false, true);
-    } else if (sg) {
-        LLVQ_LAUNCH_DOMAINS(false, true, false);
-    } else if (ctx->fast) {
-        LLVQ_LAUNCH_DOMAINS(false, false, false);
+    if (yo && sg) return LLVQ_EUNSUPPORTED;              // row-sharded: stored-gain form only
+    if (!ctx->fast) { if (yo) LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<true, false, true>), b_double); else LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<true, false, false>), b_double); }
+    else if (pipe) {
+        if (yo) LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<false, false, true>), b_double);
+        else if (sg) LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<false, true, false>), b_double);
+        else LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<false, false, false>), b_double);
     } else {
-        LLVQ_LAUNCH_DOMAINS(true, false, false);
+        if (yo) LLVQ_LAUNCH_DOMAINS((gemm_sorted_kernel<false, true>), dpi);
+        else if (sg) LLVQ_LAUNCH_DOMAINS((gemm_sorted_kernel<true, false>), dpi);
+        else LLVQ_LAUNCH_DOMAINS((gemm_sorted_kernel<false, false>), dpi);
     }
 #undef LLVQ_LAUNCH_DOMAINS
     return launch_status();
@@ -113,7 +105,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     cudaStream_t st = (cudaStream_t)stream;
     if (k_in == 0) return cudaMemsetAsync(d_y_bf16, 0, (size_t)n_out * batch * 2, st) == cudaSuccess ? LLVQ_OK : LLVQ_ECUDA;
     GemmArgs ga;
-    ga.y = d_y_bf16; ga.y_ld = n_out; ga.shard = nullptr; ga.y_f32 = 0; ga.sort_rank = nullptr; ga.nbins = 0; ga.bin_round = 0;
+    ga.y = d_y_bf16; ga.y_ld = n_out; ga.shard = nullptr; ga.y_f32 = 0;
     if (yo) {                                             // the description travels ahead of the kernel on the same stream
         ga.y = static_cast<uint16_t*>(yo->y); ga.y_ld = y_ld; ga.shard = static_cast<const YOut*>(ctx->d_shard);
         put_shard_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(*yo, static_cast<YOut*>(ctx->d_shard));   // by value: safe under stream capture
@@ -134,18 +126,22 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     ga.split = best;
     const int64_t items = row_tiles * ga.split;
     const unsigned grid = (unsigned)std::min<int64_t>(items, ctx->sm_count);
-    const size_t img = gemm_image_bytes(ctx);
+    const size_t img = ctx->fl.total;
     const size_t smem = ((img + 64 + 1023) & ~size_t(1023)) + 2 * kGemmRows * kStageK * 2 + 2 * (size_t)ga.npad * kStageK * 2;
     if (smem > 227 * 1024) return LLVQ_EUNSUPPORTED;
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (yo && sg) return LLVQ_EUNSUPPORTED;              // row-sharded: stored-gain form only
     CUtensorMap xmap;
     if (!make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
+    // codes with many classes (a warp of 32 unrelated blocks is what costs there): the kernel whose two teams order their domains; it
+    // fits for every code with class tables in global memory
     OrderArgs oa;
     if (order_args(ctx, sg ? sg->bits : 0, &oa)) {
         const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_sets = (size_t)kGemmTeams * kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2, hists = (size_t)kGemmTeams * 2 * oa.words * 4;
-        const int x_double = head + a_sets + 2 * x_set + hists <= 227 * 1024;
+        // (codes that look their classes up in global memory keep a larger L1 cache below 200 KB of shared memory: 8192 x 8192, 72 bits, batch
+        // 64: 234 us with two X buffers, 197 with one)
+        const int x_double = head + a_sets + 2 * x_set + hists <= (ctx->fast ? 227u : 200u) * 1024;
         const size_t smem_team = head + a_sets + (x_double ? 2 : 1) * x_set + hists;
         if (smem_team <= 227 * 1024) {
             GemmArgs gt = ga;
@@ -168,83 +164,13 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             return launch_status();
         }
     }
-    // codes with their class tables in shared memory and many classes (a warp of 32 unrelated blocks is what costs there):
-    // the kernel that puts every domain of 1024 blocks into the order of the sorted layout before unranking it, as many
-    // domains at a time (up to 4) as shared memory has room for beside the operand buffers
-    const int ncls = (int)ctx->host.desc.size();
-    if (ctx->fast && ctx->d_sort_rank && ncls >= 64 && ncls < 1024 && ctx->host.W + (sg ? sg->bits : 0) <= 48) {
-        const size_t head = (img + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
-                     x_set = (size_t)kDomStages * ga.npad * kStageK * 2;
-        GemmArgs gb = ga;
-        gb.nstages = (int)((ga.bpr + kDomBlocks - 1) / kDomBlocks);            // domains per row tile
-        gb.split = 1;
-        gb.sort_rank = ctx->d_sort_rank;
-        gb.nbins = (ncls + 1 + 31) / 32 * 32;                                    // one bin per class and one for "no block"
-        const size_t bins = (size_t)gb.nbins * 4 + 32 * 4 + (size_t)kDomEntries * 8;   // per ordered domain
-        const int dpi = ga.npad <= 32 ? 2 : 1;
-        gb.bin_round = 4;
-        while (gb.bin_round > dpi && head + (size_t)dpi * (a_set + x_set) + (size_t)gb.bin_round * bins > 227 * 1024) gb.bin_round -= dpi;
-        const size_t smem_bin = head + (size_t)dpi * (a_set + x_set) + (size_t)gb.bin_round * bins;
-        if (smem_bin <= 227 * 1024) {
-            const unsigned grid_bin = (unsigned)std::min<int64_t>(row_tiles * gb.nstages, ctx->sm_count);
-            gb.sp = make_split(row_tiles * gb.nstages, gb.nstages, grid_bin);
-            const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
-            const SgArgs sga = sg ? *sg : SgArgs{};
-#define LLVQ_LAUNCH_BINNED(SG, SH, RD)                                                                                          \
-    do {                                                                                                                        \
-        if (!set_smem<gemm_sorted_kernel<false, SG, SH, true, RD>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                 \
-        if (launch_pdl(gemm_sorted_kernel<false, SG, SH, true, RD>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, false), words, \
-                       d_gain_f16, sga, gb, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA;                                             \
-    } while (0)
-            if (gb.bin_round > dpi) {                    // rounds of several iterations
-                if (yo) LLVQ_LAUNCH_BINNED(false, true, true);
-                else if (sg) LLVQ_LAUNCH_BINNED(true, false, true);
-                else LLVQ_LAUNCH_BINNED(false, false, true);
-            } else {
-                if (yo) LLVQ_LAUNCH_BINNED(false, true, false);
-                else if (sg) LLVQ_LAUNCH_BINNED(true, false, false);
-                else LLVQ_LAUNCH_BINNED(false, false, false);
-            }
-#undef LLVQ_LAUNCH_BINNED
-            return launch_status();
-        }
-    }
-    // the 72-bit code at wide batches (one domain per iteration): the same with the coarse shape of the unranking as sort key,
-    // four domains ordered per round (at padded batch <= 32 the pipeline kernel on unordered chunks is faster: measured)
-    if (!ctx->fast && ctx->host.W > 64 && ctx->host.W <= 72 && ga.npad > 32 && !sg && (int)ctx->host.desc.size() <= (1 << kBigClassBits)) {
-        const size_t head = (img + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
-                     x_set = (size_t)kDomStages * ga.npad * kStageK * 2;
-        GemmArgs gb = ga;
-        gb.nstages = (int)((ga.bpr + kDomBlocks - 1) / kDomBlocks);            // domains per row tile
-        gb.split = 1;
-        gb.nbins = 160;                                                         // 128 shapes; the last bin is "no block"
-        gb.bin_round = 4;
-        const size_t bins = (size_t)gb.nbins * 4 + 32 * 4 + (size_t)kDomEntries * (8 + 4);
-        const int dpi = 1;
-        const size_t smem_bin = head + (size_t)dpi * (a_set + x_set) + (size_t)gb.bin_round * bins;
-        if (smem_bin <= 227 * 1024) {
-            const unsigned grid_bin = (unsigned)std::min<int64_t>(row_tiles * gb.nstages, ctx->sm_count);
-            gb.sp = make_split(row_tiles * gb.nstages, gb.nstages, grid_bin);
-            const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
-            if (yo) {
-                if (!set_smem<gemm_sorted_kernel<true, false, true, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
-                if (launch_pdl(gemm_sorted_kernel<true, false, true, true, true>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, true), words,
-                               d_gain_f16, SgArgs{}, gb, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA;
-            } else {
-                if (!set_smem<gemm_sorted_kernel<true, false, false, true, true>>(ctx->device, smem_bin)) return LLVQ_ECUDA;
-                if (launch_pdl(gemm_sorted_kernel<true, false, false, true, true>, grid_bin, (unsigned)kGemmThreads, smem_bin, st, fast_args(ctx, true), words,
-                               d_gain_f16, SgArgs{}, gb, dpi, xmap) != cudaSuccess) return LLVQ_ECUDA;
-            }
-            return launch_status();
-        }
-    }
     {
         // the kernel without a block barrier (see gemm_pipe_kernel), if its buffers fit
         const size_t head = (img + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2;
         const int b_double = head + 2 * a_set + 2 * x_set <= 227 * 1024;
         const size_t smem_pipe = head + 2 * a_set + (b_double ? 2 : 1) * x_set;
-        if (smem_pipe <= 227 * 1024 && (ctx->fast || ga.npad <= 32)) {    // 72-bit code at wide batches: slower than gemm_kernel (measured)
+        if (smem_pipe <= 227 * 1024) {
             GemmArgs gp = ga;
             gp.nstages = (int)((ga.bpr + kDomBlocks - 1) / kDomBlocks);        // domains per row tile
             gp.split = 1;
@@ -252,38 +178,28 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             gp.sp = make_split(row_tiles * gp.nstages, gp.nstages, grid_pipe);
             const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
             const SgArgs sga = sg ? *sg : SgArgs{};
-#define LLVQ_LAUNCH_PIPE_STORED(BIG, SG, SH)                                                                                    \
+#define LLVQ_LAUNCH_PIPE_STORED(SG, SH)                                                                                    \
     do {                                                                                                                        \
-        if (!set_smem<gemm_pipe_kernel<BIG, SG, SH, true>>(ctx->device, smem_pipe)) return LLVQ_ECUDA;                                        \
-        if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH, true>, grid_pipe, (unsigned)kGemmThreads, smem_pipe, st, fast_args(ctx, !ctx->fast), words, \
+        if (!set_smem<gemm_pipe_kernel<false, SG, SH, true>>(ctx->device, smem_pipe)) return LLVQ_ECUDA;                                        \
+        if (launch_pdl(gemm_pipe_kernel<false, SG, SH, true>, grid_pipe, (unsigned)kGemmThreads, smem_pipe, st, fast_args(ctx), words, \
                        d_gain_f16, sga, gp, b_double, xmap) != cudaSuccess) return LLVQ_ECUDA;                                        \
     } while (0)
-            if (!ctx->fast) { if (yo) LLVQ_LAUNCH_PIPE_STORED(true, false, true); else LLVQ_LAUNCH_PIPE_STORED(true, false, false); }
-            else if (yo) LLVQ_LAUNCH_PIPE_STORED(false, false, true);
-            else if (sg) LLVQ_LAUNCH_PIPE_STORED(false, true, false);
-            else LLVQ_LAUNCH_PIPE_STORED(false, false, false);
+            if (yo) LLVQ_LAUNCH_PIPE_STORED(false, true);
+            else if (sg) LLVQ_LAUNCH_PIPE_STORED(true, false);
+            else LLVQ_LAUNCH_PIPE_STORED(false, false);
 #undef LLVQ_LAUNCH_PIPE_STORED
             return launch_status();
         }
     }
-    if (yo) {
-        if (ctx->fast) {
-            if (!set_smem<gemm_kernel<false, false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemm_kernel<false, false, true>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
-        } else {
-            if (!set_smem<gemm_kernel<true, false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemm_kernel<true, false, true>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
-        }
-    } else if (sg) {
-        if (!set_smem<gemm_kernel<false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
-        if (launch_pdl(gemm_kernel<false, true>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, *sg, ga) != cudaSuccess) return LLVQ_ECUDA;
-    } else if (ctx->fast) {
-        if (!set_smem<gemm_kernel<false, false>>(ctx->device, smem)) return LLVQ_ECUDA;
-        if (launch_pdl(gemm_kernel<false, false>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
-    } else {
-        if (!set_smem<gemm_kernel<true, false>>(ctx->device, smem)) return LLVQ_ECUDA;
-        if (launch_pdl(gemm_kernel<true, false>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx, !ctx->fast), idx, d_gain_f16, SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA;
-    }
+#define LLVQ_LAUNCH_STAGES(SG, SH)                                                                                              \
+    do {                                                                                                                        \
+        if (!set_smem<gemm_kernel<SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                                \
+        if (launch_pdl(gemm_kernel<SG, SH>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx), idx, d_gain_f16, sg ? *sg : SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA; \
+    } while (0)
+    if (yo) LLVQ_LAUNCH_STAGES(false, true);
+    else if (sg) LLVQ_LAUNCH_STAGES(true, false);
+    else LLVQ_LAUNCH_STAGES(false, false);
+#undef LLVQ_LAUNCH_STAGES
     return launch_status();
 }
 
@@ -317,13 +233,13 @@ static int sort_blocks_gemm_common(const llvq_ctx* ctx, const void* d_idx, int g
     const int64_t ndomains = ((n_out + kGemmRows - 1) / kGemmRows) * ((bpr + kDomBlocks - 1) / kDomBlocks);
     const unsigned g = (unsigned)std::min<int64_t>(ndomains, 4ll * ctx->sm_count);
     if (!ctx->fast) {
-        sort_blocks_gemm_big_kernel<<<g, kDomEntries, 0, (cudaStream_t)stream>>>(fast_args(ctx, !ctx->fast), static_cast<const uint32_t*>(d_idx), n_out, bpr,
+        sort_blocks_gemm_big_kernel<<<g, kDomEntries, 0, (cudaStream_t)stream>>>(fast_args(ctx), static_cast<const uint32_t*>(d_idx), n_out, bpr,
                                                                                  ndomains, static_cast<uint32_t*>(d_sorted));
         return launch_status();
     }
     const size_t smem = ctx->fl.total + 16;
     if (!set_smem<sort_blocks_gemm_kernel>(ctx->device, smem)) return LLVQ_ECUDA;
-    sort_blocks_gemm_kernel<<<g, kDomEntries, smem, (cudaStream_t)stream>>>(fast_args(ctx, !ctx->fast), static_cast<const uint32_t*>(d_idx), ctx->d_sort_rank,
+    sort_blocks_gemm_kernel<<<g, kDomEntries, smem, (cudaStream_t)stream>>>(fast_args(ctx), static_cast<const uint32_t*>(d_idx), ctx->d_sort_rank,
                                                                            gain_bits, n_out, bpr, ndomains, static_cast<unsigned long long*>(d_sorted));
     return launch_status();
 }

@@ -33,9 +33,6 @@ struct GemmArgs {
     int64_t scratch_ld;        // row tiles * 128
     uint32_t* counters;        // [row tiles], zero on entry and on exit
     int y_f32;                 // Y holds binary32 instead of bf16 (the batch-1 product behind llvq_gemv_sorted of the 72-bit code)
-    const uint16_t* sort_rank; // stored stream ordered inside the kernel (gemm_sorted_kernel<.., kBin>): sort key of every class, else null
-    int nbins;                 // ... and the number of bins (a multiple of 32 above the largest key; the last bin is "no block")
-    int bin_round;             // ... and how many domains are ordered at a time (a multiple of the domains per iteration, at most 4)
 };
 
 __global__ void put_shard_kernel(YOut yo, YOut* dst)
@@ -63,7 +60,7 @@ __device__ __forceinline__ void group_barrier(int group)
     asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kGemmGroupThreads) : "memory");
 }
 
-template <bool kBig, bool kSg = false, bool kShard = false>
+template <bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga)
 {
@@ -120,9 +117,9 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
             const bool in = row < ga.n_out && cb < ga.bpr;
             const uint64_t b = in ? (uint64_t)(row * ga.bpr + cb) : 0ull;
             uint32_t w[12];
-            const RawBlock<kBig> raw = request_block<kBig>(stream, kSg ? nullptr : gain, fa.dc.W + (kSg ? sg.bits : 0), b, in);
+            const RawBlock<false> raw = request_block<false>(stream, kSg ? nullptr : gain, fa.dc.W + (kSg ? sg.bits : 0), b, in);
             if constexpr (kSg) block_pairs_sg(fa, T, raw.field, sg, row, in, w);
-            else block_pairs<kBig>(fa, T, raw, in, w);
+            else block_pairs<false>(fa, T, raw, in, w);
             // the MMAs of this group's previous stage read its buffers: wait for them only now, with the block already unranked
             if (uses > 0 && !mbar_wait(&bar_free[group], (uses - 1u) & 1u)) timeout = true;
             uint8_t* a_dst = a_mine + gwarp * 128 + (lane & 7) * 16;
@@ -355,22 +352,12 @@ sort_blocks_gemm_big_kernel(FastArgs fa, const uint32_t* __restrict__ stream, in
     }
 }
 
-// kBin: `sorted` points at the stored stream instead; at the start of an iteration every thread looks up the class of
-// one block per domain (S1-S2) and the CTA puts the 1024 fields of a domain into the order of the sorted layout with a
-// counting sort in shared memory (one bin per class), so that the unranking below runs on the same entries as with a
-// stream sorted at load time.  ga.bin_round domains are ordered at a time (their four block barriers are then paid once per
-// round, not once per iteration); the stream words of the next round are requested in L2 a round ahead.
-// kRound (with kBin): a round is longer than an iteration; else it is one iteration and the words come through registers.
-// kBin with kBig (class tables in global memory; rounds only): the bins are the coarse shape of the unranking (parity,
-// number of steps, steps of the first group: 128 bins) instead of the full key of the sorted layout, the entries
-// (class-local index, class | position) as in the 96-bit layout; the class look-ups of a round's domains (dependent
-// reads from L2) run side by side.
-template <bool kBig, bool kSg = false, bool kShard = false, bool kBin = false, bool kRound = false>
+// For codes whose tables leave no room for gemm_pipe_kernel's buffers.
+template <bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga, int dpi,
                    const __grid_constant__ CUtensorMap xmap)
 {
-    static_assert(!(kBin && kBig && (kSg || !kRound)), "in-kernel ordering for the codes with tables in global memory: stored gains, rounds");
     extern __shared__ __align__(1024) uint8_t smem_1k[];
     uint8_t* const smem = smem_1k;
     const uint32_t img_bytes = fa.image_bytes;
@@ -385,14 +372,6 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
     uint8_t* a_buf = smem + a_off;                                        // [dpi * 2 stages] x 24576
     const uint32_t b_stage = (uint32_t)ga.npad * kStageK * 2;
     uint8_t* b_buf = a_buf + (uint32_t)dpi * kDomStages * kAStage;         // [dpi * 2 stages] x npad * 192
-    // kBin: per domain of the iteration the bins (block counts, then the first slot of every bin), the warp totals of their prefix sum
-    // and the ordered entries
-    constexpr int kMaxRound = kRound ? 4 : 2;
-    const int nround = kBin ? ga.bin_round : 1;
-    uint32_t* bin_hist = reinterpret_cast<uint32_t*>(b_buf + (uint32_t)dpi * kDomStages * b_stage);   // [nround][nbins] counts, then first slots
-    uint32_t* bin_wt = bin_hist + nround * ga.nbins;                        // [nround][32]
-    unsigned long long* bin_ent = reinterpret_cast<unsigned long long*>(bin_wt + nround * 32);          // [nround][1024]
-    uint32_t* bin_ent2 = reinterpret_cast<uint32_t*>(bin_ent + nround * kDomEntries);                    // kBig: [nround][1024] class | position << 17
 
     pdl_launch_dependents();
     const bool image_ok = fast_load_image(smem, fa.image, fa.image_bytes, bar_img, fa.flags);
@@ -403,8 +382,6 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
     }
     const FastSmem T = fast_view(smem, fa.L);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (kBin)
-        for (int i = threadIdx.x; i < nround * ga.nbins; i += kGemmThreads) bin_hist[i] = 0u;
     if (threadIdx.x == 0) {
         mbar_init(bar_free, 1); mbar_init(bar_done, 1); mbar_init(bar_x, (uint32_t)dpi);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -427,161 +404,45 @@ gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, c
         // CTAs that share this row tile
         const uint32_t parts = dom_begin <= tile0 && tile1 <= dom_end ? 1u : split_owner(ga.sp, tile1 - 1u) - split_owner(ga.sp, tile0) + 1u;
         // the entries of an iteration are requested one iteration ahead (they come from DRAM)
-        const ulonglong2 no_entry = make_ulonglong2(kSortIndexMask, kBigNoBlock);
+        const unsigned long long no_entry = kSortIndexMask;
         auto entry_at = [&](int d, int q) {
             if (d + q >= d_end) return no_entry;
-            if (kBin) {       // a round is one iteration (no room for more): the stream words that hold the field of this thread's block
-                              // (position = thread) are requested an iteration ahead into registers; y bit 63 = no block
-                if (kRound) return no_entry;             // longer rounds ask for them in L2 instead, see below
-                const int64_t row = (int64_t)rt * kGemmRows + (threadIdx.x >> 3), cb = (int64_t)(d + q) * kDomBlocks + (threadIdx.x & 7u);
-                if (row < ga.n_out && cb < ga.bpr)
-                    return load_field_words(reinterpret_cast<const uint32_t*>(sorted), (uint64_t)(row * ga.bpr + cb), (int)fa.L.W + (kSg ? sg.bits : 0));
-                return no_entry;
-            }
             // warp 0 also issues the MMAs of every iteration: it takes the cheapest chunk of each domain (the last), the other
             // warps pair chunk w - 1 of the first domain with chunk 31 - w of the second
             const int chunk = warp == 0 ? 31 : (q == 0 ? warp - 1 : 31 - warp);
             const int64_t at = ((int64_t)rt * nd + d + q) * kDomEntries + chunk * 32 + lane;
-            if (kBig) return load_big_entry(sorted, at);
-            return make_ulonglong2(__ldg(sorted + at), 0ull);
+            return __ldg(sorted + at);
         };
-        ulonglong2 e0 = entry_at(d_begin, 0), e1 = dpi > 1 ? entry_at(d_begin, 1) : no_entry;
+        unsigned long long e0 = entry_at(d_begin, 0), e1 = dpi > 1 ? entry_at(d_begin, 1) : no_entry;
         for (int d0 = d_begin; d0 < d_end; d0 += dpi, ++uses) {
             const int nd_now = min(dpi, d_end - d0);
-            ulonglong2 cur0 = e0, cur1 = e1;
+            const unsigned long long cur0 = e0, cur1 = e1;
             e0 = entry_at(d0 + dpi, 0);
             if (dpi > 1) e1 = entry_at(d0 + dpi, 1);
-            if (kBin) {
-                const int in_round = kRound ? (d0 - d_begin) % nround : 0;  // this iteration's first domain inside the round
-                if (in_round == 0) {
-                    // ---- order the fields of the round's domains, each by the sort key of its blocks' classes
-                    const uint32_t nbins = (uint32_t)ga.nbins;
-                    const int wbits = (int)fa.L.W + (kSg ? sg.bits : 0);
-                    const int nr = min(nround, d_end - d0);                  // domains in this round
-                    const uint32_t* words = reinterpret_cast<const uint32_t*>(sorted);
-                    const int64_t row = (int64_t)rt * kGemmRows + (threadIdx.x >> 3);
-                    unsigned long long f[kMaxRound];
-                    uint32_t f2[kMaxRound];                                  // kBig: class | position << 17
-                    uint32_t key[kMaxRound], rank[kMaxRound], cnt[kMaxRound], incl[kMaxRound];
-#pragma unroll
-                    for (int r = 0; r < kMaxRound; ++r) {
-                        f[r] = kBig ? kBigNoBlock : kSortIndexMask; f2[r] = threadIdx.x << kBigClassBits;
-                        key[r] = nbins - 1u; rank[r] = cnt[r] = incl[r] = 0u;
-                        if (r >= nr) continue;
-                        const int64_t cb = (int64_t)(d0 + r) * kDomBlocks + (threadIdx.x & 7u);
-                        if (kBig) {
-                            if (row < ga.n_out && cb < ga.bpr) {
-                                uint64_t lo, hi;
-                                load_index(words, (uint64_t)(row * ga.bpr + cb), fa.dc.W, lo, hi);
-                                if (hi < fa.dc.n_hi || (hi == fa.dc.n_hi && lo < fa.dc.n_lo)) {
-                                    uint64_t local;
-                                    const uint32_t cls = (uint32_t)big_find_class(fa.dc, lo, hi, local);
-                                    const uint32_t h = __ldg(reinterpret_cast<const uint32_t*>(fa.dc.big + cls));
-                                    const uint32_t nlev = h >> 28, nlev1 = (h >> 24) & 7u, parity = (h >> 16) & 1u;
-                                    key[r] = (1u - parity) << 6 | (7u - min(nlev, 7u)) << 3 | nlev1;
-                                    f[r] = local;
-                                    f2[r] |= cls;
-                                } else {
-                                    atomicAdd(fa.bad_index, 1ull);
-                                }
-                                const int64_t cbn = cb + (int64_t)nround * kDomBlocks;
-                                if (d0 + r + nround < d_end && cbn < ga.bpr)
-                                    asm volatile("prefetch.global.L2 [%0];" ::"l"(words + (((uint64_t)(row * ga.bpr + cbn) * (uint64_t)fa.dc.W) >> 5)));
-                            }
-                        } else if (row < ga.n_out && cb < ga.bpr) {
-                            if (!kRound) f[r] = field_of_words(r == 0 ? cur0 : cur1, wbits);            // requested an iteration ago
-                            else f[r] = load_field(words, (uint64_t)(row * ga.bpr + cb), wbits);
-                            const uint64_t I = kSg ? f[r] & ((1ull << fa.L.W) - 1ull) : f[r];
-                            if (I < fa.n_points) {
-                                uint64_t local;
-                                key[r] = __ldg(ga.sort_rank + fast_find_class(T, I, local));
-                            } else {
-                                atomicAdd(fa.bad_index, 1ull);
-                                f[r] = kSortIndexMask;
-                            }
-                            // the same block of the next round: ask for its stream words in L2
-                            const int64_t cbn = cb + (int64_t)nround * kDomBlocks;
-                            if (kRound && d0 + r + nround < d_end && cbn < ga.bpr)
-                                asm volatile("prefetch.global.L2 [%0];" ::"l"(words + (((uint64_t)(row * ga.bpr + cbn) * (uint64_t)wbits) >> 5)));
-                        }
-                        rank[r] = atomicAdd(&bin_hist[r * nbins + key[r]], 1u);   // its place among the blocks of its bin
-                    }
-                    __syncthreads();
-#pragma unroll
-                    for (int r = 0; r < kMaxRound; ++r) {
-                        if (r >= nr) continue;
-                        cnt[r] = threadIdx.x < nbins ? bin_hist[r * nbins + threadIdx.x] : 0u;
-                        uint32_t v = cnt[r];
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(kFullMask, v, o); if (lane >= o) v += t; }
-                        incl[r] = v;
-                        if (lane == 31) bin_wt[r * 32 + warp] = v;
-                    }
-                    __syncthreads();
-#pragma unroll
-                    for (int r = 0; r < kMaxRound; ++r) {
-                        if (r >= nr) continue;
-                        uint32_t v = bin_wt[r * 32 + lane];                  // every warp scans the 32 warp totals
-                        const uint32_t own = v;
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(kFullMask, v, o); if (lane >= o) v += t; }
-                        const uint32_t before = __shfl_sync(kFullMask, v - own, warp);
-                        if (threadIdx.x < nbins) bin_hist[r * nbins + threadIdx.x] = before + incl[r] - cnt[r];
-                    }
-                    __syncthreads();
-#pragma unroll
-                    for (int r = 0; r < kMaxRound; ++r) {
-                        if (r >= nr) continue;
-                        const uint32_t slot = bin_hist[r * nbins + key[r]] + rank[r];
-                        if (kBig) { bin_ent[r * kDomEntries + slot] = f[r]; bin_ent2[r * kDomEntries + slot] = f2[r]; }
-                        else bin_ent[r * kDomEntries + slot] = f[r] | (unsigned long long)threadIdx.x << 48;
-                    }
-                    __syncthreads();
-                    for (int i = threadIdx.x; i < nround * (int)nbins; i += kGemmThreads) bin_hist[i] = 0u;   // for the next round (barriers follow below)
-                }
-                auto ordered = [&](int at) {                               // entry `at` of the round's ordered domains in the form the unranking takes
-                    if (!kBig) return make_ulonglong2(bin_ent[at], 0ull);
-                    const unsigned long long x = bin_ent[at];
-                    const uint32_t y2 = bin_ent2[at];
-                    return make_ulonglong2(x & ~kBigNoBlock, (x & kBigNoBlock) | (unsigned long long)(y2 & ((1u << kBigClassBits) - 1u)) << 8 |
-                                                                  (unsigned long long)(y2 >> kBigClassBits) << 32);
-                };
-                cur0 = ordered(in_round * kDomEntries + (warp == 0 ? 31 : warp - 1) * 32 + lane);
-                if (nd_now > 1) cur1 = ordered((in_round + 1) * kDomEntries + (warp == 0 ? 31 : 31 - warp) * 32 + lane);
-            }
             // ---- A: every warp unranks one chunk of 32 sorted entries per domain
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 if (q >= nd_now) break;
-                const ulonglong2 e = q == 0 ? cur0 : cur1;
-                const uint64_t field = e.x & kSortIndexMask;
+                const unsigned long long e = q == 0 ? cur0 : cur1;
+                const uint64_t field = e & kSortIndexMask;
                 const uint64_t I = kSg ? field & ((1ull << fa.L.W) - 1ull) : field;     // shape-gain form: gain index above the shape index
-                const uint32_t pos = kBig ? (uint32_t)(e.y >> 32) & 1023u : (uint32_t)(e.x >> 48);
-                const bool valid = kBig ? !(e.y >> 63) : (field != kSortIndexMask && I < fa.n_points);
+                const uint32_t pos = (uint32_t)(e >> 48);
+                const bool valid = field != kSortIndexMask && I < fa.n_points;
                 const uint32_t r = pos >> 3, c = pos & 7u;
                 const int64_t row = (int64_t)rt * kGemmRows + r, cb = (int64_t)(d0 + q) * kDomBlocks + c;
                 uint16_t gbits = 0;
                 if (!kSg && valid) gbits = ldg_u16_here(gain + row * ga.bpr + cb);
                 float gn = 0.f;                                               // the gain is converted once the block is unranked
                 uint32_t w[12];
-                if (kBig) {
-                    const int cls = valid ? (int)((uint32_t)(e.y >> 8) & 0xffffffu) : 0;
-                    DecodedBig dec{};
-                    big_decode_planes(T, fa.dc, cls, valid ? e.x : 0ull, valid, kFullMask, dec);
-                    gn = gain_to_float(gbits);
-                    expand_bf16(dec.d, gn, w);
-                    patch_id8_bf16(dec, gn, w);
-                } else {
-                    Decoded dec{};
-                    const uint32_t cls = decode_sorted_entry(fa, T, I, valid, dec);
-                    if (!kSg) gn = gain_to_float(gbits);
-                    if (kSg && valid) {
-                        const float scale = sg.row_scale ? __ldg(sg.row_scale + row) : 1.f;
-                        gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + (uint32_t)(field >> fa.L.W))),
-                                       __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
-                    }
-                    expand_bf16(dec, gn, w);
+                Decoded dec{};
+                const uint32_t cls = decode_sorted_entry(fa, T, I, valid, dec);
+                if (!kSg) gn = gain_to_float(gbits);
+                if (kSg && valid) {
+                    const float scale = sg.row_scale ? __ldg(sg.row_scale + row) : 1.f;
+                    gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + (uint32_t)(field >> fa.L.W))),
+                                   __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
                 }
+                expand_bf16(dec, gn, w);
                 // the previous MMAs read the buffers: wait for them only now, with the first chunk already unranked
                 if (q == 0) {
                     if (uses > 0 && !mbar_wait(bar_free, (uses - 1u) & 1u)) timeout = true;
@@ -675,7 +536,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga,
                  int b_double, const __grid_constant__ CUtensorMap xmap)
 {
-    static_assert(!(kStored && kBig && kSg), "no shape-gain form for the codes with tables in global memory");
+    static_assert(!(kStored && kBig), "the stored streams of codes with tables in global memory go to gemm_team_kernel");
     extern __shared__ __align__(1024) uint8_t smem_1k[];
     uint8_t* const smem = smem_1k;
     const uint32_t img_bytes = fa.image_bytes;
@@ -780,7 +641,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
             if (kStored) raw = stored_of(tk, in); else e = entry_of(tk);
             // sorted 96-bit entries name their class: its record is requested while the previous chunk is still being expanded
             uint4 rec0 = make_uint4(0u, 0u, 0u, 0u), rec1 = rec0;
-            if (kBig && !kStored) big_load_record(fa.dc, (int)((uint32_t)(e.y >> 8) & 0xffffffu), !(e.y >> 63), rec0, rec1);
+            if (kBig) big_load_record(fa.dc, (int)((uint32_t)(e.y >> 8) & 0xffffffu), !(e.y >> 63), rec0, rec1);
             while (tk < n_tickets) {
                 uint32_t tk_next = 0;
                 if (lane == 0) tk_next = atomicAdd(ticket, 1u);
@@ -793,38 +654,25 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                     uint64_t lo, hi;
                     field_value(raw, wbits, lo, hi);
                     const unsigned long long pos = (tk & 31u) * 32u + lane;
-                    e = kBig ? make_ulonglong2(lo, (in ? hi : kBigNoBlock) | pos << 32)
-                             : make_ulonglong2((in ? lo : kSortIndexMask) | pos << 48, 0ull);
+                    e = make_ulonglong2((in ? lo : kSortIndexMask) | pos << 48, 0ull);
                 }
                 const uint32_t j = tk >> 5, gd = g_base + j, b = gd & 1u;
                 const int d = d_begin + (int)j;
                 const uint64_t field = e.x & kSortIndexMask;
                 const uint64_t I = kSg ? field & ((1ull << fa.L.W) - 1ull) : field;     // shape-gain form: gain index above the shape index
                 const uint32_t pos = kBig ? (uint32_t)(e.y >> 32) & 1023u : (uint32_t)(e.x >> 48);
-                bool valid = kBig ? !(e.y >> 63) : (field != kSortIndexMask && I < fa.n_points);
-                if (kStored && kBig && valid) {                               // the stored index may be out of range: count it, treat it as no block
-                    const uint64_t hi = e.y & 0xffull;
-                    valid = hi < fa.dc.n_hi || (hi == fa.dc.n_hi && e.x < fa.dc.n_lo);
-                    if (!valid) atomicAdd(fa.bad_index, 1ull);
-                }
+                const bool valid = kBig ? !(e.y >> 63) : (field != kSortIndexMask && I < fa.n_points);
                 const uint32_t r = pos >> 3, c = pos & 7u;
                 uint16_t gbits = 0;
                 if (!kSg && valid) gbits = ldg_u16_here(gain_tile + (r * bpr + (uint32_t)d * kDomBlocks + c));
                 float gn = 0.f;                                               // the gain is converted once the block is unranked
                 uint32_t w[12];
                 if (kBig) {
-                    int cls = 0;
-                    uint64_t local = 0;
                     DecodedBig dec{};
-                    if (kStored) {
-                        if (valid) cls = big_find_class(fa.dc, e.x, e.y & 0xffull, local);
-                        big_decode_planes(T, fa.dc, cls, local, valid, kFullMask, dec);
-                    } else {
-                        big_decode_record(T, rec0, rec1, valid ? e.x : 0ull, valid, kFullMask, dec);
-                        // the next chunk's entries were requested a whole chunk ago: they are here, and their records have the
-                        // rest of this iteration to arrive
-                        big_load_record(fa.dc, (int)((uint32_t)(e_next.y >> 8) & 0xffffffu), !(e_next.y >> 63), rec0, rec1);
-                    }
+                    big_decode_record(T, rec0, rec1, valid ? e.x : 0ull, valid, kFullMask, dec);
+                    // the next chunk's entries were requested a whole chunk ago: they are here, and their records have the
+                    // rest of this iteration to arrive
+                    big_load_record(fa.dc, (int)((uint32_t)(e_next.y >> 8) & 0xffffffu), !(e_next.y >> 63), rec0, rec1);
                     gn = gain_to_float(gbits);
                     expand_bf16(dec.d, gn, w);
                     patch_id8_bf16(dec, gn, w);

@@ -185,7 +185,7 @@ bool order_args(const llvq_ctx* ctx, int gain_bits, OrderArgs* oa)
     const size_t ncls = ctx->host.desc.size();
     if (!ctx->fast) {
         oa->words = 288;                                     // 128 shapes x 2 and "no block"
-        return gain_bits == 0 && ctx->host.W > 64 && ctx->host.W <= 72 && ncls <= (1u << 17);
+        return gain_bits == 0 && ncls <= (1u << 17);
     }
     if (!ctx->d_sort_rank || ncls < 64 || ncls > 1023 || ctx->host.W + gain_bits > 64) return false;
     auto bits = [](uint64_t v) { uint32_t b = 0; while (v >> b) ++b; return b; };
