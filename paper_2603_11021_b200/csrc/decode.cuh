@@ -24,9 +24,6 @@ struct DevCode {
     int W;
 };
 
-// A decoded point: 24 signed bytes, coordinate i in byte (i & 3) of word (i >> 2).
-struct Point { uint32_t w[6]; };
-
 // ---- S1: bit unpack --------------------------------------------------------
 // Field b occupies stream bits [b*W, (b+1)*W).  Reads only the 32-bit words the field touches.
 __device__ __forceinline__ void load_index(const uint32_t* __restrict__ s, uint64_t b, int W, uint64_t& lo, uint64_t& hi)
@@ -59,28 +56,6 @@ __device__ __forceinline__ uint64_t load_field(const uint32_t* __restrict__ stre
     const uint32_t w2 = last > 64 ? __ldg(p + 2) : 0u;
     uint64_t v = (((uint64_t)w1 << 32) | w0) >> sh;
     if (sh) v |= (uint64_t)w2 << (64 - sh);
-    return W < 64 ? v & ((1ull << W) - 1) : v;
-}
-
-// The same in two steps, for a caller that requests the words well before it needs the field: the words as they are
-// (x = words 0-1, y = word 2 | bit offset << 32), and the field from them.
-__device__ __forceinline__ ulonglong2 load_field_words(const uint32_t* __restrict__ stream, uint64_t b, int W)
-{
-    const uint64_t bp = b * (uint64_t)W;
-    const uint32_t* p = stream + (bp >> 5);
-    const int sh = (int)(bp & 31);
-    const int last = sh + W;
-    const uint32_t w0 = __ldg(p);
-    const uint32_t w1 = last > 32 ? __ldg(p + 1) : 0u;
-    const uint32_t w2 = last > 64 ? __ldg(p + 2) : 0u;
-    return make_ulonglong2(((unsigned long long)w1 << 32) | w0, (unsigned long long)w2 | (unsigned long long)sh << 32);
-}
-
-__device__ __forceinline__ uint64_t field_of_words(ulonglong2 w, int W)
-{
-    const int sh = (int)(w.y >> 32);
-    uint64_t v = w.x >> sh;
-    if (sh) v |= (w.y & 0xffffffffull) << (64 - sh);
     return W < 64 ? v & ((1ull << W) - 1) : v;
 }
 
@@ -133,35 +108,6 @@ __device__ __forceinline__ void field_value(const RawField<kBig>& f, int W, uint
         else if (W < 64) lo &= (1ull << W) - 1ull;
     } else if (W < 64) {
         lo &= (1ull << W) - 1ull;
-    }
-}
-
-// q = p / d, r = p % d with magic = floor((2^64 - 1) / d): the estimate is at most one too small.
-__device__ __forceinline__ void divmod_magic(uint64_t p, uint32_t d, uint64_t magic, uint64_t& q, uint32_t& r)
-{
-    q = __umul64hi(p, magic);
-    uint64_t rem = p - q * d;
-    if (rem >= d) { rem -= d; ++q; }
-    r = (uint32_t)rem;
-}
-
-// 4 mask bits -> 4 bytes holding 0 or 1.
-__device__ __forceinline__ uint32_t spread4(uint32_t nib) { return (nib * 0x00204081u) & 0x01010101u; }
-
-// Write absolute value `val` at the positions of `mask` (positions not yet written).
-__device__ __forceinline__ void place_value(Point& pt, uint32_t mask, uint32_t val)
-{
-#pragma unroll
-    for (int i = 0; i < 6; ++i) pt.w[i] += spread4((mask >> (4 * i)) & 15u) * val;
-}
-
-// Negate the coordinates at the positions of `neg` (never zero coordinates).
-__device__ __forceinline__ void negate_at(Point& pt, uint32_t neg)
-{
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        const uint32_t sm = spread4((neg >> (4 * i)) & 15u);
-        pt.w[i] = (pt.w[i] ^ (sm * 0xFFu)) + sm;
     }
 }
 

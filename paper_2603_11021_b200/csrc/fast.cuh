@@ -369,8 +369,7 @@ __device__ __forceinline__ void expand_bytes(const Decoded& d, uint32_t out[6])
 // values per class) the upper half of the value table is not formed and the sign takes its place in the selectors: ids 4..7 are
 // the negated values then.
 // The bit planes become selectors by masks and shifts alone because of where the coordinates lie in them (coords_of): 62 instructions
-// with the
-// products; with bit i = coordinate i the planes were spread arithmetically, 122 instructions (three-layer step 93.8 -> 87.7 us).
+// with the products; with bit i = coordinate i the planes were spread arithmetically, 122 instructions (three-layer step 93.8 -> 87.7 us).
 __device__ __forceinline__ void expand_bf16(const Decoded& d, float gain, uint32_t w[12])
 {
     // bf16(gain * a) for the value ids; float(a) by the 2^23 trick (a <= 28)

@@ -98,7 +98,6 @@ namespace llvq {
 constexpr int kBigBucketBits = 20;     // buckets of the class lookup of codes with class tables in global memory (4 MB, in L2): the bisection between a bucket's first
                                        // and last class takes 1.4 steps per warp of the 72-bit code (2^16 buckets: 4.4); some buckets hold thousands of classes
 constexpr int kFastMaxLevels = 4;      // unranking steps per class on the fast path
-constexpr int kFastDescWords = 20;     // words of a class descriptor that carry data
 constexpr int kFastDescValsOdd = 18;   // words 18, 19: absolute value of id 0..7 in the numbering of the odd-only decoder form
 constexpr int kFastDescRnorm = 16;     // word holding 1 / sqrt(16 m) as binary32
 constexpr int kFastDescMagic0 = 17;    // word holding floor(2^32 / radix) of level 0 (used when the arrangement rank fits 32 bits)
