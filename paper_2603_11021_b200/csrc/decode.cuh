@@ -112,17 +112,6 @@ __device__ __forceinline__ void field_value(const RawField<kBig>& f, int W, uint
 }
 
 // ---- S7: gain ---------------------------------------------------------------
-// bf16_rn(float(gain) * float(x)): the product is exact in binary32, one rounding.
-__device__ __forceinline__ float coord(const Point& pt, int i)
-{
-    return (float)(int)(int8_t)(pt.w[i >> 2] >> (8 * (i & 3)));
-}
-
-__device__ __forceinline__ __nv_bfloat16 dequant(float gain, const Point& pt, int i)
-{
-    return __float2bfloat16_rn(gain * coord(pt, i));
-}
-
 // A 16-bit read-only load that stays where it is written among the other volatile statements (the decoders' table
 // reads): issued before a block is unranked, its result is first used when the weights are formed.
 __device__ __forceinline__ uint16_t ldg_u16_here(const uint16_t* p)
