@@ -3,16 +3,30 @@
 
 namespace {
 
+// The kernels that unrank a stream block by block deal it out in chunks of 32 blocks, one per warp of the whole grid at a time, the warps
+// of one number on all SMs before those of the next: whatever is left of the last round lies evenly over the SMs, and a short stream
+// reaches all of them.  (In tiles of 1024 blocks per CTA, 4096 x 4096 left 5 tiles to some SMs and 4 to others: 48 bits 25.6 -> 24.2
+// us, 72 bits 41.7 -> 40.5 us; 512 x 1024: 7.2 -> 5.1 and 10.2 -> 6.9 us; 8192 x 8192: 85.6 -> 83.8 us and no change.)
+__device__ __forceinline__ uint32_t first_chunk() { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+
+// How many chunks this warp takes: first_chunk() and every (32 gridDim.x)-th behind it.
+__device__ __forceinline__ uint32_t chunk_count(uint64_t nblocks)
+{
+    const uint64_t chunks = (nblocks + 31u) >> 5;
+    const uint32_t step = gridDim.x * (kFastThreads / 32);
+    return first_chunk() < chunks ? (uint32_t)((chunks - first_chunk() + step - 1u) / step) : 0u;
+}
+
+unsigned chunk_grid(const llvq_ctx* ctx, uint64_t nblocks) { return (unsigned)std::min<uint64_t>((nblocks + 31) / 32, (uint64_t)ctx->sm_count); }
 
 template <bool kBig>
 __global__ void __launch_bounds__(kFastThreads, 1)
 decode_blocks_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, uint64_t nblocks, uint2* __restrict__ out)
 {
     FAST_PROLOGUE();
-    const uint64_t ntiles = (nblocks + kFastThreads - 1) / kFastThreads;
-    uint64_t b = (uint64_t)blockIdx.x * kFastThreads + threadIdx.x;
+    uint64_t b = (uint64_t)first_chunk() * 32u + (threadIdx.x & 31u);
     RawField<kBig> raw = request_field<kBig>(stream, b, fa.dc.W, b < nblocks);
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (uint32_t left = chunk_count(nblocks); left; --left) {        // whole warps: the decoders vote
         const bool in = b < nblocks;
         const uint64_t b_next = b + (uint64_t)gridDim.x * kFastThreads;
         RawField<kBig> raw_next = request_field<kBig>(stream, b_next, fa.dc.W, b_next < nblocks);
@@ -95,19 +109,18 @@ dequant_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint
                     int64_t rows, int64_t cols, RowWalk walk, __nv_bfloat16* __restrict__ out, int64_t ld)
 {
     FAST_PROLOGUE();
+    const uint32_t b0 = first_chunk() * 32u + (threadIdx.x & 31u);
     uint32_t r = 0, cb = 0;
     if (walk.bpr) {
-        const uint32_t b0 = blockIdx.x * kFastThreads + threadIdx.x;
         r = __umulhi(b0, walk.bpr_magic);
         cb = b0 - r * walk.bpr;
         if (cb >= walk.bpr) { cb -= walk.bpr; ++r; }
     }
-    const uint64_t ntiles = (nblocks + kFastThreads - 1) / kFastThreads;
     const uint64_t total = (uint64_t)rows * (uint64_t)cols;
     const int wbits = fa.dc.W + (kSg ? sg.bits : 0);
-    uint64_t b = (uint64_t)blockIdx.x * kFastThreads + threadIdx.x, b_next = b;
+    uint64_t b = b0, b_next = b;
     RawBlock<kBig> raw_next = request_block<kBig>(stream, kSg ? nullptr : gain, wbits, b, b < nblocks);
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (uint32_t chunks = chunk_count(nblocks); chunks; --chunks) {  // whole warps: the decoders vote
         // a block's words are requested while the one before it is unranked
         RawBlock<kBig> raw = raw_next;
         use_field_from_here(raw.field);
@@ -117,7 +130,7 @@ dequant_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint
         raw_next = request_block<kBig>(stream, kSg ? nullptr : gain, wbits, b_next, b_next < nblocks);
         uint32_t w[12];
         if constexpr (kSg) block_pairs_sg(fa, T, raw.field, sg, in ? (int64_t)r : 0, in, w);   // ROWWISE only
-        else block_pairs<kBig>(fa, T, raw, in, w);                    // whole warp: the decoders vote
+        else block_pairs<kBig>(fa, T, raw, in, w);
         __nv_bfloat16* dst;
         int64_t left;
         if (walk.bpr == 0) { dst = out + b * 24; left = (int64_t)(total - b * 24); }
@@ -338,8 +351,7 @@ int llvq_decode_blocks(const llvq_ctx* ctx, const void* d_idx, uint64_t nblocks,
     // a warp of these kernels holds 32 unrelated classes: the table of small subsets (FastLayout::sub3) would almost never be taken
     // by all lanes of a step, and asking whether it can be costs more than it returns (measured), so the image goes without it
     const size_t smem = ctx->fl.total + 16;
-    const uint64_t tiles = (nblocks + kFastThreads - 1) / kFastThreads;
-    const unsigned g = (unsigned)std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count);
+    const unsigned g = chunk_grid(ctx, nblocks);
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (ctx->fast) {
         if (!set_smem<decode_blocks_fast_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
@@ -371,8 +383,7 @@ int llvq_dequant_matrix(const llvq_ctx* ctx, const void* d_idx, const uint16_t* 
     const uint64_t nblocks = layout == LLVQ_LAYOUT_FLAT ? ((uint64_t)rows * (uint64_t)cols + 23) / 24 : (uint64_t)rows * (uint64_t)bpr;
     // (image without the table of small subsets, as in llvq_decode_blocks)
     const size_t smem = ctx->fl.total + 16;
-    const uint64_t tiles = (nblocks + kFastThreads - 1) / kFastThreads;
-    const unsigned g = (unsigned)std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count);
+    const unsigned g = chunk_grid(ctx, nblocks);
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(d_w_bf16);
     if (ctx->fast) {
@@ -408,12 +419,11 @@ int llvq_dequant_matrix_sg(const llvq_ctx* ctx, const void* d_fields, int gain_b
     const uint64_t nblocks = (uint64_t)rows * (uint64_t)bpr;
     // (image without the table of small subsets, as in llvq_decode_blocks)
     const size_t smem = ctx->fl.total + 16;
-    const uint64_t tiles = (nblocks + kFastThreads - 1) / kFastThreads;
-    const unsigned g = (unsigned)std::min<uint64_t>(tiles, (uint64_t)ctx->sm_count);
+    const unsigned g = chunk_grid(ctx, nblocks);
     if (!set_smem<dequant_fast_kernel<false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
-    dequant_fast_kernel<false, true><<<g, kFastThreads, smem, (cudaStream_t)stream>>>(
-        fast_args(ctx, false), static_cast<const uint32_t*>(d_fields), nullptr, SgArgs{d_codebook_f32, d_row_scale_f32, gain_bits},
-        nblocks, rows, cols, row_walk(bpr, g), reinterpret_cast<__nv_bfloat16*>(d_w_bf16), ld);
+    if (launch_pdl(dequant_fast_kernel<false, true>, g, (unsigned)kFastThreads, smem, (cudaStream_t)stream, fast_args(ctx, false), static_cast<const uint32_t*>(d_fields),
+                   static_cast<const uint16_t*>(nullptr), SgArgs{d_codebook_f32, d_row_scale_f32, gain_bits}, nblocks, rows, cols, row_walk(bpr, g),
+                   reinterpret_cast<__nv_bfloat16*>(d_w_bf16), ld) != cudaSuccess) return LLVQ_ECUDA;
     return launch_status();
 }
 
