@@ -832,15 +832,15 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
         bool fresh = true;
         for (uint32_t d = d_begin + (uint32_t)team; d < d_end; d += kGemmTeams, ++mine) {
             // ---- order
-            OrderSpot o;
+            OrderSpot<uint64_t> o;
+            o.b0 = 0;
             o.row = rt * kGemmRows + (tid >> 3);
-            o.b0 = (uint64_t)rt * kGemmRows * ga.bpr;
-            o.b = (tid >> 3) * bpr + d * kDomBlocks + (tid & 7u);
+            o.b = (uint64_t)o.row * bpr + (d * kDomBlocks + (tid & 7u));
             o.pos = tid;
             o.there = d * kDomBlocks + (tid & 7u) < bpr;
             order_piece<kBig, kSg, kGemmTeamThreads>(fa, T, sg, oa, stream, hists + ((uint32_t)team * 2u + (mine & 1u)) * oa.words,
                                                hists + ((uint32_t)team * 2u + ((mine & 1u) ^ 1u)) * oa.words, ent, ent2, team, tid, o, (uint32_t)ga.n_out,
-                                               64u * bpr, 64u, (uint32_t)kGemmTeamThreads, [&] {
+                                               (uint64_t)bpr * 64u, 64u, (uint32_t)kGemmTeamThreads, [&] {
                 // the entries go over what the previous MMAs read
                 if (mine > 0 && !mbar_wait(bar_free + team, (mine - 1u) & 1u)) timeout = true;
                 if (x_double && tid == 0) request_x(smem_u32(x_mine), &xmap, (int)d, ga.npad, bar_x + team);

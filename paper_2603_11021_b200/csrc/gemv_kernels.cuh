@@ -681,7 +681,7 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
             const uint32_t narrow = nchunks <= 8u ? 2u : nchunks <= 16u ? 1u : 0u, c = tid & (127u >> narrow), r = tid >> (7u - narrow);
             uint32_t kq;
             const uint32_t rg = split_row(sp, u0 + (c >> 2), kq);
-            OrderSpot o;
+            OrderSpot<uint32_t> o;
             o.row = rg * kGemvGroupRows + r;
             o.b0 = (uint64_t)rg0 * kGemvGroupRows * bpr;
             o.b = (o.row - rg0 * kGemvGroupRows) * bpr + kq * 4u + (c & 3u);

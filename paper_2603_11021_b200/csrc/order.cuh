@@ -19,10 +19,14 @@ struct OrderArgs {
 
 // Where the blocks of a thread lie in a piece: numbers b0 + b, b0 + b + b_step, .. in the stream, rows row, row + row_step, .. (there
 // are n_out), position codes pos, pos + pos_step, ..; none of them where the column or the unit does not exist (!there).
-// b counts from the first block of a run of rows short enough for its bits to be counted in 32 bits.
+// Count: what the bits of b and the steps are counted in.  Nothing limits the length of a row of the batched products: 64 bits, with
+// b0 = 0.  A row of the GEMV has its slice of x in shared memory (192 bytes per 4 blocks of 227 KB), and the at most 1024 + 32
+// rows of a pass then hold less than 2^23 blocks: 32 bits behind b0, their first block (11008 x 4096: 53.3 us, with 64 bits 53.4).
+template <typename Count>
 struct OrderSpot {
     uint64_t b0;
-    uint32_t b, row, pos;
+    Count b;
+    uint32_t row, pos;
     bool there;
 };
 
@@ -32,10 +36,10 @@ __device__ __forceinline__ void team_barrier(int team, int threads) { asm volati
 // histogram (zero on entry) and the next one's (zeroed here).  The entries go to ent (with kBig the class-local index) and, with
 // kBig, ent2 (class | position << 17, bit 31 = no block); on return the piece is complete.
 // before_write(): what has to be awaited before ent may be written.
-template <bool kBig, bool kSg, int kThreads, typename Before>
+template <bool kBig, bool kSg, int kThreads, typename Count, typename Before>
 __device__ __forceinline__ void order_piece(const FastArgs& fa, const FastSmem& T, const SgArgs& sg, const OrderArgs& oa, const uint32_t* __restrict__ stream,
                                             uint32_t* hist, uint32_t* hist_next, unsigned long long* ent, uint32_t* ent2, int team, uint32_t tid,
-                                            const OrderSpot& o, uint32_t n_out, uint32_t b_step, uint32_t row_step, uint32_t pos_step, Before before_write)
+                                            const OrderSpot<Count>& o, uint32_t n_out, Count b_step, uint32_t row_step, uint32_t pos_step, Before before_write)
 {
     constexpr int kEach = kOrderBlocks / kThreads;
     const uint32_t lane = tid & 31u;
@@ -47,12 +51,13 @@ __device__ __forceinline__ void order_piece(const FastArgs& fa, const FastSmem& 
         RawField<kBig> raw[kEach];
         const uint64_t bits0 = o.b0 * (uint64_t)wbits;
         const uint32_t* base = stream + (bits0 >> 5);
-        const uint32_t bits = o.b * (uint32_t)wbits + ((uint32_t)bits0 & 31u), step = b_step * (uint32_t)wbits;
+        const Count bits = o.b * (Count)wbits + ((uint32_t)bits0 & 31u), step = b_step * (Count)wbits;
         uint32_t in = 0;
 #pragma unroll
         for (int q = 0; q < kEach; ++q) {
             const bool there = o.there && o.row + (uint32_t)q * row_step < n_out;
-            raw[q] = request_field_at<kBig>(base, bits + (uint32_t)q * step, wbits, there);
+            const Count at = bits + (uint32_t)q * step;
+            raw[q] = request_field_at<kBig>(base + (at >> 5), (uint32_t)at & 31u, wbits, there);
             in |= (uint32_t)there << q;
         }
         if constexpr (kBig) {
