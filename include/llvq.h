@@ -235,6 +235,7 @@ int llvq_gemv_sorted_sg(const llvq_ctx* ctx, const void* d_sorted, int gain_bits
  * fed to the tensor cores, accumulation in binary32.
  * d_x_bf16: device, [batch][k_in] bf16 bits, 16-byte aligned, k_in % 8 == 0.
  * d_y_bf16: device, [batch][n_out] bf16 bits.  1 <= batch <= 64.
+ * Codes whose class tables stay in global memory, and the sorted layouts: k_in <= 2^30 (LLVQ_EUNSUPPORTED beyond).
  */
 int llvq_gemm_small_batch(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f16,
                           int64_t n_out, int64_t k_in, const uint16_t* d_x_bf16,

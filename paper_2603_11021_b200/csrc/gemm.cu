@@ -9,6 +9,10 @@ namespace {
 #include "gemv_kernels.cuh"
 #include "gemm_kernels.cuh"
 
+// The kernels that take X by TMA name its columns by signed 32-bit coordinates (past 2^31 they wrapped, and the copy faulted); up to here a
+// box's offset in bytes stays below 2^31 too.  Longer rows of a stored stream go to gemm_kernel, which reads X by plain loads.
+constexpr int64_t kMaxMapColumns = 1ll << 30;
+
 // The tensor map of X [batch][k_in] bf16 (16-byte aligned, k_in a multiple of 8): boxes of 64 columns x npad rows, 128-byte swizzle.
 bool make_x_map(const uint16_t* d_x, int64_t k_in, int batch, int npad, CUtensorMap* map)
 {
@@ -43,6 +47,7 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
                         const uint16_t* d_x_bf16, int batch, uint16_t* d_y_bf16, float* scratch, uint32_t* counters, void* stream,
                         const YOut* yo = nullptr, int64_t y_ld = 0, const SgArgs* sg = nullptr, int y_f32 = 0)
 {
+    if (k_in > kMaxMapColumns) return LLVQ_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     GemmArgs ga;
@@ -100,6 +105,8 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
                 const SgArgs* sg = nullptr, const YOut* yo = nullptr, int64_t y_ld = 0)
 {
     if (n_out == 0) return LLVQ_OK;
+    const bool mapped = k_in <= kMaxMapColumns;
+    if (!mapped && !ctx->fast) return LLVQ_EUNSUPPORTED;  // gemm_kernel reads class tables in shared memory
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
@@ -132,11 +139,11 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (yo && sg) return LLVQ_EUNSUPPORTED;              // row-sharded: stored-gain form only
     CUtensorMap xmap;
-    if (!make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
+    if (mapped && !make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
     // codes with many classes (a warp of 32 unrelated blocks is what costs there): the kernel whose two teams order their domains; it
     // fits for every code with class tables in global memory
     OrderArgs oa;
-    if (order_args(ctx, sg ? sg->bits : 0, &oa)) {
+    if (mapped && order_args(ctx, sg ? sg->bits : 0, &oa)) {
         const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_sets = (size_t)kGemmTeams * kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2, hists = (size_t)kGemmTeams * 2 * oa.words * 4;
         // (codes that look their classes up in global memory keep a larger L1 cache below 200 KB of shared memory: 8192 x 8192, 72 bits, batch
@@ -164,7 +171,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             return launch_status();
         }
     }
-    {
+    if (mapped) {
         // the kernel without a block barrier (see gemm_pipe_kernel), if its buffers fit
         const size_t head = (img + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2;

@@ -40,3 +40,32 @@ def test_rows_of_a_tile_beyond_2_to_the_32_bits(code):
     share = k_in // torch.cuda.get_device_properties(0).multi_processor_count
     assert gemm_error(y[:, first:].float().cpu().numpy(), want, share) <= TOL_BF16_OUT
     assert P.llvq_last_error(ctx) == (0, 0)
+
+
+def test_columns_beyond_2_to_the_31():
+    # the column coordinates of a TMA copy are signed 32-bit numbers
+    import paper_2603_11021_b200 as P
+    k_in = 2 ** 31 + 4800
+    nblocks = -(-k_in // 24)
+    x = torch.zeros((1, k_in), dtype=torch.bfloat16, device="cuda")
+    x[0, 0], x[0, 24 * (nblocks - 100)] = 3.0, 5.0
+    gain = torch.full((nblocks,), 0.5, dtype=torch.half, device="cuda")
+    for code in [(2, 2), (2, 8)]:
+        ctx = P.Context(*code, device=0)
+        stream = torch.zeros(ctx.index_bytes(nblocks), dtype=torch.uint8, device="cuda")      # field 0: the point (4, 4, 0, ..)
+        assert P.llvq_gemm_small_batch(ctx, stream, gain, 1, k_in, x).item() == 16.0
+        assert P.llvq_last_error(ctx) == (0, 0)
+
+
+def test_rows_too_long_for_the_kernels_that_copy_x_by_tma_are_refused():
+    # refused by the size alone, before anything is launched
+    import paper_2603_11021_b200 as P
+    k_in, some = 2 ** 30 + 8, torch.zeros(64, device="cuda").data_ptr()
+    L = P.load_library()
+    for code in [(2, 2), (2, 8), (2, 53)]:
+        ctx = P.Context(*code, device=0)
+        args = (ctx._h, some, some, 1, k_in, some, 1, some, None)
+        assert L.llvq_gemm_small_batch_sorted(*args) == 3
+        if code == (2, 53):
+            assert L.llvq_gemm_small_batch(*args) == 3
+            assert L.llvq_gemv_sorted(ctx._h, some, some, 1, k_in, some, some, P.LLVQ_F32, None) == 3
