@@ -56,7 +56,7 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
         ga.y = static_cast<uint16_t*>(yo->y); ga.y_ld = y_ld; ga.shard = static_cast<const YOut*>(ctx->d_shard);
         put_shard_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(*yo, static_cast<YOut*>(ctx->d_shard));   // by value: safe under stream capture
     }
-    ga.n_out = n_out; ga.k_in = k_in; ga.bpr = (k_in + 23) / 24;
+    ga.n_out = n_out; ga.k_in = k_in; ga.bpr = (k_in + 23) / 24; ga.gain_row = (uint32_t)(2 * ga.bpr);
     ga.batch = batch; ga.npad = (batch + 15) / 16 * 16;
     ga.nstages = (int)((ga.bpr + kDomBlocks - 1) / kDomBlocks);              // domains per row tile
     ga.x = d_x_bf16; ga.scratch = scratch; ga.counters = counters;
@@ -117,7 +117,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
         ga.y = static_cast<uint16_t*>(yo->y); ga.y_ld = y_ld; ga.shard = static_cast<const YOut*>(ctx->d_shard);
         put_shard_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(*yo, static_cast<YOut*>(ctx->d_shard));   // by value: safe under stream capture
     }
-    ga.n_out = n_out; ga.k_in = k_in; ga.bpr = (k_in + 23) / 24;
+    ga.n_out = n_out; ga.k_in = k_in; ga.bpr = (k_in + 23) / 24; ga.gain_row = (uint32_t)(2 * ga.bpr);
     ga.batch = batch; ga.npad = (batch + 15) / 16 * 16;
     ga.nstages = (int)((ga.bpr + kStageBlocks - 1) / kStageBlocks);
     ga.x = d_x_bf16; ga.scratch = scratch; ga.counters = counters;
@@ -141,9 +141,10 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     CUtensorMap xmap;
     if (mapped && !make_x_map(d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
     // codes with many classes (a warp of 32 unrelated blocks is what costs there): the kernel whose two teams order their domains; it
-    // fits for every code with class tables in global memory
+    // fits for every code with class tables in global memory.  (For the other codes it counts the blocks of a row tile in 32 bits: 8192 x 8192
+    // batch 16: 102.0 us, with 64 bits 102.4)
     OrderArgs oa;
-    if (mapped && order_args(ctx, sg ? sg->bits : 0, &oa)) {
+    if (mapped && (!ctx->fast || kGemmRows * ga.bpr <= 1ll << 32) && order_args(ctx, sg ? sg->bits : 0, &oa)) {
         const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_sets = (size_t)kGemmTeams * kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2, hists = (size_t)kGemmTeams * 2 * oa.words * 4;
         // (codes that look their classes up in global memory keep a larger L1 cache below 200 KB of shared memory: 8192 x 8192, 72 bits, batch

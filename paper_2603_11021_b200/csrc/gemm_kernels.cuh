@@ -25,6 +25,7 @@ struct GemmArgs {
     int batch, npad;
     int nstages, split;        // gemm_kernel: 96-column stages and pieces of K
     Split sp;                  // the kernels on domains: which CTA works on which
+    uint32_t gain_row;         // bytes of gains per row of blocks (below 2^32: k_in <= kMaxMapColumns)
     const uint16_t* x;
     uint16_t* y;               // Y [batch][y_ld] bf16, at the first row of this launch's rows
     int64_t y_ld;
@@ -53,6 +54,12 @@ __device__ __forceinline__ void gemm_store(const GemmArgs& ga, int n, int64_t or
         const int np = ga.shard->n_peer;
         for (int p = 0; p < np; ++p) reinterpret_cast<__nv_bfloat16*>(ga.shard->peer[p])[at] = h;
     }
+}
+
+// Gain of the block in row r of a row tile and column block cb.  A tile may hold more than 2^32 blocks.
+__device__ __forceinline__ const uint16_t* gain_at(const GemmArgs& ga, const uint16_t* gain_tile, uint32_t r, uint32_t cb)
+{
+    return reinterpret_cast<const uint16_t*>(reinterpret_cast<const uint8_t*>(gain_tile + cb) + (uint64_t)r * ga.gain_row);
 }
 
 __device__ __forceinline__ void group_barrier(int group)
@@ -632,7 +639,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
             auto stored_of = [&](uint32_t t, bool& in) {
                 const uint32_t pos = (t & 31u) * 32u + lane, c0 = ((uint32_t)d_begin + (t >> 5)) * kDomBlocks + (pos & 7u), r0 = pos >> 3;
                 in = t < n_tickets && (int64_t)rt * kGemmRows + r0 < ga.n_out && c0 < bpr;
-                return request_field<kBig>(reinterpret_cast<const uint32_t*>(sorted), (uint64_t)rt * kGemmRows * ga.bpr + (r0 * bpr + c0), wbits, in);
+                return request_field<kBig>(reinterpret_cast<const uint32_t*>(sorted), ((uint64_t)rt * kGemmRows + r0) * bpr + c0, wbits, in);
             };
             uint32_t tk = (uint32_t)warp - 1u;
             ulonglong2 e = no_entry;
@@ -664,7 +671,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 const bool valid = kBig ? !(e.y >> 63) : (field != kSortIndexMask && I < fa.n_points);
                 const uint32_t r = pos >> 3, c = pos & 7u;
                 uint16_t gbits = 0;
-                if (!kSg && valid) gbits = ldg_u16_here(gain_tile + (r * bpr + (uint32_t)d * kDomBlocks + c));
+                if (!kSg && valid) gbits = ldg_u16_here(gain_at(ga, gain_tile, r, (uint32_t)d * kDomBlocks + c));
                 float gn = 0.f;                                               // the gain is converted once the block is unranked
                 uint32_t w[12];
                 if (kBig) {
@@ -869,7 +876,7 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
                 else { const uint32_t y = q == 0 ? e2[0] : e2[1]; b.valid = !(y >> 31); b.pos = (y >> 17) & 1023u; }
                 const uint32_t r = b.pos >> 3, c = b.pos & 7u;
                 uint16_t gbits = 0;
-                if (!kSg && b.valid) gbits = ldg_u16_here(gain_tile + (r * bpr + d * kDomBlocks + c));
+                if (!kSg && b.valid) gbits = ldg_u16_here(kBig ? gain_at(ga, gain_tile, r, d * kDomBlocks + c) : gain_tile + (r * bpr + d * kDomBlocks + c));
                 float gn = 0.f;                                           // the gain is converted once the block is unranked
                 uint32_t w[12];
                 if constexpr (kBig) {

@@ -42,6 +42,28 @@ def test_rows_of_a_tile_beyond_2_to_the_32_bits(code):
     assert P.llvq_last_error(ctx) == (0, 0)
 
 
+def test_gains_of_a_tile_beyond_2_to_the_32_blocks():
+    # field 0 is the point (4, 4, 0, ..), so a row is known from its gains: zero but for the last rows, whose gains lie 2^32 behind those of
+    # row 0.  A code of few classes, one of many, one with class tables in global memory
+    import paper_2603_11021_b200 as P
+    n_out, bpr = 128, 2 ** 32 // 127 // 8 * 8 + 8
+    assert 127 * bpr >= 2 ** 32
+    k_in = 24 * bpr
+    gain = torch.zeros(n_out * bpr, dtype=torch.half, device="cuda")
+    gain[125 * bpr:] = 0.5
+    x = torch.zeros((1, k_in), dtype=torch.bfloat16, device="cuda")
+    x[0, ::24 * 1024] = 1.0                                # whole numbers: exact in binary32 whatever the order of the sums
+    want = 2.0 * x.count_nonzero().item()
+    for code in [(2, 2), (2, 8), (2, 53)]:
+        ctx = P.Context(*code, device=0)
+        stream = torch.zeros(ctx.index_bytes(n_out * bpr), dtype=torch.uint8, device="cuda")
+        y = P.llvq_gemm_small_batch(ctx, stream, gain, n_out, k_in, x).float()
+        assert y[0, 125:].tolist() == pytest.approx([want] * 3, rel=2.0 ** -8), code      # the rounding of the bf16 output
+        assert not y[0, :125].any(), code
+        assert P.llvq_last_error(ctx) == (0, 0)
+        del stream
+
+
 def test_columns_beyond_2_to_the_31():
     # the column coordinates of a TMA copy are signed 32-bit numbers
     import paper_2603_11021_b200 as P
