@@ -657,18 +657,18 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 RawField<kBig> raw_next{};
                 bool in_next = false;
                 if (kStored) raw_next = stored_of(tk_next, in_next); else e_next = entry_of(tk_next);
-                if (kStored) {                                              // this chunk's blocks in the form of the sorted layout's entries
-                    uint64_t lo, hi;
-                    field_value(raw, wbits, lo, hi);
-                    const unsigned long long pos = (tk & 31u) * 32u + lane;
-                    e = make_ulonglong2((in ? lo : kSortIndexMask) | pos << 48, 0ull);
+                if (kStored) {                                              // a field may take all 64 bits: its position is known from the ticket
+                    uint64_t lo, none;
+                    field_value(raw, wbits, lo, none);
+                    e.x = lo;
                 }
                 const uint32_t j = tk >> 5, gd = g_base + j, b = gd & 1u;
                 const int d = d_begin + (int)j;
-                const uint64_t field = e.x & kSortIndexMask;
+                const uint64_t field = kStored ? (uint64_t)e.x : e.x & kSortIndexMask;
                 const uint64_t I = kSg ? field & ((1ull << fa.L.W) - 1ull) : field;     // shape-gain form: gain index above the shape index
-                const uint32_t pos = kBig ? (uint32_t)(e.y >> 32) & 1023u : (uint32_t)(e.x >> 48);
-                const bool valid = kBig ? !(e.y >> 63) : (field != kSortIndexMask && I < fa.n_points);
+                const uint32_t pos = kBig ? (uint32_t)(e.y >> 32) & 1023u : kStored ? (tk & 31u) * 32u + lane : (uint32_t)(e.x >> 48);
+                const bool there = kStored ? in : field != kSortIndexMask;
+                const bool valid = kBig ? !(e.y >> 63) : (there && I < fa.n_points);
                 const uint32_t r = pos >> 3, c = pos & 7u;
                 uint16_t gbits = 0;
                 if (!kSg && valid) gbits = ldg_u16_here(gain_at(ga, gain_tile, r, (uint32_t)d * kDomBlocks + c));
@@ -687,7 +687,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                     Decoded dec{};
                     uint32_t cls;
                     if (kStored) {
-                        if (field != kSortIndexMask && !valid) atomicAdd(fa.bad_index, 1ull);
+                        if (there && !valid) atomicAdd(fa.bad_index, 1ull);
                         uint64_t local = 0;
                         cls = valid ? fast_find_class(T, I, local) : 0u;
                         fast_decode_local<-1>(T, cls, local, valid, kFullMask, dec);
