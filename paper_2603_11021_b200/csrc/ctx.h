@@ -5,6 +5,7 @@
 #include <cstdint>
 
 #include "decode.cuh"
+#include "launch_host.h"
 #include "tables.h"
 
 // Device tables of the encoder (point -> index): present for codes the encoder supports.
@@ -25,6 +26,8 @@ struct llvq_ctx {
     void* d_blob = nullptr;          // one allocation holding every device table
     unsigned long long* d_err = nullptr;
     int sm_count = 0;
+    size_t smem_most = 0;            // shared memory that one block may have on the device
+    mutable llvq::SmemLimits smem_limits;
     float* d_scratch = nullptr;      // split-K accumulation buffer of the small-batch GEMM, kept all-zero between calls
     uint32_t* d_counters = nullptr;  // per row tile arrival counters, kept zero between calls
     void* d_shard = nullptr;         // device copy of the destinations (peers' Y and flags) of the row-sharded GEMM in flight

@@ -536,7 +536,7 @@ int llvq_encode_blocks(const llvq_ctx* ctx, const float* d_v_f32, uint64_t nbloc
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t smem = kEncWarps * sizeof(WarpTables) + sizeof(GolayTrio);
-    if (cudaFuncSetAttribute(encode_search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return LLVQ_ECUDA;
+    if (!allow_smem<encode_search_kernel>(ctx->smem_limits, ctx->smem_most, smem)) return LLVQ_ECUDA;
     PatternSteps steps;
     for (int o = 0; o < 3; ++o)
         for (int j = 0; j < 4; ++j) { steps.lo[o][j] = (ctx->trio.pat[o][j] & 15u) * 8u; steps.hi[o][j] = (uint32_t)(ctx->trio.pat[o][j] >> 4) * 8u; }

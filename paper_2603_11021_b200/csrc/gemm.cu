@@ -81,7 +81,7 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
     if (smem > 227 * 1024 || (!ctx->fast && !pipe)) return LLVQ_EUNSUPPORTED;      // (the pipeline's buffers fit for every code of the second kind)
 #define LLVQ_LAUNCH_DOMAINS(K, LAST)                                                                                          \
     do {                                                                                                                     \
-        if (!set_smem<K>(ctx->device, smem)) return LLVQ_ECUDA;                                                               \
+        if (!set_smem<K>(ctx, smem)) return LLVQ_ECUDA;                                                               \
         if (launch_pdl(K, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx), static_cast<const unsigned long long*>(p), d_gain_f16, \
                        sga, ga, LAST, xmap) != cudaSuccess) return LLVQ_ECUDA;                                                \
     } while (0)
@@ -165,7 +165,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_TEAM(BIG, SG, SH)                                                                                              \
     do {                                                                                                                     \
-        if (!set_smem<gemm_team_kernel<BIG, SG, SH>>(ctx->device, smem_team)) return LLVQ_ECUDA;                                   \
+        if (!set_smem<gemm_team_kernel<BIG, SG, SH>>(ctx, smem_team)) return LLVQ_ECUDA;                                   \
         if (launch_pdl(gemm_team_kernel<BIG, SG, SH>, grid_team, (unsigned)kGemmThreads, smem_team, st, fast_args(ctx, false), idx, oa, d_gain_f16, sga, gt, \
                        x_double, xmap) != cudaSuccess) return LLVQ_ECUDA;                                                     \
     } while (0)
@@ -193,7 +193,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_PIPE_STORED(SG, SH)                                                                                    \
     do {                                                                                                                        \
-        if (!set_smem<gemm_pipe_kernel<false, SG, SH, true>>(ctx->device, smem_pipe)) return LLVQ_ECUDA;                                        \
+        if (!set_smem<gemm_pipe_kernel<false, SG, SH, true>>(ctx, smem_pipe)) return LLVQ_ECUDA;                                        \
         if (launch_pdl(gemm_pipe_kernel<false, SG, SH, true>, grid_pipe, (unsigned)kGemmThreads, smem_pipe, st, fast_args(ctx), words, \
                        d_gain_f16, sga, gp, b_double, xmap) != cudaSuccess) return LLVQ_ECUDA;                                        \
     } while (0)
@@ -206,7 +206,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     }
 #define LLVQ_LAUNCH_STAGES(SG, SH)                                                                                              \
     do {                                                                                                                        \
-        if (!set_smem<gemm_kernel<SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                                \
+        if (!set_smem<gemm_kernel<SG, SH>>(ctx, smem)) return LLVQ_ECUDA;                                                \
         if (launch_pdl(gemm_kernel<SG, SH>, grid, (unsigned)kGemmThreads, smem, st, fast_args(ctx), idx, d_gain_f16, sg ? *sg : SgArgs{}, ga) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
     if (yo) LLVQ_LAUNCH_STAGES(false, true);
@@ -251,7 +251,7 @@ static int sort_blocks_gemm_common(const llvq_ctx* ctx, const void* d_idx, int g
         return launch_status();
     }
     const size_t smem = ctx->fl.total + 16;
-    if (!set_smem<sort_blocks_gemm_kernel>(ctx->device, smem)) return LLVQ_ECUDA;
+    if (!set_smem<sort_blocks_gemm_kernel>(ctx, smem)) return LLVQ_ECUDA;
     sort_blocks_gemm_kernel<<<g, kDomEntries, smem, (cudaStream_t)stream>>>(fast_args(ctx), static_cast<const uint32_t*>(d_idx), ctx->d_sort_rank,
                                                                            gain_bits, n_out, bpr, ndomains, static_cast<unsigned long long*>(d_sorted));
     return launch_status();

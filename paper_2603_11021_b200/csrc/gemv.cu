@@ -111,7 +111,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
         const FastArgs fa = fast_args(ctx, ext_bin);
 #define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
     do {                                                                                                                   \
-        if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx->device, smem_bin)) return LLVQ_ECUDA;                                          \
+        if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx, smem_bin)) return LLVQ_ECUDA;                                          \
         if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
                        bpr, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
@@ -125,7 +125,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
         const FastArgs fa = fast_args(ctx, ext_order);
 #define LLVQ_LAUNCH_ORDER(BF16, SG, SH)                                                                               \
     do {                                                                                                                   \
-        if (!set_smem<gemv_order_kernel<BF16, SG, SH>>(ctx->device, smem_order)) return LLVQ_ECUDA;                   \
+        if (!set_smem<gemv_order_kernel<BF16, SG, SH>>(ctx, smem_order)) return LLVQ_ECUDA;                   \
         if (launch_pdl(gemv_order_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_order, st, fa, idx, oa, d_gain_f16, sga, sp, n_out, k_in, \
                        bpr, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;              \
     } while (0)
@@ -139,7 +139,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const FastArgs fa = fast_args(ctx, ext_direct);
 #define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH)                                                                        \
     do {                                                                                                           \
-        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                               \
+        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH>>(ctx, smem)) return LLVQ_ECUDA;                               \
         if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, sp, per_pass, n_out, k_in, bpr, d_x_bf16, yo, \
                        ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;                         \
     } while (0)
@@ -206,7 +206,7 @@ static int sort_blocks_common(const llvq_ctx* ctx, const void* d_fields, int gai
     const int64_t units = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
     const unsigned g = (unsigned)std::min<int64_t>(units, ctx->sm_count);
     const size_t smem = ctx->fl.total + 16;
-    if (!set_smem<sort_blocks_kernel>(ctx->device, smem)) return LLVQ_ECUDA;
+    if (!set_smem<sort_blocks_kernel>(ctx, smem)) return LLVQ_ECUDA;
     sort_blocks_kernel<<<g, kSortThreads, smem, (cudaStream_t)stream>>>(fast_args(ctx), static_cast<const uint32_t*>(d_fields), ctx->d_sort_rank, gain_bits,
                                                                        make_split(units, nq, g), n_out, bpr, static_cast<unsigned long long*>(d_sorted));
     return launch_status();
@@ -245,7 +245,7 @@ static int gemv_sorted_common(const llvq_ctx* ctx, const void* d_sorted, const u
     const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_SORTED(BF16, SG, SH)                                                                                \
     do {                                                                                                                \
-        if (!set_smem<gemv_sorted_kernel<BF16, SG, SH>>(ctx->device, smem)) return LLVQ_ECUDA;                                        \
+        if (!set_smem<gemv_sorted_kernel<BF16, SG, SH>>(ctx, smem)) return LLVQ_ECUDA;                                        \
         if (launch_pdl(gemv_sorted_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem, st, fa, sp, d_gain_f16, sga, split, n_out, k_in, bpr, \
                        acc_floats, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;          \
     } while (0)
@@ -349,10 +349,10 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         const size_t smem_ov = ov_bytes();
         if (one_pass && max_groups <= kGemvGroupsPerPass && smem_ov <= kSmemLimit) {
             if (y_dtype == LLVQ_BF16) {
-                if (!set_smem<gemv_sorted_overlap_kernel<true>>(ctx->device, smem_ov)) return LLVQ_ECUDA;
+                if (!set_smem<gemv_sorted_overlap_kernel<true>>(ctx, smem_ov)) return LLVQ_ECUDA;
                 if (launch_pdl(gemv_sorted_overlap_kernel<true>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, shift, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
             } else {
-                if (!set_smem<gemv_sorted_overlap_kernel<false>>(ctx->device, smem_ov)) return LLVQ_ECUDA;
+                if (!set_smem<gemv_sorted_overlap_kernel<false>>(ctx, smem_ov)) return LLVQ_ECUDA;
                 if (launch_pdl(gemv_sorted_overlap_kernel<false>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, shift, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
             }
             return launch_status();
@@ -360,16 +360,16 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     }
     if (sorted) {
         if (y_dtype == LLVQ_BF16) {
-            if (!set_smem<gemv_sorted_multi_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemv_sorted_multi_kernel<true>>(ctx, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemv_sorted_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         } else {
-            if (!set_smem<gemv_sorted_multi_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
+            if (!set_smem<gemv_sorted_multi_kernel<false>>(ctx, smem)) return LLVQ_ECUDA;
             if (launch_pdl(gemv_sorted_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
         }
     } else {
 #define LLVQ_LAUNCH_MULTI(K, ...)                                                                                                  \
     do {                                                                                                                           \
-        if (!set_smem<K>(ctx->device, smem)) return LLVQ_ECUDA;                                                                     \
+        if (!set_smem<K>(ctx, smem)) return LLVQ_ECUDA;                                                                     \
         if (launch_pdl(K, g, (unsigned)kSortThreads, smem, st, fa, __VA_ARGS__, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
         const bool bf16 = y_dtype == LLVQ_BF16;

@@ -7,7 +7,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -274,20 +273,11 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, 
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
-// Allow `bytes` of dynamic shared memory for a kernel on the current device (`device`).  The runtime keeps the setting, so it is
-// asked only when a launch needs more than any before it.
+// Whether a launch of the kernel on the context's device, which is current, can have `bytes` of dynamic shared memory.
 template <auto kKernel>
-bool set_smem(int device, size_t bytes)
+bool set_smem(const llvq_ctx* ctx, size_t bytes)
 {
-    static std::atomic<uint32_t> allowed[64];
-    std::atomic<uint32_t>* const have = device < 64 ? &allowed[device] : nullptr;
-    if (have && have->load(std::memory_order_acquire) >= bytes) return true;
-    if (cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
-    if (have) {
-        uint32_t seen = have->load(std::memory_order_relaxed);
-        while (seen < bytes && !have->compare_exchange_weak(seen, (uint32_t)bytes, std::memory_order_release)) {}
-    }
-    return true;
+    return allow_smem<kKernel>(ctx->smem_limits, ctx->smem_most, bytes);
 }
 
 int check_common(const llvq_ctx* ctx, const void* d_idx)

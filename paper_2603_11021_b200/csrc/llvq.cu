@@ -161,6 +161,7 @@ int llvq_create(llvq_ctx** out, int m_lo, int m_hi, int device)
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return LLVQ_ECUDA; }
     ctx->sm_count = prop.multiProcessorCount;
+    ctx->smem_most = prop.sharedMemPerBlockOptin;
 
     const HostTables& h = ctx->host;
     const size_t ncls = h.desc.size();
@@ -354,11 +355,11 @@ int llvq_decode_blocks(const llvq_ctx* ctx, const void* d_idx, uint64_t nblocks,
     const unsigned g = chunk_grid(ctx, nblocks);
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (ctx->fast) {
-        if (!set_smem<decode_blocks_fast_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
+        if (!set_smem<decode_blocks_fast_kernel<false>>(ctx, smem)) return LLVQ_ECUDA;
         if (launch_pdl(decode_blocks_fast_kernel<false>, g, (unsigned)kFastThreads, smem, (cudaStream_t)stream, fast_args(ctx, false), idx, nblocks,
                        reinterpret_cast<uint2*>(d_points)) != cudaSuccess) return LLVQ_ECUDA;
     } else {
-        if (!set_smem<decode_blocks_fast_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
+        if (!set_smem<decode_blocks_fast_kernel<true>>(ctx, smem)) return LLVQ_ECUDA;
         if (launch_pdl(decode_blocks_fast_kernel<true>, g, (unsigned)kFastThreads, smem, (cudaStream_t)stream, fast_args(ctx, false), idx, nblocks,
                        reinterpret_cast<uint2*>(d_points)) != cudaSuccess) return LLVQ_ECUDA;
     }
@@ -387,11 +388,11 @@ int llvq_dequant_matrix(const llvq_ctx* ctx, const void* d_idx, const uint16_t* 
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(d_w_bf16);
     if (ctx->fast) {
-        if (!set_smem<dequant_fast_kernel<false>>(ctx->device, smem)) return LLVQ_ECUDA;
+        if (!set_smem<dequant_fast_kernel<false>>(ctx, smem)) return LLVQ_ECUDA;
         if (launch_pdl(dequant_fast_kernel<false, false>, g, (unsigned)kFastThreads, smem, st, fast_args(ctx, false), idx, d_gain_f16, SgArgs{}, (uint64_t)nblocks,
                        rows, cols, row_walk(bpr, g), w, ld) != cudaSuccess) return LLVQ_ECUDA;
     } else {
-        if (!set_smem<dequant_fast_kernel<true>>(ctx->device, smem)) return LLVQ_ECUDA;
+        if (!set_smem<dequant_fast_kernel<true>>(ctx, smem)) return LLVQ_ECUDA;
         if (launch_pdl(dequant_fast_kernel<true, false>, g, (unsigned)kFastThreads, smem, st, fast_args(ctx, false), idx, d_gain_f16, SgArgs{}, (uint64_t)nblocks,
                        rows, cols, row_walk(bpr, g), w, ld) != cudaSuccess) return LLVQ_ECUDA;
     }
@@ -420,7 +421,7 @@ int llvq_dequant_matrix_sg(const llvq_ctx* ctx, const void* d_fields, int gain_b
     // (image without the table of small subsets, as in llvq_decode_blocks)
     const size_t smem = ctx->fl.total + 16;
     const unsigned g = chunk_grid(ctx, nblocks);
-    if (!set_smem<dequant_fast_kernel<false, true>>(ctx->device, smem)) return LLVQ_ECUDA;
+    if (!set_smem<dequant_fast_kernel<false, true>>(ctx, smem)) return LLVQ_ECUDA;
     if (launch_pdl(dequant_fast_kernel<false, true>, g, (unsigned)kFastThreads, smem, (cudaStream_t)stream, fast_args(ctx, false), static_cast<const uint32_t*>(d_fields),
                    static_cast<const uint16_t*>(nullptr), SgArgs{d_codebook_f32, d_row_scale_f32, gain_bits}, nblocks, rows, cols, row_walk(bpr, g),
                    reinterpret_cast<__nv_bfloat16*>(d_w_bf16), ld) != cudaSuccess) return LLVQ_ECUDA;
