@@ -13,30 +13,6 @@ namespace {
 // box's offset in bytes stays below 2^31 too.  Longer rows of a stored stream go to gemm_kernel, which reads X by plain loads.
 constexpr int64_t kMaxMapColumns = 1ll << 30;
 
-// The tensor map of X [batch][k_in] bf16 (16-byte aligned, k_in a multiple of 8): boxes of 64 columns x npad rows, 128-byte swizzle.
-// The driver's function asks for a current context, which a thread has only once a runtime call has bound the device's: a thread whose first
-// such call this is binds it here (the calls before it, of PyTorch's allocator and stream included, need none).
-bool make_x_map(int device, const uint16_t* d_x, int64_t k_in, int batch, int npad, CUtensorMap* map)
-{
-    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static const Encode encode = [] {                    // the driver's function, without linking against the driver library
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult found;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
-            found != cudaDriverEntryPointSuccess) fn = nullptr;
-        return reinterpret_cast<Encode>(fn);
-    }();
-    if (!encode) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)k_in, (cuuint64_t)batch}, strides[1] = {(cuuint64_t)k_in * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)npad}, steps[2] = {1, 1};
-    auto made = [&] {
-        return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(d_x), dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    return made() || (cudaSetDevice(device) == cudaSuccess && made());
-}
-
 int check_gemm_args(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f16, int64_t n_out, int64_t k_in,
                     const uint16_t* d_x_bf16, int batch, const uint16_t* d_y_bf16)
 {
@@ -143,8 +119,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     if (smem > 227 * 1024) return LLVQ_EUNSUPPORTED;
     const uint32_t* idx = static_cast<const uint32_t*>(d_idx);
     if (yo && sg) return LLVQ_EUNSUPPORTED;              // row-sharded: stored-gain form only
-    CUtensorMap xmap;
-    if (mapped && !make_x_map(ctx->device, d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
+    CUtensorMap xmap;                                    // made for the kernels that take X by TMA
     // codes with many classes (a warp of 32 unrelated blocks is what costs there): the kernel whose two teams order their domains; it
     // fits for every code with class tables in global memory.  (For the other codes it counts the blocks of a row tile in 32 bits: 8192 x 8192
     // batch 16: 102.0 us, with 64 bits 102.4)
@@ -163,6 +138,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             const unsigned grid_team = (unsigned)std::min<int64_t>(row_tiles * gt.nstages, ctx->sm_count);
             gt.sp = make_split(row_tiles * gt.nstages, gt.nstages, grid_team);
             const SgArgs sga = sg ? *sg : SgArgs{};
+            if (!make_x_map(ctx->device, d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
 #define LLVQ_LAUNCH_TEAM(BIG, SG, SH)                                                                                              \
     do {                                                                                                                     \
         if (!set_smem<gemm_team_kernel<BIG, SG, SH>>(ctx, smem_team)) return LLVQ_ECUDA;                                   \
@@ -191,6 +167,7 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
             gp.sp = make_split(row_tiles * gp.nstages, gp.nstages, grid_pipe);
             const unsigned long long* words = static_cast<const unsigned long long*>(d_idx);
             const SgArgs sga = sg ? *sg : SgArgs{};
+            if (!make_x_map(ctx->device, d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
 #define LLVQ_LAUNCH_PIPE_STORED(SG, SH)                                                                                    \
     do {                                                                                                                        \
         if (!set_smem<gemm_pipe_kernel<false, SG, SH, true>>(ctx, smem_pipe)) return LLVQ_ECUDA;                                        \

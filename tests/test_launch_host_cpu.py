@@ -66,3 +66,41 @@ int main()
 def test_two_threads_that_need_different_sizes(tmp_path, a, b):
     r = _run(tmp_path, SMEM.replace("SIZE_A", str(a)).replace("SIZE_B", str(b)))
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+# a look-up of the driver's function that fails is made again by the next call; a thread without a context gets one
+X_MAP = r"""
+#include "launch_host.h"
+#include <cstdio>
+
+static int lookups, encodes;
+static bool bound;
+
+static CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
+                       const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill)
+{
+    ++encodes;
+    return bound && dims[0] == 48 && dims[1] == 3 && strides[0] == 96 && box[1] == 16 ? CUDA_SUCCESS : CUDA_ERROR_INVALID_CONTEXT;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** fn, unsigned, unsigned long long, cudaDriverEntryPointQueryResult* r)
+{
+    *fn = lookups ? reinterpret_cast<void*>(encode) : nullptr;
+    *r = lookups++ ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+    return cudaSuccess;
+}
+cudaError_t cudaSetDevice(int device) { bound = device == 5; return cudaSuccess; }
+
+int main()
+{
+    CUtensorMap map;
+    bool ok[3];
+    for (bool& o : ok) o = llvq::make_x_map(5, nullptr, 48, 3, 16, &map);
+    std::printf("%d %d %d, %d look-ups, %d calls\n", ok[0], ok[1], ok[2], lookups, encodes);
+    return !ok[0] && ok[1] && ok[2] && lookups == 2 && encodes == 3 ? 0 : 1;
+}
+"""
+
+
+def test_tensor_map_of_x_after_a_failed_look_up_and_without_a_context(tmp_path):
+    r = _run(tmp_path, X_MAP)
+    assert r.returncode == 0, r.stdout + r.stderr
