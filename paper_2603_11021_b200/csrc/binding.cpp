@@ -7,6 +7,7 @@
 // CUDA stream address or None (PyTorch's current stream), and returns the output tensor, or a nonzero LLVQ status as an int
 // for the caller to raise.  Violated expectations raise AssertionError, tensors of the wrong kind TypeError.
 #include <torch/csrc/Dtype.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <ATen/ops/empty.h>
@@ -100,19 +101,17 @@ int call(F f)
 int y_code(at::ScalarType t) { return t == at::kFloat ? LLVQ_F32 : LLVQ_BF16; }
 uint64_t blocks_of(int64_t rows, int64_t cols) { return (uint64_t)rows * (uint64_t)((cols + 23) / 24); }
 
+// C++ exceptions become the Python ones that PyTorch's own functions raise for them (torch.OutOfMemoryError and so on).
 #define LLVQ_FUNC(name, count)                                                                                    \
     PyObject* name##_body(Args& A);                                                                               \
     PyObject* name(PyObject*, PyObject* const* args, Py_ssize_t n)                                                 \
     {                                                                                                             \
+        HANDLE_TH_ERRORS                                                                                          \
         if (n != count) { PyErr_Format(PyExc_TypeError, #name " takes %d arguments", count); return nullptr; }    \
         Args A{args};                                                                                             \
-        try {                                                                                                     \
-            PyObject* r = name##_body(A);                                                                         \
-            return A.ok ? r : nullptr;                                                                            \
-        } catch (const std::exception& e) {                                                                       \
-            PyErr_SetString(PyExc_RuntimeError, e.what());                                                        \
-            return nullptr;                                                                                       \
-        }                                                                                                         \
+        PyObject* r = name##_body(A);                                                                             \
+        return A.ok ? r : nullptr;                                                                                \
+        END_HANDLE_TH_ERRORS                                                                                      \
     }                                                                                                             \
     PyObject* name##_body(Args& A)
 
