@@ -99,6 +99,8 @@ int call(F f)
 }
 
 int y_code(at::ScalarType t) { return t == at::kFloat ? LLVQ_F32 : LLVQ_BF16; }
+// Whether w has room for rows x cols with leading dimension ld (the product may exceed 64 bits).
+bool holds(const at::Tensor& w, int64_t rows, int64_t cols, int64_t ld) { return rows == 0 || (__int128)w.numel() >= ((__int128)rows - 1) * ld + cols; }
 uint64_t blocks_of(int64_t rows, int64_t cols) { return (uint64_t)rows * (uint64_t)((cols + 23) / 24); }
 
 // C++ exceptions become the Python ones that PyTorch's own functions raise for them (torch.OutOfMemoryError and so on).
@@ -290,7 +292,7 @@ LLVQ_FUNC(dequant, 9)
     A.expect(w.scalar_type() == at::kBFloat16 && g->scalar_type() == at::kHalf);
     const uint64_t nblocks = layout == LLVQ_LAYOUT_FLAT ? ((uint64_t)rows * (uint64_t)cols + 23) / 24 : blocks_of(rows, cols);
     A.expect((uint64_t)g->numel() >= nblocks && bytes_of(*idx) >= llvq_index_bytes(ctx, nblocks));
-    A.expect(rows == 0 || w.numel() >= (rows - 1) * ld + cols);
+    A.expect(holds(w, rows, cols, ld));
     const void* pi = A.device(idx, "d_idx");
     const uint16_t* pg = static_cast<const uint16_t*>(A.device(g, "d_gain"));
     uint16_t* pw = static_cast<uint16_t*>(A.device(&w, "d_w"));
@@ -309,7 +311,7 @@ LLVQ_FUNC(dequant_sg, 10)
     if (!A.ok) return nullptr;
     at::Tensor w = w0 ? *w0 : new_tensor({rows, ld}, at::kBFloat16, *f);
     A.expect(w.scalar_type() == at::kBFloat16);
-    if (!A.expect(rows == 0 || w.numel() >= (rows - 1) * ld + cols)) return nullptr;
+    if (!A.expect(holds(w, rows, cols, ld))) return nullptr;
     const SgPtrs p = sg_args(A, cb, rs, bits, rows);
     A.expect(bytes_of(*f) >= llvq_field_bytes(ctx, blocks_of(rows, cols), (int)bits));
     const void* pf = A.device(f, "d_fields");
