@@ -123,7 +123,7 @@ LLVQ_FUNC(gemv, 10)
     const llvq_ctx* ctx = A.context(0);
     const at::Tensor *w = A.tensor(1, "d_idx"), *g = A.tensor(2, "d_gain"), *x = A.tensor(5, "d_x"), *y0 = A.tensor_or_none(6, "d_y");
     const int64_t n_out = A.integer(3), k_in = A.integer(4);
-    const at::ScalarType yt = A.dtype(7);
+    const at::ScalarType yt = y0 ? y0->scalar_type() : A.dtype(7);
     const bool sorted = A.a[9] == Py_True;
     if (!A.ok) return nullptr;
     at::Tensor y = y0 ? *y0 : new_tensor({n_out}, yt, *w);
@@ -159,7 +159,7 @@ LLVQ_FUNC(gemv_sg, 12)
     const at::Tensor *w = A.tensor(1, "d_fields"), *cb = A.tensor(3, "d_codebook"), *rs = A.tensor_or_none(4, "d_row_scale"),
                      *x = A.tensor(7, "d_x"), *y0 = A.tensor_or_none(8, "d_y");
     const int64_t bits = A.integer(2), n_out = A.integer(5), k_in = A.integer(6);
-    const at::ScalarType yt = A.dtype(9);
+    const at::ScalarType yt = y0 ? y0->scalar_type() : A.dtype(9);
     const bool sorted = A.a[11] == Py_True;
     if (!A.ok) return nullptr;
     at::Tensor y = y0 ? *y0 : new_tensor({n_out}, yt, *w);

@@ -20,3 +20,15 @@ def test_a_leading_dimension_that_wraps_is_too_long_for_the_output(ctx):
         P.llvq_dequant_matrix(ctx, idx, gain, rows, 1, P.LLVQ_LAYOUT_ROWWISE, w, ld)
     with pytest.raises(AssertionError):
         P.llvq_dequant_matrix_sg(ctx, idx, 0, torch.ones(1), None, rows, 1, w, ld)
+
+
+def test_the_type_of_an_output_is_not_asked_for_where_the_output_is_given(ctx):
+    import paper_2603_11021_b200 as P
+    idx, gain = torch.zeros(ctx.index_bytes(8), dtype=torch.uint8), torch.zeros(8, dtype=torch.half)
+    x, y = torch.zeros(24, dtype=torch.bfloat16), torch.zeros(8)
+    with pytest.raises(TypeError, match="contiguous CUDA tensor"):       # as far as a CPU tensor gets
+        P.llvq_gemv(ctx, idx, gain, 8, 24, x, y, y_dtype=None)
+    with pytest.raises(TypeError, match="contiguous CUDA tensor"):
+        P.llvq_gemv_sg(ctx, idx, 0, torch.ones(1), None, 8, 24, x, y, y_dtype=None)
+    with pytest.raises(TypeError, match="torch.dtype"):
+        P.llvq_gemv(ctx, idx, gain, 8, 24, x, y_dtype="float32")
