@@ -242,7 +242,7 @@ LLVQ_FUNC(gemv_multi, 5)
     const llvq_ctx* ctx = A.context(0);
     const at::ScalarType yt = A.dtype(2);
     const bool sorted = A.a[4] == Py_True;
-    if (!A.ok) return nullptr;
+    if (!A.expect(yt == at::kFloat || yt == at::kBFloat16)) return nullptr;
     PyObject* mats = PySequence_Fast(A.a[1], "mats must be a sequence");
     if (!mats) { A.ok = false; return nullptr; }
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(mats);

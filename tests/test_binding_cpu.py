@@ -32,3 +32,14 @@ def test_the_type_of_an_output_is_not_asked_for_where_the_output_is_given(ctx):
         P.llvq_gemv_sg(ctx, idx, 0, torch.ones(1), None, 8, 24, x, y, y_dtype=None)
     with pytest.raises(TypeError, match="torch.dtype"):
         P.llvq_gemv(ctx, idx, gain, 8, 24, x, y_dtype="float32")
+
+
+@pytest.mark.parametrize("sorted_layout", [False, True])
+@pytest.mark.parametrize("dtype", [torch.int8, torch.float16, torch.float64])
+def test_outputs_of_several_products_are_binary32_or_bf16(ctx, dtype, sorted_layout):
+    # anything else was written as bf16, two bytes per element whatever its width
+    import paper_2603_11021_b200 as P
+    idx, gain = torch.zeros(ctx.index_bytes(8), dtype=torch.uint8), torch.zeros(8, dtype=torch.half)
+    mat = (idx, gain, 8, 24, torch.zeros(24, dtype=torch.bfloat16), torch.zeros(8, dtype=dtype))
+    with pytest.raises(AssertionError):
+        (P.llvq_gemv_sorted_multi if sorted_layout else P.llvq_gemv_multi)(ctx, [mat], y_dtype=dtype)
