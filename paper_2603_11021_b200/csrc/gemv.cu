@@ -12,20 +12,24 @@ namespace {
 
 constexpr size_t kSmemLimit = 227 * 1024;
 
-// Shared memory of gemv_bin_kernel for `su` units per segment, and whether the table of small subsets still fits.
-void bin_smem(const llvq_ctx* ctx, int64_t nq, int su, size_t& bytes, bool& ext)
+// Shared memory of gemv_bin_kernel, and whether the table of small subsets still fits.  acc_floats = room for the row sums, cut down to one
+// copy per row where rows are so long that x needs the space.
+void bin_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext, uint32_t& acc_floats)
 {
-    const size_t rest = 16 + (size_t)nq * 48 * 4 + kSortAccFloats * 4 + 16 + 2 * 1024 * 4 + (size_t)su * 32 * (8 + 2);
-    ext = ctx->fl.total_ext + rest <= kSmemLimit;
-    bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest;
+    const size_t rest = 16 + (size_t)nq * 48 * 4 + 16 + 2 * 1024 * 4 + (size_t)kBinSegUnits * 32 * (8 + 2);
+    acc_floats = kSortAccFloats;
+    while (acc_floats > kGemvGroupsPerPass * kGemvGroupRows && ctx->fl.total + rest + acc_floats * 4 > kSmemLimit) acc_floats /= 2;
+    ext = ctx->fl.total_ext + rest + acc_floats * 4 <= kSmemLimit;
+    bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest + acc_floats * 4;
 }
 
-bool bin_kernel_serves(const llvq_ctx* ctx, int64_t nq, const SgArgs* sg)
+// Whether gemv_bin_kernel takes a matrix; order = gemv_order_kernel takes it too, which is preferred to cut row sums.
+bool bin_kernel_serves(const llvq_ctx* ctx, int64_t nq, const SgArgs* sg, bool order)
 {
-    size_t bytes; bool ext;
-    bin_smem(ctx, nq, kBinSegUnits, bytes, ext);
+    size_t bytes; bool ext; uint32_t acc_floats;
+    bin_smem(ctx, nq, bytes, ext, acc_floats);
     return (!sg || sg->bits <= 5) && ctx->fast && ctx->d_sort_rank && ctx->host.desc.size() >= 64 && ctx->host.W <= 48 && bytes <= kSmemLimit &&
-           nq < (1ll << 24);
+           nq < (1ll << 24) && (acc_floats == kSortAccFloats || !order);
 }
 
 // Stored streams of codes with many classes: gemv_bin_kernel while a CTA's range is one of its segments (it orders the whole range at
@@ -101,19 +105,18 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     if (shard && sg) return LLVQ_EUNSUPPORTED;
     // codes with many classes (a warp of unrelated blocks is what costs there): the kernels that order the blocks before they unrank
     // them; the others, and rows too long for their buffers, go to the direct kernel
-    int seg_units = kBinSegUnits;
-    size_t smem_bin; bool ext_bin;
-    bin_smem(ctx, nq, seg_units, smem_bin, ext_bin);
+    size_t smem_bin; bool ext_bin; uint32_t acc_floats;
+    bin_smem(ctx, nq, smem_bin, ext_bin, acc_floats);
     OrderArgs oa;
     size_t smem_order; bool ext_order;
     const bool order = order_smem(ctx, nq, sg ? sg->bits : 0, oa, smem_order, ext_order);
-    if (bin_kernel_serves(ctx, nq, sg) && (one_segment(upc) || !order)) {
+    if (bin_kernel_serves(ctx, nq, sg, order) && (one_segment(upc) || !order)) {
         const FastArgs fa = fast_args(ctx, ext_bin);
 #define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
     do {                                                                                                                   \
         if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx, smem_bin)) return LLVQ_ECUDA;                                          \
         if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
-                       bpr, seg_units, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
+                       bpr, acc_floats, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
         if (shard)   { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, true); else LLVQ_LAUNCH_BIN(false, false, true); }
         else if (sg) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, true, false); else LLVQ_LAUNCH_BIN(false, true, false); }
@@ -318,9 +321,9 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);
     else {
         const bool order = order_smem(ctx, max_nq, 0, oa, smem, ext);
-        bin = bin_kernel_serves(ctx, max_nq, nullptr) && (bin || !order);
+        bin = bin_kernel_serves(ctx, max_nq, nullptr, order) && (bin || !order);
         if (!bin && !order) return LLVQ_EUNSUPPORTED;
-        if (bin) bin_smem(ctx, max_nq, kBinSegUnits, smem, ext);
+        if (bin) bin_smem(ctx, max_nq, smem, ext, acc_floats);
     }
     if (smem > kSmemLimit) return LLVQ_EUNSUPPORTED;
     DeviceGuard guard(ctx->device);
@@ -373,7 +376,7 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         if (launch_pdl(K, g, (unsigned)kSortThreads, smem, st, fa, __VA_ARGS__, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
         const bool bf16 = y_dtype == LLVQ_BF16;
-        if (bin) { if (bf16) LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<true>, ctx->d_sort_rank, mm); else LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<false>, ctx->d_sort_rank, mm); }
+        if (bin) { if (bf16) LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<true>, ctx->d_sort_rank, mm, acc_floats); else LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<false>, ctx->d_sort_rank, mm, acc_floats); }
         else     { if (bf16) LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel<true>, oa, mm, (uint32_t)max_nq); else LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel<false>, oa, mm, (uint32_t)max_nq); }
 #undef LLVQ_LAUNCH_MULTI
     }

@@ -776,30 +776,30 @@ gemv_order_multi_kernel(FastArgs fa, OrderArgs oa, const __grid_constant__ GemvM
 // and then proceeds like gemv_sorted_kernel on those entries (S3-S8): a warp takes 32 consecutive entries, runs
 // the one unranker form they need and each lane forms its own dot product.
 // ===========================================================================
-constexpr int kBinSegUnits = 256;                    // at most 8192 blocks per segment (halved while shared memory is short)
+constexpr int kBinSegUnits = 256;                    // at most 8192 blocks per segment
 constexpr int kBinPerThread = kBinSegUnits * 32 / kSortThreads;   // 8
 
 template <bool kOutBf16, bool kSg, bool kShard>
 __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem& T, uint8_t* staging, const uint32_t* __restrict__ stream,
                                               const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, const SgArgs& sg,
-                                              const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, int seg_units,
+                                              const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, uint32_t acc_floats,
                                               const uint16_t* __restrict__ x, const YOut& yo, float* __restrict__ scratch,
                                               uint32_t* __restrict__ counters, int64_t slot0)
 {
     const uint32_t nq = sp.per_row;
     uint32_t* xs = reinterpret_cast<uint32_t*>(staging);            // [nq * 4][12] packed bf16 pairs of x
-    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [kSortAccFloats]
-    uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + kSortAccFloats);
+    float* acc = reinterpret_cast<float*>(xs + nq * 48);            // [acc_floats]
+    uint32_t* last_flag = reinterpret_cast<uint32_t*>(acc + acc_floats);
     uint32_t* next_chunk = last_flag + 1;
     uint32_t* hist = last_flag + 4;                                  // [1024] bins in sort order; later their first slots
     uint32_t* cursor = hist + 1024;                                  // [1024]
-    unsigned long long* ent = reinterpret_cast<unsigned long long*>(cursor + 1024);   // [seg_units * 32] class-local index | position << 48
-    uint16_t* ent_cls = reinterpret_cast<uint16_t*>(ent + seg_units * 32);            // [seg_units * 32] class (| gain index << 10), 0xffff = no block
+    unsigned long long* ent = reinterpret_cast<unsigned long long*>(cursor + 1024);   // [kBinSegUnits * 32] class-local index | position << 48
+    uint16_t* ent_cls = reinterpret_cast<uint16_t*>(ent + kBinSegUnits * 32);         // [kBinSegUnits * 32] class (| gain index << 10), 0xffff = no block
     stage_x(xs, x, k_in, nq * 48, threadIdx.x, blockDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t kWarps = blockDim.x >> 5;
     for_each_sorted_segment(sp, blockIdx.x, [&](uint32_t tu0, uint32_t tu1, uint32_t rg0, uint32_t rg1, bool first, bool last) {
-        const uint32_t shift = acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, kSortAccFloats);
+        const uint32_t shift = acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, acc_floats);
         if (first)
             for (uint32_t i = threadIdx.x; i < (rg1 - rg0 + 1u) * kGemvGroupRows << shift; i += blockDim.x) acc[i] = 0.f;
         hist[threadIdx.x] = 0; cursor[threadIdx.x] = 0;
@@ -906,25 +906,25 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
         const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
         finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
         __syncthreads();
-    }, (uint32_t)seg_units);
+    }, (uint32_t)kBinSegUnits);
 }
 
 template <bool kOutBf16, bool kSg = false, bool kShard = false>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_bin_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, SgArgs sg,
-                Split sp, int64_t n_out, int64_t k_in, int64_t bpr, int seg_units, const uint16_t* __restrict__ x, YOut yo,
+                Split sp, int64_t n_out, int64_t k_in, int64_t bpr, uint32_t acc_floats, const uint16_t* __restrict__ x, YOut yo,
                 float* __restrict__ scratch, uint32_t* __restrict__ counters)
 {
     prefetch_stored_span<kSg>(fa, stream, gain, sg, sp, n_out, bpr);       // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
-    gemv_bin_body<kOutBf16, kSg, kShard>(fa, T, staging, stream, sort_rank, gain, sg, sp, n_out, k_in, (uint32_t)bpr, seg_units, x, yo, scratch, counters, 0);
+    gemv_bin_body<kOutBf16, kSg, kShard>(fa, T, staging, stream, sort_rank, gain, sg, sp, n_out, k_in, (uint32_t)bpr, acc_floats, x, yo, scratch, counters, 0);
     if (kShard) shard_arrive(yo);
 }
 
 // Several independent matrices on their stored streams in one launch.
 template <bool kOutBf16>
 __global__ void __launch_bounds__(kSortThreads, 1)
-gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const __grid_constant__ GemvMulti mm, float* __restrict__ scratch,
+gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const __grid_constant__ GemvMulti mm, uint32_t acc_floats, float* __restrict__ scratch,
                       uint32_t* __restrict__ counters)
 {
     prefetch_stored_span<false>(fa, static_cast<const uint32_t*>(mm.m[0].weights), mm.m[0].gain, SgArgs{}, mm.m[0].sp, mm.m[0].n_out, mm.m[0].bpr);
@@ -937,7 +937,7 @@ gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const
         YOut yo{};
         yo.y = M.y;
         gemv_bin_body<kOutBf16, false, false>(fa, T, staging, static_cast<const uint32_t*>(M.weights), sort_rank, M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
-                                              (uint32_t)M.bpr, kBinSegUnits, M.x, yo, scratch, counters, M.slot0);
+                                              (uint32_t)M.bpr, acc_floats, M.x, yo, scratch, counters, M.slot0);
         __syncthreads();
     }
 }

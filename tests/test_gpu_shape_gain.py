@@ -220,3 +220,17 @@ def test_gemm_small_batch_sg(lib, ctxs, codes, code, bits, n_out, k_in, batch):
     yv = lib.llvq_gemv_sg(ctx, to_dev_u8(stream), bits, _f32(cb), _f32(rs), n_out, k_in, to_dev_bf16(x[0]), y_dtype=torch.bfloat16)
     assert gemv_error(y1[0].float().cpu().numpy(), yv.float().cpu().numpy().astype(np.float64)) <= 2.0 ** -7
     assert lib.llvq_last_error(ctx) == (0, 0)
+
+
+# rows around the longest that leave room for all copies of the row sums beside the ordered blocks of a thread block, and around the longest
+# that leave room for one (a field of 49 bits is ordered in this kernel alone)
+@pytest.mark.parametrize("k_in", [24 * 4 * 135, 24 * 4 * 136 - 16, 14336, 24 * 4 * 199, 24 * 4 * 200 - 24])
+def test_gemv_of_long_rows_with_a_gain_bit(oracle_mod, k_in):
+    import paper_2603_11021_b200 as P
+    ctx, o, n_out, bits = P.Context(2, 13, device=0), oracle_mod.Code(2, 13), 203, 1
+    stream, _ = gen.make_layer_sg(o.N, o.W, bits, n_out, k_in, seed=6)
+    cb, rs, x = np.array([4.3, 5.4], dtype=np.float32), gen.row_scales_f32(n_out, seed=6), gen.normal_bf16((1, k_in), seed=6)
+    want = o.gemm_sg(stream, bits, cb, rs, n_out, k_in, x, threads=4)[0]
+    y = P.llvq_gemv_sg(ctx, to_dev_u8(stream), bits, torch.from_numpy(cb).cuda(), torch.from_numpy(rs).cuda(), n_out, k_in, to_dev_bf16(x[0]))
+    assert gemv_error(y.cpu().numpy(), want) <= 1e-3       # binary32 sums
+    assert P.llvq_last_error(ctx) == (0, 0)
