@@ -16,7 +16,7 @@ import os
 
 import torch
 
-from .build import LIB, NATIVE
+from .build import LIB, NATIVE, native_matches, native_stamp
 
 __all__ = [
     "Context", "llvq_decode_blocks", "llvq_dequant_matrix", "llvq_gemv", "llvq_gemm_small_batch", "llvq_gemm_small_batch_noalloc",
@@ -82,6 +82,8 @@ def load_library() -> ctypes.CDLL:
         raise ImportError(f"{LIB} not found: run `python -m paper_2603_11021_b200.build` (needs nvcc); there is no fallback path")
     if not os.path.exists(NATIVE):
         raise ImportError(f"{NATIVE} not found: run `python -m paper_2603_11021_b200.build`; there is no fallback path")
+    if not native_matches():
+        raise ImportError(f"{NATIVE} is not {native_stamp()}: run `python -m paper_2603_11021_b200.build`")
     lib = ctypes.CDLL(LIB)
     vp, i64, u64 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_uint64
     lib.llvq_create.argtypes = [ctypes.POINTER(vp), ctypes.c_int, ctypes.c_int, ctypes.c_int]

@@ -44,9 +44,28 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Build libllvq.so and _native.so next to this file; returns the library's path."""
     if force or is_stale():
         _build_library(verbose)
-    if force or not os.path.exists(NATIVE) or any(os.path.getmtime(NATIVE) < os.path.getmtime(f) for f in [BINDING] + _headers()):
+    if force or native_is_stale():
         _build_native()
     return LIB
+
+
+def native_stamp() -> str:
+    """What _native.so is compiled against beside its sources: it holds inline code of PyTorch's and Python's headers."""
+    import sys
+    import torch
+    return f"built for torch {torch.__version__}, cxx11 {int(torch.compiled_with_cxx11_abi())}, python {sys.version_info.major}.{sys.version_info.minor}"
+
+
+def native_matches() -> bool:
+    """Whether _native.so, which carries its stamp, was built for the PyTorch and Python that run."""
+    with open(NATIVE, "rb") as f:
+        return native_stamp().encode() + b"\0" in f.read()
+
+
+def native_is_stale() -> bool:
+    if not os.path.exists(NATIVE) or not native_matches():
+        return True
+    return any(os.path.getmtime(NATIVE) < os.path.getmtime(f) for f in [BINDING] + _headers())
 
 
 def _build_native() -> None:
@@ -58,6 +77,7 @@ def _build_native() -> None:
     tmp = NATIVE + f".{os.getpid()}.tmp"
     subprocess.check_call([
         os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+        f'-DLLVQ_BUILT_FOR="{native_stamp()}"',
         "-I", os.path.join(ROOT, "include"), "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
         "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], BINDING, "-o", tmp, "-L", PKG, "-lllvq",
         "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"])

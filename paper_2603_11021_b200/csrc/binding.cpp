@@ -414,4 +414,10 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Entry points of libllvq
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }
+// (LLVQ_BUILT_FOR: the PyTorch and Python whose headers this was compiled with, looked for in the file before it is loaded)
+PyMODINIT_FUNC PyInit__native()
+{
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", LLVQ_BUILT_FOR) != 0) { Py_DECREF(m); return nullptr; }
+    return m;
+}

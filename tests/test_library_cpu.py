@@ -55,3 +55,14 @@ def test_unsupported_codes_are_rejected(lib):
         assert L.llvq_create(ctypes.byref(h), m_lo, m_hi, -1) == 3
         assert not h.value
     assert L.llvq_create(None, 2, 2, -1) == 1
+
+
+def test_native_module_of_another_pytorch_is_rebuilt_and_not_loaded(lib, monkeypatch):
+    import torch
+    from paper_2603_11021_b200 import build
+    assert not build.native_is_stale() and build.native_matches()
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + "1")
+    assert build.native_is_stale()
+    monkeypatch.setattr(lib, "_lib", None)
+    with pytest.raises(ImportError, match="built for"):
+        lib.load_library()
