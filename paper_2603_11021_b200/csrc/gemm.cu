@@ -23,7 +23,7 @@ int check_gemm_args(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_ga
     return LLVQ_OK;
 }
 
-// Enqueue gemm_sorted_kernel on a stream sorted by llvq_sort_blocks_gemm.
+// Enqueue gemm_pipe_kernel on a stream sorted by llvq_sort_blocks_gemm.
 int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_gain_f16, int64_t n_out, int64_t k_in,
                         const uint16_t* d_x_bf16, int batch, uint16_t* d_y_bf16, float* scratch, uint32_t* counters, void* stream,
                         const YOut* yo = nullptr, int64_t y_ld = 0, const SgArgs* sg = nullptr, int y_f32 = 0)
@@ -41,40 +41,32 @@ int launch_gemm_domains(const llvq_ctx* ctx, const void* p, const uint16_t* d_ga
     ga.batch = batch; ga.npad = (batch + 15) / 16 * 16;
     ga.nstages = (int)((ga.bpr + kDomBlocks - 1) / kDomBlocks);              // domains per row tile
     ga.x = d_x_bf16; ga.scratch = scratch; ga.counters = counters;
-    int dpi = ga.npad <= 32 ? 2 : 1;                                         // gemm_sorted_kernel: domains unranked per iteration (shared memory decides)
     const int64_t row_tiles = (n_out + kGemmRows - 1) / kGemmRows;
     ga.scratch_ld = row_tiles * kGemmRows;
     ga.split = 1;
     const unsigned grid = (unsigned)std::min<int64_t>(row_tiles * ga.nstages, ctx->sm_count);
     ga.sp = make_split(row_tiles * ga.nstages, ga.nstages, grid);
-    // gemm_pipe_kernel: two A buffer sets and two X buffer sets, or one X set when two do not fit; else the kernel with the block barrier
+    // two A buffer sets, and two X buffer sets or one when two do not fit (with one everything fits for every code that has a sorted
+    // layout: at most 223232 bytes).  Class tables in global memory: see the rule on 200 KB in launch_gemm
     const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_set = (size_t)kDomStages * kGemmRows * kStageK * 2,
                  x_set = (size_t)kDomStages * ga.npad * kStageK * 2;
-    int pipe = 0, b_double = 0;
-    size_t smem = head + (size_t)dpi * (a_set + x_set);
-    if (head + 2 * a_set + 2 * x_set <= (ctx->fast ? 227u : 200u) * 1024) { pipe = 1; b_double = 1; smem = head + 2 * a_set + 2 * x_set; }
-    else if (head + 2 * a_set + x_set <= 227 * 1024) { pipe = 1; smem = head + 2 * a_set + x_set; }
-    if (smem > 227 * 1024 || (!ctx->fast && !pipe)) return LLVQ_EUNSUPPORTED;      // (the pipeline's buffers fit for every code of the second kind)
-#define LLVQ_LAUNCH_DOMAINS(K, LAST)                                                                                          \
+    const int b_double = head + 2 * a_set + 2 * x_set <= (ctx->fast ? 227u : 200u) * 1024;
+    const size_t smem = head + 2 * a_set + (b_double ? 2 : 1) * x_set;
+    if (smem > 227 * 1024) return LLVQ_EUNSUPPORTED;
+#define LLVQ_LAUNCH_DOMAINS(BIG, SG, SH)                                                                                          \
     do {                                                                                                                     \
-        if (!set_smem<K>(ctx, smem)) return LLVQ_ECUDA;                                                               \
-        if (launch_pdl(K, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx), static_cast<const unsigned long long*>(p), d_gain_f16, \
-                       sga, ga, LAST, xmap) != cudaSuccess) return LLVQ_ECUDA;                                                \
+        if (!set_smem<gemm_pipe_kernel<BIG, SG, SH>>(ctx, smem)) return LLVQ_ECUDA;                                           \
+        if (launch_pdl(gemm_pipe_kernel<BIG, SG, SH>, grid, (unsigned)kGemmThreads, smem, (cudaStream_t)stream, fast_args(ctx), \
+                       static_cast<const unsigned long long*>(p), d_gain_f16, sga, ga, b_double, xmap) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
     const SgArgs sga = sg ? *sg : SgArgs{};
     CUtensorMap xmap;
     if (!make_x_map(ctx->device, d_x_bf16, k_in, batch, ga.npad, &xmap)) return LLVQ_ECUDA;
     if (yo && sg) return LLVQ_EUNSUPPORTED;              // row-sharded: stored-gain form only
-    if (!ctx->fast) { if (yo) LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<true, false, true>), b_double); else LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<true, false, false>), b_double); }
-    else if (pipe) {
-        if (yo) LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<false, false, true>), b_double);
-        else if (sg) LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<false, true, false>), b_double);
-        else LLVQ_LAUNCH_DOMAINS((gemm_pipe_kernel<false, false, false>), b_double);
-    } else {
-        if (yo) LLVQ_LAUNCH_DOMAINS((gemm_sorted_kernel<false, true>), dpi);
-        else if (sg) LLVQ_LAUNCH_DOMAINS((gemm_sorted_kernel<true, false>), dpi);
-        else LLVQ_LAUNCH_DOMAINS((gemm_sorted_kernel<false, false>), dpi);
-    }
+    if (yo) { if (ctx->fast) LLVQ_LAUNCH_DOMAINS(false, false, true); else LLVQ_LAUNCH_DOMAINS(true, false, true); }
+    else if (sg) LLVQ_LAUNCH_DOMAINS(false, true, false);
+    else if (ctx->fast) LLVQ_LAUNCH_DOMAINS(false, false, false);
+    else LLVQ_LAUNCH_DOMAINS(true, false, false);
 #undef LLVQ_LAUNCH_DOMAINS
     return launch_status();
 }

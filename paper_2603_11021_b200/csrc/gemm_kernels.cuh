@@ -1,7 +1,7 @@
 // The fused dequant + small-batch GEMM kernels (tcgen05, accumulator in tensor memory): the kernel with two thread
-// groups on alternating stages, the sorted layouts (sort kernels and the consumer with a block barrier), and the
-// kernel without a block barrier that both entry points run for the 48-bit codes.  Included by gemm.cu inside its
-// unnamed namespace, after kernels_common.cuh and gemv_kernels.cuh (shard_arrive).
+// groups on alternating stages, the kernels that make the sorted layouts, the pipeline kernel that consumes them (and stored streams of few
+// classes), and the kernel whose two teams order a stored stream of many classes.  Included by gemm.cu inside its unnamed
+// namespace, after kernels_common.cuh, order.cuh and gemv_kernels.cuh (shard_arrive).
 #pragma once
 
 // ===========================================================================
@@ -218,10 +218,8 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
 // A domain is 128 rows x 8 column blocks (1024 blocks, two 96-column MMA stages); the stream holds the domains
 // row tile major, each domain's blocks ordered like the GEMV's sorted layout (decoder form, unranking steps,
 // class), one 64-bit entry per block: the stored index unchanged (48 bits) + position in the domain (row * 8 +
-// column block, 10 bits, stored in the high 16).  The kernel runs the whole CTA on one accumulator: per
-// iteration it unranks one domain (padded batch > 32) or two (warp w takes the w-th chunk of the first and the
-// (31-w)-th of the second: both are ordered from expensive to cheap, so the pairs balance), writing the bf16
-// weights straight to their place in the K-major A tiles, then one thread issues the tcgen05 MMAs of those stages.
+// column block, 10 bits, stored in the high 16).  gemm_pipe_kernel unranks them, writing the bf16 weights straight to
+// their place in the K-major A tiles.
 // ===========================================================================
 constexpr int kDomBlocks = 8;                          // column blocks per domain
 constexpr int kDomEntries = kGemmRows * kDomBlocks;    // 1024
@@ -359,178 +357,8 @@ sort_blocks_gemm_big_kernel(FastArgs fa, const uint32_t* __restrict__ stream, in
     }
 }
 
-// For codes whose tables leave no room for gemm_pipe_kernel's buffers.
-template <bool kSg = false, bool kShard = false>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg, GemmArgs ga, int dpi,
-                   const __grid_constant__ CUtensorMap xmap)
-{
-    extern __shared__ __align__(1024) uint8_t smem_1k[];
-    uint8_t* const smem = smem_1k;
-    const uint32_t img_bytes = fa.image_bytes;
-    uint64_t* bar_img = reinterpret_cast<uint64_t*>(smem + img_bytes);
-    uint64_t* bar_free = bar_img + 1;                                     // the MMAs reading the A / B buffers are done
-    uint64_t* bar_done = bar_img + 2;                                     // the accumulator of this item is complete
-    uint64_t* bar_x = bar_img + 3;                                        // the X slices of the iteration are in the buffer
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_img + 5);
-    uint32_t* last_flag = tmem_slot + 1;
-    const uint32_t a_off = (img_bytes + 64 + 1023) & ~1023u;
-    constexpr uint32_t kAStage = kGemmRows * kStageK * 2;                  // 24576
-    uint8_t* a_buf = smem + a_off;                                        // [dpi * 2 stages] x 24576
-    const uint32_t b_stage = (uint32_t)ga.npad * kStageK * 2;
-    uint8_t* b_buf = a_buf + (uint32_t)dpi * kDomStages * kAStage;         // [dpi * 2 stages] x npad * 192
-
-    pdl_launch_dependents();
-    const bool image_ok = fast_load_image(smem, fa.image, fa.image_bytes, bar_img, fa.flags);
-    pdl_wait();                                        // also when the image did not arrive: the dependents of this launch rely on it
-    if (!image_ok) {
-        if (kShard) shard_arrive(*ga.shard);           // the peers must not wait for this rank
-        return;
-    }
-    const FastSmem T = fast_view(smem, fa.L);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        mbar_init(bar_free, 1); mbar_init(bar_done, 1); mbar_init(bar_x, (uint32_t)dpi);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    const uint32_t idesc = instr_desc_bf16_m128((uint32_t)ga.npad);
-    const uint32_t nd = ga.sp.per_row;                                     // domains per row tile
-    // every CTA takes an equal contiguous range of the row_tiles * nd domains (row tile major); the parts of a row
-    // tile that end up in different CTAs are summed through the scratch, as in the GEMV
-    const uint32_t dom_begin = split_begin(ga.sp, blockIdx.x), dom_end = split_begin(ga.sp, blockIdx.x + 1u);
-    uint32_t uses = 0, done = 0;
-    bool timeout = false;
-    for (uint32_t rt = split_row(ga.sp, dom_begin); rt * nd < dom_end; ++rt) {
-        const uint32_t tile0 = rt * nd, tile1 = tile0 + nd;
-        const int d_begin = (int)(max(dom_begin, tile0) - tile0), d_end = (int)(min(dom_end, tile1) - tile0);
-        // CTAs that share this row tile
-        const uint32_t parts = dom_begin <= tile0 && tile1 <= dom_end ? 1u : split_owner(ga.sp, tile1 - 1u) - split_owner(ga.sp, tile0) + 1u;
-        // the entries of an iteration are requested one iteration ahead (they come from DRAM)
-        const unsigned long long no_entry = kSortIndexMask;
-        auto entry_at = [&](int d, int q) {
-            if (d + q >= d_end) return no_entry;
-            // warp 0 also issues the MMAs of every iteration: it takes the cheapest chunk of each domain (the last), the other
-            // warps pair chunk w - 1 of the first domain with chunk 31 - w of the second
-            const int chunk = warp == 0 ? 31 : (q == 0 ? warp - 1 : 31 - warp);
-            const int64_t at = ((int64_t)rt * nd + d + q) * kDomEntries + chunk * 32 + lane;
-            return __ldg(sorted + at);
-        };
-        unsigned long long e0 = entry_at(d_begin, 0), e1 = dpi > 1 ? entry_at(d_begin, 1) : no_entry;
-        for (int d0 = d_begin; d0 < d_end; d0 += dpi, ++uses) {
-            const int nd_now = min(dpi, d_end - d0);
-            const unsigned long long cur0 = e0, cur1 = e1;
-            e0 = entry_at(d0 + dpi, 0);
-            if (dpi > 1) e1 = entry_at(d0 + dpi, 1);
-            // ---- A: every warp unranks one chunk of 32 sorted entries per domain
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (q >= nd_now) break;
-                const unsigned long long e = q == 0 ? cur0 : cur1;
-                const uint64_t field = e & kSortIndexMask;
-                const uint64_t I = kSg ? field & ((1ull << fa.L.W) - 1ull) : field;     // shape-gain form: gain index above the shape index
-                const uint32_t pos = (uint32_t)(e >> 48);
-                const bool valid = field != kSortIndexMask && I < fa.n_points;
-                const uint32_t r = pos >> 3, c = pos & 7u;
-                const int64_t row = (int64_t)rt * kGemmRows + r, cb = (int64_t)(d0 + q) * kDomBlocks + c;
-                uint16_t gbits = 0;
-                if (!kSg && valid) gbits = ldg_u16_here(gain + row * ga.bpr + cb);
-                float gn = 0.f;                                               // the gain is converted once the block is unranked
-                uint32_t w[12];
-                Decoded dec{};
-                const uint32_t cls = decode_sorted_entry(fa, T, I, valid, dec);
-                if (!kSg) gn = gain_to_float(gbits);
-                if (kSg && valid) {
-                    const float scale = sg.row_scale ? __ldg(sg.row_scale + row) : 1.f;
-                    gn = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + (uint32_t)(field >> fa.L.W))),
-                                   __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
-                }
-                expand_bf16(dec, gn, w);
-                // the previous MMAs read the buffers: wait for them only now, with the first chunk already unranked
-                if (q == 0) {
-                    if (uses > 0 && !mbar_wait(bar_free, (uses - 1u) & 1u)) timeout = true;
-                    if (threadIdx.x == 0)
-                        for (int st = 0; st < dpi; ++st) {
-                            if (st < nd_now) request_x(smem_u32(b_buf) + (uint32_t)st * kDomStages * b_stage, &xmap, d0 + st, ga.npad, bar_x);
-                            else mbar_expect(bar_x, 0u);
-                        }
-                }
-                uint8_t* a_dst = a_buf + (uint32_t)(q * kDomStages + (c >> 2)) * kAStage + (r >> 3) * 128u + (r & 7u) * 16u + 3u * (c & 3u) * 2048u;
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-                    *reinterpret_cast<uint4*>(a_dst + j * 2048) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
-            }
-            fence_async_smem();
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                if (!mbar_wait(bar_x, uses & 1u)) timeout = true;
-                tc_fence_after();
-                for (int st = 0; st < nd_now; ++st)
-                    domain_mmas(tmem, smem_u32(a_buf) + (uint32_t)st * kDomStages * kAStage, smem_u32(b_buf) + (uint32_t)st * kDomStages * b_stage, ga.npad,
-                                idesc, d0 == d_begin && st == 0);
-                umma_commit(bar_free);
-                if (d0 + dpi >= d_end) umma_commit(bar_done);
-            }
-        }
-        // ---- epilogue: accumulator -> scratch (split-K) or Y
-        const bool has = d_end > d_begin;
-        if (warp < 4 && has) {
-            if (!mbar_wait(bar_done, done & 1u)) timeout = true;
-            tc_fence_after();
-            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
-            for (int c0 = 0; c0 < ga.npad; c0 += 16) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-                if (orow < ga.n_out) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int n = c0 + i;
-                        if (n < ga.batch) {
-                            if (parts == 1u) gemm_store<kShard>(ga, n, orow, v[i]);
-                            else atomicAdd(ga.scratch + (int64_t)n * ga.scratch_ld + orow, v[i]);
-                        }
-                    }
-                }
-            }
-            tc_fence_before();
-        }
-        done += has;
-        if (parts > 1u) {
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) *last_flag = (atomicAdd(ga.counters + rt, 1u) == parts - 1u);
-            __syncthreads();
-            if (*last_flag) {
-                __threadfence();
-                for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
-                    const int n = i / kGemmRows;
-                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
-                    if (orow < ga.n_out) {
-                        float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
-                        gemm_store<kShard>(ga, n, orow, __ldcg(sp));
-                        __stcg(sp, 0.f);
-                    }
-                }
-                if (threadIdx.x == 0) ga.counters[rt] = 0u;
-            }
-        }
-        __syncthreads();
-    }
-    if (timeout) atomicOr(fa.flags, 1u);
-    if (kShard) {
-        __threadfence_system();                           // this thread's stores to the peers' copies, before the CTA counts itself in
-        shard_arrive(*ga.shard);
-    }
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, kTmemCols);
-}
-
-// The same product for padded batch <= 32, where two domains' tiles fit: the two buffer sets alternate between
-// consecutive domains and nobody waits for the whole CTA.  Warps 1..31 unrank: the chunks of 32 sorted entries of a
+// The product from a sorted layout: two buffer sets alternate between consecutive domains (two A tiles; two X slices, or one where
+// shared memory has room for no more) and nobody waits for the whole CTA.  Warps 1..31 unrank: the chunks of 32 sorted entries of a
 // row tile are handed out by a ticket counter (ticket t = chunk t % 32 of the tile's domain t / 32, so from expensive
 // to cheap inside a domain), a warp always holding its next ticket with that chunk's entries already requested.
 // It unranks the chunk, waits (rarely) until the MMAs that read this buffer two domains ago are done, writes its
