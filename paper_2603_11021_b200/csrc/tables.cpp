@@ -112,7 +112,6 @@ bool fill_descriptor(const HostTables& t, const ClassInfo& c, ClassDesc& d, int&
     d.parity = (uint8_t)c.parity; d.w = (uint8_t)c.w; d.B = (uint8_t)c.B; d.m = (uint32_t)c.m;
     d.A = (uint16_t)c.A;
     d.goff = (uint16_t)(c.parity ? 0 : t.woff[c.w]);
-    d.magicA = ~0ull / c.A;
     int n46 = 0;
     for (size_t i = 0; i < c.values.size(); ++i)
         if (c.values[i] % 8 == 4 || c.values[i] % 8 == 6) n46 += c.mults[i];
@@ -132,7 +131,6 @@ bool fill_descriptor(const HostTables& t, const ClassInfo& c, ClassDesc& d, int&
             LevelDesc& l = d.lev[nlev++];
             l.radix = t.pascal[n * 25 + gm[i]];
             l.k = (uint8_t)gm[i]; l.val = (uint8_t)gv[i]; l.n = (uint8_t)n; l.pad = 0;
-            l.magic = ~0ull / l.radix;
             n -= gm[i];
             ++steps;
         }

@@ -12,17 +12,15 @@ typedef unsigned __int128 u128;
 constexpr int kDim = 24;
 constexpr int kMaxLevels = 8;
 
-// One "choose k of the slots still free" step of the arrangement unranking
-// (App. A step 4).  magic = floor((2^64 - 1) / radix) for division by multiply-high.
+// One "choose k of the slots still free" step of the arrangement unranking (App. A step 4).
 struct LevelDesc {
     uint32_t radix;   // C(n, k)
     uint8_t k;        // slots taken by this value
     uint8_t val;      // absolute value placed
     uint8_t n;        // slots free before this step
     uint8_t pad;
-    uint64_t magic;
 };
-static_assert(sizeof(LevelDesc) == 16, "LevelDesc layout");
+static_assert(sizeof(LevelDesc) == 8, "LevelDesc layout");
 
 // Everything the kernels need to rebuild a point of one class from its
 // class-local index (App. A steps 3-4).  Group 1 = positions F1(c) (values
@@ -40,11 +38,9 @@ struct ClassDesc {
     uint16_t goff;     // first admissible codeword in the sorted Golay table
     uint16_t A;        // number of admissible codewords
     uint32_t m;        // shell
-    uint64_t magicA;   // floor((2^64 - 1) / A)
-    uint64_t reserved;
     LevelDesc lev[kMaxLevels];   // group-1 steps first, then group-0 steps
 };
-static_assert(sizeof(ClassDesc) == 32 + 16 * kMaxLevels, "ClassDesc layout");
+static_assert(sizeof(ClassDesc) == 16 + 8 * kMaxLevels, "ClassDesc layout");
 
 // Compact form of ClassDesc for the codes whose class tables stay in global memory (32 bytes, two 16-byte loads): the
 // radix of a step is C(free slots, k) from the Pascal triangle in shared memory and its reciprocals come from two tables
