@@ -114,7 +114,7 @@ __device__ __forceinline__ int coset_point(double u, uint32_t c, int pi, int lan
 // lattice point is farther from u by a margin far above any binary64 rounding.
 // Bound: the integer / logic pipe (78 % busy, 818 instructions per decode; the shared-memory pipe is at 54 %).  Scoring the 8192
 // cosets one by one took about 6000 instructions and was bound by bank conflicts: 38.9 -> 1.13 ms for the 699 050 vectors of a
-// 4096 x 4096 matrix (EUCLIDEAN, indexing included), 32.0 -> 2.06 ms for the 174 763 of 1024 x 4096 (ANGULAR, 12 decodes each).
+// 4096 x 4096 matrix (EUCLIDEAN, indexing included), 32.0 -> 2.06 ms for the 174 763 of 1024 x 4096 (ANGULAR on shells 2..12, 11 decodes each).
 // Steps on the way: rows of 128 bytes per (parity, nibble) read by the 16 lanes of one parity instead of rows shared by both
 // parities (1.38 -> 1.31 ms), roundings by additions instead of conversions and 24 warps drawing their vectors from a shared
 // counter instead of fixed strides (-> 1.13 ms).

@@ -119,8 +119,9 @@ int launch_gemm(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     if (mapped && (!ctx->fast || kGemmRows * ga.bpr <= 1ll << 32) && order_args(ctx, sg ? sg->bits : 0, &oa)) {
         const size_t head = (ctx->fl.total + 64 + 1023) & ~size_t(1023), a_sets = (size_t)kGemmTeams * kDomStages * kGemmRows * kStageK * 2,
                      x_set = (size_t)kDomStages * ga.npad * kStageK * 2, hists = (size_t)kGemmTeams * 2 * oa.words * 4;
-        // (codes that look their classes up in global memory keep a larger L1 cache below 200 KB of shared memory: 8192 x 8192, 72 bits, batch
-        // 64: 234 us with two X buffers, 197 with one)
+        // (codes that look their classes up in global memory keep a larger L1 cache below 200 KB of shared memory: 8192 x 8192, two X buffers
+        // above 200 KB / one below, batch 48 and 64: shells 2..20 166 / 148 and 169 / 151 us, 2..30 192 / 164 and 196 / 167, 2..53 231 / 195
+        // and 234 / 198; the sorted layouts within 1 %)
         const int x_double = head + a_sets + 2 * x_set + hists <= (ctx->fast ? 227u : 200u) * 1024;
         const size_t smem_team = head + a_sets + (x_double ? 2 : 1) * x_set + hists;
         if (smem_team <= 227 * 1024) {

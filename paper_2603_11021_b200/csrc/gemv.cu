@@ -33,7 +33,9 @@ bool bin_kernel_serves(const llvq_ctx* ctx, int64_t nq, const SgArgs* sg, bool o
 }
 
 // Stored streams of codes with many classes: gemv_bin_kernel while a CTA's range is one of its segments (it orders the whole range at
-// once, so the warps share classes best), else gemv_order_kernel, whose teams order small pieces and unrank others meanwhile.
+// once, so the warps share classes best), else gemv_order_kernel, whose teams order small pieces and unrank others meanwhile.  Rows of
+// 4096, shells 2..13, gemv_bin_kernel / gemv_order_kernel in us by units per CTA: 19 11.7 / 13.8, 74 16.2 / 16.6, 149 23.7 / 26.9, 205 30.0 /
+// 30.2, 256 35.2 / 33.9, 298 43.8 / 41.8, 400 54.5 / 53.7, 521 70.9 / 67.1; 595 (8192 x 8192) 82.8 / 71.9.
 bool one_segment(int64_t units_per_cta) { return units_per_cta <= kBinSegUnits; }
 
 // Whether gemv_order_kernel takes a matrix of nq units per row group; its shared memory, and whether the table of small subsets

@@ -626,8 +626,8 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
 // team orders a piece, its warps take 32 consecutive entries at a time, run the one unranker form they need, and each lane
 // forms its own dot product, as in gemv_sorted_kernel.  A share's pieces are of equal size (the teams drift apart by
 // themselves: first pieces of 8, 16, 24 and 32 units made shares of two pieces slower and long ones no faster).  28672 x 8192:
-// 278 -> 235 us, 8192 x 8192: 82 -> 71 us against gemv_bin_kernel, which orders up to 8192 blocks at a time as a phase of the
-// whole block and is the faster one while that is the CTA's whole range (4096 x 4096: 23.5 against 26 us).
+// 278 -> 235 us, 8192 x 8192: 82 -> 72 us, 11008 x 4096: 54.5 -> 53.7 us against gemv_bin_kernel, which orders up to 8192 blocks at a
+// time as a phase of the whole block and is the faster one while that is the CTA's whole range (4096 x 4096: 23.7 against 26.9 us).
 // ===========================================================================
 constexpr int kOrderTeams = 4;
 constexpr int kTeamThreads = kSortThreads / kOrderTeams;

@@ -42,8 +42,8 @@ _SCALE = {"byte": 1.0, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9, "ns": 1.0, "us"
 
 
 # what the fused GEMV kernels are compiled from (the default set of sources a counter file vouches for)
-GEMV_SOURCES = ["tables.h", "tables.cpp", "ctx.h", "decode.cuh", "fast.cuh", "big.cuh", "umma.cuh", "kernels_common.cuh", "gemv_kernels.cuh",
-                "gemv.cu"]
+GEMV_SOURCES = ["tables.h", "tables.cpp", "ctx.h", "launch_host.h", "decode.cuh", "fast.cuh", "big.cuh", "umma.cuh", "kernels_common.cuh", "order.cuh",
+                "gemv_kernels.cuh", "gemv.cu"]
 
 
 def source_hash(names=None) -> str:

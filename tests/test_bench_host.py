@@ -114,3 +114,16 @@ def test_counter_file_vouches_for_its_sources_only(tmp_path):
     stale.write_text(json.dumps({"duration_ns": 1.0, "sources": ["tables.h"], "source_hash": "0" * 16}))
     assert nc.load(str(stale)) is None and nc.load(str(tmp_path / "missing.json")) is None
     assert nc.source_hash(["tables.h"]) != nc.source_hash(["tables.h", "fast.cuh"])
+
+
+def test_the_default_sources_are_all_that_the_gemv_kernels_include():
+    import re
+    from paper_2603_11021_b200 import ncu_counters as nc
+    csrc, seen, todo = os.path.join(nc.PKG, "csrc"), set(), ["gemv.cu"]
+    while todo:
+        name = todo.pop()
+        if name not in seen and os.path.exists(os.path.join(csrc, name)):
+            seen.add(name)
+            with open(os.path.join(csrc, name)) as f:
+                todo += re.findall(r'#include "([^"]+)"', f.read())
+    assert seen <= set(nc.GEMV_SOURCES)
