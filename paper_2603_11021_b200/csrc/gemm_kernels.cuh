@@ -443,7 +443,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
                 for (uint32_t j = 0; j < n_dom; ++j) {
                     if (b_double && j + 1 < n_dom) stage_b(j + 1);
                     const uint32_t gd = g_base + j, b = gd & 1u, bx = b_double ? b : 0u;
-                    if (!mbar_wait(bar_full + b, (gd >> 1) & 1u)) timeout = true;
+                    if (!mbar_wait_copies(bar_full + b, (gd >> 1) & 1u)) timeout = true;
                     tc_fence_after();
                     domain_mmas(tmem, smem_u32(a_buf) + b * kDomStages * kAStage, smem_u32(b_buf) + bx * kDomStages * b_stage, ga.npad, idesc, j == 0);
                     umma_commit(bar_free + b);
@@ -737,7 +737,7 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
                     if (i_tile > 0u && !mbar_wait(bar_free + (team ^ 1), before & 1u)) timeout = true;
                     request_x(smem_u32(x_mine), &xmap, (int)d, ga.npad, bar_x + team);
                 }
-                if (!mbar_wait(bar_x + team, mine & 1u)) timeout = true;
+                if (!mbar_wait_copies(bar_x + team, mine & 1u)) timeout = true;
                 tc_fence_after();
                 domain_mmas(tmem + 64u * (uint32_t)team, smem_u32(a_mine), smem_u32(x_mine), ga.npad, idesc, fresh);
                 umma_commit(bar_free + team);

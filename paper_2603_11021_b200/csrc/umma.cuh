@@ -29,6 +29,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
     return done != 0;
 }
 
+// The same where the phase counts copies into this block's shared memory: when the limit runs out, waits as long again before it returns
+// false, so that a late copy does not land in the memory of whichever block comes next.
+__device__ __forceinline__ bool mbar_wait_copies(uint64_t* bar, uint32_t parity)
+{
+    if (mbar_wait(bar, parity)) return true;
+    mbar_wait(bar, parity);
+    return false;
+}
+
 // Whether the phase has completed, without waiting.
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity)
 {
