@@ -49,3 +49,31 @@ def test_products_from_a_new_thread(code, batch):
         torch.cuda.synchronize()
         assert (got.float() == 2.0 * (k_in // 24)).all(), name
     assert P.llvq_last_error(ctx) == (0, 0)
+
+
+def test_first_launches_of_a_context_inside_a_capture():
+    # the kernels have been launched before, by another context: what the host settles for a new one is no work on the stream
+    import paper_2603_11021_b200 as P
+    n_out, k_in, batch = 256, 480, 16
+    nblocks = n_out * (k_in // 24)
+    gain = torch.full((nblocks,), 0.25, dtype=torch.half, device="cuda")
+    x = torch.ones((batch, k_in), dtype=torch.bfloat16, device="cuda")
+    y, yb = torch.empty(n_out, device="cuda"), torch.empty((batch, n_out), dtype=torch.bfloat16, device="cuda")
+    for capture in (False, True):
+        ctx = P.Context(2, 13, device=0)
+        stream = torch.zeros(ctx.index_bytes(nblocks), dtype=torch.uint8, device="cuda")
+        y.fill_(-1.0), yb.fill_(-1.0)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        if capture:
+            with torch.cuda.graph(graph):
+                P.llvq_gemv(ctx, stream, gain, n_out, k_in, x[0], y)
+                P.llvq_gemm_small_batch(ctx, stream, gain, n_out, k_in, x, yb)
+            graph.replay()
+        else:
+            P.llvq_gemv(ctx, stream, gain, n_out, k_in, x[0], y)
+            P.llvq_gemm_small_batch(ctx, stream, gain, n_out, k_in, x, yb)
+        torch.cuda.synchronize()
+        assert (y == 2.0 * (k_in // 24)).all() and (yb.float() == 2.0 * (k_in // 24)).all()
+        assert P.llvq_last_error(ctx) == (0, 0)
+        del graph
