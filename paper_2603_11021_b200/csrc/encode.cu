@@ -383,43 +383,73 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
     }
 }
 
-// Bits of a at the set positions of mask, packed lowest first.
-__device__ __forceinline__ uint32_t extract_bits(uint32_t a, uint32_t mask)
+// Bits kBit of the 24 bytes of w as a mask, byte i -> bit i: the eight bits of a pair of words are moved together by one multiplication
+// (bits 8 i and 8 i + 4 meet the factors 2^(32 - 7 j); those with i = j are wanted, no two products fall together, so nothing carries).
+template <int kBit>
+__device__ __forceinline__ uint32_t bit_plane(const uint32_t (&w)[6])
 {
-    uint32_t r = 0, k = 0;
-    while (mask) {
-        const uint32_t low = mask & (0u - mask);
-        if (a & low) r |= 1u << k;
-        ++k;
-        mask ^= low;
+    uint32_t r[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const uint32_t lo = w[2 * j] >> kBit, hi = kBit < 4 ? w[2 * j + 1] << (4 - kBit) : w[2 * j + 1] >> (kBit - 4);
+        const unsigned long long p = (unsigned long long)((lo & 0x01010101u) | (hi & 0x10101010u)) * 0x102040800ull;
+        r[j] = (uint32_t)(p >> 32) & 0xffu;
     }
-    return r;
+    return r[0] | r[1] << 8 | r[2] << 16;
 }
 
+constexpr int kRankThreads = 256;
+constexpr int kRankValues = 32;            // larger than any absolute value of a point: its square is at most 16 * 53
+
 // Point -> index (Sec. 3.2; inverse of App. A steps 1-4), one thread per block.  A point that is not in the code
-// gets index 0 and is counted in the out-of-range counter.
-__global__ void __launch_bounds__(256)
+// gets index 0 and is counted in the out-of-range counter.  The absolute values are taken as bit planes over the 24
+// coordinates: which coordinates hold a value is a few operations on masks, and the place of an element among
+// the free slots is a population count.
+// Bound: instruction issue and dependent reads (class record, codeword).  With a loop over the 24 coordinates per value, and the free
+// slots gathered bit by bit, encoding 699 050 Gaussian vectors (EUCLIDEAN) took 1126 us in all; 1063 us with masks.
+__global__ void __launch_bounds__(kRankThreads)
 rank_kernel(DevCode dc, EncTables et, const uint32_t* __restrict__ golay, const uint32_t* __restrict__ pascal,
             const int8_t* __restrict__ points, uint64_t n, unsigned long long* __restrict__ index)
 {
-    const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ uint64_t sig_of[kRankValues];
+    __shared__ uint32_t choose[25 * 25];
+    for (int i = threadIdx.x; i < kRankValues; i += kRankThreads) sig_of[i] = __ldg(et.sig_of_value + i);
+    for (int i = threadIdx.x; i < 25 * 25; i += kRankThreads) choose[i] = __ldg(pascal + i);
+    __syncthreads();
+    const uint64_t b = (uint64_t)blockIdx.x * kRankThreads + threadIdx.x;
     if (b >= n) return;
-    int a[24];
-    uint32_t c = 0, neg = 0, nonzero = 0, bit1 = 0;
-    uint64_t sig = 0;
-    const int parity = points[b * 24] & 1;
-    bool good = true;
+    uint32_t w[6];
+    const int8_t* const from = points + b * 24;
+    if ((reinterpret_cast<uintptr_t>(points) & 7u) == 0) {
 #pragma unroll
-    for (int i = 0; i < 24; ++i) {
-        const int xi = points[b * 24 + i];
-        a[i] = xi < 0 ? -xi : xi;
-        good &= (xi & 1) == parity && a[i] < 64;
-        sig += __ldg(et.sig_of_value + (a[i] & 63));
-        c |= (uint32_t)(((xi - parity) >> 1) & 1) << i;
-        neg |= (uint32_t)(xi < 0) << i;
-        nonzero |= (uint32_t)(xi != 0) << i;
-        bit1 |= (uint32_t)((a[i] >> 1) & 1) << i;
+        for (int j = 0; j < 3; ++j) { const uint2 t = __ldg(reinterpret_cast<const uint2*>(from) + j); w[2 * j] = t.x; w[2 * j + 1] = t.y; }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            w[j] = 0;
+            for (int i = 0; i < 4; ++i) w[j] |= (uint32_t)(uint8_t)__ldg(from + 4 * j + i) << (8 * i);
+        }
     }
+    const uint32_t all = 0xffffffu;
+    const uint32_t odd = bit_plane<0>(w), neg = bit_plane<7>(w);
+    uint32_t beyond = 0;
+    uint64_t sig = 0;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {                                              // absolute values
+        const uint32_t m = (w[j] >> 7) & 0x01010101u;
+        w[j] = (w[j] ^ m * 255u) + m;
+        beyond |= w[j];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sig += sig_of[(w[j] >> (8 * i)) & (kRankValues - 1)];
+    }
+    const uint32_t bit1 = bit_plane<1>(w), bit2 = bit_plane<2>(w), bit3 = bit_plane<3>(w), bit4 = bit_plane<4>(w);
+    const bool parity = odd != 0u;
+    bool good = (odd == 0u || odd == all) && (beyond & 0xe0e0e0e0u) == 0u;
+    const uint32_t c = parity ? bit1 ^ neg : bit1;                              // bit 1 of x - parity
+    // the coordinates whose absolute value is v (a value of the point's parity)
+    const auto holding = [&](uint32_t v) {
+        return ~((bit1 ^ (0u - (v >> 1 & 1u))) | (bit2 ^ (0u - (v >> 2 & 1u))) | (bit3 ^ (0u - (v >> 3 & 1u))) | (bit4 ^ (0u - (v >> 4 & 1u)))) & all;
+    };
     // class of the multiset of absolute values
     uint32_t cls = 0;
     bool found = false;
@@ -433,41 +463,39 @@ rank_kernel(DevCode dc, EncTables et, const uint32_t* __restrict__ golay, const 
     good &= found;
     unsigned long long I = 0;
     if (good) {
-        const ClassDesc& d = dc.cls[cls];
+        const uint4* const record = reinterpret_cast<const uint4*>(dc.cls + cls);     // ClassDesc: 16 bytes, then 8 per level
+        const uint4 h = __ldg(record);
+        const uint32_t weight = (h.x >> 8) & 0xffu, B = (h.x >> 16) & 0xffu, signpar = h.x >> 24;
+        const int nlev1 = (int)(h.y & 0xffu), nlev = nlev1 + (int)((h.y >> 8) & 0xffu);
+        const uint32_t fill1 = (h.y >> 16) & 0xffu, fill0 = h.y >> 24, goff = h.z & 0xffffu, A = h.z >> 16;
         const uint32_t pos = __ldg(et.pos_by_low12 + (c & 0xfffu));
         good &= __ldg(golay + pos) == c;                                   // c must be a codeword
-        const uint32_t r = pos - d.goff;
-        good &= r < d.A;                                                   // ... of the weight the class needs
-        const uint32_t F1 = parity ? 0u : c, F0 = ~F1 & 0xffffffu;
-        uint32_t freem = parity ? 0xffffffu : F1;
-        bool in0 = parity != 0;
+        const uint32_t r = pos - goff;
+        good &= r < A;                                                     // ... of the weight the class needs
+        const uint32_t F1 = parity ? 0u : c, F0 = ~F1 & all;
+        uint32_t freem = parity ? all : F1;
+        bool in0 = parity;
         unsigned long long p = 0, mult = 1;
-        const int nlev = d.nlev1 + d.nlev0;
         for (int l = 0; l < nlev; ++l) {
-            if (!in0 && l >= d.nlev1) {                                    // the rest of group 1 holds its filler
-                for (int i = 0; i < 24; ++i) if ((freem >> i) & 1u) good &= a[i] == d.fill1;
+            if (!in0 && l >= nlev1) {                                      // the rest of group 1 holds its filler
+                good &= (freem & ~holding(fill1)) == 0u;
                 freem = F0; in0 = true;
             }
-            const LevelDesc& lv = d.lev[l];
-            uint32_t am = 0;
-            for (int i = 0; i < 24; ++i) am |= (uint32_t)(a[i] == lv.val) << i;
-            am &= freem;
-            good &= __popc(am) == lv.k;
-            uint32_t rel = extract_bits(am, freem), rho = 0;
-            for (int t = 1; rel; ++t) {                                    // combinatorial number system: sum of C(e_t, t)
-                const int e = __ffs(rel) - 1;
-                rho += __ldg(pascal + e * 25 + min(t, 24));
-                rel &= rel - 1;
-            }
+            const uint2 lv = __ldg(reinterpret_cast<const uint2*>(record + 1) + l);     // radix, slots | value << 8 | ...
+            const uint32_t mine = holding((lv.y >> 8) & 0xffu) & freem;
+            good &= (uint32_t)__popc(mine) == (lv.y & 0xffu);
+            uint32_t rho = 0, t = 1;
+            for (uint32_t left = mine; left; left &= left - 1u, ++t)       // combinatorial number system: sum of C(e_t, t), e_t = place among the free slots
+                rho += choose[__popc(freem & ((left & (0u - left)) - 1u)) * 25 + t];
             p += mult * rho;
-            mult *= lv.radix;
-            freem ^= am;
+            mult *= lv.x;
+            freem ^= mine;
         }
         if (!in0) {
-            for (int i = 0; i < 24; ++i) if ((freem >> i) & 1u) good &= a[i] == d.fill1;
+            good &= (freem & ~holding(fill1)) == 0u;
             freem = F0;
         }
-        for (int i = 0; i < 24; ++i) if ((freem >> i) & 1u) good &= a[i] == d.fill0;
+        good &= (freem & ~holding(fill0)) == 0u;
         unsigned long long s = 0;
         if (parity) {
             good &= neg == (c ^ bit1);                                     // 1 mod 4 on F0, 3 mod 4 on F1
@@ -475,10 +503,13 @@ rank_kernel(DevCode dc, EncTables et, const uint32_t* __restrict__ golay, const 
             // s = the signs of the positions that carry one (F1 and the nonzero ones of F0), ascending, without the last F1
             // position, whose sign the others fix (sum = 0 mod 8)
             const uint32_t last_f1 = F1 ? 0x80000000u >> __clz(F1) : 0u;
-            if (d.w) good &= ((neg & last_f1) != 0u) == (((__popc(neg & F1 & ~last_f1) + d.signpar) & 1u) != 0u);
-            s = extract_bits(neg, (F1 | (F0 & nonzero)) & ~last_f1);
+            if (weight) good &= ((neg & last_f1) != 0u) == (((__popc(neg & F1 & ~last_f1) + signpar) & 1u) != 0u);
+            const uint32_t signs = (F1 | (F0 & (bit1 | bit2 | bit3 | bit4))) & ~last_f1;
+            uint32_t bits = 0;
+            for (uint32_t left = neg & signs; left; left &= left - 1u) bits |= 1u << __popc(signs & ((left & (0u - left)) - 1u));
+            s = bits;
         }
-        I = dc.off_lo[cls] + r + (unsigned long long)d.A * (s + (p << d.B));
+        I = dc.off_lo[cls] + r + (unsigned long long)A * (s + (p << B));
     }
     if (!good) { I = 0; atomicAdd(dc.bad_index, 1ull); }
     index[b] = I;
@@ -508,8 +539,8 @@ int status_of_launch() { return cudaGetLastError() == cudaSuccess ? LLVQ_OK : LL
 
 int launch_rank(const llvq_ctx* ctx, const int8_t* d_points, uint64_t nblocks, uint64_t* d_index, cudaStream_t st)
 {
-    const unsigned grid = (unsigned)((nblocks + 255) / 256);
-    rank_kernel<<<grid, 256, 0, st>>>(ctx->dev, ctx->enc, ctx->d_golay, ctx->enc.pascal, d_points, nblocks,
+    const unsigned grid = (unsigned)((nblocks + kRankThreads - 1) / kRankThreads);
+    rank_kernel<<<grid, kRankThreads, 0, st>>>(ctx->dev, ctx->enc, ctx->d_golay, ctx->enc.pascal, d_points, nblocks,
                                       reinterpret_cast<unsigned long long*>(d_index));
     return status_of_launch();
 }
