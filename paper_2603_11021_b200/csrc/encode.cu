@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "ctx.h"
 #include "tables.h"
@@ -17,13 +18,14 @@ using namespace llvq;
 namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
-constexpr int kEncWarps = 24;              // vectors in flight per CTA (one CTA per SM), one warp each
 constexpr uint32_t kFlagSearchGaveUp = 4u; // LLVQ_FLAG_SEARCH_GAVE_UP
 
 constexpr int kMaxShell = 53;              // llvq_create's limit
 constexpr int kMaxCand = 64;               // cosets re-scored in binary64 per search; more (massive ties) means all 8192 are
 
-// Units of the first stage of the search: costs and moves are whole numbers of 1 / kCostScale.  The largest rounding error
+// ---- the careful search: one vector per warp ----
+
+// Units of its first stage: costs and moves are whole numbers of 1 / kCostScale.  The largest rounding error
 // of a coordinate costs 1/4, i.e. 2046: sixteen of them stay below 2^15.
 constexpr float kCostScale = 8184.f;
 // Two cosets whose first-stage costs differ by more than this are in the same order in exact arithmetic: a cost carries at
@@ -33,7 +35,7 @@ constexpr uint32_t kParityBit = 0x8000u;   // where a cost carries the parity of
 constexpr uint32_t kParityCode = 0x7676u;  // a byte-permute selector XOR this trades places with the one of the other parity
 constexpr uint32_t kSelEven = 0x3244u;     // {high half of the first operand} stays high, low half zero; ^ kParityCode: moved low
 
-// Per-warp scratch of the lattice search.
+// Per-warp scratch of the careful search.
 struct __align__(128) WarpTables {
     uint2 nib[2][6][16];    // [parity][4 coordinates][bit pattern n]: {cost | move << 16, parity code | move of pattern ~n << 16}; rows of 128 bytes
     uint4 pk[24][2];        // [coordinate, octad by octad][parity] w(b), w(b + 2), w(b + 2), w(b) for offset b = parity:
@@ -95,32 +97,26 @@ __device__ __forceinline__ int coset_point(double u, uint32_t c, int pi, int lan
     return x;
 }
 
-// Nearest point of the unbounded lattice to u (one coordinate per lane, lanes 0..23; all in units of the integer
-// coordinates).  Every lattice point is b + 4 z with b_i = parity + 2 c_i, c a Golay codeword, and sum z = parity
-// (mod 2) (the sum rules of Sec. 2.4: all Golay weights are multiples of 4).  For each of the 2 x 4096 cosets the
-// best z is the rounded one, with the coordinate of largest rounding error moved to its other neighbour when the
-// sum rule fails.
-// Two stages.  The first finds the smallest cost over all cosets in whole numbers, along a trio of octads (GolayTrio): per
-// parity and octad pattern {w, ~w} the best cost for an even and for an odd sum of z (a move included where the rounded z has
-// the other parity), packed as two 16-bit halves; over the 512 triples those add up, the even and odd sums of three octads
-// combining to the parity the coset needs.  A minimum over the parities of the three octads never moves more than one
-// coordinate where one move is the better choice, so this is the minimum over the 8192 cosets.  A lane holds (parity, x,
-// half of the a): 32 pairs (a, b), three instructions each with the packed add-and-minimum of this architecture.
-// Every coset within kCostMargin of the smallest cost is then listed (usually one) and evaluated in binary64, coordinate by
-// coordinate in lane order, one rounding per operation: its point, and, if there are several, the squared distance as the
-// sum over the coordinates in order.  The smallest distance wins, the lowest (parity, codeword position) among equal ones;
-// inside a coset the first coordinate with the largest error moves.  The result does not depend on the first stage's
-// rounding.  Returns the coordinate of this lane (0 for lanes >= 24) and the squared norm of the point; unique = every other
-// lattice point is farther from u by a margin far above any binary64 rounding.
-// Bound: the integer / logic pipe (78 % busy, 818 instructions per decode; the shared-memory pipe is at 54 %).  Scoring the 8192
-// cosets one by one took about 6000 instructions and was bound by bank conflicts: 38.9 -> 1.13 ms for the 699 050 vectors of a
-// 4096 x 4096 matrix (EUCLIDEAN, indexing included), 32.0 -> 2.06 ms for the 174 763 of 1024 x 4096 (ANGULAR on shells 2..12, 11 decodes each).
-// Steps on the way: rows of 128 bytes per (parity, nibble) read by the 16 lanes of one parity instead of rows shared by both
-// parities (1.38 -> 1.31 ms), roundings by additions instead of conversions and 24 warps drawing their vectors from a shared
-// counter instead of fixed strides (-> 1.13 ms).
-__device__ __forceinline__ int lattice_nearest(WarpTables& W, const GolayTrio& S, const PatternSteps& steps,
-                                               const uint32_t (&row)[6], const uint32_t* __restrict__ golay, const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
+// Nearest point of the unbounded lattice to u (one coordinate per lane, lanes 0..23), as nearest_pairs below finds it, for the
+// inputs to which two cosets are so close that whole-number costs do not tell them apart (about one in sixty).
+// First stage: per parity and octad pattern {w, ~w} the best cost for an even and for an odd sum of z (a move included where the
+// rounded z has the other parity), the minimum over the 512 triples of patterns that are codewords (GolayTrio); a lane holds (parity, x,
+// half of the a).  Every coset within kCostMargin of the smallest cost is then listed and evaluated in binary64, coordinate by
+// coordinate in lane order, one rounding per operation: its point, and, if there are several, the squared distance as the sum over
+// the coordinates in order.  The smallest distance wins, the lowest (parity, codeword position) among equal ones; inside a coset the
+// first coordinate with the largest error moves.  The result does not depend on the first stage's rounding.  Returns the coordinate of
+// this lane (0 for lanes >= 24) and the squared norm of the point; unique = every other lattice point is farther from u by a margin
+// far above any binary64 rounding.
+__device__ __noinline__ int nearest_careful(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
+                                            const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
 {
+    uint32_t row[6];                                             // where the nibbles of pattern (x, 4 h) of every octad are
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+        const uint32_t p = S.pat[o][(lane & 7) * 8 + ((lane >> 1) & 4)], t = (uint32_t)__cvta_generic_to_shared(&W.nib[lane >> 4][2 * o][0]);
+        row[2 * o] = t ^ (p & 15u) * 8u;
+        row[2 * o + 1] = (t + 128u) ^ (p >> 4) * 8u;
+    }
     const float uq = __shfl_sync(kFull, (float)u, lane < 24 ? S.coord[lane] : lane);   // octad order
     if (lane < 24) {
         uint32_t w[4];
@@ -263,123 +259,654 @@ __device__ __forceinline__ int lattice_nearest(WarpTables& W, const GolayTrio& S
     return best_x;
 }
 
-// One warp per input vector; inputs are binary32 values, all scoring runs in binary64 with one rounding per operation and
-// sums over the coordinates in order.  EUCLIDEAN: if the nearest lattice point of the input lies in the code it is the
+// ---- the search: two lanes per vector ----
+
+// Units of the costs below: whole numbers of 1 / kPairScale.  Three octads cost at most 6 of the squares of the half spacing
+// that a coordinate's offset is measured in (an octad with a move at most 2, two of them together at most 4 before the better
+// combination is taken), 65400: 16 bits.
+constexpr float kPairRoot = 104.403065f;   // sqrt(kPairScale)
+constexpr float kPairScale = 10900.f;
+// As kCostMargin: a sum of 24 costs carries 24 roundings of half a unit and 0.6 from binary32 errors (|u| up to 30).
+constexpr uint32_t kPairMargin = 26u;
+// The costs of the eight codewords of one triple of patterns are formed again from binary32 sums, 2.1 units off at most: what lies
+// more than this above the smallest whole-number cost (12.6 off at most) is farther than the coset that has it.
+constexpr uint32_t kWordMargin = 15u;
+
+// Two forms of the kernel: kPairs = two lanes per vector, 16 warps of 16 vectors, all warps of the CTA in step (below); else one warp
+// per vector, 24 warps, nearest_careful alone.
+template <bool kPairs> constexpr int kEncWarps = kPairs ? 16 : 24;
+template <bool kPairs> constexpr int kEncVecs = kPairs ? 16 : 1;          // vectors of a warp
+// Shared memory of a warp: costs of the patterns of the six nibbles, [nibble][pattern][vector] (or the scratch of nearest_careful), and the
+// inputs, [coordinate][vector].
+constexpr uint32_t kNibRow = 16 * sizeof(uint2), kNibTable = 16 * kNibRow, kNibBytes = 6 * kNibTable;
+static_assert(sizeof(WarpTables) + 24 <= kNibBytes, "nearest_careful works where the costs were");
+template <bool kPairs> constexpr uint32_t kEncWarpBytes = kPairs ? kNibBytes : (uint32_t)sizeof(WarpTables) + 128u;
+template <bool kPairs> constexpr size_t kEncSmem = kEncWarps<kPairs> * (kEncWarpBytes<kPairs> + 24 * kEncVecs<kPairs> * sizeof(float)) + sizeof(GolayTrio) + (kPairs ? kNibTable : 128);
+
+// The patterns of a codeword on the three octads are x ^ a, x ^ b, x ^ a ^ b with x and a, b from two [8, 4] codes whose sums are
+// the even words (Turyn's construction; GolayTrio has the order of coordinates in which these are the same two for every octad).
+__device__ constexpr uint32_t turyn_a(uint32_t a)
+{
+    constexpr uint32_t a0 = kTurynA[0], a1 = kTurynA[1], a2 = kTurynA[2];
+    return (a & 1 ? a0 : 0u) ^ (a & 2 ? a1 : 0u) ^ (a & 4 ? a2 : 0u);
+}
+__device__ constexpr uint32_t turyn_x(uint32_t x)
+{
+    constexpr uint32_t x0 = kTurynX[0], x1 = kTurynX[1], x2 = kTurynX[2];
+    return (x & 1 ? x0 : 0u) ^ (x & 2 ? x1 : 0u) ^ (x & 4 ? x2 : 0u);
+}
+
+__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y)
+{
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+
+__device__ __forceinline__ uint32_t half_of(uint32_t v, int pi) { return pi ? v >> 16 : v & 0xffffu; }
+
+// Costs of a part of the coordinates for an even and for an odd sum of its z, parity 0 of the lattice in the low halves, parity 1 in the high ones.
+struct Cost {
+    uint32_t even, odd;
+};
+__device__ __forceinline__ Cost operator+(const Cost& a, const Cost& b)
+{
+    return {__viaddmin_u16x2(a.odd, b.odd, a.even + b.even), __viaddmin_u16x2(a.odd, b.even, a.even + b.odd)};
+}
+
+// Cost of octad pattern `p` (of the a-code; the tables' addresses carry the x) or its complement, whichever is cheaper; lo, hi:
+// where the costs of the octad's nibbles 0 are, with the x in the row bits.
+__device__ __forceinline__ Cost pattern_cost(uint32_t lo, uint32_t hi, uint32_t p, uint32_t octad)
+{
+    const uint2 l = lds64((lo ^ (p & 15u) * kNibRow) + octad * 2u * kNibTable), h = lds64((hi ^ (p >> 4) * kNibRow) + octad * 2u * kNibTable);
+    const uint2 lc = lds64((lo ^ (~p & 15u) * kNibRow) + octad * 2u * kNibTable), hc = lds64((hi ^ (~p >> 4 & 15u) * kNibRow) + octad * 2u * kNibTable);
+    Cost c;
+    c.even = __viaddmin_u16x2(lc.y, hc.y, __viaddmin_u16x2(lc.x, hc.x, __viaddmin_u16x2(l.y, h.y, l.x + h.x)));
+    c.odd = __viaddmin_u16x2(lc.y, hc.x, __viaddmin_u16x2(lc.x, hc.y, __viaddmin_u16x2(l.y, h.x, l.x + h.y)));
+    return c;
+}
+
+// What a search returns; both lanes of a vector hold the same, but for x: half of the point each.
+struct Nearest {
+    uint32_t x[3];          // coordinates 12 q .. 12 q + 11 as signed bytes (q = 0, 1: the lane of the pair; the halves of the warp)
+    int norm2;              // squared norm of the point
+    double dot;             // its inner product with u
+    bool unique;            // every other lattice point is farther from u by a margin far above any binary64 rounding
+};
+
+// nearest_careful for u = (v rn) radius (v[stride i] holds coordinate i), one vector for the whole warp.
+__device__ __forceinline__ void nearest_of_warp(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
+                                                const uint16_t* __restrict__ pos_by_low12, const float* v, int stride, double rn, double radius, int lane,
+                                                int8_t* point, int& norm2, double& dot, bool& unique)
+{
+    const double u = lane < 24 ? __dmul_rn(__dmul_rn((double)v[stride * lane], rn), radius) : 0.0;
+    const int xi = nearest_careful(W, S, steps, golay, pos_by_low12, u, lane, norm2, unique);
+    dot = u * (double)xi;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) dot += __shfl_xor_sync(kFull, dot, o);
+    if (lane < 24) point[lane] = (int8_t)xi;
+}
+
+// Vectors of a CTA that wait for nearest_careful, and its answers.
+// More vectors per SM than this: two lanes take a vector, else a warp does.  Two lanes per vector use the chip best, but a CTA works on 256 vectors at a time
+// for some 15 us; shells 2..13 and 2..12, us for a warp per vector / two lanes: EUCLIDEAN 12 000 vectors 53 / 69, 30 000 87 / 87, 80 000 174 / 151;
+// ANGULAR 5000 76 / 90, 12 000 132 / 178, 30 000 278 / 207.
+constexpr uint64_t kPairsFromEuclidean = 208, kPairsFromAngular = 128;
+constexpr int kFew = 40;                   // no more vectors than this left in a CTA: all of them go to nearest_careful (EUCLIDEAN 867 -> 761 us with the wider loads)
+constexpr uint32_t kPendingMost = 48;
+struct Pending {
+    double rn, radius, dot;
+    const float* v;
+    int norm2;
+    bool unique;
+    alignas(4) int8_t x[24];
+};
+struct PendingList {
+    Pending list[kPendingMost];
+    uint32_t count;
+};
+
+// Nearest point of the unbounded lattice to u = (v rn) radius, every operation rounded once to binary64 (v[16 i] holds coordinate i; v s1 s2
+// is u in binary32; all in units of the integer coordinates).  Every lattice point is b + 4 z with b_i = parity + 2 c_i, c a
+// Golay codeword, and sum z = parity (mod 2) (the sum rules of Sec. 2.4: all Golay weights are multiples of 4).  For each of the
+// 2 x 4096 cosets the best z is the rounded one, with the coordinate of largest rounding error moved to its other neighbour when
+// the sum rule fails.
+// Two stages.  The first finds the coset of smallest cost in whole numbers.  Every part of the coordinates has
+// two costs, for an even and for an odd sum of its z, 16 bits each for either parity of the lattice in one word; two parts combine by
+// two additions and two add-and-minimum.  Coordinates combine to pairs and nibbles (tables in shared memory), these to the 64 patterns
+// {w, ~w} of an octad, and the Golay code is the 512 triples (x, a, b) of such patterns (Turyn's construction).  Choosing a
+// neighbour per part moves more than one coordinate only where that costs no less than one move, so this is the minimum over the
+// cosets.  A lane makes three of the six tables and takes four of the eight x.  If the best (x, parity) leads all others by more than the
+// rounding of the costs, its 64 triples are looked at again, then the best triple's eight codewords, and the coset that is left is
+// evaluated as the oracle does: coordinate by coordinate, one binary64 rounding per operation, the first coordinate with the
+// largest error moving where the sum rule asks for it.  Wherever a second candidate lies within the margin (one vector in
+// sixty) the vector goes to nearest_careful, one per warp.  So the result does not depend on the first stage's rounding.
+// Bound: instruction issue (55 % of the slots) and the load / store pipe by turns: the warps in step read their tables together and then
+// compute together.  Against nearest_careful for every vector, 24 warps: 818 -> 430 warp instructions per search; 699 050 vectors EUCLIDEAN
+// 1063 -> 737 us, 174 763 ANGULAR on shells 2..12 2035 -> 796 us (of it 2035 -> 1430 by the radii left out).
+// All threads of the CTA call this together; `wanted` = this lane's vector is to be searched, `few` = so few of the CTA's are that
+// nearest_careful takes them all.
+// The block barriers keep the warps in step: the code is long (some 1500 instructions once through, half of them four times), and warps that are
+// each somewhere else in it fetch more instructions than the SM delivers (2 warps per scheduler: 3.0 of 5.8 stall cycles per
+// instruction were fetches; 0.1 of 3.9 with the barriers, 1329 -> 942 us for the 174 763 vectors of the ANGULAR case).
+__device__ __forceinline__ void nearest_pairs(uint32_t nib, const float* v, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
+                                              const uint16_t* __restrict__ pos_by_low12, WarpTables& careful, PendingList& pending, float s1, float s2, double rn,
+                                              double radius, bool wanted, bool few, int warp, int lane, Nearest& r)
+{
+    const int q = lane >> 4;
+    bool settled = false;
+    if (!few) {
+        const uint32_t tab = nib + 8u * (uint32_t)(lane & 15);
+        const uint32_t* const coords = reinterpret_cast<const uint32_t*>(S.coord);
+#pragma unroll 1
+        for (uint32_t g = 3u * (uint32_t)q; g < 3u * (uint32_t)q + 3u; ++g) {
+            const uint32_t four = coords[g];
+            Cost n[4][2];                                            // by bit of the codeword
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float t0 = v[16u * ((four >> (8 * k)) & 31u)] * s1 * s2 * 0.25f;
+                uint32_t w[2][2];
+#pragma unroll
+                for (int pi = 0; pi < 2; ++pi) {
+                    // rounding by adding 1.5 * 2^23 (the parity of z is then the last bit), whole numbers from adding 2^23: no conversions
+                    const float t = pi ? t0 - 0.25f : t0, tr = t + 12582912.f, err = t - (tr - 12582912.f);
+                    const float a = fabsf(err) * kPairRoot, b = kPairRoot - a, c = 0.5f * kPairRoot - a, d = 0.5f * kPairRoot + a;
+                    uint32_t sel = (__float_as_uint(tr) & 1u) * 0x4444u ^ 0x5410u;
+                    if (pi == 1 && k == 0) sel ^= g == 4u ? 0x4444u : 0u;    // octad 2 of parity 1 is kept odd sum first: totals then have the parity that the cosets ask for
+                    w[pi][0] = __byte_perm(__float_as_uint(fmaf(a, a, 8388608.f)), __float_as_uint(fmaf(b, b, 8388608.f)), sel);
+                    // an offset larger by 2 moves t by a half: the error becomes 1/2 - |err|, and z one less where err was negative
+                    sel ^= (uint32_t)((int)__float_as_uint(err) >> 31) & 0x4444u;
+                    w[pi][1] = __byte_perm(__float_as_uint(fmaf(c, c, 8388608.f)), __float_as_uint(fmaf(d, d, 8388608.f)), sel);
+                }
+#pragma unroll
+                for (int b = 0; b < 2; ++b) n[k][b] = {__byte_perm(w[0][b], w[1][b], 0x5410), __byte_perm(w[0][b], w[1][b], 0x7632)};
+            }
+            Cost pair[2][4];
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) pair[p][b] = n[2 * p][b & 1] + n[2 * p + 1][b >> 1];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const Cost c = pair[0][i & 3] + pair[1][i >> 2];
+                sts64(tab + g * kNibTable + (uint32_t)i * kNibRow, c.even, c.odd);
+            }
+        }
+        uint32_t best = 0xffffu, second = 0xffffu, group = 0;        // group: 2 x + parity
+        uint32_t kept[8];                                            // the smallest costs of that x, by a
+#pragma unroll
+        for (int i = 0; i < 8; ++i) kept[i] = 0u;
+#pragma unroll 1
+        for (uint32_t x = 4u * (uint32_t)q; x < 4u * (uint32_t)q + 4u; ++x) {
+            __syncthreads();
+            const uint32_t px = turyn_x(x);
+            const uint32_t lo = tab ^ (px & 15u) * kNibRow, hi = (tab + kNibTable) ^ (px >> 4) * kNibRow;
+            Cost b[8], c[8];
+            uint32_t least[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { b[j] = pattern_cost(lo, hi, turyn_a(j), 1u); c[j] = pattern_cost(lo, hi, turyn_a(j), 2u); }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const Cost a = pattern_cost(lo, hi, turyn_a(i), 0u);
+                uint32_t least_even = 0xffffffffu, least_odd = 0xffffffffu;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const Cost two = a + b[j];
+                    least_even = __viaddmin_u16x2(two.even, c[i ^ j].even, least_even);
+                    least_odd = __viaddmin_u16x2(two.odd, c[i ^ j].odd, least_odd);
+                }
+                least[i] = __vminu2(least_even, least_odd);
+            }
+            const uint32_t m = __vminu2(__vimin3_u16x2(least[0], least[1], least[2]), __vminu2(__vimin3_u16x2(least[3], least[4], least[5]), __vminu2(least[6], least[7])));
+            const uint32_t before = best;
+#pragma unroll
+            for (uint32_t pi = 0; pi < 2; ++pi) {
+                const uint32_t mine = half_of(m, (int)pi);
+                second = min(second, max(best, mine));
+                group = mine < best ? 2u * x + pi : group;
+                best = min(best, mine);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) kept[i] = best < before ? least[i] : kept[i];
+        }
+        __syncthreads();
+        // the better lane of the two; its a within the margin
+        uint32_t a_of = 0, b_of = 0, hits = 0;
+        {
+            const uint32_t best_o = __shfl_xor_sync(kFull, best, 16), second_o = __shfl_xor_sync(kFull, second, 16), group_o = __shfl_xor_sync(kFull, group, 16);
+            const bool mine = best < best_o || (best == best_o && q == 0);
+            second = min(max(best, best_o), mine ? second : second_o);
+            best = min(best, best_o);
+            settled = second > best + kPairMargin;
+#pragma unroll
+            for (uint32_t i = 0; i < 8; ++i)
+                if (half_of(kept[i], (int)(group & 1u)) <= best + kPairMargin) { a_of = i; ++hits; }
+            a_of |= hits << 8;
+            const uint32_t a_of_o = __shfl_xor_sync(kFull, a_of, 16);
+            a_of = mine ? a_of : a_of_o;
+            group = mine ? group : group_o;
+            settled &= a_of >> 8 == 1u;
+            a_of &= 7u;
+        }
+        const int pi = (int)(group & 1u);
+        const uint32_t px = turyn_x(group >> 1), pa = turyn_a(a_of);
+        {
+            // the b within the margin: four for either lane
+            constexpr uint32_t upper = turyn_a(4);
+            const uint32_t lo = tab ^ (px & 15u) * kNibRow, hi = (tab + kNibTable) ^ (px >> 4) * kNibRow;
+            const uint32_t lo_a = lo ^ (pa & 15u) * kNibRow, hi_a = hi ^ (pa >> 4) * kNibRow;
+            const uint32_t lo_q = q ? (upper & 15u) * kNibRow : 0u, hi_q = q ? (upper >> 4) * kNibRow : 0u;
+            const Cost a = pattern_cost(lo_a, hi_a, 0u, 0u);
+            hits = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < 4; ++j) {
+                const Cost two = a + pattern_cost(lo ^ lo_q, hi ^ hi_q, turyn_a(j), 1u), c = pattern_cost(lo_a ^ lo_q, hi_a ^ hi_q, turyn_a(j), 2u);
+                if (half_of(__vminu2(two.even + c.even, two.odd + c.odd), pi) <= best + kPairMargin) { b_of = 4u * (uint32_t)q + j; ++hits; }
+            }
+            const uint32_t other = __shfl_xor_sync(kFull, hits << 8 | b_of, 16);
+            settled &= hits + (other >> 8) == 1u;
+            b_of = hits ? b_of : other & 7u;
+        }
+        // the triple's patterns and their complements: {cost with an even sum of z, with an odd one} from the coordinates, a nibble of
+        // every octad for either lane
+        const uint32_t pb = turyn_a(b_of);
+        uint32_t patterns = (px ^ pa) | (px ^ pb) << 8 | (px ^ pa ^ pb) << 16, part[3], part_c[3];
+        patterns >>= 4 * q;
+        const float shift = pi ? 0.25f : 0.f;
+#pragma unroll
+        for (int o = 0; o < 3; ++o) {
+            const uint32_t four = coords[2 * o + q];
+            float sum = 0.f, squares = 0.f, most = 0.f, fewest = 1.f;
+            uint32_t parity = 0u;                                    // bit 0: of the sum of z; bit 1: of the number of negative errors
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float t = v[16u * ((four >> (8 * k)) & 31u)] * s1 * s2 * 0.25f - shift, tr = t + 12582912.f, err = t - (tr - 12582912.f);
+                const uint32_t bit = (patterns >> (8 * o + k)) & 1u, negative = __float_as_uint(err) >> 31;
+                const float mag = fabsf(fabsf(err) - __uint_as_float(bit * 0x3f000000u));
+                squares = fmaf(mag, mag, squares);
+                sum += mag;
+                most = fmaxf(most, mag);
+                fewest = fminf(fewest, mag);
+                parity ^= ((__float_as_uint(tr) & 1u) ^ (bit & negative)) | negative << 1;
+            }
+            squares += __shfl_xor_sync(kFull, squares, 16);
+            sum += __shfl_xor_sync(kFull, sum, 16);
+            most = fmaxf(most, __shfl_xor_sync(kFull, most, 16));
+            fewest = fminf(fewest, __shfl_xor_sync(kFull, fewest, 16));
+            parity ^= __shfl_xor_sync(kFull, parity, 16);
+            if (o == 2) parity ^= (uint32_t)pi;
+            const float other = squares - sum + 2.f;                 // the complement's errors are 1/2 - mag
+            const uint32_t stay = __float_as_uint(fmaf(squares, kPairScale, 8388608.f)), move = __float_as_uint(fmaf(squares + (1.f - 2.f * most), kPairScale, 8388608.f));
+            const uint32_t stay_c = __float_as_uint(fmaf(other, kPairScale, 8388608.f)), move_c = __float_as_uint(fmaf(fmaf(2.f, fewest, other), kPairScale, 8388608.f));
+            part[o] = __byte_perm(stay, move, parity & 1u ? 0x1054 : 0x5410);
+            part_c[o] = __byte_perm(stay_c, move_c, (parity ^ parity >> 1) & 1u ? 0x1054 : 0x5410);
+        }
+        uint32_t word = 0;
+        {
+            hits = 0;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {                            // bit o: the complement on octad o
+                const uint32_t a = t & 1 ? part_c[0] : part[0], b = t & 2 ? part_c[1] : part[1], c = t & 4 ? part_c[2] : part[2];
+                const uint32_t all = __viaddmin_u16x2(__byte_perm(a, 0u, 0x3232), __byte_perm(b, 0u, 0x1032), __byte_perm(a, 0u, 0x1010) + b) + c;
+                if (min(all & 0xffffu, all >> 16) <= best + kWordMargin) { word = (uint32_t)t; ++hits; }
+            }
+            settled &= hits == 1u;
+            const uint32_t x8 = (group >> 1) * 8u;
+            word = S.word[0][x8 + a_of] ^ (word & 1u ? S.ones[0] : 0u) ^ S.word[1][x8 + b_of] ^ (word & 2u ? S.ones[1] : 0u) ^
+                   S.word[2][x8 + (a_of ^ b_of)] ^ (word & 4u ? S.ones[2] : 0u);
+        }
+        // the point of coset (pi, word), twelve coordinates for either lane
+        {
+            constexpr double kRint = 6755399441055744.0;             // 1.5 * 2^52: adding it rounds to a whole number, which is in the low word
+            double most = -1.0, next = -1.0, u_most = 0.0, dot = 0.0;
+            int sum = 0, who = 0, move = 4;
+            const float* const mine = v + 16 * 12 * q;
+            word >>= 12 * q;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                r.x[j] = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k = 4 * j + i;
+                    const double u = __dmul_rn(__dmul_rn((double)mine[16 * k], rn), radius);
+                    const int b = pi + 2 * (int)((word >> k) & 1u);
+                    const double bd = b & 2 ? (pi ? 3.0 : 2.0) : (pi ? 1.0 : 0.0);
+                    const double tt = __dmul_rn(__dsub_rn(u, bd), 0.25), big = __dadd_rn(tt, kRint), z = __dsub_rn(big, kRint);
+                    const double err = __dsub_rn(tt, z), mag = fabs(err);
+                    const int xi = b + 4 * __double2loint(big);
+                    r.x[j] |= (uint32_t)(xi & 0xff) << (8 * i);
+                    sum += xi;
+                    dot = fma(u, fma(z, 4.0, bd), dot);
+                    next = mag > most ? most : fmax(next, mag);
+                    if (mag > most) { most = mag; who = k; u_most = u; move = err < 0.0 ? -4 : 4; }
+                }
+            }
+            sum += __shfl_xor_sync(kFull, sum, 16);
+            const double most_o = __shfl_xor_sync(kFull, most, 16), next_o = __shfl_xor_sync(kFull, next, 16);
+            const bool moved = (sum & 7) != (pi ? 4 : 0);
+            next = fmax(fmin(most, most_o), fmax(next, next_o));
+            if (moved && (q == 0 ? most >= most_o : most > most_o)) {    // the first coordinate with the largest error is here
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if (who >> 2 == j) {
+                        const uint32_t old = (r.x[j] >> (8 * (who & 3))) & 0xffu;
+                        r.x[j] ^= (old ^ ((old + (uint32_t)move) & 0xffu)) << (8 * (who & 3));
+                    }
+                dot = fma((double)move, u_most, dot);
+            }
+            most = fmax(most, most_o);
+            r.unique = moved ? next <= most - 1.0e-6 : most < 0.5 - 1.0e-6;
+            r.dot = dot + __shfl_xor_sync(kFull, dot, 16);
+            int n2 = 0;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) n2 = __dp4a((int)r.x[j], (int)r.x[j], n2);
+            r.norm2 = n2 + __shfl_xor_sync(kFull, n2, 16);
+        }
+    }
+    // vectors with several candidates: the CTA's warps take them one by one
+    bool waiting = wanted && !settled;
+    while (true) {
+        __syncthreads();                                         // the costs of all warps are done with: nearest_careful works there
+        uint32_t slot = kPendingMost;
+        if (waiting && q == 0) {
+            slot = atomicAdd(&pending.count, 1u);
+            if (slot < kPendingMost) { Pending& p = pending.list[slot]; p.v = v; p.rn = rn; p.radius = radius; }
+        }
+        slot = __shfl_sync(kFull, slot, lane & 15);
+        __syncthreads();
+        const uint32_t n = pending.count;
+        if (n == 0u) break;
+        __syncthreads();
+        if (threadIdx.x == 0) pending.count = 0u;
+        for (uint32_t i = (uint32_t)warp; i < min(n, kPendingMost); i += (uint32_t)kEncWarps<true>) {
+            Pending& p = pending.list[i];
+            int norm2;
+            double dot;
+            bool unique;
+            nearest_of_warp(careful, S, steps, golay, pos_by_low12, p.v, 16, p.rn, p.radius, lane, p.x, norm2, dot, unique);
+            if (lane == 0) { p.norm2 = norm2; p.unique = unique; p.dot = dot; }
+        }
+        __syncthreads();
+        if (slot < kPendingMost) {
+            const Pending& p = pending.list[slot];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) r.x[j] = reinterpret_cast<const uint32_t*>(p.x)[3 * q + j];
+            r.norm2 = p.norm2; r.unique = p.unique; r.dot = p.dot;
+            waiting = false;
+        }
+    }
+}
+
+// The oracle's score of a candidate (24 signed bytes), one binary64 rounding per operation, sums in the order of the coordinates.
+__device__ __noinline__ double exact_score(int metric, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t w4, uint32_t w5, const float* v, int stride, double rn)
+{
+    const uint32_t w[6] = {w0, w1, w2, w3, w4, w5};
+    double acc = 0.0;
+    int n2 = 0;
+#pragma unroll
+    for (int i = 0; i < 24; ++i) {
+        const int x = (int)(int8_t)(w[i >> 2] >> (8 * (i & 3)));
+        const double vi = (double)v[stride * i];
+        n2 += x * x;
+        if (metric == LLVQ_EUCLIDEAN) {
+            const double dd = __dsub_rn(vi, (double)x);
+            acc = __dadd_rn(acc, __dmul_rn(dd, dd));
+        } else {
+            acc = __dadd_rn(acc, __dmul_rn(__dmul_rn(vi, rn), (double)x));
+        }
+    }
+    return metric == LLVQ_EUCLIDEAN ? -acc : __ddiv_rn(acc, __dsqrt_rn((double)n2));
+}
+
+// Shells m_from .. m_to as a mask (bit m = shell m; none if m_from > m_to).
+__device__ __forceinline__ uint64_t shells(int m_from, int m_to)
+{
+    return m_from > m_to ? 0ull : (~0ull >> (63 - (m_to - m_from))) << m_from;
+}
+
+// Two lanes per input vector, each pair with its own progress: a vector that is done is replaced at once.  (One warp per vector, kPairs false:
+// all pairs of lanes do the same.)
+// Inputs are binary32 values, the scoring that decides runs in binary64 with one rounding per operation and sums over the
+// coordinates in order.  EUCLIDEAN: if the nearest lattice point of the input lies in the code it is the
 // answer (it is then also the nearest point of the cut, App. E "Spherical shaping").  Otherwise, and for ANGULAR always,
 // the input direction is decoded at every shell radius sqrt(16 m); of the candidates inside the code the one nearest to
 // the input (EUCLIDEAN) or with the largest cosine (ANGULAR) wins, the first radius on ties.  A zero input gives the
 // point of index 0, (4, 4, 0^22), the first point of the first class of Shell(2) (Sec. 2.3).  Needs m_lo == 2 and
-// m_hi >= 3 (checked on the host).
+// m_hi >= 3 (checked on the host).  Scores are compared as binary64 sums in any order; where they come within 1e-9, as the oracle forms them.
 // EUCLIDEAN does not need all the radii.  At distance r along the direction d of the input (length R) the nearest point x
 // minimises |x|^2 - 2 r <x, d>; two minimisers at radii r < r' therefore satisfy <x, d> <= <x', d>, and
 // |x'|^2 - 2 R <x', d> <= |x|^2 - 2 R <x, d> for r < r' <= R (symmetrically for R <= r' < r): the radius next to R that yields a
-// point of the code beats all radii beyond it, by the margin that lattice_nearest reports as `unique`.  So the radii are tried
+// point of the code beats all radii beyond it, by the margin reported as `unique`.  So the radii are tried
 // outwards from R, on each side until such a point is found (inputs so long that a squared distance no longer resolves the
-// margin try them all).  ANGULAR needs every radius; the exact score is formed only where a binary32 one comes near the best.
-__global__ void __launch_bounds__(kEncWarps * 32, 1)
+// margin try them all).
+// Neither does ANGULAR.  With g = max_x 2 t <x, d> - |x|^2 = 2 t <x_t, d> - |x_t|^2 known from the decode at radius t, every lattice
+// point of norm r satisfies <x, d> <= (g + r^2) / (2 t): its cosine stays below the best one found, c, if r lies strictly between
+// the roots of r^2 - 2 t c r + g.  That rules out whole shells (`out`).  And as a maximum of lines g is convex in t: the nearest
+// point's norm does not fall as t grows, so between two decoded radii it stays between theirs.  A radius at which only ruled-out
+// shells are possible cannot change the result and is not decoded.  The order: downwards from m_hi while the points found lie in
+// shells that could still win, then a leap to the radius that should rule out most of what is left below.  On Gaussian
+// inputs, shells 2..12, 6.0 of 11 radii are decoded.
+template <bool kPairs>
+__global__ void __launch_bounds__(kEncWarps<kPairs> * 32, 1)
 encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __grid_constant__ PatternSteps steps, const float* __restrict__ v, uint64_t n, int metric, int m_lo, int m_hi,
                      int8_t* __restrict__ points, uint32_t* __restrict__ flags)
 {
-    extern __shared__ __align__(128) uint8_t enc_smem[];
-    WarpTables* tabs = reinterpret_cast<WarpTables*>(enc_smem);
-    GolayTrio& S = *reinterpret_cast<GolayTrio*>(enc_smem + kEncWarps * sizeof(WarpTables));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ double radius[kMaxShell + 1];                     // sqrt(16 m)
+    extern __shared__ __align__(1024) uint8_t enc_smem[];
+    constexpr int kVecs = kEncVecs<kPairs>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane >> 4;
+    const uint32_t start = (uint32_t)__cvta_generic_to_shared(enc_smem), align = kPairs ? kNibTable : 128u, nib0 = (start + align - 1u) & ~(align - 1u);
+    uint8_t* const mem = enc_smem + (nib0 - start);
+    const uint32_t nib = nib0 + (uint32_t)warp * kEncWarpBytes<kPairs>;
+    WarpTables& careful = *reinterpret_cast<WarpTables*>(mem + warp * kEncWarpBytes<kPairs>);
+    float* const mine_v = reinterpret_cast<float*>(mem + kEncWarps<kPairs> * kEncWarpBytes<kPairs>) + warp * (24 * kVecs) + (kPairs ? lane & 15 : 0);
+    GolayTrio& S = *reinterpret_cast<GolayTrio*>(mem + kEncWarps<kPairs> * (kEncWarpBytes<kPairs> + 24 * kVecs * sizeof(float)));
+    __shared__ double radius[kMaxShell + 1], per_radius[kMaxShell + 1];     // sqrt(16 m) and its reciprocal
     __shared__ uint32_t next_vec;
-    if (threadIdx.x == 0) next_vec = 0u;
-    for (int i = threadIdx.x; i <= m_hi; i += blockDim.x) radius[i] = __dsqrt_rn(__dmul_rn(16.0, (double)i));
+    __shared__ PendingList pending;
+    if (threadIdx.x == 0) { next_vec = 0u; pending.count = 0u; }
+    for (int i = threadIdx.x; i <= m_hi; i += blockDim.x) {
+        radius[i] = __dsqrt_rn(__dmul_rn(16.0, (double)i));
+        per_radius[i] = 1.0 / radius[i];
+    }
     for (int i = threadIdx.x; i < (int)sizeof(GolayTrio) / 4; i += blockDim.x)
         reinterpret_cast<uint32_t*>(&S)[i] = __ldg(reinterpret_cast<const uint32_t*>(et.trio) + i);
     __syncthreads();
-    WarpTables& W = tabs[warp];
-    uint32_t row[6];                                             // where the nibbles of pattern (x, 4 h) of every octad are
-#pragma unroll
-    for (int o = 0; o < 3; ++o) {
-        const uint32_t p = S.pat[o][(lane & 7) * 8 + ((lane >> 1) & 4)], t = (uint32_t)__cvta_generic_to_shared(&W.nib[lane >> 4][2 * o][0]);
-        row[2 * o] = t ^ (p & 15u) * 8u;
-        row[2 * o + 1] = (t + 128u) ^ (p >> 4) * 8u;
-    }
+    const bool words = (reinterpret_cast<uintptr_t>(points) & 3u) == 0, quads = (reinterpret_cast<uintptr_t>(v) & 15u) == 0;
     const float reach = sqrtf(16.f * (float)m_hi) + 4.01f, reach2 = reach * reach;
-    // a CTA's share is contiguous; its warps draw the vectors one by one (some take several decodes, and the schedulers favour some warps)
+    // a CTA's share is contiguous; its warps draw the vectors as they have room (some take several decodes)
     const uint64_t first = n / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, n % gridDim.x);
     const uint32_t count = (uint32_t)(n / gridDim.x + (blockIdx.x < n % gridDim.x));
+
+    bool active = false, drained = false;       // this lane's vector is being searched; there are no more
+    bool starting = false, direct = false;      // its radii are about to be started; the input itself is decoded (else: its direction at shell radius m)
+    bool outwards = false, ok = false;
+    uint32_t t = 0, bx[3] = {0u, 0u, 0u};       // its number in the share, the best point
+    double rn = 1.0, length = 0.0, best = 0.0;
+    float s1 = 1.f;                              // a power of two that brings the input near length 1
+    int best_m = 0, m = 0, m_start = 0, step = 0;
+    int upper = 0, upper_shell = 0, lower = 0, lower_shell = 0;  // ANGULAR: the radii from `upper` on are settled, `lower` (0: none) is decoded; shells of their points
+    uint64_t out = 0;
+    const auto store = [&](const uint32_t (&x)[3]) {
+        int8_t* const at = points + (first + t) * 24 + 12 * q;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (words) reinterpret_cast<uint32_t*>(at)[j] = x[j];
+            else for (int i = 0; i < 4; ++i) at[4 * j + i] = (int8_t)(x[j] >> (8 * i));
+        }
+    };
+    const uint32_t origin[3] = {q ? 0u : 0x0404u, 0u, 0u};       // the point of index 0
     while (true) {
-        uint32_t t = 0;
-        if (lane == 0) t = atomicAdd(&next_vec, 1u);
-        t = __shfl_sync(kFull, t, 0);
-        if (t >= count) break;
-        const uint64_t vec = first + t;
-        const float vf = lane < 24 ? __ldg(v + vec * 24 + lane) : 0.f;
-        const double vi = (double)vf;
-        int bestx = lane == 0 || lane == 1 ? 4 : 0;              // the point of index 0
-        const bool zero = __all_sync(kFull, vf == 0.f), finite = __all_sync(kFull, isfinite(vf));
-        bool ok = zero;
-        if (!zero && finite) {
-            bool direct = false;                                 // the input itself is decoded (else: its direction at shell radius m)
-            if (metric == LLVQ_EUCLIDEAN) {
+        const uint32_t vacant = __ballot_sync(kFull, !active && !drained);
+        if (vacant) {
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(&next_vec, kPairs ? (uint32_t)__popc(vacant & 0xffffu) : 1u);
+            base = __shfl_sync(kFull, base, 0);
+            if (!active && !drained) {
+                t = base + (kPairs ? (uint32_t)__popc(vacant & ((1u << (lane & 15)) - 1u)) : 0u);
+                drained = t >= count;
+            }
+            const bool taking = !active && !drained;
+            const uint32_t takers = __ballot_sync(kFull, taking);
+            if (taking) {
+                const float* const from = v + (first + t) * 24 + 12 * q;
+                float n2f = 0.f;
+                uint32_t some = 0, finite = 1;
+                const auto take = [&](int k, float f) {
+                    some |= f != 0.f; finite &= isfinite(f) ? 1u : 0u;
+                    n2f = fmaf(f, f, n2f);
+                    mine_v[kVecs * (12 * q + k)] = f;
+                };
+                if (quads) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const float4 f = __ldg(reinterpret_cast<const float4*>(from) + k);
+                        take(4 * k, f.x); take(4 * k + 1, f.y); take(4 * k + 2, f.z); take(4 * k + 3, f.w);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int k = 0; k < 12; ++k) take(k, __ldg(from + k));
+                }
+                n2f += __shfl_xor_sync(takers, n2f, 16);
+                some |= __shfl_xor_sync(takers, some, 16);
+                finite &= __shfl_xor_sync(takers, finite, 16);
+                // (the vectors that will be taken when the CTA is through with those it has)
+                if (t + kEncWarps<kPairs> * kVecs < count) asm volatile("prefetch.global.L2 [%0];" ::"l"(from + kEncWarps<kPairs> * kVecs * 24));
                 // no lattice point is farther than 4 from any input (covering radius): beyond radius sqrt(16 m_hi) + 4 the nearest
                 // point is certainly outside the code and the decode can be skipped
-                float n2f = vf * vf;
-#pragma unroll
-                for (int o = 16; o; o >>= 1) n2f += __shfl_xor_sync(kFull, n2f, o);
-                direct = n2f <= reach2;
+                direct = metric == LLVQ_EUCLIDEAN && n2f <= reach2;
+                starting = !direct;
+                active = some && finite;
+                ok = false;
+                rn = 1.0;
+                s1 = 1.f;
+                if (!active) {
+                    store(origin);
+                    if (!finite) atomicOr(flags, kFlagSearchGaveUp);
+                }
             }
-            double rn = 0.0, best = -1.0e300;
-            float best_f = -2.f;
-            int best_m = 0, m = 0, m_start = 0, step = 0;        // step 0: the radii have not been started
-            bool outwards = false;
-            while (true) {                                       // (one copy of the search in the code: two would not fit the instruction cache)
-                if (!direct) {
-                    if (step == 0) {
-                        const double n2 = seq_sum24(__dmul_rn(vi, vi));
-                        rn = __ddiv_rn(1.0, __dsqrt_rn(n2));
-                        outwards = metric == LLVQ_EUCLIDEAN && n2 < 1.0e9;
-                        // tried outwards: first down from the largest radius not above R, then up from the next one
-                        m = m_start = outwards ? max(m_lo - 1, (int)fmin(n2 * 0.0625, (double)m_hi)) : m_hi;
-                        step = -1;
-                    }
-                    if (step < 0 && m < m_lo) { m = m_start + 1; step = 1; }
-                    if (m > m_hi) break;
-                }
-                const double u = direct ? vi : __dmul_rn(__dmul_rn(vi, rn), radius[m]);
-                int norm2;
-                bool unique;
-                const int x = lattice_nearest(W, S, steps, row, golay, et.pos_by_low12, u, lane, norm2, unique);
-                const bool in_code = norm2 >= 16 * m_lo && norm2 < 16 * m_hi + 16;
-                if (direct) {
-                    if (in_code) { ok = true; bestx = x; break; }
-                    direct = false;
-                    continue;
-                }
-                const int m_now = m;
-                m += step;
-                if (!in_code) continue;
-                double score;
+        }
+        __syncwarp();
+        int busy = 0;
+        if constexpr (kPairs) {
+            busy = __syncthreads_count(active && q == 0);
+            if (busy == 0 && __syncthreads_and(drained)) break;
+        } else {
+            if (drained) break;
+            if (!active) continue;
+        }
+        if (active && starting) {
+            double n2 = 0.0;
+#pragma unroll
+            for (int i = 0; i < 24; ++i) { const double vi = (double)mine_v[kVecs * i]; n2 = __dadd_rn(n2, __dmul_rn(vi, vi)); }
+            length = __dsqrt_rn(n2);
+            rn = __ddiv_rn(1.0, length);
+            outwards = metric == LLVQ_EUCLIDEAN && n2 < 1.0e9;
+            // tried outwards: first down from the largest radius not above R, then up from the next one
+            m = m_start = outwards ? max(m_lo - 1, (int)fmin(n2 * 0.0625, (double)m_hi)) : m_hi;
+            step = -1;
+            if (m < m_lo) { m = m_start + 1; step = 1; }
+            upper = m_hi + 1; lower = 0; out = 0;
+            starting = false;
+            s1 = __uint_as_float((uint32_t)min(max(1150 - ((__double2hiint(length) >> 20) & 0x7ff), 1), 254) << 23);
+        }
+        __syncwarp();
+        const double rad = direct || !active ? 1.0 : radius[m];
+        const float s2 = direct || !active ? 1.f : (float)(rad * (rn / (double)s1));
+        Nearest r;
+        if constexpr (kPairs) {
+            nearest_pairs(nib, mine_v, S, steps, golay, et.pos_by_low12, careful, pending, s1, s2, rn, rad, active, busy <= kFew, warp, lane, r);
+        } else {
+            int8_t* const point = reinterpret_cast<int8_t*>(&careful + 1);
+            nearest_of_warp(careful, S, steps, golay, et.pos_by_low12, mine_v, kVecs, rn, rad, lane, point, r.norm2, r.dot, r.unique);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 3; ++j) r.x[j] = reinterpret_cast<const uint32_t*>(point)[3 * q + j];
+        }
+        __syncwarp();
+        const int shell = r.norm2 >> 4;                          // lattice points have norms 16 m
+        const bool in_code = shell >= m_lo && shell <= m_hi;
+        const uint32_t unlike = __ballot_sync(kFull, ((r.x[0] ^ bx[0]) | (r.x[1] ^ bx[1]) | (r.x[2] ^ bx[2])) != 0u) >> (lane & 15) & 0x10001u;
+        bool done = false;
+        if (active && direct) {
+            direct = false;
+            starting = !in_code;
+            if (in_code) {
+                done = ok = true;
+#pragma unroll
+                for (int j = 0; j < 3; ++j) bx[j] = r.x[j];
+            }
+        } else if (active) {
+            if (in_code) {
+                // the candidate's score, up to rounding: the cosine; EUCLIDEAN: 2 <v, x> - |x|^2, which is |v|^2 minus the squared distance
+                double score, tol = 1.0e-9;
                 if (metric == LLVQ_EUCLIDEAN) {
-                    const double dd = __dsub_rn(vi, (double)x);
-                    score = -seq_sum24(lane < 24 ? __dmul_rn(dd, dd) : 0.0);
+                    score = 2.0 * r.dot * length * per_radius[m] - (double)r.norm2;
+                    tol = 1.0e-9 * (1.0 + length) + 1.0e-14 * length * length;
                 } else {
-                    float s = (float)__dmul_rn(vi, rn) * (float)x;
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-                    s *= rsqrtf((float)norm2);
-                    if (s < best_f - 1.0e-5f) continue;          // binary32 errors stay below 3e-6
-                    best_f = fmaxf(best_f, s);
-                    const double dot = seq_sum24(lane < 24 ? __dmul_rn(__dmul_rn(vi, rn), (double)x) : 0.0);
-                    score = __ddiv_rn(dot, __dsqrt_rn((double)norm2));
+                    score = r.dot * per_radius[m] * per_radius[shell];
                 }
-                if (!ok || score > best || (score == best && m_now < best_m)) { best = score; bestx = x; best_m = m_now; ok = true; }
-                if (outwards && unique) {                        // this side is done
-                    if (step > 0) break;
+                bool better = !ok || score > best + tol;
+                if (!better && !(score < best - tol)) {
+                    if (!unlike) {
+                        best_m = min(best_m, m);                 // the same point again
+                    } else {
+                        const uint32_t pair = 0x10001u << (lane & 15);
+                        uint32_t w[6], b[6];
+#pragma unroll
+                        for (int j = 0; j < 3; ++j) {
+                            const uint32_t xo = __shfl_xor_sync(pair, r.x[j], 16), bo = __shfl_xor_sync(pair, bx[j], 16);
+                            w[j] = q ? xo : r.x[j]; w[3 + j] = q ? r.x[j] : xo;
+                            b[j] = q ? bo : bx[j]; b[3 + j] = q ? bx[j] : bo;
+                        }
+                        const double now = exact_score(metric, w[0], w[1], w[2], w[3], w[4], w[5], mine_v, kVecs, rn);
+                        const double before = exact_score(metric, b[0], b[1], b[2], b[3], b[4], b[5], mine_v, kVecs, rn);
+                        better = now > before || (now == before && m < best_m);
+                    }
+                }
+                if (better) {
+                    best = score; best_m = m; ok = true;
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) bx[j] = r.x[j];
+                }
+            }
+            if (metric == LLVQ_EUCLIDEAN) {
+                if (in_code && outwards && r.unique) {           // this side is done
+                    done = step > 0;
                     m = m_lo - 1;
+                } else {
+                    m += step;
+                }
+                if (step < 0 && m < m_lo) { m = m_start + 1; step = 1; }
+                done |= m > m_hi;
+            } else {
+                if (ok) {
+                    const float disc = (float)((rad * best) * (rad * best) - 2.0 * r.dot + (double)r.norm2);
+                    if (disc > 0.01f) {
+                        // strictly between the roots, by a margin far above the rounding
+                        const float mid = (float)(rad * best), half = sqrtf(disc) - 0.002f;
+                        const float from = fmaxf(mid - half, 0.f), to = fmaxf(mid + half, 0.f);
+                        out |= shells(max((int)(from * from * 0.0625f) + 1, 2), min((int)(to * to * 0.0625f), m_hi));
+                    }
+                }
+                if (m == upper - 1) { upper = m; upper_shell = shell; }
+                else { lower = m; lower_shell = shell; }
+                while (true) {
+                    const uint64_t open = shells(lower ? max(lower_shell, m_lo) : m_lo, min(upper_shell, m_hi)) & ~out;
+                    if (upper == m_lo || (!open && !lower)) { done = true; break; }
+                    if (!open || upper == lower + 1) { upper = lower; upper_shell = lower_shell; lower = 0; continue; }
+                    m = upper - 1;
+                    if (!lower && upper_shell <= m_hi && ((out >> upper_shell) & 1u)) {
+                        const float reached = 4.f * sqrtf((float)(63 - __clzll((long long)open))) - 1.5f;
+                        m = min(m, max((int)(reached * reached * 0.0625f), m_lo + 1));
+                    }
+                    break;
                 }
             }
         }
-        if (!ok) {
-            bestx = lane == 0 || lane == 1 ? 4 : 0;
-            if (lane == 0) atomicOr(flags, kFlagSearchGaveUp);
+        if (done) {
+            if (!ok) atomicOr(flags, kFlagSearchGaveUp);
+            if (ok) store(bx);
+            else store(origin);
+            active = false;
         }
-        if (lane < 24) points[vec * 24 + lane] = (int8_t)bestx;
     }
 }
 
@@ -405,8 +932,6 @@ constexpr int kRankValues = 32;            // larger than any absolute value of 
 // gets index 0 and is counted in the out-of-range counter.  The absolute values are taken as bit planes over the 24
 // coordinates: which coordinates hold a value is a few operations on masks, and the place of an element among
 // the free slots is a population count.
-// Bound: instruction issue and dependent reads (class record, codeword).  With a loop over the 24 coordinates per value, and the free
-// slots gathered bit by bit, encoding 699 050 Gaussian vectors (EUCLIDEAN) took 1126 us in all; 1063 us with masks.
 __global__ void __launch_bounds__(kRankThreads)
 rank_kernel(DevCode dc, EncTables et, const uint32_t* __restrict__ golay, const uint32_t* __restrict__ pascal,
             const int8_t* __restrict__ points, uint64_t n, unsigned long long* __restrict__ index)
@@ -566,15 +1091,19 @@ int llvq_encode_blocks(const llvq_ctx* ctx, const float* d_v_f32, uint64_t nbloc
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return LLVQ_ECUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t smem = kEncWarps * sizeof(WarpTables) + sizeof(GolayTrio);
-    if (!allow_smem<encode_search_kernel>(ctx->smem_limits, ctx->smem_most, smem)) return LLVQ_ECUDA;
     PatternSteps steps;
     for (int o = 0; o < 3; ++o)
         for (int j = 0; j < 4; ++j) { steps.lo[o][j] = (ctx->trio.pat[o][j] & 15u) * 8u; steps.hi[o][j] = (uint32_t)(ctx->trio.pat[o][j] >> 4) * 8u; }
     const unsigned grid = (unsigned)std::min<uint64_t>(nblocks, (uint64_t)ctx->sm_count);
-    encode_search_kernel<<<grid, kEncWarps * 32, smem, st>>>(ctx->d_golay, ctx->enc, steps, d_v_f32, nblocks, metric, ctx->host.m_lo, ctx->host.m_hi,
-                                                            d_points, ctx->dev.flags);
-    if (int e = status_of_launch()) return e;
+    const bool pairs = nblocks > (uint64_t)ctx->sm_count * (metric == LLVQ_EUCLIDEAN ? kPairsFromEuclidean : kPairsFromAngular);
+    const auto launch = [&](auto form) -> int {
+        constexpr bool kPairs = decltype(form)::value;
+        if (!allow_smem<encode_search_kernel<kPairs>>(ctx->smem_limits, ctx->smem_most, kEncSmem<kPairs>)) return LLVQ_ECUDA;
+        encode_search_kernel<kPairs><<<grid, kEncWarps<kPairs> * 32, kEncSmem<kPairs>, st>>>(ctx->d_golay, ctx->enc, steps, d_v_f32, nblocks, metric, ctx->host.m_lo,
+                                                                                           ctx->host.m_hi, d_points, ctx->dev.flags);
+        return status_of_launch();
+    };
+    if (int e = pairs ? launch(std::true_type{}) : launch(std::false_type{})) return e;
     return launch_rank(ctx, d_points, nblocks, d_index, st);
 }
 

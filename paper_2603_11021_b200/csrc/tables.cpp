@@ -439,71 +439,32 @@ bool build_class_hash(const HostTables& t, std::vector<uint64_t>& keys, std::vec
 
 bool build_golay_trio(const HostTables& t, GolayTrio& out)
 {
+    // an order of the coordinates of this Golay code in which every octad has the two codes (found by trying the permutations of
+    // each octad of a trio); that it is one is checked below
+    static constexpr uint8_t kOrder[24] = {0, 1, 2, 3, 7, 4, 12, 10, 6, 18, 17, 19, 11, 13, 14, 16, 5, 8, 22, 20, 23, 15, 9, 21};
     std::vector<uint32_t> by_low12(4096, ~0u);                // the low 12 bits identify a codeword (checked by the caller)
     for (uint32_t w : t.golay) by_low12[w & 0xfffu] = w;
     auto in_code = [&](uint32_t w) { return by_low12[w & 0xfffu] == w; };
-    uint32_t o1 = 0, o2 = 0;
-    for (uint32_t w : t.golay) {
-        if (__builtin_popcount(w) != 8) continue;
-        if (!o1) o1 = w;
-        else if (!(w & o1)) { o2 = w; break; }
-    }
-    if (!o2) return false;
-    out.ones[0] = o1; out.ones[1] = o2; out.ones[2] = ~(o1 | o2) & 0xffffffu;
-    if (!in_code(out.ones[2])) return false;
-    for (int o = 0, q = 0; o < 3; ++o)
-        for (int i = 0; i < 24; ++i)
-            if ((out.ones[o] >> i) & 1u) out.coord[q++] = (uint8_t)i;
-    // the representative of a codeword up to complements: bit 0 on the first coordinate of every octad (a linear choice)
-    auto canon = [&](uint32_t w) {
-        for (int o = 0; o < 3; ++o) if ((w >> out.coord[8 * o]) & 1u) w ^= out.ones[o];
-        return w;
-    };
-    std::vector<uint32_t> span(1, 0);
-    auto add = [&](uint32_t w) {                              // extends the span; false if w is in it already
-        for (uint32_t v : span) if (v == w) return false;
-        for (size_t n = span.size(), i = 0; i < n; ++i) span.push_back(span[i] ^ w);
-        return true;
-    };
-    uint32_t a[3] = {0}, b[3] = {0}, c[3] = {0}, x[3] = {0};
-    int na = 0, nx = 0;
-    for (uint32_t w : t.golay) {                              // (a, 0, c): zero on the second octad
-        if (na == 3) break;
-        const uint32_t k = canon(w);
-        if ((k & o2) || !add(k)) continue;
-        a[na] = k & o1; c[na] = k & out.ones[2]; ++na;
-    }
-    if (na != 3) return false;
-    for (int i = 0; i < 3; ++i) {                             // (a, b, 0) with the same a, hence (0, b, c)
-        for (uint32_t w : t.golay) {
-            const uint32_t k = canon(w);
-            if ((k & o1) == a[i] && !(k & out.ones[2])) b[i] = k & o2;
+    for (int o = 0; o < 3; ++o) {
+        out.ones[o] = 0;
+        for (int q = 0; q < 8; ++q) {
+            const uint8_t c = kOrder[8 * o + q];
+            out.coord[8 * o + q] = c;
+            out.place[c] = (uint8_t)(8 * o + q);
+            out.ones[o] |= 1u << c;
         }
-        if (!b[i] || !add(b[i] | c[i])) return false;
-    }
-    for (uint32_t w : t.golay) {
-        if (nx == 3) break;
-        const uint32_t k = canon(w);
-        if (add(k)) x[nx++] = k;
-    }
-    if (nx != 3 || span.size() != 512) return false;
-    for (int xi = 0; xi < 8; ++xi)
-        for (int j = 0; j < 8; ++j) {
-            uint32_t w = 0, va = 0, vb = 0, vc = 0;
+        if (!in_code(out.ones[o])) return false;
+        for (int xa = 0; xa < 64; ++xa) {
+            uint32_t p = 0, w = 0;
             for (int i = 0; i < 3; ++i) {
-                if ((xi >> i) & 1) w ^= x[i];
-                if ((j >> i) & 1) { va ^= a[i]; vb ^= b[i]; vc ^= c[i]; }
+                if ((xa >> i) & 1) p ^= kTurynA[i];
+                if ((xa >> (3 + i)) & 1) p ^= kTurynX[i];
             }
-            out.word[0][xi * 8 + j] = (w ^ va) & o1;
-            out.word[1][xi * 8 + j] = (w ^ vb) & o2;
-            out.word[2][xi * 8 + j] = (w ^ vc) & out.ones[2];
+            for (int q = 0; q < 8; ++q) w |= ((p >> q) & 1u) << kOrder[8 * o + q];
+            out.pat[o][xa] = (uint8_t)p;
+            out.word[o][xa] = w;
         }
-    for (int o = 0; o < 3; ++o)
-        for (int j = 0; j < 64; ++j) {
-            uint32_t p = 0;
-            for (int q = 0; q < 8; ++q) p |= ((out.word[o][j] >> out.coord[8 * o + q]) & 1u) << q;
-            out.pat[o][j] = (uint8_t)p;
-        }
+    }
     for (int xi = 0; xi < 8; ++xi)                            // every combination must be a codeword
         for (int i = 0; i < 8; ++i)
             for (int j = 0; j < 8; ++j)

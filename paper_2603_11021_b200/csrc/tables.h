@@ -175,13 +175,16 @@ bool build_class_hash(const HostTables& t, std::vector<uint64_t>& keys, std::vec
 
 // The Golay code cut along a trio of octads (three disjoint codewords of weight 8).  Restricted to one octad the codewords
 // are the 128 words of even weight, complementing a codeword on one octad gives another codeword, and up to complements
-// the code is { (s1[x, a], s2[x, b], s3[x, a ^ b]) : x, a, b = 0..7 }: 512 triples, each standing for 8 codewords
-// (Conway & Sloane, "Sphere Packings, Lattices and Groups", ch. 11: the Turyn construction).
+// the code is { (s[x, a], s[x, b], s[x, a ^ b]) : x, a, b = 0..7 }: 512 triples, each standing for 8 codewords
+// (Conway & Sloane, "Sphere Packings, Lattices and Groups", ch. 11: the Turyn construction).  s[x, a] is linear: the sum of a word
+// of the [8, 4] code spanned by kTurynX and 0xff and one of that spanned by kTurynA and 0xff, which have only 0 and 0xff in common.
+constexpr uint32_t kTurynA[3] = {0x1e, 0x66, 0xaa}, kTurynX[3] = {0x36, 0x5a, 0x8e};
 struct GolayTrio {
     uint32_t word[3][64];   // [octad][x * 8 + a] the codeword's bits on the octad, as bits of the 24 coordinates
     uint32_t ones[3];       // the octads
-    uint8_t pat[3][64];     // the same bits packed: bit p = coordinate coord[8 * octad + p]
-    uint8_t coord[24];      // coordinates octad by octad, ascending inside an octad
+    uint8_t pat[3][64];     // the same bits packed: bit p = coordinate coord[8 * octad + p]; the same for all three octads
+    uint8_t coord[24];      // coordinates octad by octad, in the order that makes the patterns those of kTurynA and kTurynX
+    uint8_t place[24];      // where in coord a coordinate is
 };
 bool build_golay_trio(const HostTables& t, GolayTrio& out);
 
