@@ -351,7 +351,7 @@ __device__ __forceinline__ void nearest_of_warp(WarpTables& W, const GolayTrio& 
 // ANGULAR 5000 76 / 90, 12 000 132 / 178, 30 000 278 / 207.
 constexpr uint64_t kPairsFromEuclidean = 208, kPairsFromAngular = 128;
 constexpr int kFew = 40;                   // no more vectors than this left in a CTA: all of them go to nearest_careful (EUCLIDEAN 867 -> 761 us with the wider loads)
-constexpr uint32_t kPendingMost = 48;
+constexpr uint32_t kPendingMost = 48, kPendingEnough = 14;
 struct Pending {
     double rn, radius, dot;
     const float* v;
@@ -379,17 +379,19 @@ struct PendingList {
 // evaluated as the oracle does: coordinate by coordinate, one binary64 rounding per operation, the first coordinate with the
 // largest error moving where the sum rule asks for it.  Wherever a second candidate lies within the margin (one vector in
 // sixty) the vector goes to nearest_careful, one per warp.  So the result does not depend on the first stage's rounding.
-// Bound: instruction issue (55 % of the slots) and the load / store pipe by turns: the warps in step read their tables together and then
-// compute together.  Against nearest_careful for every vector, 24 warps: 818 -> 430 warp instructions per search; 699 050 vectors EUCLIDEAN
-// 1063 -> 737 us, 174 763 ANGULAR on shells 2..12 2035 -> 796 us (of it 2035 -> 1430 by the radii left out).
-// All threads of the CTA call this together; `wanted` = this lane's vector is to be searched, `few` = so few of the CTA's are that
-// nearest_careful takes them all.
+// Bound: the logic pipe (62 % busy, issue 57 %) and what a block barrier costs.  Against nearest_careful for every vector, 24 warps: 818 -> 400 warp
+// instructions per search; 699 050 vectors EUCLIDEAN 1063 -> 669 us, 174 763 ANGULAR on shells 2..12 2035 -> 722 us (of it 2035 -> 1430 by the
+// radii left out).
+// All threads of the CTA call this together; `wanted` = this lane's vector is to be searched, `waiting` = it is on the list for
+// nearest_careful at `spot`, `few` = so few of the CTA's are left that nearest_careful takes them all.  Returns whether r is the answer
+// for this lane's vector.  (The list is worked off when almost every warp gets one of it, not after every search: 709 -> 695 us EUCLIDEAN.)
 // The block barriers keep the warps in step: the code is long (some 1500 instructions once through, half of them four times), and warps that are
 // each somewhere else in it fetch more instructions than the SM delivers (2 warps per scheduler: 3.0 of 5.8 stall cycles per
-// instruction were fetches; 0.1 of 3.9 with the barriers, 1329 -> 942 us for the 174 763 vectors of the ANGULAR case).
-__device__ __forceinline__ void nearest_pairs(uint32_t nib, const float* v, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
+// instruction were fetches; 0.1 of 3.9 with the barriers, 1329 -> 942 us for the 174 763 vectors of the ANGULAR case).  One per search:
+// with one per x the warps read their tables all at the same time and then computed (737 and 796 us, 709 and 762 with one per search).
+__device__ __forceinline__ bool nearest_pairs(uint32_t nib, const float* v, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
                                               const uint16_t* __restrict__ pos_by_low12, WarpTables& careful, PendingList& pending, float s1, float s2, double rn,
-                                              double radius, bool wanted, bool few, int warp, int lane, Nearest& r)
+                                              double radius, bool wanted, bool& waiting, uint32_t& spot, bool few, int warp, int lane, Nearest& r)
 {
     const int q = lane >> 4;
     bool settled = false;
@@ -436,7 +438,6 @@ __device__ __forceinline__ void nearest_pairs(uint32_t nib, const float* v, cons
         for (int i = 0; i < 8; ++i) kept[i] = 0u;
 #pragma unroll 1
         for (uint32_t x = 4u * (uint32_t)q; x < 4u * (uint32_t)q + 4u; ++x) {
-            __syncthreads();
             const uint32_t px = turyn_x(x);
             const uint32_t lo = tab ^ (px & 15u) * kNibRow, hi = (tab + kNibTable) ^ (px >> 4) * kNibRow;
             Cost b[8], c[8];
@@ -445,15 +446,18 @@ __device__ __forceinline__ void nearest_pairs(uint32_t nib, const float* v, cons
             for (int j = 0; j < 8; ++j) { b[j] = pattern_cost(lo, hi, turyn_a(j), 1u); c[j] = pattern_cost(lo, hi, turyn_a(j), 2u); }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const Cost a = pattern_cost(lo, hi, turyn_a(i), 0u);
-                uint32_t least_even = 0xffffffffu, least_odd = 0xffffffffu;
+                // the other two octads together for an even and for an odd sum of this one's z: four instructions for each b (six with the
+                // first two octads combined first: 695 -> 669 us EUCLIDEAN, 749 -> 722 us ANGULAR)
+                uint32_t even = 0xffffffffu, odd = 0xffffffffu;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const Cost two = a + b[j];
-                    least_even = __viaddmin_u16x2(two.even, c[i ^ j].even, least_even);
-                    least_odd = __viaddmin_u16x2(two.odd, c[i ^ j].odd, least_odd);
+                    even = __viaddmin_u16x2(b[j].even, c[i ^ j].even, even);
+                    odd = __viaddmin_u16x2(b[j].odd, c[i ^ j].even, odd);
+                    even = __viaddmin_u16x2(b[j].odd, c[i ^ j].odd, even);
+                    odd = __viaddmin_u16x2(b[j].even, c[i ^ j].odd, odd);
                 }
-                least[i] = __vminu2(least_even, least_odd);
+                const Cost a = pattern_cost(lo, hi, turyn_a(i), 0u);
+                least[i] = __viaddmin_u16x2(a.odd, odd, a.even + even);
             }
             const uint32_t m = __vminu2(__vimin3_u16x2(least[0], least[1], least[2]), __vminu2(__vimin3_u16x2(least[3], least[4], least[5]), __vminu2(least[6], least[7])));
             const uint32_t before = best;
@@ -601,19 +605,22 @@ __device__ __forceinline__ void nearest_pairs(uint32_t nib, const float* v, cons
             r.norm2 = n2 + __shfl_xor_sync(kFull, n2, 16);
         }
     }
-    // vectors with several candidates: the CTA's warps take them one by one
-    bool waiting = wanted && !settled;
+    // vectors with several candidates wait until there is one for almost every warp, or nothing else to do
+    bool found = wanted && settled;
+    waiting |= wanted && !settled;
     while (true) {
         __syncthreads();                                         // the costs of all warps are done with: nearest_careful works there
-        uint32_t slot = kPendingMost;
-        if (waiting && q == 0) {
-            slot = atomicAdd(&pending.count, 1u);
-            if (slot < kPendingMost) { Pending& p = pending.list[slot]; p.v = v; p.rn = rn; p.radius = radius; }
+        if (waiting && spot >= kPendingMost) {
+            uint32_t mine = 0;
+            if (q == 0) {
+                mine = atomicAdd(&pending.count, 1u);
+                if (mine < kPendingMost) { Pending& p = pending.list[mine]; p.v = v; p.rn = rn; p.radius = radius; }
+            }
+            spot = __shfl_sync(__activemask(), mine, lane & 15);
         }
-        slot = __shfl_sync(kFull, slot, lane & 15);
         __syncthreads();
         const uint32_t n = pending.count;
-        if (n == 0u) break;
+        if (n < (few ? 1u : kPendingEnough)) break;
         __syncthreads();
         if (threadIdx.x == 0) pending.count = 0u;
         for (uint32_t i = (uint32_t)warp; i < min(n, kPendingMost); i += (uint32_t)kEncWarps<true>) {
@@ -625,14 +632,18 @@ __device__ __forceinline__ void nearest_pairs(uint32_t nib, const float* v, cons
             if (lane == 0) { p.norm2 = norm2; p.unique = unique; p.dot = dot; }
         }
         __syncthreads();
-        if (slot < kPendingMost) {
-            const Pending& p = pending.list[slot];
+        if (waiting && spot < kPendingMost) {
+            const Pending& p = pending.list[spot];
 #pragma unroll
             for (int j = 0; j < 3; ++j) r.x[j] = reinterpret_cast<const uint32_t*>(p.x)[3 * q + j];
             r.norm2 = p.norm2; r.unique = p.unique; r.dot = p.dot;
             waiting = false;
+            found = true;
         }
+        spot = kPendingMost;
+        if (n <= kPendingMost) break;
     }
+    return found;
 }
 
 // The oracle's score of a candidate (24 signed bytes), one binary64 rounding per operation, sums in the order of the coordinates.
@@ -717,6 +728,8 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
 
     bool active = false, drained = false;       // this lane's vector is being searched; there are no more
     bool starting = false, direct = false;      // its radii are about to be started; the input itself is decoded (else: its direction at shell radius m)
+    bool waiting = false;                       // it is on the list for nearest_careful, at `spot`
+    uint32_t spot = kPendingMost;
     bool outwards = false, ok = false;
     uint32_t t = 0, bx[3] = {0u, 0u, 0u};       // its number in the share, the best point
     double rn = 1.0, length = 0.0, best = 0.0;
@@ -785,9 +798,12 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
         }
         __syncwarp();
         int busy = 0;
+        bool few = false, found = true;
         if constexpr (kPairs) {
             busy = __syncthreads_count(active && q == 0);
             if (busy == 0 && __syncthreads_and(drained)) break;
+            // (also where all that are left wait)
+            few = busy <= kFew || __syncthreads_count(active && !waiting) == 0;
         } else {
             if (drained) break;
             if (!active) continue;
@@ -812,7 +828,7 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
         const float s2 = direct || !active ? 1.f : (float)(rad * (rn / (double)s1));
         Nearest r;
         if constexpr (kPairs) {
-            nearest_pairs(nib, mine_v, S, steps, golay, et.pos_by_low12, careful, pending, s1, s2, rn, rad, active, busy <= kFew, warp, lane, r);
+            found = nearest_pairs(nib, mine_v, S, steps, golay, et.pos_by_low12, careful, pending, s1, s2, rn, rad, active && !waiting, waiting, spot, few, warp, lane, r);
         } else {
             int8_t* const point = reinterpret_cast<int8_t*>(&careful + 1);
             nearest_of_warp(careful, S, steps, golay, et.pos_by_low12, mine_v, kVecs, rn, rad, lane, point, r.norm2, r.dot, r.unique);
@@ -825,7 +841,8 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
         const bool in_code = shell >= m_lo && shell <= m_hi;
         const uint32_t unlike = __ballot_sync(kFull, ((r.x[0] ^ bx[0]) | (r.x[1] ^ bx[1]) | (r.x[2] ^ bx[2])) != 0u) >> (lane & 15) & 0x10001u;
         bool done = false;
-        if (active && direct) {
+        if (!found || !active) {
+        } else if (direct) {
             direct = false;
             starting = !in_code;
             if (in_code) {
@@ -833,7 +850,7 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
 #pragma unroll
                 for (int j = 0; j < 3; ++j) bx[j] = r.x[j];
             }
-        } else if (active) {
+        } else {
             if (in_code) {
                 // the candidate's score, up to rounding: the cosine; EUCLIDEAN: 2 <v, x> - |x|^2, which is |v|^2 minus the squared distance
                 double score, tol = 1.0e-9;
