@@ -61,6 +61,14 @@ void sorted_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext, uint
     bytes = (ext ? ctx->fl.total_ext : ctx->fl.total) + rest + acc_floats * 4;
 }
 
+// Where every unit of a matrix has a warp of its own, codes with many classes have nothing to gain from ordering their blocks first: the direct kernel with
+// binary32 FMAs.  Shells 2..13, us for gemv_bin_kernel / the direct kernel by units per CTA (of 148): 1 10.4 / 6.2, 5 10.2 / 6.6, 10 9.9 / 6.4, 13 9.0 / 7.0,
+// 19 10.7 / 7.3, 27 10.0 / 8.3; with two rounds 37 13.1 / 13.2.
+constexpr int64_t kOneRound = 32;
+// With two CTAs per row group, or one, a row's sum takes one exchange or none instead of a tree of them: about 1 us, which some ten units more per CTA cost
+// (512 x 1024 7.9 -> 6.6 us, 1000 x 1000 8.0 -> 6.4).
+constexpr int64_t kMoreUnits = 10;
+
 // Shared by llvq_gemv, llvq_gemv_sg and llvq_gemv_rowshard: exactly one of d_gain_f16 / sg is used.
 int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f16, const SgArgs* sg, int64_t n_out, int64_t k_in,
                        const uint16_t* d_x_bf16, const YOut& yo, int y_dtype, void* stream)
@@ -91,8 +99,16 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const size_t smem = (ext_direct ? ctx->fl.total_ext : ctx->fl.total) + rest;
     if (smem > kSmemMax || n_out > 64ll * kMaxScratchRows) return LLVQ_EUNSUPPORTED;
     const int64_t units = ((n_out + kGemvGroupRows - 1) / kGemvGroupRows) * nq;
-    const unsigned g = (unsigned)std::min<int64_t>(units, ctx->sm_count);
-    const Split sp = make_split(units, nq, g);
+    unsigned g = (unsigned)std::min<int64_t>(units, ctx->sm_count);
+    const bool one_round = units <= kOneRound * g;
+    if (one_round) {
+        const int64_t groups = units / nq, per_group = std::min<int64_t>(ctx->sm_count / groups, 2);
+        if (per_group > 0) {
+            const int64_t most = (nq + per_group - 1) / per_group;
+            if (most <= kOneRound && most <= (units + g - 1) / g + kMoreUnits) g = (unsigned)std::min(groups * per_group, units);
+        }
+    }
+    const Split sp = make_gemv_split(units, nq, g, n_out);
     // warps per CTA: the count in [28, 32] that wastes the fewest warp slots on the units of one CTA
     const int64_t upc = (units + g - 1) / g;
     int warps = 32; double best_eff = 0.0;
@@ -112,7 +128,11 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     OrderArgs oa;
     size_t smem_order; bool ext_order;
     const bool order = order_smem(ctx, nq, sg ? sg->bits : 0, oa, smem_order, ext_order);
-    if (bin_kernel_serves(ctx, nq, sg, order) && (one_segment(upc) || !order)) {
+    const bool bin = bin_kernel_serves(ctx, nq, sg, order) && (one_segment(upc) || !order);
+    const size_t rest_fma = rest_x + kSortAccFloats * 4;
+    const bool ext_fma = ctx->fl.total_ext + rest_fma <= kSmemLimit, fma = one_round && (bin || order) && ctx->fl.total + rest_fma <= kSmemLimit;
+    const size_t smem_fma = (ext_fma ? ctx->fl.total_ext : ctx->fl.total) + rest_fma;
+    if (bin && !fma) {
         const FastArgs fa = fast_args(ctx, ext_bin);
 #define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
     do {                                                                                                                   \
@@ -126,7 +146,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
 #undef LLVQ_LAUNCH_BIN
         return launch_status();
     }
-    if (order) {
+    if (order && !fma) {
         const FastArgs fa = fast_args(ctx, ext_order);
 #define LLVQ_LAUNCH_ORDER(BF16, SG, SH)                                                                               \
     do {                                                                                                                   \
@@ -141,18 +161,23 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
 #undef LLVQ_LAUNCH_ORDER
         return launch_status();
     }
-    const FastArgs fa = fast_args(ctx, ext_direct);
-#define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH)                                                                        \
+    const FastArgs fa = fast_args(ctx, fma ? ext_fma : ext_direct);
+#define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH, FMA)                                                                   \
     do {                                                                                                           \
-        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH>>(ctx, smem)) return LLVQ_ECUDA;                               \
-        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH>, g, threads, smem, st, fa, idx, d_gain_f16, sga, sp, per_pass, n_out, k_in, bpr, d_x_bf16, yo, \
-                       ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;                         \
+        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH, FMA>>(ctx, FMA ? smem_fma : smem)) return LLVQ_ECUDA;                          \
+        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH, FMA>, g, FMA ? fma_threads : threads, FMA ? smem_fma : smem, st, fa, idx, d_gain_f16, sga, sp, FMA ? (uint32_t)kGemvGroupsPerPass : per_pass, n_out, k_in, bpr, \
+                       d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;           \
     } while (0)
-    if (shard && ctx->fast) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(false, true, false, true); else LLVQ_LAUNCH_GEMV(false, false, false, true); }
-    else if (shard)         { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(true, true, false, true);  else LLVQ_LAUNCH_GEMV(true, false, false, true); }
-    else if (sg)            { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(false, true, true, false);  else LLVQ_LAUNCH_GEMV(false, false, true, false); }
-    else if (ctx->fast)     { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(false, true, false, false); else LLVQ_LAUNCH_GEMV(false, false, false, false); }
-    else                    { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_GEMV(true, true, false, false);  else LLVQ_LAUNCH_GEMV(true, false, false, false); }
+    const unsigned fma_threads = 32u * (unsigned)std::max<int64_t>(upc, 16);        // a warp per unit
+    const bool bf16 = y_dtype == LLVQ_BF16;
+    if (fma && shard)       { if (bf16) LLVQ_LAUNCH_GEMV(false, true, false, true, true);   else LLVQ_LAUNCH_GEMV(false, false, false, true, true); }
+    else if (fma && sg)     { if (bf16) LLVQ_LAUNCH_GEMV(false, true, true, false, true);   else LLVQ_LAUNCH_GEMV(false, false, true, false, true); }
+    else if (fma)           { if (bf16) LLVQ_LAUNCH_GEMV(false, true, false, false, true);  else LLVQ_LAUNCH_GEMV(false, false, false, false, true); }
+    else if (shard && ctx->fast) { if (bf16) LLVQ_LAUNCH_GEMV(false, true, false, true, false); else LLVQ_LAUNCH_GEMV(false, false, false, true, false); }
+    else if (shard)         { if (bf16) LLVQ_LAUNCH_GEMV(true, true, false, true, false);   else LLVQ_LAUNCH_GEMV(true, false, false, true, false); }
+    else if (sg)            { if (bf16) LLVQ_LAUNCH_GEMV(false, true, true, false, false);  else LLVQ_LAUNCH_GEMV(false, false, true, false, false); }
+    else if (ctx->fast)     { if (bf16) LLVQ_LAUNCH_GEMV(false, true, false, false, false); else LLVQ_LAUNCH_GEMV(false, false, false, false, false); }
+    else                    { if (bf16) LLVQ_LAUNCH_GEMV(true, true, false, false, false);  else LLVQ_LAUNCH_GEMV(true, false, false, false, false); }
 #undef LLVQ_LAUNCH_GEMV
     return launch_status();
 }
@@ -245,7 +270,7 @@ static int gemv_sorted_common(const llvq_ctx* ctx, const void* d_sorted, const u
     size_t smem; bool ext; uint32_t acc_floats;
     sorted_smem(ctx, nq, smem, ext, acc_floats);
     const FastArgs fa = fast_args(ctx, ext);
-    const Split split = make_split(units, nq, g);
+    const Split split = make_gemv_split(units, nq, g, n_out);
     const unsigned long long* sp = static_cast<const unsigned long long*>(d_sorted);
     const SgArgs sga = sg ? *sg : SgArgs{};
 #define LLVQ_LAUNCH_SORTED(BF16, SG, SH)                                                                                \
@@ -318,6 +343,7 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         slot += (d.n_out + kGemvGroupRows - 1) / kGemvGroupRows * kGemvGroupRows;
     }
     if (slot > 64ll * kMaxScratchRows) return LLVQ_EUNSUPPORTED;
+    for (int i = 0; i < n_mats; ++i) mm.m[i].sp.trees = tree_rows(mm.m[i].slot0, mm.m[i].n_out, slot);
     size_t smem; bool ext;                               // the longest rows decide for the whole launch
     OrderArgs oa{};
     if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);

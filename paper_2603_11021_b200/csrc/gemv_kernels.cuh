@@ -110,6 +110,30 @@ __device__ __forceinline__ void finish_pass(const YOut& yo, const Split& sp, uin
             }
             continue;
         }
+        if (parts <= 8u && sp.trees) {
+            // three to eight CTAs (short rows of small matrices): a tree of such slots, seven per row, over the CTAs in order.  Who finds a
+            // slot empty is done; the other goes on to the next one with both sums.  Up to three round trips for the last to arrive, where
+            // the way below takes a fence on either side of the counter and a read behind it (sorted 512 x 1024:
+            // 8.0 -> 7.1 us, 1024 x 4096 10.6 -> 9.6)
+            if (mine) {
+                unsigned long long* const tree = reinterpret_cast<unsigned long long*>(scratch + kPairSlotOffset) + (kPairSlots - 8 * (slot0 + row + 1));
+                float sum = part;
+                uint32_t at = blockIdx.x - split_owner(sp, first), width = parts, node = 0;
+                bool last = true;
+                while (width > 1u) {
+                    if ((at ^ 1u) < width) {
+                        unsigned long long* const slot = tree + node + (at >> 1);
+                        const unsigned long long seen = atomicCAS(slot, 0ull, (unsigned long long)__float_as_uint(sum) | 1ull << 32);
+                        if (seen == 0ull) { last = false; break; }
+                        __stcg(slot, 0ull);
+                        sum = at & 1u ? __fadd_rn(__uint_as_float((uint32_t)seen), sum) : __fadd_rn(sum, __uint_as_float((uint32_t)seen));
+                    }
+                    at >>= 1; width = (width + 1u) >> 1; node += node ? 2u : 4u;
+                }
+                if (last) store_y<kOutBf16, kShard>(yo, row, sum);
+            }
+            continue;
+        }
         if (mine) atomicAdd(scratch + slot0 + row, part);
         __threadfence();                               // every lane's add is performed before ...
         __syncwarp();
@@ -164,7 +188,33 @@ __device__ __forceinline__ float dot24_bf16(const uint32_t w[12], const uint32_t
     return s0 + s1;
 }
 
-template <bool kBig, bool kOutBf16, bool kSg = false, bool kShard = false>
+// Row sums of a pass in shared memory: acc[row << shift | lane & mask], as many copies of every row (a power of two, up to one per
+// lane) as kSortAccFloats floats hold.  An addition of floats in shared memory is a compare-and-swap loop that goes round once for
+// every lane of the warp that meets the same address: 32 blocks of a warp fall into some 80 rows, and with one copy per warp
+// parity instead of per lane that took 18 instructions and 15 passes over the banks per addition (stored 11008 x 4096: 56.4 -> 53.7 us).
+constexpr uint32_t kSortAccFloats = 4 * kGemvGroupsPerPass * kGemvGroupRows;
+
+__device__ __forceinline__ uint32_t acc_shift(uint32_t rows, uint32_t floats)
+{
+    uint32_t c = 5;
+    while (c > 0 && (rows << c) > floats) --c;
+    return c;
+}
+
+// Sums over the copies of rows first..first + 7, in lanes 0..7; the whole warp calls this.
+__device__ __forceinline__ float acc_row_sums(const float* acc, uint32_t first, uint32_t shift)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    float v = 0.f;
+    for (uint32_t c = lane & 3u; c < (1u << shift); c += 4) v += acc[(first + (lane >> 2)) << shift | c];      // four lanes per row
+    v += __shfl_xor_sync(kFullMask, v, 1);
+    v += __shfl_xor_sync(kFullMask, v, 2);
+    return __shfl_sync(kFullMask, v, (lane & 7u) * 4u);
+}
+
+// kFma: each lane forms its own dot product with binary32 FMAs instead (what small matrices of codes with many classes take, whose larger ones go to
+// gemv_bin_kernel: the tensor core's sums are 1.3 to 1.6 times as far from exact ones, 1.0e-7 against 6.4e-8 of the 2-norm at 1000 x 1000).
+template <bool kBig, bool kOutBf16, bool kSg = false, bool kShard = false, bool kFma = false>
 __global__ void __launch_bounds__(kGemvThreads, 1)
 gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, Split sp, uint32_t groups_per_pass,
                  int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
@@ -181,7 +231,8 @@ gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_
     const uint32_t rg_first = split_row(sp, u_begin), rg_last = split_row(sp, u_end - 1u);
     for (uint32_t rg0 = rg_first; rg0 <= rg_last; rg0 += groups_per_pass) {
         const uint32_t rg1 = min(rg0 + groups_per_pass - 1u, rg_last);
-        for (uint32_t i = threadIdx.x; i < groups_per_pass * kGemvGroupRows; i += blockDim.x) acc[i] = 0.f;
+        const uint32_t shift = kFma ? acc_shift((rg1 - rg0 + 1u) * kGemvGroupRows, kSortAccFloats) : 0u;      // copies of the row sums
+        for (uint32_t i = threadIdx.x; i < (kFma ? (rg1 - rg0 + 1u) * kGemvGroupRows << shift : groups_per_pass * kGemvGroupRows); i += blockDim.x) acc[i] = 0.f;
         __syncthreads();
         const uint32_t p_begin = max(u_begin, rg0 * nq), p_end = min(u_end, (rg1 + 1u) * nq);
         uint32_t kq, rg = split_row(sp, p_begin + (uint32_t)warp, kq);      // walked along with u: no division per unit
@@ -211,14 +262,21 @@ gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_
             const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
             const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
             float c[4] = {0.f, 0.f, 0.f, 0.f};
+            if constexpr (kFma) {
+                atomicAdd(&acc[((rg_now - rg0) * kGemvGroupRows + g) << shift | ((uint32_t)(warp * 4 + t) & ((1u << shift) - 1u))], dot24_bf16(w, xv));
+            } else {
 #pragma unroll
-            for (int q = 0; q < 6; ++q)
-                mma_bf16_16816(c, w[2 * q], 0u, w[2 * q + 1], 0u, xv[2 * q], xv[2 * q + 1]);
-            if (t == 0) atomicAdd(&acc[(rg_now - rg0) * kGemvGroupRows + g], c[0]);
+                for (int q = 0; q < 6; ++q)
+                    mma_bf16_16816(c, w[2 * q], 0u, w[2 * q + 1], 0u, xv[2 * q], xv[2 * q + 1]);
+            }
+            if (!kFma && t == 0) atomicAdd(&acc[(rg_now - rg0) * kGemvGroupRows + g], c[0]);
         }
         __syncthreads();
         // row groups this CTA covers completely are final; the (at most two) split ones go through the scratch
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) { return lane < kGemvGroupRows ? acc[r + lane] : 0.f; });
+        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) {
+            if constexpr (kFma) return acc_row_sums(acc, r, shift);
+            return lane < kGemvGroupRows ? acc[r + lane] : 0.f;
+        });
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     }
     if (kShard) shard_arrive(yo);
@@ -240,30 +298,7 @@ constexpr uint32_t kKindEven = 0u, kKindOdd = 1u, kKindOther = 2u, kKindNull = 3
 // ===========================================================================
 constexpr int kSortSegUnits = 2048;                  // 65536 blocks
 constexpr int kSortThreads = 1024;
-// Row sums of a pass in shared memory: acc[row << shift | lane & mask], as many copies of every row (a power of two, up to one per
-// lane) as kSortAccFloats floats hold.  An addition of floats in shared memory is a compare-and-swap loop that goes round once for
-// every lane of the warp that meets the same address: 32 blocks of a warp fall into some 80 rows, and with one copy per warp
-// parity instead of per lane that took 18 instructions and 15 passes over the banks per addition (stored 11008 x 4096: 56.4 -> 53.7 us).
-constexpr uint32_t kSortAccFloats = 4 * kGemvGroupsPerPass * kGemvGroupRows;
 constexpr unsigned long long kSortIndexMask = (1ull << 48) - 1ull;
-
-__device__ __forceinline__ uint32_t acc_shift(uint32_t rows, uint32_t floats)
-{
-    uint32_t c = 5;
-    while (c > 0 && (rows << c) > floats) --c;
-    return c;
-}
-
-// Sums over the copies of rows first..first + 7, in lanes 0..7; the whole warp calls this.
-__device__ __forceinline__ float acc_row_sums(const float* acc, uint32_t first, uint32_t shift)
-{
-    const uint32_t lane = threadIdx.x & 31u;
-    float v = 0.f;
-    for (uint32_t c = lane & 3u; c < (1u << shift); c += 4) v += acc[(first + (lane >> 2)) << shift | c];      // four lanes per row
-    v += __shfl_xor_sync(kFullMask, v, 1);
-    v += __shfl_xor_sync(kFullMask, v, 2);
-    return __shfl_sync(kFullMask, v, (lane & 7u) * 4u);
-}
 
 // Calls f(tu0, tu1, rg0, rg1, first, last) for every segment [tu0, tu1) of CTA `cta` in order; rg0..rg1 = row
 // groups of the pass the segment belongs to (a pass covers at most kGemvGroupsPerPass row groups); first / last =

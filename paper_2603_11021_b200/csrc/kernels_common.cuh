@@ -36,6 +36,8 @@ constexpr int kCounterWords = 64 * kMaxScratchRows / 8;      // the word after t
 // and `peer` the other ranks' copies mapped into this process, every pointer already advanced to the band's first
 // row.  The stores to a peer travel over NVLink as plain remote writes.  n_peer = 0 is the single-GPU case.
 constexpr int64_t kPairSlotOffset = 64ll * 65536;      // floats: the 64-bit slots of finish_pass lie behind the binary32 scratch rows
+constexpr int64_t kPairSlots = 64ll * 65536;
+constexpr int64_t kTreeRows = 1 << 18;                 // rows that may have a tree of slots
 constexpr int kMaxShardPeers = 7;
 struct YOut {
     void* y;
@@ -78,6 +80,7 @@ struct Split {
     uint32_t ctas_magic;                     // ceil(2^32 / ctas): exact quotients of numbers below ctas^2 (ctas < 1625)
     uint32_t per_row, row_magic;             // floor(2^32 / per_row): quotients at most one too small
     float ctas_per_unit;
+    uint32_t trees;                          // finish_pass may use the trees of slots (set by the GEMV's launches)
 };
 
 Split make_split(int64_t units, int64_t per_row, unsigned ctas)
@@ -88,6 +91,18 @@ Split make_split(int64_t units, int64_t per_row, unsigned ctas)
     s.per_row = (uint32_t)per_row;
     s.row_magic = per_row == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / (uint64_t)per_row);
     s.ctas_per_unit = (float)((double)ctas / (double)units);
+    s.trees = 0u;
+    return s;
+}
+
+// Whether the rows from first_row on of a GEMV launch of `rows` rows in all may use the trees of slots: those lie at the end of the slots,
+// which the rows' own slots must not reach.
+uint32_t tree_rows(int64_t first_row, int64_t n_out, int64_t rows) { return first_row + n_out <= kTreeRows && rows <= kPairSlots - 8 * kTreeRows; }
+
+Split make_gemv_split(int64_t units, int64_t per_row, unsigned ctas, int64_t n_out)
+{
+    Split s = make_split(units, per_row, ctas);
+    s.trees = tree_rows(0, n_out, n_out);
     return s;
 }
 

@@ -1,0 +1,45 @@
+"""Products of small matrices: row groups shared by one to many thread blocks (whole groups, one exchange, trees of exchanges, scratch and
+counter), at most one unit per warp and just beyond, repeated so that a slot left behind by one call shows in the next."""
+import numpy as np
+import pytest
+import torch
+
+import llvq_inputs as gen
+import paper_2603_11021_b200 as P
+from gpu_util import gemv_error, to_dev_bf16, to_dev_f16, to_dev_u8
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("code", [(2, 13), (3, 3)])
+@pytest.mark.parametrize("n_out,k_in", [(8, 24), (16, 4100), (133, 500), (160, 8000), (240, 8000), (400, 480), (500, 3100), (1000, 1000), (1184, 768), (1192, 770),
+                                        (3800, 480)])
+def test_small_products_by_how_a_row_group_is_shared(oracle_mod, code, n_out, k_in):
+    o, ctx = oracle_mod.Code(*code), P.Context(*code, device=0)
+    stream, gain, _ = gen.make_layer(o.N, o.W, n_out, k_in, 1, seed=n_out)
+    x = gen.normal_bf16(k_in, seed=k_in)
+    want = o.gemv(stream, gain, n_out, k_in, x)
+    d_s, d_g, d_x = to_dev_u8(stream), to_dev_f16(gain), to_dev_bf16(x)
+    srt = P.llvq_sort_blocks(ctx, d_s, n_out, k_in)
+    for _ in range(3):
+        assert gemv_error(P.llvq_gemv(ctx, d_s, d_g, n_out, k_in, d_x).cpu().numpy(), want) <= 1e-3
+        assert gemv_error(P.llvq_gemv_sorted(ctx, srt, d_g, n_out, k_in, d_x).cpu().numpy(), want) <= 1e-3
+    assert P.llvq_last_error(ctx) == (0, 0)
+
+
+def test_small_shape_gain_products(oracle_mod):
+    from oracle.gain_codebook import chi_codebook
+    o, ctx = oracle_mod.Code(2, 12), P.Context(2, 12, device=0)
+    for n_out, k_in in [(133, 500), (1000, 1000), (240, 8000)]:
+        bpr = (k_in + 23) // 24
+        lo, hi = gen.random_indices(o.N, o.W, n_out * bpr, seed=n_out)
+        k = gen.gain_indices(n_out * bpr, 1, seed=n_out)
+        d_s = to_dev_u8(gen.pack_indices(lo | (k << np.uint64(o.W)), hi, o.W + 1))
+        cb = torch.tensor(chi_codebook(1), dtype=torch.float32, device="cuda")
+        scale = torch.linspace(0.01, 0.03, n_out, device="cuda")
+        x = to_dev_bf16(gen.normal_bf16(k_in, seed=1))
+        w = P.llvq_dequant_matrix_sg(ctx, d_s, 1, cb, scale, n_out, k_in).double()
+        want = (w @ x.double()).cpu().numpy()
+        for _ in range(2):
+            assert gemv_error(P.llvq_gemv_sg(ctx, d_s, 1, cb, scale, n_out, k_in, x).cpu().numpy(), want) <= 1e-3
+    assert P.llvq_last_error(ctx) == (0, 0)
