@@ -107,16 +107,9 @@ __device__ __forceinline__ int coset_point(double u, uint32_t c, int pi, int lan
 // first coordinate with the largest error moves.  The result does not depend on the first stage's rounding.  Returns the coordinate of
 // this lane (0 for lanes >= 24) and the squared norm of the point; unique = every other lattice point is farther from u by a margin
 // far above any binary64 rounding.
-__device__ __noinline__ int nearest_careful(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
-                                            const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
+__device__ __forceinline__ int nearest_careful_from(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t (&row)[6],
+                                                    const uint32_t* __restrict__ golay, const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
 {
-    uint32_t row[6];                                             // where the nibbles of pattern (x, 4 h) of every octad are
-#pragma unroll
-    for (int o = 0; o < 3; ++o) {
-        const uint32_t p = S.pat[o][(lane & 7) * 8 + ((lane >> 1) & 4)], t = (uint32_t)__cvta_generic_to_shared(&W.nib[lane >> 4][2 * o][0]);
-        row[2 * o] = t ^ (p & 15u) * 8u;
-        row[2 * o + 1] = (t + 128u) ^ (p >> 4) * 8u;
-    }
     const float uq = __shfl_sync(kFull, (float)u, lane < 24 ? S.coord[lane] : lane);   // octad order
     if (lane < 24) {
         uint32_t w[4];
@@ -259,6 +252,25 @@ __device__ __noinline__ int nearest_careful(WarpTables& W, const GolayTrio& S, c
     return best_x;
 }
 
+// Where the nibbles of pattern (x, 4 h) of every octad are in W.
+__device__ __forceinline__ void pattern_rows(WarpTables& W, const GolayTrio& S, int lane, uint32_t (&row)[6])
+{
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+        const uint32_t p = S.pat[o][(lane & 7) * 8 + ((lane >> 1) & 4)], t = (uint32_t)__cvta_generic_to_shared(&W.nib[lane >> 4][2 * o][0]);
+        row[2 * o] = t ^ (p & 15u) * 8u;
+        row[2 * o + 1] = (t + 128u) ^ (p >> 4) * 8u;
+    }
+}
+
+__device__ __noinline__ int nearest_careful(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
+                                            const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
+{
+    uint32_t row[6];
+    pattern_rows(W, S, lane, row);
+    return nearest_careful_from(W, S, steps, row, golay, pos_by_low12, u, lane, norm2, unique);
+}
+
 // ---- the search: two lanes per vector ----
 
 // Units of the costs below: whole numbers of 1 / kPairScale.  Three octads cost at most 6 of the squares of the half spacing
@@ -332,24 +344,20 @@ struct Nearest {
     bool unique;            // every other lattice point is farther from u by a margin far above any binary64 rounding
 };
 
-// nearest_careful for u = (v rn) radius (v[stride i] holds coordinate i), one vector for the whole warp.
-__device__ __forceinline__ void nearest_of_warp(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t* __restrict__ golay,
-                                                const uint16_t* __restrict__ pos_by_low12, const float* v, int stride, double rn, double radius, int lane,
-                                                int8_t* point, int& norm2, double& dot, bool& unique)
+// <u, x>, a coordinate per lane.
+__device__ __forceinline__ double dot_of_warp(double u, int xi)
 {
-    const double u = lane < 24 ? __dmul_rn(__dmul_rn((double)v[stride * lane], rn), radius) : 0.0;
-    const int xi = nearest_careful(W, S, steps, golay, pos_by_low12, u, lane, norm2, unique);
-    dot = u * (double)xi;
+    double dot = u * (double)xi;
 #pragma unroll
     for (int o = 16; o; o >>= 1) dot += __shfl_xor_sync(kFull, dot, o);
-    if (lane < 24) point[lane] = (int8_t)xi;
+    return dot;
 }
 
 // Vectors of a CTA that wait for nearest_careful, and its answers.
 // More vectors per SM than this: two lanes take a vector, else a warp does.  Two lanes per vector use the chip best, but a CTA works on 256 vectors at a time
-// for some 15 us; shells 2..13 and 2..12, us for a warp per vector / two lanes: EUCLIDEAN 12 000 vectors 53 / 69, 30 000 87 / 87, 80 000 174 / 151;
-// ANGULAR 5000 76 / 90, 12 000 132 / 178, 30 000 278 / 207.
-constexpr uint64_t kPairsFromEuclidean = 208, kPairsFromAngular = 128;
+// for some 15 us; shells 2..13 and 2..12, us for a warp per vector / two lanes: EUCLIDEAN 12 000 vectors 50 / 69, 30 000 79 / 87, 40 000 98 / 112;
+// ANGULAR 5000 71 / 90, 15 700 148 / 190, 25 000 240 / 196.
+constexpr uint64_t kPairsFromEuclidean = 352, kPairsFromAngular = 136;
 constexpr int kFew = 40;                   // no more vectors than this left in a CTA: all of them go to nearest_careful (EUCLIDEAN 867 -> 761 us with the wider loads)
 constexpr uint32_t kPendingMost = 48, kPendingEnough = 14;
 struct Pending {
@@ -626,9 +634,11 @@ __device__ __forceinline__ bool nearest_pairs(uint32_t nib, const float* v, cons
         for (uint32_t i = (uint32_t)warp; i < min(n, kPendingMost); i += (uint32_t)kEncWarps<true>) {
             Pending& p = pending.list[i];
             int norm2;
-            double dot;
             bool unique;
-            nearest_of_warp(careful, S, steps, golay, pos_by_low12, p.v, 16, p.rn, p.radius, lane, p.x, norm2, dot, unique);
+            const double u = lane < 24 ? __dmul_rn(__dmul_rn((double)p.v[16 * lane], p.rn), p.radius) : 0.0;
+            const int xi = nearest_careful(careful, S, steps, golay, pos_by_low12, u, lane, norm2, unique);
+            const double dot = dot_of_warp(u, xi);
+            if (lane < 24) p.x[lane] = (int8_t)xi;
             if (lane == 0) { p.norm2 = norm2; p.unique = unique; p.dot = dot; }
         }
         __syncthreads();
@@ -726,6 +736,8 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
     const uint64_t first = n / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, n % gridDim.x);
     const uint32_t count = (uint32_t)(n / gridDim.x + (blockIdx.x < n % gridDim.x));
 
+    [[maybe_unused]] uint32_t row[6];
+    if constexpr (!kPairs) pattern_rows(careful, S, lane, row);
     bool active = false, drained = false;       // this lane's vector is being searched; there are no more
     bool starting = false, direct = false;      // its radii are about to be started; the input itself is decoded (else: its direction at shell radius m)
     bool waiting = false;                       // it is on the list for nearest_careful, at `spot`
@@ -759,27 +771,36 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
             const bool taking = !active && !drained;
             const uint32_t takers = __ballot_sync(kFull, taking);
             if (taking) {
-                const float* const from = v + (first + t) * 24 + 12 * q;
                 float n2f = 0.f;
                 uint32_t some = 0, finite = 1;
-                const auto take = [&](int k, float f) {
-                    some |= f != 0.f; finite &= isfinite(f) ? 1u : 0u;
-                    n2f = fmaf(f, f, n2f);
-                    mine_v[kVecs * (12 * q + k)] = f;
-                };
-                if (quads) {
+                const float* const from = v + (first + t) * 24 + (kPairs ? 12 * q : 0);
+                if constexpr (kPairs) {
+                    const auto take = [&](int k, float f) {
+                        some |= f != 0.f; finite &= isfinite(f) ? 1u : 0u;
+                        n2f = fmaf(f, f, n2f);
+                        mine_v[kVecs * (12 * q + k)] = f;
+                    };
+                    if (quads) {
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const float4 f = __ldg(reinterpret_cast<const float4*>(from) + k);
-                        take(4 * k, f.x); take(4 * k + 1, f.y); take(4 * k + 2, f.z); take(4 * k + 3, f.w);
-                    }
-                } else {
+                        for (int k = 0; k < 3; ++k) {
+                            const float4 f = __ldg(reinterpret_cast<const float4*>(from) + k);
+                            take(4 * k, f.x); take(4 * k + 1, f.y); take(4 * k + 2, f.z); take(4 * k + 3, f.w);
+                        }
+                    } else {
 #pragma unroll 4
-                    for (int k = 0; k < 12; ++k) take(k, __ldg(from + k));
+                        for (int k = 0; k < 12; ++k) take(k, __ldg(from + k));
+                    }
+                    n2f += __shfl_xor_sync(takers, n2f, 16);
+                    some |= __shfl_xor_sync(takers, some, 16);
+                    finite &= __shfl_xor_sync(takers, finite, 16);
+                } else {
+                    const float f = lane < 24 ? __ldg(from + lane) : 0.f;
+                    if (lane < 24) mine_v[lane] = f;
+                    n2f = f * f;
+#pragma unroll
+                    for (int o = 16; o; o >>= 1) n2f += __shfl_xor_sync(kFull, n2f, o);
+                    some = __any_sync(kFull, f != 0.f); finite = __all_sync(kFull, isfinite(f));
                 }
-                n2f += __shfl_xor_sync(takers, n2f, 16);
-                some |= __shfl_xor_sync(takers, some, 16);
-                finite &= __shfl_xor_sync(takers, finite, 16);
                 // (the vectors that will be taken when the CTA is through with those it has)
                 if (t + kEncWarps<kPairs> * kVecs < count) asm volatile("prefetch.global.L2 [%0];" ::"l"(from + kEncWarps<kPairs> * kVecs * 24));
                 // no lattice point is farther than 4 from any input (covering radius): beyond radius sqrt(16 m_hi) + 4 the nearest
@@ -831,7 +852,10 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
             found = nearest_pairs(nib, mine_v, S, steps, golay, et.pos_by_low12, careful, pending, s1, s2, rn, rad, active && !waiting, waiting, spot, few, warp, lane, r);
         } else {
             int8_t* const point = reinterpret_cast<int8_t*>(&careful + 1);
-            nearest_of_warp(careful, S, steps, golay, et.pos_by_low12, mine_v, kVecs, rn, rad, lane, point, r.norm2, r.dot, r.unique);
+            const double u = lane < 24 ? __dmul_rn(__dmul_rn((double)mine_v[lane], rn), rad) : 0.0;
+            const int xi = nearest_careful_from(careful, S, steps, row, golay, et.pos_by_low12, u, lane, r.norm2, r.unique);
+            r.dot = direct ? 0.0 : dot_of_warp(u, xi);           // (not looked at where the input itself was decoded)
+            if (lane < 24) point[lane] = (int8_t)xi;
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < 3; ++j) r.x[j] = reinterpret_cast<const uint32_t*>(point)[3 * q + j];
