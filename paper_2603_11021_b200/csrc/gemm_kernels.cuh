@@ -56,6 +56,61 @@ __device__ __forceinline__ void gemm_store(const GemmArgs& ga, int n, int64_t or
     }
 }
 
+// Carries a finished accumulator of row tile rt out, a quarter of its rows and 16 of its columns per warp (a warp reaches the rows 32 (warp & 3) on): into the
+// scratch where CTAs share the tile, else to Y.  second = the accumulator 64 columns on belongs to the same tile.  With four warps taking all columns one
+// after the other, and the shared tile then read, converted and cleared value by value, a tile's end grew with the batch: sorted, shells 2..13, batch 64,
+// 512 x 1024 17.2 -> 12.8 us, 4096 x 4096 39.8 -> 31.6, 8192 x 8192 87.6 -> 79.5; batch 16 30.3 -> 30.1 and 77.0 -> 76.8.
+template <bool kShard>
+__device__ __forceinline__ void carry_out(const GemmArgs& ga, uint32_t tmem, bool second, bool shared_tile, uint32_t rt, int warp, int lane)
+{
+    const int c0 = (warp >> 2) * 16;
+    const uint32_t from = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
+    const int64_t orow = (int64_t)rt * kGemmRows + (warp & 3) * 32 + lane;
+    float v[16];
+    tmem_ld16(from, v);
+    if (second) {
+        float v1[16];
+        tmem_ld16(from + 64u, v1);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] += v1[i];
+    }
+    if (orow < ga.n_out) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int n = c0 + i;
+            if (n < ga.batch) {
+                if (!shared_tile) gemm_store<kShard>(ga, n, orow, v[i]);
+                else atomicAdd(ga.scratch + (int64_t)n * ga.scratch_ld + orow, v[i]);
+            }
+        }
+    }
+}
+
+// Y of row tile rt from the scratch, which is left at zero; all threads of the CTA that arrived last.  Four of a thread's values are asked for together (all
+// eight of a batch of 64 in one go cost the main loop registers: batch 16 1 to 4 % slower).
+template <bool kShard>
+__device__ __forceinline__ void convert_tile(const GemmArgs& ga, uint32_t rt)
+{
+    static_assert(kGemmThreads % kGemmRows == 0, "a thread has one row of the tile");
+    constexpr int kAhead = 4, kStep = kGemmThreads / kGemmRows;
+    const int64_t orow = (int64_t)rt * kGemmRows + threadIdx.x % kGemmRows;
+    if (orow >= ga.n_out) return;
+    float* at = ga.scratch + (int64_t)(threadIdx.x / kGemmRows) * ga.scratch_ld + orow;
+    const int64_t step = (int64_t)kStep * ga.scratch_ld;
+#pragma unroll 1
+    for (int n = (int)(threadIdx.x / kGemmRows); n < ga.batch; n += kAhead * kStep, at += kAhead * step) {
+        float v[kAhead];
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) v[j] = n + j * kStep < ga.batch ? __ldcg(at + j * step) : 0.f;
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j)
+            if (n + j * kStep < ga.batch) {
+                gemm_store<kShard>(ga, n + j * kStep, orow, v[j]);
+                __stcg(at + j * step, 0.f);
+            }
+    }
+}
+
 // Gain of the block in row r of a row tile and column block cb.  A tile may hold more than 2^32 blocks.
 __device__ __forceinline__ const uint16_t* gain_at(const GemmArgs& ga, const uint16_t* gain_tile, uint32_t r, uint32_t cb)
 {
@@ -156,30 +211,11 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
         }
         // ---- epilogue: accumulators -> scratch (split-K) or Y
         const bool has0 = s_end > s_begin, has1 = s_end > s_begin + 1;
-        if (warp < 4) {
-            if (has0 && !mbar_wait(&bar_done[0], done[0] & 1u)) timeout = true;
+        if (has0 && (warp >> 2) * 16 < ga.npad) {
+            if (!mbar_wait(&bar_done[0], done[0] & 1u)) timeout = true;
             if (has1 && !mbar_wait(&bar_done[1], done[1] & 1u)) timeout = true;
             tc_fence_after();
-            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
-            for (int c0 = 0; c0 < ga.npad && has0; c0 += 16) {
-                float v[16], v1[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-                if (has1) {
-                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + 64u + (uint32_t)c0, v1);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] += v1[i];
-                }
-                if (orow < ga.n_out) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int n = c0 + i;
-                        if (n < ga.batch) {
-                            if (ga.split == 1) gemm_store<kShard>(ga, n, orow, v[i]);
-                            else atomicAdd(ga.scratch + (int64_t)n * ga.scratch_ld + orow, v[i]);
-                        }
-                    }
-                }
-            }
+            carry_out<kShard>(ga, tmem, has1, ga.split > 1, (uint32_t)rt, warp, lane);
             tc_fence_before();
         }
         done[0] += has0; done[1] += has1;
@@ -190,15 +226,7 @@ gemm_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __
             __syncthreads();
             if (*last_flag) {
                 __threadfence();
-                for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
-                    const int n = i / kGemmRows;
-                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
-                    if (orow < ga.n_out) {
-                        float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
-                        gemm_store<kShard>(ga, n, orow, __ldcg(sp));
-                        __stcg(sp, 0.f);
-                    }
-                }
+                convert_tile<kShard>(ga, (uint32_t)rt);
                 if (threadIdx.x == 0) ga.counters[rt] = 0u;
             }
         }
@@ -549,24 +577,10 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
         g_base += n_dom;
         const bool has = d_end > d_begin;
         // ---- epilogue: accumulator -> scratch (split-K) or Y
-        if (warp < 4 && has) {
+        if (has && (warp >> 2) * 16 < ga.npad) {
             if (!mbar_wait(bar_done, done & 1u)) timeout = true;
             tc_fence_after();
-            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
-            for (int c0 = 0; c0 < ga.npad; c0 += 16) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-                if (orow < ga.n_out) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int n = c0 + i;
-                        if (n < ga.batch) {
-                            if (parts == 1u) gemm_store<kShard>(ga, n, orow, v[i]);
-                            else atomicAdd(ga.scratch + (int64_t)n * ga.scratch_ld + orow, v[i]);
-                        }
-                    }
-                }
-            }
+            carry_out<kShard>(ga, tmem, false, parts > 1u, rt, warp, lane);
             tc_fence_before();
         }
         done += has;
@@ -577,15 +591,7 @@ gemm_pipe_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, con
             __syncthreads();
             if (*last_flag) {
                 __threadfence();
-                for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
-                    const int n = i / kGemmRows;
-                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
-                    if (orow < ga.n_out) {
-                        float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
-                        gemm_store<kShard>(ga, n, orow, __ldcg(sp));
-                        __stcg(sp, 0.f);
-                    }
-                }
+                convert_tile<kShard>(ga, (uint32_t)rt);
                 if (threadIdx.x == 0) ga.counters[rt] = 0u;
             }
         }
@@ -747,31 +753,11 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
         const uint32_t n0 = (d_end - d_begin + 1u) / 2u, n1 = (d_end - d_begin) / 2u;
         // ---- epilogue: accumulators -> scratch (split-K) or Y
         __syncthreads();                                                  // both teams' MMAs of this tile are issued
-        if (warp < 4 && n0 > 0) {
+        if (n0 > 0 && (warp >> 2) * 16 < ga.npad) {
             if (!mbar_wait(bar_free, (base[0] + n0 - 1u) & 1u)) timeout = true;
             if (n1 > 0 && !mbar_wait(bar_free + 1, (base[1] + n1 - 1u) & 1u)) timeout = true;
             tc_fence_after();
-            const int64_t orow = (int64_t)rt * kGemmRows + warp * 32 + lane;
-            for (int c0 = 0; c0 < ga.npad; c0 += 16) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-                if (n1 > 0) {
-                    float v1[16];
-                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + 64u + (uint32_t)c0, v1);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] += v1[i];
-                }
-                if (orow < ga.n_out) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int n = c0 + i;
-                        if (n < ga.batch) {
-                            if (parts == 1u) gemm_store<kShard>(ga, n, orow, v[i]);
-                            else atomicAdd(ga.scratch + (int64_t)n * ga.scratch_ld + orow, v[i]);
-                        }
-                    }
-                }
-            }
+            carry_out<kShard>(ga, tmem, n1 > 0, parts > 1u, rt, warp, lane);
             tc_fence_before();
         }
         base[0] += n0; base[1] += n1;
@@ -782,15 +768,7 @@ gemm_team_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa,
             __syncthreads();
             if (*last_flag) {
                 __threadfence();
-                for (int i = threadIdx.x; i < kGemmRows * ga.batch; i += kGemmThreads) {
-                    const int n = i / kGemmRows;
-                    const int64_t orow = (int64_t)rt * kGemmRows + (i % kGemmRows);
-                    if (orow < ga.n_out) {
-                        float* sp = ga.scratch + (int64_t)n * ga.scratch_ld + orow;
-                        gemm_store<kShard>(ga, n, orow, __ldcg(sp));
-                        __stcg(sp, 0.f);
-                    }
-                }
+                convert_tile<kShard>(ga, (uint32_t)rt);
                 if (threadIdx.x == 0) ga.counters[rt] = 0u;
             }
         }
