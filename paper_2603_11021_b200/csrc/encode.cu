@@ -355,9 +355,9 @@ __device__ __forceinline__ double dot_of_warp(double u, int xi)
 
 // Vectors of a CTA that wait for nearest_careful, and its answers.
 // More vectors per SM than this: two lanes take a vector, else a warp does.  Two lanes per vector use the chip best, but a CTA works on 256 vectors at a time
-// for some 15 us; shells 2..13 and 2..12, us for a warp per vector / two lanes: EUCLIDEAN 12 000 vectors 50 / 69, 30 000 79 / 87, 40 000 98 / 112;
+// for some 15 us; shells 2..13 and 2..12, us for a warp per vector / two lanes: EUCLIDEAN 12 000 vectors 50 / 69, 30 000 79 / 87, 40 000 98 / 112, 52 000 113 / 118;
 // ANGULAR 5000 71 / 90, 15 700 148 / 190, 25 000 240 / 196.
-constexpr uint64_t kPairsFromEuclidean = 352, kPairsFromAngular = 136;
+constexpr uint64_t kPairsFromEuclidean = 384, kPairsFromAngular = 136;
 constexpr int kFew = 40;                   // no more vectors than this left in a CTA: all of them go to nearest_careful (EUCLIDEAN 867 -> 761 us with the wider loads)
 constexpr uint32_t kPendingMost = 48, kPendingEnough = 14;
 struct Pending {

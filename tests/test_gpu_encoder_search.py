@@ -9,7 +9,7 @@ import paper_2603_11021_b200 as P
 
 pytestmark = pytest.mark.gpu
 
-PAIRS_FROM = {"EUCLIDEAN": 352, "ANGULAR": 136}           # vectors per SM beyond which two lanes take a vector
+PAIRS_FROM = {"EUCLIDEAN": 384, "ANGULAR": 136}           # vectors per SM beyond which two lanes take a vector
 
 
 def _inputs(n, seed, grid=7):
