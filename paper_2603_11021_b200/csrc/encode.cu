@@ -618,14 +618,14 @@ __device__ __forceinline__ bool nearest_pairs(uint32_t nib, const float* v, cons
     waiting |= wanted && !settled;
     while (true) {
         __syncthreads();                                         // the costs of all warps are done with: nearest_careful works there
-        if (waiting && spot >= kPendingMost) {
-            uint32_t mine = 0;
-            if (q == 0) {
-                mine = atomicAdd(&pending.count, 1u);
-                if (mine < kPendingMost) { Pending& p = pending.list[mine]; p.v = v; p.rn = rn; p.radius = radius; }
-            }
-            spot = __shfl_sync(__activemask(), mine, lane & 15);
+        const bool listing = waiting && spot >= kPendingMost;
+        uint32_t mine = 0;
+        if (listing && q == 0) {
+            mine = atomicAdd(&pending.count, 1u);
+            if (mine < kPendingMost) { Pending& p = pending.list[mine]; p.v = v; p.rn = rn; p.radius = radius; }
         }
+        mine = __shfl_sync(kFull, mine, lane & 15);              // all lanes: those that list their vector need not have stayed together
+        if (listing) spot = mine;
         __syncthreads();
         const uint32_t n = pending.count;
         if (n < (few ? 1u : kPendingEnough)) break;
