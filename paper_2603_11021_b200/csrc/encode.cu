@@ -440,6 +440,7 @@ __device__ __forceinline__ bool nearest_pairs(uint32_t nib, const float* v, cons
                 sts64(tab + g * kNibTable + (uint32_t)i * kNibRow, c.even, c.odd);
             }
         }
+        __syncwarp();                                                // either lane of a vector reads the tables that the other one made
         uint32_t best = 0xffffu, second = 0xffffu, group = 0;        // group: 2 x + parity
         uint32_t kept[8];                                            // the smallest costs of that x, by a
 #pragma unroll
@@ -761,6 +762,7 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
     while (true) {
         const uint32_t vacant = __ballot_sync(kFull, !active && !drained);
         if (vacant) {
+            __syncwarp();                                        // the inputs that are about to be replaced are no longer read (a vote orders no memory)
             uint32_t base = 0;
             if (lane == 0) base = atomicAdd(&next_vec, kPairs ? (uint32_t)__popc(vacant & 0xffffu) : 1u);
             base = __shfl_sync(kFull, base, 0);

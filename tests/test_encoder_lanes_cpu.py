@@ -1,7 +1,7 @@
 """The encoder's search with a thread block of lanes that do not run in step (no GPU).  CUDA promises that lanes of a warp meet only where a barrier, a
 shuffle or a vote says so.  Here the kernel's own text runs on the CPU, every lane on a stack of its own, and whoever runs goes on to the next
-such meeting before anyone else moves: a value read before its writer has been there is the stale one, and a shuffle from a lane that is not
-among those named is an error, as is a meeting that some lane never comes to."""
+such meeting before anyone else moves.  Errors are a shuffle from a lane that is not among those named, a meeting that some lane never comes
+to, and a table entry read or overwritten with no barrier between the lanes that share it."""
 import os
 import re
 import shutil
@@ -47,7 +47,7 @@ struct Lane {
     ucontext_t at;
     std::vector<char> stack = std::vector<char>(256 * 1024);
     enum { kRuns, kAtWarp, kAtBlock, kDone } state = kRuns;
-    uint32_t mask = 0;
+    uint32_t mask = 0, orders = 1;       // orders: barriers of the warp or the block this lane has passed
     uint64_t value = 0, seen[32];        // what this lane brought; what everyone brought (block: the total)
 };
 static std::vector<Lane> lanes;
@@ -88,7 +88,7 @@ static uint64_t meet_block(uint64_t value)
         if (l.state != Lane::kAtBlock) { leave(me); return me.seen[0]; }
         total += l.value;
     }
-    for (Lane& l : lanes) { l.state = Lane::kRuns; l.seen[0] = total; }
+    for (Lane& l : lanes) { l.state = Lane::kRuns; l.seen[0] = total; ++l.orders; }
     return total;
 }
 
@@ -126,7 +126,7 @@ template <typename T> static T __shfl_sync(uint32_t mask, T v, int from)
     return as<T>(meet(mask, bits_of(v)).seen[from & 31]);
 }
 template <typename T> static T __shfl_xor_sync(uint32_t mask, T v, int other) { return __shfl_sync(mask, v, (int)(threadIdx.x & 31) ^ other); }
-static void __syncwarp(uint32_t mask = ~0u) { meet(mask, 0); }
+static void __syncwarp() { ++meet(~0u, 0).orders; }
 static uint32_t __ballot_sync(uint32_t mask, bool p)
 {
     Lane& me = meet(mask, p);
@@ -180,8 +180,30 @@ static int __double2loint(double v) { return (int)(uint32_t)as<uint64_t>(v); }
 static int __double2hiint(double v) { return (int)(as<uint64_t>(v) >> 32); }
 alignas(1024) static uint8_t enc_smem[232448];
 static size_t __cvta_generic_to_shared(const void* p) { return (size_t)(static_cast<const uint8_t*>(p) - enc_smem); }
-static uint2 read_shared(uint32_t a) { if (a % 8 || a + 8 > sizeof enc_smem) fail("read outside shared memory"); uint2 v; std::memcpy(&v, enc_smem + a, 8); return v; }
-static void write_shared(uint32_t a, uint32_t x, uint32_t y) { if (a % 8 || a + 8 > sizeof enc_smem) fail("write outside shared memory"); const uint2 v{x, y}; std::memcpy(enc_smem + a, &v, 8); }
+// Shared memory, 8 bytes at a time: lanes of a warp see each other's only across a barrier (shuffles and votes order no memory).
+static struct { uint32_t writer, written, read[32]; } uses[sizeof enc_smem / 8];
+static uint2 read_shared(uint32_t a)
+{
+    if (a % 8 || a + 8 > sizeof enc_smem) fail("read outside shared memory");
+    auto& u = uses[a / 8];
+    const uint32_t now = lanes[threadIdx.x].orders;
+    if (u.writer != threadIdx.x && u.written >= now) fail("read of what another lane wrote, with no barrier between them");
+    u.read[threadIdx.x & 31] = now;
+    uint2 v;
+    std::memcpy(&v, enc_smem + a, 8);
+    return v;
+}
+static void write_shared(uint32_t a, uint32_t x, uint32_t y)
+{
+    if (a % 8 || a + 8 > sizeof enc_smem) fail("write outside shared memory");
+    auto& u = uses[a / 8];
+    const uint32_t now = lanes[threadIdx.x].orders;
+    for (uint32_t i = 0; i < 32; ++i)
+        if (i != (threadIdx.x & 31) && u.read[i] >= now) fail("write over what another lane has read, with no barrier between them");
+    u.writer = threadIdx.x; u.written = now;
+    const uint2 v{x, y};
+    std::memcpy(enc_smem + a, &v, 8);
+}
 """
 
 MAIN = r"""
@@ -246,3 +268,11 @@ def test_list_of_waiting_vectors(oracle_mod, search, metric, m_hi, descending):
     v = (np.random.default_rng(22).standard_normal((40, 24)) * 2.5).astype(np.float32)
     v[::4] = np.round(v[::4] * 2) / 2
     _check(oracle_mod, search, v, metric, m_hi, descending)
+
+
+@pytest.mark.parametrize("descending", [False, True])
+def test_tables_are_read_after_all_their_lanes_have_written(oracle_mod, search, descending):
+    # near points of the code: one candidate each, all of them found in the tables; more vectors than a block has at a time, so that some are replaced
+    rng, o = np.random.default_rng(23), oracle_mod.Code(2, 13)
+    v = o.unrank([o.N // 330 * j + 5 for j in range(330)]) + 0.3 * rng.standard_normal((330, 24))
+    _check(oracle_mod, search, v.astype(np.float32), "EUCLIDEAN", 13, descending)
