@@ -256,14 +256,16 @@ gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_
             u += kWarps; kq += kWarps;
             raw_next = request(u);
             uint32_t w[12];
-            if constexpr (kSg) block_pairs_sg(fa, T, raw.field, sg, (int64_t)rg_now * kGemvGroupRows + g, in_now, w);
-            else block_pairs<kBig>(fa, T, raw, in_now, w);
+            [[maybe_unused]] bool valid;
+            if constexpr (kSg) valid = block_pairs_sg(fa, T, raw.field, sg, (int64_t)rg_now * kGemvGroupRows + g, in_now, w);
+            else valid = block_pairs<kBig>(fa, T, raw, in_now, w);
             const uint4* xb = reinterpret_cast<const uint4*>(xs + cb_now * 12u);
             const uint4 x0 = xb[0], x1 = xb[1], x2 = xb[2];
             const uint32_t xv[12] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w, x2.x, x2.y, x2.z, x2.w};
             float c[4] = {0.f, 0.f, 0.f, 0.f};
             if constexpr (kFma) {
-                atomicAdd(&acc[((rg_now - rg0) * kGemvGroupRows + g) << shift | ((uint32_t)(warp * 4 + t) & ((1u << shift) - 1u))], dot24_bf16(w, xv));
+                // a block whose index is out of range adds nothing, whatever its gain and its slice of x are (as in gemv_bin_kernel)
+                atomicAdd(&acc[((rg_now - rg0) * kGemvGroupRows + g) << shift | ((uint32_t)(warp * 4 + t) & ((1u << shift) - 1u))], valid ? dot24_bf16(w, xv) : 0.f);
             } else {
 #pragma unroll
                 for (int q = 0; q < 6; ++q)

@@ -150,7 +150,8 @@ __device__ __forceinline__ RawBlock<kBig> request_block(const uint32_t* __restri
 }
 
 // The table-driven decoder of the codes whose class tables stay in global memory, from the stored stream.
-__device__ __forceinline__ void block_planes_big(const FastArgs& fa, const FastSmem& T, const RawField<true>& f, bool in, DecodedBig& d)
+// These return whether the block exists and its index is in range; the weights of one that is not are zeros times its gain.
+__device__ __forceinline__ bool block_planes_big(const FastArgs& fa, const FastSmem& T, const RawField<true>& f, bool in, DecodedBig& d)
 {
     uint64_t lo, hi;
     field_value(f, fa.dc.W, lo, hi);
@@ -159,15 +160,17 @@ __device__ __forceinline__ void block_planes_big(const FastArgs& fa, const FastS
     uint64_t local = 0;
     const int cls = valid ? big_find_class(fa.dc, lo, hi, local) : 0;
     big_decode_planes(T, fa.dc, cls, local, valid, kFullMask, d);
+    return valid;
 }
 
-__device__ __forceinline__ void block_planes(const FastArgs& fa, const FastSmem& T, const RawField<false>& f, bool in, Decoded& d)
+__device__ __forceinline__ bool block_planes(const FastArgs& fa, const FastSmem& T, const RawField<false>& f, bool in, Decoded& d)
 {
     uint64_t I, none;
     field_value(f, (int)fa.L.W, I, none);
     const bool valid = in && I < fa.n_points;
     if (in && !valid) atomicAdd(fa.bad_index, 1ull);
     fast_decode(T, I, valid, d);
+    return valid;
 }
 
 template <bool kBig>
@@ -188,18 +191,20 @@ __device__ __forceinline__ void block_bytes(const FastArgs& fa, const FastSmem& 
 }
 
 template <bool kBig>
-__device__ __forceinline__ void block_pairs(const FastArgs& fa, const FastSmem& T, const RawBlock<kBig>& r, bool in, uint32_t w[12])
+__device__ __forceinline__ bool block_pairs(const FastArgs& fa, const FastSmem& T, const RawBlock<kBig>& r, bool in, uint32_t w[12])
 {
     if constexpr (kBig) {
         DecodedBig d{};
-        block_planes_big(fa, T, r.field, in, d);
+        const bool valid = block_planes_big(fa, T, r.field, in, d);
         const float g = gain_to_float(r.gain);
         expand_bf16(d.d, g, w);
         patch_id8_bf16(d, g, w);
+        return valid;
     } else {
         Decoded d;
-        block_planes(fa, T, r.field, in, d);
+        const bool valid = block_planes(fa, T, r.field, in, d);
         expand_bf16(d, gain_to_float(r.gain), w);
+        return valid;
     }
 }
 
@@ -212,7 +217,7 @@ struct SgArgs {
     int bits;
 };
 
-__device__ __forceinline__ void block_pairs_sg(const FastArgs& fa, const FastSmem& T, const RawField<false>& raw,
+__device__ __forceinline__ bool block_pairs_sg(const FastArgs& fa, const FastSmem& T, const RawField<false>& raw,
                                                const SgArgs& sg, int64_t row, bool in, uint32_t w[12])
 {
     uint64_t f, none;
@@ -231,6 +236,7 @@ __device__ __forceinline__ void block_pairs_sg(const FastArgs& fa, const FastSme
         g = __fmul_rn(__fmul_rn(scale, __ldg(sg.codebook + k)), __uint_as_float(T.desc[cls * kFastDescStride + kFastDescRnorm]));
     }
     expand_bf16(d, g, w);
+    return valid;
 }
 
 // Programmatic dependent launch: a GEMV kernel lets the next kernel of the stream start early (its thread blocks

@@ -43,3 +43,34 @@ def test_small_shape_gain_products(oracle_mod):
         for _ in range(2):
             assert gemv_error(P.llvq_gemv_sg(ctx, d_s, 1, cb, scale, n_out, k_in, x).cpu().numpy(), want) <= 1e-3
     assert P.llvq_last_error(ctx) == (0, 0)
+
+
+@pytest.mark.parametrize("blocks", [31, 32, 33])          # units per thread block where every group of 8 rows has one: the two kernels' border lies at 32
+@pytest.mark.parametrize("gain_bits", [None, 1])
+def test_out_of_range_blocks_add_nothing_whatever_they_meet(oracle_mod, blocks, gain_bits):
+    code = (2, 13) if gain_bits is None else (2, 12)
+    o, ctx = oracle_mod.Code(*code), P.Context(*code, device=0)
+    n_out, k_in = 8 * torch.cuda.get_device_properties(0).multi_processor_count, 96 * blocks
+    bpr, row = k_in // 24, 777
+    lo, hi = gen.random_indices(o.N, o.W, n_out * bpr, seed=blocks)
+    x = gen.normal_bf16(k_in, seed=1)
+    for at in (3, bpr - 1):
+        lo[row * bpr + at] = o.N                          # the first index that is out of range ...
+    d_x = to_dev_bf16(x)
+    d_x[24 * 3 + 5], d_x[24 * (bpr - 1)] = float("inf"), float("nan")       # ... meets what is not finite
+    x[24 * 3:24 * 4] = x[24 * (bpr - 1):] = 0
+    if gain_bits is None:
+        gain = gen.make_layer(o.N, o.W, n_out, k_in, 1, seed=2)[1]
+        gain[row * bpr + 3] = 0x7c00
+        d_s, d_g = to_dev_u8(gen.pack_indices(lo, hi, o.W)), to_dev_f16(gain)
+        y = P.llvq_gemv(ctx, d_s, d_g, n_out, k_in, d_x)
+        w = P.llvq_dequant_matrix(ctx, d_s, d_g, n_out, k_in, P.LLVQ_LAYOUT_ROWWISE)
+    else:
+        k = gen.gain_indices(n_out * bpr, gain_bits, seed=2)
+        d_s = to_dev_u8(gen.pack_indices(lo | (k << np.uint64(o.W)), hi, o.W + gain_bits))
+        cb, scale = torch.tensor([4.3, 5.4], device="cuda"), torch.full((n_out,), 0.02, device="cuda")
+        y = P.llvq_gemv_sg(ctx, d_s, gain_bits, cb, scale, n_out, k_in, d_x)
+        w = P.llvq_dequant_matrix_sg(ctx, d_s, gain_bits, cb, scale, n_out, k_in)
+    terms = torch.where(to_dev_bf16(x) == 0, 0.0, w[row].double() * to_dev_bf16(x).double())
+    assert abs(y[row].item() - terms.sum().item()) <= 100 * 2.0 ** -24 * terms.abs().sum().item()      # a term goes through fewer than 100 binary32 additions
+    assert P.llvq_last_error(ctx)[0] == 4                 # two blocks, counted by the product and by the dequantizer
