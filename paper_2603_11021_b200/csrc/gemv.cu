@@ -134,40 +134,46 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     const size_t smem_fma = (ext_fma ? ctx->fl.total_ext : ctx->fl.total) + rest_fma;
     if (bin && !fma) {
         const FastArgs fa = fast_args(ctx, ext_bin);
-#define LLVQ_LAUNCH_BIN(BF16, SG, SH)                                                                                      \
+#define LLVQ_LAUNCH_BIN_T(BF16, SG, SH, TREES)                                                                             \
     do {                                                                                                                   \
-        if (!set_smem<gemv_bin_kernel<BF16, SG, SH>>(ctx, smem_bin)) return LLVQ_ECUDA;                                          \
-        if (launch_pdl(gemv_bin_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
+        if (!set_smem<gemv_bin_kernel<BF16, SG, SH, TREES>>(ctx, smem_bin)) return LLVQ_ECUDA;                                   \
+        if (launch_pdl(gemv_bin_kernel<BF16, SG, SH, TREES>, g, (unsigned)kSortThreads, smem_bin, st, fa, idx, ctx->d_sort_rank, d_gain_f16, sga, sp, n_out, k_in, \
                        bpr, acc_floats, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
     } while (0)
+#define LLVQ_LAUNCH_BIN(BF16, SG, SH) do { if (sp.trees) LLVQ_LAUNCH_BIN_T(BF16, SG, SH, true); else LLVQ_LAUNCH_BIN_T(BF16, SG, SH, false); } while (0)
         if (shard)   { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, true); else LLVQ_LAUNCH_BIN(false, false, true); }
         else if (sg) { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, true, false); else LLVQ_LAUNCH_BIN(false, true, false); }
         else         { if (y_dtype == LLVQ_BF16) LLVQ_LAUNCH_BIN(true, false, false); else LLVQ_LAUNCH_BIN(false, false, false); }
 #undef LLVQ_LAUNCH_BIN
+#undef LLVQ_LAUNCH_BIN_T
         return launch_status();
     }
     if (order && !fma) {
         const FastArgs fa = fast_args(ctx, ext_order);
-#define LLVQ_LAUNCH_ORDER(BF16, SG, SH)                                                                               \
+#define LLVQ_LAUNCH_ORDER_T(BF16, SG, SH, TREES)                                                                      \
     do {                                                                                                                   \
-        if (!set_smem<gemv_order_kernel<BF16, SG, SH>>(ctx, smem_order)) return LLVQ_ECUDA;                   \
-        if (launch_pdl(gemv_order_kernel<BF16, SG, SH>, g, (unsigned)kSortThreads, smem_order, st, fa, idx, oa, d_gain_f16, sga, sp, n_out, k_in, \
+        if (!set_smem<gemv_order_kernel<BF16, SG, SH, TREES>>(ctx, smem_order)) return LLVQ_ECUDA;                   \
+        if (launch_pdl(gemv_order_kernel<BF16, SG, SH, TREES>, g, (unsigned)kSortThreads, smem_order, st, fa, idx, oa, d_gain_f16, sga, sp, n_out, k_in, \
                        bpr, d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;              \
     } while (0)
         const bool bf16 = y_dtype == LLVQ_BF16;
+#define LLVQ_LAUNCH_ORDER(BF16, SG, SH) do { if (sp.trees) LLVQ_LAUNCH_ORDER_T(BF16, SG, SH, true); else LLVQ_LAUNCH_ORDER_T(BF16, SG, SH, false); } while (0)
         if (shard)   { if (bf16) LLVQ_LAUNCH_ORDER(true, false, true); else LLVQ_LAUNCH_ORDER(false, false, true); }
         else if (sg) { if (bf16) LLVQ_LAUNCH_ORDER(true, true, false); else LLVQ_LAUNCH_ORDER(false, true, false); }
         else         { if (bf16) LLVQ_LAUNCH_ORDER(true, false, false); else LLVQ_LAUNCH_ORDER(false, false, false); }
 #undef LLVQ_LAUNCH_ORDER
+#undef LLVQ_LAUNCH_ORDER_T
         return launch_status();
     }
     const FastArgs fa = fast_args(ctx, fma ? ext_fma : ext_direct);
-#define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH, FMA)                                                                   \
+#define LLVQ_LAUNCH_GEMV_T(BIG, BF16, SG, SH, FMA, TREES)                                                          \
     do {                                                                                                           \
-        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH, FMA>>(ctx, FMA ? smem_fma : smem)) return LLVQ_ECUDA;                          \
-        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH, FMA>, g, FMA ? fma_threads : threads, FMA ? smem_fma : smem, st, fa, idx, d_gain_f16, sga, sp, FMA ? (uint32_t)kGemvGroupsPerPass : per_pass, n_out, k_in, bpr, \
+        if (!set_smem<gemv_fast_kernel<BIG, BF16, SG, SH, FMA, TREES>>(ctx, FMA ? smem_fma : smem)) return LLVQ_ECUDA;                          \
+        if (launch_pdl(gemv_fast_kernel<BIG, BF16, SG, SH, FMA, TREES>, g, FMA ? fma_threads : threads, FMA ? smem_fma : smem, st, fa, idx, d_gain_f16, sga, sp, FMA ? (uint32_t)kGemvGroupsPerPass : per_pass, n_out, k_in, bpr, \
                        d_x_bf16, yo, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;           \
     } while (0)
+#define LLVQ_LAUNCH_GEMV(BIG, BF16, SG, SH, FMA)                                                                   \
+    do { if (sp.trees) LLVQ_LAUNCH_GEMV_T(BIG, BF16, SG, SH, FMA, true); else LLVQ_LAUNCH_GEMV_T(BIG, BF16, SG, SH, FMA, false); } while (0)
     const unsigned fma_threads = 32u * (unsigned)std::max<int64_t>(upc, 16);        // a warp per unit
     const bool bf16 = y_dtype == LLVQ_BF16;
     if (fma && shard)       { if (bf16) LLVQ_LAUNCH_GEMV(false, true, false, true, true);   else LLVQ_LAUNCH_GEMV(false, false, false, true, true); }
@@ -179,6 +185,7 @@ int gemv_common(const llvq_ctx* ctx, const void* d_idx, const uint16_t* d_gain_f
     else if (ctx->fast)     { if (bf16) LLVQ_LAUNCH_GEMV(false, true, false, false, false); else LLVQ_LAUNCH_GEMV(false, false, false, false, false); }
     else                    { if (bf16) LLVQ_LAUNCH_GEMV(true, true, false, false, false);  else LLVQ_LAUNCH_GEMV(true, false, false, false, false); }
 #undef LLVQ_LAUNCH_GEMV
+#undef LLVQ_LAUNCH_GEMV_T
     return launch_status();
 }
 
@@ -343,7 +350,11 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         slot += (d.n_out + kGemvGroupRows - 1) / kGemvGroupRows * kGemvGroupRows;
     }
     if (slot > 64ll * kMaxScratchRows) return LLVQ_EUNSUPPORTED;
-    for (int i = 0; i < n_mats; ++i) mm.m[i].sp.trees = tree_rows(mm.m[i].slot0, mm.m[i].n_out, slot);
+    bool trees = false;
+    for (int i = 0; i < n_mats; ++i) {
+        mm.m[i].sp.trees = tree_rows(mm.m[i].sp, mm.m[i].slot0, mm.m[i].n_out, slot);
+        trees = trees || mm.m[i].sp.trees;
+    }
     size_t smem; bool ext;                               // the longest rows decide for the whole launch
     OrderArgs oa{};
     if (sorted) sorted_smem(ctx, max_nq, smem, ext, acc_floats);
@@ -359,6 +370,17 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
     cudaStream_t st = (cudaStream_t)stream;
     const FastArgs fa = fast_args(ctx, ext);
     const unsigned g = (unsigned)ctx->sm_count;
+    const bool bf16 = y_dtype == LLVQ_BF16;
+#define LLVQ_LAUNCH_MULTI_T(K, BYTES, ...)                                                                                                      \
+    do {                                                                                                                                        \
+        if (!set_smem<K>(ctx, BYTES)) return LLVQ_ECUDA;                                                                                        \
+        if (launch_pdl(K, g, (unsigned)kSortThreads, BYTES, st, fa, __VA_ARGS__, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
+    } while (0)
+#define LLVQ_LAUNCH_MULTI(K, BYTES, ...)                                                                                    \
+    do {                                                                                                                    \
+        if (trees) { if (bf16) LLVQ_LAUNCH_MULTI_T((K<true, true>), BYTES, __VA_ARGS__); else LLVQ_LAUNCH_MULTI_T((K<false, true>), BYTES, __VA_ARGS__); } \
+        else { if (bf16) LLVQ_LAUNCH_MULTI_T((K<true, false>), BYTES, __VA_ARGS__); else LLVQ_LAUNCH_MULTI_T((K<false, false>), BYTES, __VA_ARGS__); } \
+    } while (0)
     if (sorted && n_mats >= 2) {
         // the kernel without a barrier between the matrices, when every CTA's share of every matrix is one segment and
         // one pass and three sets of (x, row sums) fit beside the tables
@@ -379,35 +401,15 @@ static int gemv_multi_common(const llvq_ctx* ctx, const llvq_gemv_desc* descs, i
         while (shift > 2 && ov_bytes() > kSmemLimit) --shift;
         const size_t smem_ov = ov_bytes();
         if (one_pass && max_groups <= kGemvGroupsPerPass && smem_ov <= kSmemLimit) {
-            if (y_dtype == LLVQ_BF16) {
-                if (!set_smem<gemv_sorted_overlap_kernel<true>>(ctx, smem_ov)) return LLVQ_ECUDA;
-                if (launch_pdl(gemv_sorted_overlap_kernel<true>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, shift, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
-            } else {
-                if (!set_smem<gemv_sorted_overlap_kernel<false>>(ctx, smem_ov)) return LLVQ_ECUDA;
-                if (launch_pdl(gemv_sorted_overlap_kernel<false>, g, (unsigned)kSortThreads, smem_ov, st, fa, mm, xs_words, acc_rows, shift, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
-            }
+            LLVQ_LAUNCH_MULTI(gemv_sorted_overlap_kernel, smem_ov, mm, xs_words, acc_rows, shift);
             return launch_status();
         }
     }
-    if (sorted) {
-        if (y_dtype == LLVQ_BF16) {
-            if (!set_smem<gemv_sorted_multi_kernel<true>>(ctx, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_sorted_multi_kernel<true>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
-        } else {
-            if (!set_smem<gemv_sorted_multi_kernel<false>>(ctx, smem)) return LLVQ_ECUDA;
-            if (launch_pdl(gemv_sorted_multi_kernel<false>, g, (unsigned)kSortThreads, smem, st, fa, mm, acc_floats, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA;
-        }
-    } else {
-#define LLVQ_LAUNCH_MULTI(K, ...)                                                                                                  \
-    do {                                                                                                                           \
-        if (!set_smem<K>(ctx, smem)) return LLVQ_ECUDA;                                                                     \
-        if (launch_pdl(K, g, (unsigned)kSortThreads, smem, st, fa, __VA_ARGS__, ctx->d_scratch, ctx->d_counters) != cudaSuccess) return LLVQ_ECUDA; \
-    } while (0)
-        const bool bf16 = y_dtype == LLVQ_BF16;
-        if (bin) { if (bf16) LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<true>, ctx->d_sort_rank, mm, acc_floats); else LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel<false>, ctx->d_sort_rank, mm, acc_floats); }
-        else     { if (bf16) LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel<true>, oa, mm, (uint32_t)max_nq); else LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel<false>, oa, mm, (uint32_t)max_nq); }
+    if (sorted) { if (bf16) LLVQ_LAUNCH_MULTI_T(gemv_sorted_multi_kernel<true>, smem, mm, acc_floats); else LLVQ_LAUNCH_MULTI_T(gemv_sorted_multi_kernel<false>, smem, mm, acc_floats); }
+    else if (bin) LLVQ_LAUNCH_MULTI(gemv_bin_multi_kernel, smem, ctx->d_sort_rank, mm, acc_floats);
+    else LLVQ_LAUNCH_MULTI(gemv_order_multi_kernel, smem, oa, mm, (uint32_t)max_nq);
 #undef LLVQ_LAUNCH_MULTI
-    }
+#undef LLVQ_LAUNCH_MULTI_T
     return launch_status();
 }
 

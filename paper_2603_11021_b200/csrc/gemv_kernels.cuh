@@ -75,7 +75,11 @@ __device__ __forceinline__ void stage_x(uint32_t* xs, const uint16_t* __restrict
 // by exactly two CTAs take a shorter way, below).
 // The caller puts a __syncthreads() before (sums complete) and after (sums may be cleared) the call.
 // slot0 (a multiple of 8) = first scratch row / pair slot of this matrix when one launch works on several matrices.
-template <bool kOutBf16, bool kShard, typename RowSums>
+// kTrees = the trees of slots are part of the kernel, for launches some of whose groups are shared by three CTAs or more: where none is, their code
+// alone cost the kernels on stored streams 0.1 to 0.2 us (72-bit code, 1400 x 1000 9.38 us without, 9.59 with it; shells 3, 2048 x 1024 5.00 and
+// 5.09) and gemv_sorted_overlap_kernel nine registers.  gemv_sorted_kernel always has it: it comes out faster with it (1400 x 1000 6.53 us, 6.64 without;
+// shape-gain 4096 x 11008 38.5 and 39.2).
+template <bool kOutBf16, bool kShard, bool kTrees, typename RowSums>
 __device__ __forceinline__ void finish_pass(const YOut& yo, const Split& sp, uint32_t rg0, uint32_t rg1, uint32_t u_begin, uint32_t u_end,
                                             int64_t n_out, float* __restrict__ scratch, uint32_t* __restrict__ counters, RowSums row_sums,
                                             int64_t slot0 = 0, int warp_of = -1, int nwarps_of = 0)
@@ -110,7 +114,7 @@ __device__ __forceinline__ void finish_pass(const YOut& yo, const Split& sp, uin
             }
             continue;
         }
-        if (parts <= 8u && sp.trees) {
+        if (kTrees && parts <= 8u && sp.trees) {
             // three to eight CTAs (short rows of small matrices): a tree of such slots, seven per row, over the CTAs in order.  Who finds a
             // slot empty is done; the other goes on to the next one with both sums.  Up to three round trips for the last to arrive, where
             // the way below takes a fence on either side of the counter and a read behind it (sorted 512 x 1024:
@@ -214,7 +218,7 @@ __device__ __forceinline__ float acc_row_sums(const float* acc, uint32_t first, 
 
 // kFma: each lane forms its own dot product with binary32 FMAs instead (what small matrices of codes with many classes take, whose larger ones go to
 // gemv_bin_kernel: the tensor core's sums are 1.3 to 1.6 times as far from exact ones, 1.0e-7 against 6.4e-8 of the 2-norm at 1000 x 1000).
-template <bool kBig, bool kOutBf16, bool kSg = false, bool kShard = false, bool kFma = false>
+template <bool kBig, bool kOutBf16, bool kSg, bool kShard, bool kFma, bool kTrees>
 __global__ void __launch_bounds__(kGemvThreads, 1)
 gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, SgArgs sg, Split sp, uint32_t groups_per_pass,
                  int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
@@ -275,7 +279,7 @@ gemv_fast_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_
         }
         __syncthreads();
         // row groups this CTA covers completely are final; the (at most two) split ones go through the scratch
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) {
+        finish_pass<kOutBf16, kShard, kTrees>(yo, sp, rg0, rg1, u_begin, u_end, n_out, scratch, counters, [&](uint32_t r) {
             if constexpr (kFma) return acc_row_sums(acc, r, shift);
             return lane < kGemvGroupRows ? acc[r + lane] : 0.f;
         });
@@ -498,12 +502,12 @@ __device__ __forceinline__ void gemv_sorted_body(const FastArgs& fa, const FastS
         // end of the pass: row groups this CTA covers completely are final; the split ones go through the scratch
         auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
         const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
+        finish_pass<kOutBf16, kShard, true>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     });
 }
 
-template <bool kOutBf16, bool kSg = false, bool kShard = false>
+template <bool kOutBf16, bool kSg, bool kShard>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_sorted_kernel(FastArgs fa, const unsigned long long* __restrict__ sorted, const uint16_t* __restrict__ gain, SgArgs sg,
                    Split sp, int64_t n_out, int64_t k_in, int64_t bpr, uint32_t acc_floats, const uint16_t* __restrict__ x, YOut yo,
@@ -549,7 +553,7 @@ struct OverlapSet {
     uint32_t pad;
 };
 
-template <bool kOutBf16>
+template <bool kOutBf16, bool kTrees>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, int xs_words, int acc_rows, uint32_t shift, float* __restrict__ scratch,
                            uint32_t* __restrict__ counters)
@@ -644,7 +648,7 @@ gemv_sorted_overlap_kernel(FastArgs fa, const __grid_constant__ GemvMulti mm, in
             YOut yo{};
             yo.y = M.y;
             auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
-            finish_pass<kOutBf16, false>(yo, sp, rg0, split_row(sp, ue - 1u), ub, ue, M.n_out, scratch, counters, row_sums, M.slot0, 0, 1);
+            finish_pass<kOutBf16, false, kTrees>(yo, sp, rg0, split_row(sp, ue - 1u), ub, ue, M.n_out, scratch, counters, row_sums, M.slot0, 0, 1);
             __syncwarp();
             if (i + kOverlapSets < mm.n) {
                 if (lane == 0) { ctl[set].next_chunk = 0u; ctl[set].arrived = 0u; }
@@ -689,7 +693,7 @@ __device__ __forceinline__ void prefetch_stored_span(const FastArgs& fa, const u
 }
 
 // One matrix; `piece` = pieces this team has been through.
-template <bool kOutBf16, bool kSg, bool kShard>
+template <bool kOutBf16, bool kSg, bool kShard, bool kTrees>
 __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSmem& T, const OrderArgs& oa, uint32_t* xs, uint8_t* areas,
                                                 const uint32_t* __restrict__ stream, const uint16_t* __restrict__ gain, const SgArgs& sg, const Split& sp,
                                                 int64_t n_out, int64_t k_in, uint32_t bpr, const uint16_t* __restrict__ x, const YOut& yo,
@@ -760,7 +764,7 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
         }
         __syncthreads();
         const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, [&](uint32_t i) { return acc_row_sums(acc, i, shift); }, slot0);
+        finish_pass<kOutBf16, kShard, kTrees>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, [&](uint32_t i) { return acc_row_sums(acc, i, shift); }, slot0);
         __syncthreads();                                   // the sums are read above: the next pass may clear them only now
     }, 1u << 30);
 }
@@ -772,7 +776,7 @@ __device__ __forceinline__ void gemv_order_body(const FastArgs& fa, const FastSm
     for (uint32_t i = threadIdx.x; i < kOrderTeams * 2 * oa.words; i += blockDim.x) reinterpret_cast<uint32_t*>(areas + 16)[i] = 0u; \
     uint32_t piece = 0;
 
-template <bool kOutBf16, bool kSg = false, bool kShard = false>
+template <bool kOutBf16, bool kSg, bool kShard, bool kTrees>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_order_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa, const uint16_t* __restrict__ gain, SgArgs sg,
                   Split sp, int64_t n_out, int64_t k_in, int64_t bpr, const uint16_t* __restrict__ x, YOut yo,
@@ -781,12 +785,12 @@ gemv_order_kernel(FastArgs fa, const uint32_t* __restrict__ stream, OrderArgs oa
     prefetch_stored_span<kSg>(fa, stream, gain, sg, sp, n_out, bpr);       // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
     ORDER_PROLOGUE(sp.per_row);
-    gemv_order_body<kOutBf16, kSg, kShard>(fa, T, oa, xs, areas, stream, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0, piece);
+    gemv_order_body<kOutBf16, kSg, kShard, kTrees>(fa, T, oa, xs, areas, stream, gain, sg, sp, n_out, k_in, (uint32_t)bpr, x, yo, scratch, counters, 0, piece);
     if (kShard) shard_arrive(yo);
 }
 
 // Several independent matrices on their stored streams in one launch; max_nq = the largest number of units per row group.
-template <bool kOutBf16>
+template <bool kOutBf16, bool kTrees>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_order_multi_kernel(FastArgs fa, OrderArgs oa, const __grid_constant__ GemvMulti mm, uint32_t max_nq, float* __restrict__ scratch,
                         uint32_t* __restrict__ counters)
@@ -801,7 +805,7 @@ gemv_order_multi_kernel(FastArgs fa, OrderArgs oa, const __grid_constant__ GemvM
                                         mm.m[i + 1].n_out, mm.m[i + 1].bpr);
         YOut yo{};
         yo.y = M.y;
-        gemv_order_body<kOutBf16, false, false>(fa, T, oa, xs, areas, static_cast<const uint32_t*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
+        gemv_order_body<kOutBf16, false, false, kTrees>(fa, T, oa, xs, areas, static_cast<const uint32_t*>(M.weights), M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
                                                        (uint32_t)M.bpr, M.x, yo, scratch, counters, M.slot0, piece);
     }
 }
@@ -816,7 +820,7 @@ gemv_order_multi_kernel(FastArgs fa, OrderArgs oa, const __grid_constant__ GemvM
 constexpr int kBinSegUnits = 256;                    // at most 8192 blocks per segment
 constexpr int kBinPerThread = kBinSegUnits * 32 / kSortThreads;   // 8
 
-template <bool kOutBf16, bool kSg, bool kShard>
+template <bool kOutBf16, bool kSg, bool kShard, bool kTrees>
 __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem& T, uint8_t* staging, const uint32_t* __restrict__ stream,
                                               const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, const SgArgs& sg,
                                               const Split& sp, int64_t n_out, int64_t k_in, uint32_t bpr, uint32_t acc_floats,
@@ -941,12 +945,12 @@ __device__ __forceinline__ void gemv_bin_body(const FastArgs& fa, const FastSmem
         if (!last) return;
         auto row_sums = [&](uint32_t r) { return acc_row_sums(acc, r, shift); };
         const uint32_t ub = split_begin(sp, blockIdx.x), ue = split_begin(sp, blockIdx.x + 1u);     // recomputed here: not kept across the main loop
-        finish_pass<kOutBf16, kShard>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
+        finish_pass<kOutBf16, kShard, kTrees>(yo, sp, rg0, rg1, ub, ue, n_out, scratch, counters, row_sums, slot0);
         __syncthreads();
     }, (uint32_t)kBinSegUnits);
 }
 
-template <bool kOutBf16, bool kSg = false, bool kShard = false>
+template <bool kOutBf16, bool kSg, bool kShard, bool kTrees>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_bin_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t* __restrict__ sort_rank, const uint16_t* __restrict__ gain, SgArgs sg,
                 Split sp, int64_t n_out, int64_t k_in, int64_t bpr, uint32_t acc_floats, const uint16_t* __restrict__ x, YOut yo,
@@ -954,12 +958,12 @@ gemv_bin_kernel(FastArgs fa, const uint32_t* __restrict__ stream, const uint16_t
 {
     prefetch_stored_span<kSg>(fa, stream, gain, sg, sp, n_out, bpr);       // while the table image is on its way
     FAST_PROLOGUE(if (kShard) shard_arrive(yo));
-    gemv_bin_body<kOutBf16, kSg, kShard>(fa, T, staging, stream, sort_rank, gain, sg, sp, n_out, k_in, (uint32_t)bpr, acc_floats, x, yo, scratch, counters, 0);
+    gemv_bin_body<kOutBf16, kSg, kShard, kTrees>(fa, T, staging, stream, sort_rank, gain, sg, sp, n_out, k_in, (uint32_t)bpr, acc_floats, x, yo, scratch, counters, 0);
     if (kShard) shard_arrive(yo);
 }
 
 // Several independent matrices on their stored streams in one launch.
-template <bool kOutBf16>
+template <bool kOutBf16, bool kTrees>
 __global__ void __launch_bounds__(kSortThreads, 1)
 gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const __grid_constant__ GemvMulti mm, uint32_t acc_floats, float* __restrict__ scratch,
                       uint32_t* __restrict__ counters)
@@ -973,7 +977,7 @@ gemv_bin_multi_kernel(FastArgs fa, const uint16_t* __restrict__ sort_rank, const
                                      mm.m[i + 1].n_out, mm.m[i + 1].bpr);
         YOut yo{};
         yo.y = M.y;
-        gemv_bin_body<kOutBf16, false, false>(fa, T, staging, static_cast<const uint32_t*>(M.weights), sort_rank, M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
+        gemv_bin_body<kOutBf16, false, false, kTrees>(fa, T, staging, static_cast<const uint32_t*>(M.weights), sort_rank, M.gain, SgArgs{}, M.sp, M.n_out, M.k_in,
                                               (uint32_t)M.bpr, acc_floats, M.x, yo, scratch, counters, M.slot0);
         __syncthreads();
     }

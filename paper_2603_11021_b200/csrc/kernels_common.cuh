@@ -80,7 +80,7 @@ struct Split {
     uint32_t ctas_magic;                     // ceil(2^32 / ctas): exact quotients of numbers below ctas^2 (ctas < 1625)
     uint32_t per_row, row_magic;             // floor(2^32 / per_row): quotients at most one too small
     float ctas_per_unit;
-    uint32_t trees;                          // finish_pass may use the trees of slots (set by the GEMV's launches)
+    uint32_t trees;                          // finish_pass takes the trees of slots (set by the GEMV's launches)
 };
 
 Split make_split(int64_t units, int64_t per_row, unsigned ctas)
@@ -95,14 +95,17 @@ Split make_split(int64_t units, int64_t per_row, unsigned ctas)
     return s;
 }
 
-// Whether the rows from first_row on of a GEMV launch of `rows` rows in all may use the trees of slots: those lie at the end of the slots,
-// which the rows' own slots must not reach.
-uint32_t tree_rows(int64_t first_row, int64_t n_out, int64_t rows) { return first_row + n_out <= kTreeRows && rows <= kPairSlots - 8 * kTreeRows; }
+// Whether the rows of a GEMV launch from first_row on (of `rows` rows in all) take the trees of slots.  Three CTAs or more share a row group only where
+// it holds the whole range of one and a unit on either side; and the trees lie at the end of the slots, which the rows' own slots must not reach.
+uint32_t tree_rows(const Split& s, int64_t first_row, int64_t n_out, int64_t rows)
+{
+    return s.per_row >= s.each + 2u && first_row + n_out <= kTreeRows && rows <= kPairSlots - 8 * kTreeRows;
+}
 
 Split make_gemv_split(int64_t units, int64_t per_row, unsigned ctas, int64_t n_out)
 {
     Split s = make_split(units, per_row, ctas);
-    s.trees = tree_rows(0, n_out, n_out);
+    s.trees = tree_rows(s, 0, n_out, n_out);
     return s;
 }
 

@@ -74,3 +74,24 @@ def test_out_of_range_blocks_add_nothing_whatever_they_meet(oracle_mod, blocks, 
     terms = torch.where(to_dev_bf16(x) == 0, 0.0, w[row].double() * to_dev_bf16(x).double())
     assert abs(y[row].item() - terms.sum().item()) <= 100 * 2.0 ** -24 * terms.abs().sum().item()      # a term goes through fewer than 100 binary32 additions
     assert P.llvq_last_error(ctx)[0] == 4                 # two blocks, counted by the product and by the dequantizer
+
+
+def test_groups_shared_by_many_and_by_two_in_one_launch(oracle_mod):
+    # the trees of slots serve the first and the last of these matrices, the pairs of slots the other one
+    o, ctx = oracle_mod.Code(2, 13), P.Context(2, 13, device=0)
+    mats, want = [], []
+    for n_out, k_in in [(240, 8000), (4096, 480), (1000, 1000)]:
+        stream, gain, _ = gen.make_layer(o.N, o.W, n_out, k_in, 1, seed=n_out)
+        x = gen.normal_bf16(k_in, seed=k_in)
+        want.append(o.gemv(stream, gain, n_out, k_in, x))
+        mats.append((to_dev_u8(stream), to_dev_f16(gain), n_out, k_in, to_dev_bf16(x)))
+    y = [torch.empty(m[2], dtype=torch.float32, device="cuda") for m in mats]
+    stored = [m + (out,) for m, out in zip(mats, y)]
+    srt = [(P.llvq_sort_blocks(ctx, m[0], m[2], m[3]),) + m[1:] for m in stored]
+    for multi, args in [(P.llvq_gemv_multi, stored), (P.llvq_gemv_sorted_multi, srt), (P.llvq_gemv_sorted_multi, srt[:2]), (P.llvq_gemv_multi, stored)]:
+        for out in y:
+            out.fill_(-1)
+        multi(ctx, args)
+        for out, w in zip(y[:len(args)], want):
+            assert gemv_error(out.cpu().numpy(), w) <= 1e-3
+    assert P.llvq_last_error(ctx) == (0, 0)
