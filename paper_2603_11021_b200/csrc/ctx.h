@@ -35,7 +35,7 @@ struct llvq_ctx {
     llvq::FastLayout fl{};
     const uint8_t* d_image = nullptr;
     uint64_t largest_class = 0;      // points of the largest class
-    bool can_encode = false;         // m_lo == 2, m_hi >= 6, indices fit 64 bits
+    bool can_encode = false;         // m_lo == 2, m_hi >= 3, indices fit 64 bits
     EncTables enc{};
     llvq::GolayTrio trio{};
     const uint32_t* d_golay = nullptr;   // [4096] sorted codewords in global memory

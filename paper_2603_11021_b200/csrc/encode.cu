@@ -353,13 +353,18 @@ __device__ __forceinline__ double dot_of_warp(double u, int xi)
     return dot;
 }
 
-// Vectors of a CTA that wait for nearest_careful, and its answers.
 // More vectors per SM than this: two lanes take a vector, else a warp does.  Two lanes per vector use the chip best, but a CTA works on 256 vectors at a time
-// for some 15 us; shells 2..13 and 2..12, us for a warp per vector / two lanes: EUCLIDEAN 12 000 vectors 50 / 69, 30 000 79 / 87, 40 000 98 / 112, 52 000 113 / 118;
-// ANGULAR 5000 71 / 90, 15 700 148 / 190, 25 000 240 / 196.
+// for some 15 us.  Gaussian inputs, us for a warp per vector / two lanes by vectors per SM (of 148):
+//   EUCLIDEAN shells 2..13  260 87 / 100  330 104 / 112  384 114 / 114  450 128 / 126;  both are equal at 265 (2..3), 365 (2..5), 385 (2..8), 430 (2..20), 460 (2..24)
+//   ANGULAR   shells 2..13  100 143 / 181  136 184 / 190  150 200 / 193  200 255 / 200;  both are equal at 115 (2..3), 130 (2..5), 136 (2..8), 148 (2..20), 145 (2..24)
+// Inputs on a coarse grid, most of which have several nearest cosets, would be better off with a warp per vector (EUCLIDEAN, 174 763 vectors: integers 557 /
+// 908, halves 404 / 475, quarters 336 / 338), which the host cannot know; a block that changes over when it meets them costs all inputs 2.5 % and gains those 4 %.
 constexpr uint64_t kPairsFromEuclidean = 384, kPairsFromAngular = 136;
-constexpr int kFew = 40;                   // no more vectors than this left in a CTA: all of them go to nearest_careful (EUCLIDEAN 867 -> 761 us with the wider loads)
+// No more vectors than this left in a CTA: all of them go to nearest_careful.  The two metrics' largest cases, us: never (0) 817 / 869, 16 690 / 745, 40 670 / 721,
+// 80 656 / 712.
+constexpr int kFew = 40;
 constexpr uint32_t kPendingMost = 48, kPendingEnough = 14;
+// A vector of a CTA that waits for nearest_careful, and the answer.
 struct Pending {
     double rn, radius, dot;
     const float* v;

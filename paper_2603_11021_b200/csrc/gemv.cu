@@ -66,7 +66,9 @@ void sorted_smem(const llvq_ctx* ctx, int64_t nq, size_t& bytes, bool& ext, uint
 // 19 10.7 / 7.3, 27 10.0 / 8.3; with two rounds 37 13.1 / 13.2.
 constexpr int64_t kOneRound = 32;
 // With two CTAs per row group, or one, a row's sum takes one exchange or none instead of a tree of them: about 1 us, which some ten units more per CTA cost
-// (512 x 1024 7.9 -> 6.6 us, 1000 x 1000 8.0 -> 6.4).
+// (512 x 1024 7.9 -> 6.7 us, 1000 x 1000 8.0 -> 6.4).  The same cut serves the codes that stay with the direct kernel as it was, us without / with it:
+// 72 bits 600 x 1000 9.5 / 8.5, 304 x 2880 10.2 / 9.9, 1100 x 2900 12.8 / 11.9; shells 3 600 x 1920 5.2 / 4.8, 1000 x 2000 5.7 / 4.9; shells 2..11 with two gain
+// bits 640 x 1900 7.4 / 6.9.  Six more units per CTA and no row whole is where it loses most: 400 x 4000 7.9 / 8.0, 72 bits 10.4 / 10.9.
 constexpr int64_t kMoreUnits = 10;
 
 // Shared by llvq_gemv, llvq_gemv_sg and llvq_gemv_rowshard: exactly one of d_gain_f16 / sg is used.

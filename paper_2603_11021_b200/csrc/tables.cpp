@@ -450,7 +450,6 @@ bool build_golay_trio(const HostTables& t, GolayTrio& out)
         for (int q = 0; q < 8; ++q) {
             const uint8_t c = kOrder[8 * o + q];
             out.coord[8 * o + q] = c;
-            out.place[c] = (uint8_t)(8 * o + q);
             out.ones[o] |= 1u << c;
         }
         if (!in_code(out.ones[o])) return false;

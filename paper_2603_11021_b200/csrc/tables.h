@@ -184,7 +184,6 @@ struct GolayTrio {
     uint32_t ones[3];       // the octads
     uint8_t pat[3][64];     // the same bits packed: bit p = coordinate coord[8 * octad + p]; the same for all three octads
     uint8_t coord[24];      // coordinates octad by octad, in the order that makes the patterns those of kTurynA and kTurynX
-    uint8_t place[24];      // where in coord a coordinate is
 };
 bool build_golay_trio(const HostTables& t, GolayTrio& out);
 
