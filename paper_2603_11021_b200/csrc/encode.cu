@@ -43,6 +43,7 @@ struct __align__(128) WarpTables {
     uint32_t cand[kMaxCand - 1];
     uint32_t ncand;
 };
+static_assert((kMaxCand - 1) * 24 <= sizeof(WarpTables::nib) && 24 * sizeof(double) <= sizeof(WarpTables::pk), "the candidates' points and the input take the tables' place");
 
 // Nibbles of the octad patterns [octad][a = 1..3] (x = 0), times 8 (the row bytes of WarpTables::nib they select): patterns are
 // linear in (x, a), so the address of a pattern is that of (x, a & 4) XOR one of these.
@@ -230,21 +231,53 @@ __device__ __forceinline__ int nearest_careful_from(WarpTables& W, const GolayTr
     if (listed == 1u) {
         const uint32_t k = W.cand[0];
         best_x = coset_point(u, k & 0xffffffu, (int)(k >> 24), lane, unique);
-    } else {
+    } else if (listed <= (uint32_t)(kMaxCand - 1)) {
+        // the candidates' points one after the other, their squared distances a lane each: 24 dependent additions for all of them together
         unique = false;
-        const uint32_t n = listed > (uint32_t)(kMaxCand - 1) ? 8192u : listed;      // too many near-ties to list: every coset
-        double best_d2 = 1.0e300;
-        uint32_t best_id = 0xffffffffu;
-        best_x = 0;
-        for (uint32_t t = 0; t < n; ++t) {
-            uint32_t id = t, c;
-            if (listed > (uint32_t)(kMaxCand - 1)) c = __ldg(golay + (t & 4095u));
-            else { c = W.cand[t] & 0xffffffu; id = W.cand[t] >> 24 << 12 | __ldg(pos_by_low12 + (c & 0xfffu)); }
+        int8_t* const points = reinterpret_cast<int8_t*>(W.nib);                    // the costs are done with
+        double* const us = reinterpret_cast<double*>(W.pk);
+        if (lane < 24) us[lane] = u;
+        for (uint32_t t = 0; t < listed; ++t) {
+            const uint32_t k = W.cand[t];
             bool alone;
-            const int x = coset_point(u, c, (int)(id >> 12), lane, alone);
+            const int x = coset_point(u, k & 0xffffffu, (int)(k >> 24), lane, alone);
+            if (lane < 24) points[24 * t + (uint32_t)lane] = (int8_t)x;
+        }
+        __syncwarp();
+        unsigned long long best_d2 = ~0ull;                                         // the bits of numbers that are not negative are in their order
+        uint32_t best_id = 0xffffffffu, best_t = 0;
+        for (uint32_t t = (uint32_t)lane; t < listed; t += 32u) {
+            const uint32_t k = W.cand[t], id = k >> 24 << 12 | __ldg(pos_by_low12 + (k & 0xfffu));
+            double acc = 0.0;
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+                const uint32_t four = reinterpret_cast<const uint32_t*>(points)[6u * t + (uint32_t)j];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const double dd = __dsub_rn(us[4 * j + i], (double)(int8_t)(four >> (8 * i)));
+                    acc = __dadd_rn(acc, __dmul_rn(dd, dd));
+                }
+            }
+            const unsigned long long d2 = (unsigned long long)__double_as_longlong(acc);
+            if (d2 < best_d2 || (d2 == best_d2 && id < best_id)) { best_d2 = d2; best_id = id; best_t = t; }
+        }
+        const uint32_t hi = __reduce_min_sync(kFull, (uint32_t)(best_d2 >> 32));
+        const bool in_hi = (uint32_t)(best_d2 >> 32) == hi;
+        const uint32_t lo = __reduce_min_sync(kFull, in_hi ? (uint32_t)best_d2 : 0xffffffffu);
+        const bool nearest = in_hi && (uint32_t)best_d2 == lo;
+        const uint32_t first = __reduce_min_sync(kFull, nearest ? best_id : 0xffffffffu);
+        best_t = __shfl_sync(kFull, best_t, __ffs(__ballot_sync(kFull, nearest && best_id == first)) - 1);
+        best_x = lane < 24 ? (int)points[24u * best_t + (uint32_t)lane] : 0;
+    } else {                                                                        // too many near-ties to list: every coset
+        unique = false;
+        double best_d2 = 1.0e300;
+        best_x = 0;
+        for (uint32_t t = 0; t < 8192u; ++t) {                                      // in the order that decides between equal ones
+            bool alone;
+            const int x = coset_point(u, __ldg(golay + (t & 4095u)), (int)(t >> 12), lane, alone);
             const double dd = __dsub_rn(u, (double)x);
             const double d2 = seq_sum24(lane < 24 ? __dmul_rn(dd, dd) : 0.0);
-            if (d2 < best_d2 || (d2 == best_d2 && id < best_id)) { best_d2 = d2; best_id = id; best_x = x; }
+            if (d2 < best_d2) { best_d2 = d2; best_x = x; }
         }
     }
     norm2 = __reduce_add_sync(kFull, best_x * best_x);
