@@ -108,6 +108,10 @@ __device__ __forceinline__ int coset_point(double u, uint32_t c, int pi, int lan
 // first coordinate with the largest error moves.  The result does not depend on the first stage's rounding.  Returns the coordinate of
 // this lane (0 for lanes >= 24) and the squared norm of the point; unique = every other lattice point is farther from u by a margin
 // far above any binary64 rounding.
+// kTogether: the squared distances of several candidates are formed a lane each.  With 16 warps there is little to hide a chain of 24 additions per candidate
+// behind (two lanes per vector, 174 763 integer vectors EUCLIDEAN 915 -> 710 us, Gaussian ones 215 -> 213); with 24 the code costs searches that need none of
+// it more than it gains (52 000 Gaussian vectors 109.5 -> 111.5 us, 30 000 on half integers 97 -> 100).
+template <bool kTogether>
 __device__ __forceinline__ int nearest_careful_from(WarpTables& W, const GolayTrio& S, const PatternSteps& steps, const uint32_t (&row)[6],
                                                     const uint32_t* __restrict__ golay, const uint16_t* __restrict__ pos_by_low12, double u, int lane, int& norm2, bool& unique)
 {
@@ -231,7 +235,7 @@ __device__ __forceinline__ int nearest_careful_from(WarpTables& W, const GolayTr
     if (listed == 1u) {
         const uint32_t k = W.cand[0];
         best_x = coset_point(u, k & 0xffffffu, (int)(k >> 24), lane, unique);
-    } else if (listed <= (uint32_t)(kMaxCand - 1)) {
+    } else if (kTogether && listed <= (uint32_t)(kMaxCand - 1)) {
         // the candidates' points one after the other, their squared distances a lane each: 24 dependent additions for all of them together
         unique = false;
         int8_t* const points = reinterpret_cast<int8_t*>(W.nib);                    // the costs are done with
@@ -268,16 +272,21 @@ __device__ __forceinline__ int nearest_careful_from(WarpTables& W, const GolayTr
         const uint32_t first = __reduce_min_sync(kFull, nearest ? best_id : 0xffffffffu);
         best_t = __shfl_sync(kFull, best_t, __ffs(__ballot_sync(kFull, nearest && best_id == first)) - 1);
         best_x = lane < 24 ? (int)points[24u * best_t + (uint32_t)lane] : 0;
-    } else {                                                                        // too many near-ties to list: every coset
+    } else {
         unique = false;
+        const uint32_t n = listed > (uint32_t)(kMaxCand - 1) ? 8192u : listed;      // too many near-ties to list: every coset
         double best_d2 = 1.0e300;
+        uint32_t best_id = 0xffffffffu;
         best_x = 0;
-        for (uint32_t t = 0; t < 8192u; ++t) {                                      // in the order that decides between equal ones
+        for (uint32_t t = 0; t < n; ++t) {
+            uint32_t id = t, c;
+            if (listed > (uint32_t)(kMaxCand - 1)) c = __ldg(golay + (t & 4095u));
+            else { c = W.cand[t] & 0xffffffu; id = W.cand[t] >> 24 << 12 | __ldg(pos_by_low12 + (c & 0xfffu)); }
             bool alone;
-            const int x = coset_point(u, __ldg(golay + (t & 4095u)), (int)(t >> 12), lane, alone);
+            const int x = coset_point(u, c, (int)(id >> 12), lane, alone);
             const double dd = __dsub_rn(u, (double)x);
             const double d2 = seq_sum24(lane < 24 ? __dmul_rn(dd, dd) : 0.0);
-            if (d2 < best_d2) { best_d2 = d2; best_x = x; }
+            if (d2 < best_d2 || (d2 == best_d2 && id < best_id)) { best_d2 = d2; best_id = id; best_x = x; }
         }
     }
     norm2 = __reduce_add_sync(kFull, best_x * best_x);
@@ -301,7 +310,7 @@ __device__ __noinline__ int nearest_careful(WarpTables& W, const GolayTrio& S, c
 {
     uint32_t row[6];
     pattern_rows(W, S, lane, row);
-    return nearest_careful_from(W, S, steps, row, golay, pos_by_low12, u, lane, norm2, unique);
+    return nearest_careful_from<true>(W, S, steps, row, golay, pos_by_low12, u, lane, norm2, unique);
 }
 
 // ---- the search: two lanes per vector ----
@@ -390,13 +399,15 @@ __device__ __forceinline__ double dot_of_warp(double u, int xi)
 // for some 15 us.  Gaussian inputs, us for a warp per vector / two lanes by vectors per SM (of 148):
 //   EUCLIDEAN shells 2..13  260 87 / 100  330 104 / 112  384 114 / 114  450 128 / 126;  both are equal at 265 (2..3), 365 (2..5), 385 (2..8), 430 (2..20), 460 (2..24)
 //   ANGULAR   shells 2..13  100 143 / 181  136 184 / 190  150 200 / 193  200 255 / 200;  both are equal at 115 (2..3), 130 (2..5), 136 (2..8), 148 (2..20), 145 (2..24)
-// Inputs on a coarse grid, most of which have several nearest cosets, would be better off with a warp per vector (EUCLIDEAN, 174 763 vectors: integers 557 /
-// 908, halves 404 / 475, quarters 336 / 338), which the host cannot know; a block that changes over when it meets them costs all inputs 2.5 % and gains those 4 %.
+// EUCLIDEAN inputs on a coarse grid, many of which have several nearest cosets, would be better off with a warp per vector (us, a warp, before there were two forms / two lanes: 60 000
+// vectors of integers 222 / 300, halves 158 / 203, quarters 140 / 162; 174 763 vectors 532 / 670, 376 / 407, 332 / 313), which the host cannot know; a block
+// that changes over when it meets them costs all inputs 2.5 % and gains those 4 %.
 constexpr uint64_t kPairsFromEuclidean = 384, kPairsFromAngular = 136;
 // No more vectors than this left in a CTA: all of them go to nearest_careful.  The two metrics' largest cases, us: never (0) 817 / 869, 16 690 / 745, 40 670 / 721,
 // 80 656 / 712.
 constexpr int kFew = 40;
-constexpr uint32_t kPendingMost = 48, kPendingEnough = 14;
+// The longest list: as many as shared memory has room for.  174 763 integer vectors 710 us with 48, 670 with 96; Gaussian ones 213 with either.
+constexpr uint32_t kPendingMost = 96, kPendingEnough = 14;
 // A vector of a CTA that waits for nearest_careful, and the answer.
 struct Pending {
     double rn, radius, dot;
@@ -893,7 +904,7 @@ encode_search_kernel(const uint32_t* __restrict__ golay, EncTables et, const __g
         } else {
             int8_t* const point = reinterpret_cast<int8_t*>(&careful + 1);
             const double u = lane < 24 ? __dmul_rn(__dmul_rn((double)mine_v[lane], rn), rad) : 0.0;
-            const int xi = nearest_careful_from(careful, S, steps, row, golay, et.pos_by_low12, u, lane, r.norm2, r.unique);
+            const int xi = nearest_careful_from<false>(careful, S, steps, row, golay, et.pos_by_low12, u, lane, r.norm2, r.unique);
             r.dot = direct ? 0.0 : dot_of_warp(u, xi);           // (not looked at where the input itself was decoded)
             if (lane < 24) point[lane] = (int8_t)xi;
             __syncwarp();

@@ -95,3 +95,12 @@ def test_angular_search_at_extreme_lengths_with_two_lanes_per_vector(oracle_mod,
     want, _ = o.encode(v.astype(np.float64), oracle_mod.ANGULAR, threads=16)
     pts, _, which = _pair_form((2, 12), scaled, "ANGULAR")
     assert np.array_equal(pts, want[which])
+
+
+def test_more_vectors_wait_than_a_block_lists(oracle_mod):
+    # of integers every other vector has several nearest cosets (some 140 of the 256 that a thread block has at a time, up to 32 each), midpoints have up to 48
+    o = oracle_mod.Code(2, 13)
+    distinct = np.concatenate([np.round(np.random.default_rng(12).standard_normal((600, 24)) * 2.5), _edge_inputs(o, "midpoints", 157)]).astype(np.float32)
+    want, index = o.encode(distinct.astype(np.float64), oracle_mod.EUCLIDEAN, threads=16)
+    pts, idx, which = _pair_form((2, 13), distinct, "EUCLIDEAN", seed=4)
+    assert np.array_equal(pts, want[which]) and np.array_equal(idx, np.array(index, dtype=np.uint64)[which])
